@@ -739,10 +739,12 @@ inline void tc_destroy(TcState& tc) {
     tc.best = nullptr; tc.done = nullptr; tc.lse_part = nullptr; tc.ready = false;
 }
 
-inline bool tc_usable(const TcState& tc, int rows, int K, int n, bool force) {
-    if (!tc.ready) return false;
-    if (rows < TC_BM || K < TC_BK || K % 8 != 0 || n < 1 || n > 256) return false;
-    return force || n >= 16;
+inline bool tc_usable(const TcState& tc, int rows, int K, int n) {
+    return tc.ready && rows >= TC_BM && K >= TC_BK && K % 8 == 0 && n >= 1 && n <= 256;
+}
+inline bool tc_resident(const TcState& tc, const __nv_bfloat16* W) {        // a model weight, converted at init
+    auto it = tc.weights.find(W);
+    return it != tc.weights.end() && it->second.resident;
 }
 
 // 2-d tensor map [outer][inner] of 2-byte floats with a [box_outer][64] box and 128-byte swizzle

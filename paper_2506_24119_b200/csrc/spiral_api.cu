@@ -66,7 +66,11 @@ namespace {
 inline size_t meta_args_offset(int max_batch) { return (((size_t)5 * max_batch + 2) * sizeof(int32_t) + 7) & ~(size_t)7; }
 constexpr int META_RING = 16;
 constexpr int MAX_PIECES = 4;
-constexpr int TC_MIN_BATCH = 16;    // below this the batch is no dense contraction: CUDA-core GEMV
+// Batches below this use the CUDA-core GEMV for weights the context does not own (spiral_linear on a matrix of the
+// caller's): converting the matrix for one such call costs more than the call.  The model's own weights have their
+// fp16 copies from init and go through the tensor-core kernel at every batch size: it streams them at the memory's
+// pace whatever the batch (N is padded to 16), the GEMV at 2.7 TB/s with one row and less with more.
+constexpr int TC_MIN_BATCH = 16;
 
 // per-kernel timing (spiral_profile): one record = a pair of events around one launch
 struct ProfRec { int cls; cudaEvent_t e0, e1; };
@@ -353,7 +357,7 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
     int rc = tc_init(c->tc, device, max_batch);
     if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
     if (rc != SPIRAL_OK) { free_ctx(c); return rc; }
-    if (c->tc.ready && max_batch >= TC_MIN_BATCH) {
+    if (c->tc.ready) {
         struct M { const bf16* w; int rows, k; };
         std::vector<M> mats;
         for (int l = 0; l < L; ++l) {
@@ -364,7 +368,7 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
         }
         mats.push_back({c->lm_head, d->vocab, d->d_model});
         for (const M& m : mats) {
-            if (!tc_usable(c->tc, m.rows, m.k, max_batch, false)) continue;
+            if (!tc_usable(c->tc, m.rows, m.k, max_batch)) continue;
             rc = tc_register_weight(c->tc, m.w, m.rows, m.k, true, 0, &c->launches, nullptr);
             if (rc == SPIRAL_OK && m.w != c->lm_head) {
                 int np = tc_max_pieces(c->tc, m.rows, m.k);
@@ -386,7 +390,7 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
         // dense append path: needs every layer matrix on the tensor-core path
         c->pf_ready = true;
         for (const M& m : mats)
-            if (m.w != c->lm_head && !tc_usable(c->tc, m.rows, m.k, max_batch, false)) c->pf_ready = false;
+            if (m.w != c->lm_head && !tc_usable(c->tc, m.rows, m.k, max_batch)) c->pf_ready = false;
         if (c->pf_ready) {
             rc = pf_gemm_setup();
             e = cudaSuccess;
@@ -670,7 +674,8 @@ static int launch_linear(spiral_ctx* c, int cls, const bf16* W, int rows, int K,
 static int launch_linear_impl(spiral_ctx* c, const bf16* W, int rows, int K, const __half* X, int n, float* y_direct,
                               int path, Pieces* out, cudaStream_t st) {
     float* y = y_direct ? y_direct : c->pieces;
-    if (path != 1 && !y_direct && tc_usable(c->tc, rows, K, n, path == 2)) {
+    if (path != 1 && !y_direct && tc_usable(c->tc, rows, K, n) &&
+        (path == 2 || n >= TC_MIN_BATCH || tc_resident(c->tc, W))) {
         int rc = tc_linear(c->tc, W, rows, K, X, n, c->pieces, c->pieces_elems, out, c->status, st, &c->launches);
         if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
         if (rc != SPIRAL_ERR_UNSUPPORTED || path == 2) return rc;
@@ -772,7 +777,7 @@ static int run_layers(spiral_ctx* c, spiral_kv* kv, int n, cudaStream_t st) {
 // LM head (+ sampling, + logits for the caller) for the n rows of ctx->h, as the step's StepArgs say.
 static int run_head_impl(spiral_ctx* c, int n, cudaStream_t st) {
     const spiral_model_desc& d = c->d;
-    if (tc_usable(c->tc, d.vocab, d.d_model, n, false)) {
+    if (tc_usable(c->tc, d.vocab, d.d_model, n)) {
         int rc = tc_lm_head(c->tc, c->lm_head, d.vocab, d.d_model, c->h, n, meta_args(c), c->status, st, &c->launches);
         if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
         if (rc != SPIRAL_ERR_UNSUPPORTED) return rc;
@@ -1624,7 +1629,7 @@ extern "C" int spiral_selftest_wait_timeout(spiral_ctx* ctx, spiral_kv* kv, int 
     const spiral_model_desc& d = ctx->d;
     const int qd = d.n_q_heads * d.head_dim;
     const int n = std::min(ctx->max_batch, 16);
-    if (which == 0 && !tc_usable(ctx->tc, d.d_model, qd, n, true)) return SPIRAL_ERR_UNSUPPORTED;
+    if (which == 0 && !tc_usable(ctx->tc, d.d_model, qd, n)) return SPIRAL_ERR_UNSUPPORTED;
     if (which == 1 && kv->seq_len[0] < 1) return SPIRAL_ERR_INVALID;
     CU_TRY(cudaStreamSynchronize(st));
     const unsigned long long short_ns = 1000000ull, normal_ns = TMA_WAIT_NS;
