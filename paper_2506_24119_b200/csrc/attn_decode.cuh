@@ -14,9 +14,19 @@
 // part of (q * scale) in the cache's 2-byte type, rows 8..15 the low part, so one MMA yields the
 // product with a query mantissa twice as long (row g + row g+8); the softmax weights in P.V are
 // split the same way.  Online softmax runs in the exp2 domain with fp32 running max / sum.
-// A range that covers only part of a (game, head) item publishes a partial (m, l, o); the range
-// that publishes last folds the item's partials in range order (so the result does not depend on
-// which one that is) and emits the normalised output.
+//
+// How the ranges lie and how items that several warps share are put together:
+//   spread  every item of the step fits whole ranges (all games hold the same number of pages, and a multiple of it is
+//           within a quarter of the even cut): range r belongs to warp r / grid of CTA r % grid, no item is shared.
+//   block   everything else.  CTA c owns the units [c Rc, (c + 1) Rc) and deals them evenly to its eight warps.  A warp
+//           leaves the partial result (max, sum, output) of an item it shares with its neighbours in shared memory;
+//           after one CTA barrier the eight warps add the partials up, one query head at a time, and emit the items
+//           that lie inside the CTA.  An item that several CTAs share (at most two per CTA) costs one partial per CTA
+//           in global memory; the CTA that publishes last adds them in CTA order, so the result does not depend on
+//           which one that is.
+// With ranges dealt to single warps all over the GPU, as before, an item of a long context was shared by up to 20 warps
+// and one warp alone added their partials, a serial chain of L2 round trips: 24 us per layer for one game at 900 tokens
+// (3.7 MB), 92 us for 18 games at 1-15 K tokens (295 MB, 42 us of streaming).
 #pragma once
 #include <cuda.h>
 
@@ -30,7 +40,7 @@ namespace spiral {
 constexpr int ATTN_PAGE = 16;          // tokens per page the kernel is built for
 constexpr int ATTN_WARPS = 8;
 constexpr int ATTN_STAGES = 2;         // per-warp ring depth (a third stage only adds queueing: 8 warps x 3 x 8 KB oversubscribes the memory system)
-constexpr int ATTN_RMIN = 4;           // ranges are never cut shorter than this many pages
+constexpr int ATTN_CTA_MIN = ATTN_WARPS;   // block form: a CTA owns at least a page per warp
 constexpr int ATTN_MAX_SLOTS = 256;    // batch slots per launch
 
 struct AttnParams {
@@ -39,14 +49,14 @@ struct AttnParams {
     const int32_t* game;            // [n]
     const int32_t* ctx_len;         // [n]; tokens attended = ctx_len[i] + len_add
     const int32_t* cum;             // [n + 1] running count of (head, page) units before each slot, then
-                                    // cum[n + 1] = pages per work range (both written by the host per step)
+                                    // cum[n + 1] = pages per work range: > 0 spread form (per warp), < 0 block form
+                                    // (minus the pages per CTA); written by the host per step
     int len_add;
     int n, max_pages, n_pages, layer, n_q_heads, n_kv_heads, group;
-    int n_workers;                  // warps of the attention grid
     float scale_log2;               // log2(e) / sqrt(head_dim)
-    float* o_part;                  // [n_workers + n * n_kv_heads][group][head_dim]
-    float* m_part;                  // [n_workers + n * n_kv_heads][group]   (log2 domain)
-    float* l_part;
+    float* o_part;                  // [2 grid][group][head_dim]: partials of items shared between CTAs; CTA c keeps the
+    float* m_part;                  // [2 grid][group]  (log2 domain)   one that began before it in 2 c, the one that
+    float* l_part;                  //                                  goes on after it in 2 c + 1
     int* item_cnt;                  // [n * n_kv_heads] partials published per item; zero between launches
     __half* out_f16;                // [n][n_q_heads * head_dim] (input of the output projection) and / or
     float* out_f32;                 // the same in fp32; either may be null
@@ -55,31 +65,25 @@ struct AttnParams {
                                     // first wait has to run out and the warp has to unwind
 };
 
-// Host side of the schedule: unit prefix over the slots and the pages per work range.  The even
-// cut is ceil(U / workers); a range length up to a quarter above it is preferred when it makes fewer
-// (game, head) items straddle a range boundary, because every straddling item costs a merge of
-// partials at the end of the kernel (with equal-length games one item per range avoids them all).
-inline void attn_host_plan(const int* tokens, int n, int n_kv_heads, int n_workers, int32_t* cum_out /* n + 2 */) {
+// Host side of the schedule: unit prefix over the slots and the pages per work range (see the top of the file).
+inline void attn_host_plan(const int* tokens, int n, int n_kv_heads, int grid, int32_t* cum_out /* n + 2 */) {
     cum_out[0] = 0;
-    for (int i = 0; i < n; ++i) cum_out[i + 1] = cum_out[i] + n_kv_heads * ((tokens[i] + ATTN_PAGE - 1) / ATTN_PAGE);
-    const long long U = cum_out[n];
-    int r0 = (int)((U + n_workers - 1) / n_workers);
-    if (r0 < ATTN_RMIN) r0 = ATTN_RMIN;
-    int best_r = r0;
-    long long best_splits = -1;
-    const int r_hi = r0 + (r0 + 3) / 4;
-    for (int r = r0; r <= r_hi && best_splits != 0; ++r) {
-        long long splits = 0;
-        for (int i = 0; i < n; ++i) {
-            const int pages = (cum_out[i + 1] - cum_out[i]) / n_kv_heads;
-            for (int h = 0; h < n_kv_heads; ++h) {
-                const long long ua = cum_out[i] + (long long)h * pages;
-                splits += (ua / r) != ((ua + pages - 1) / r);
-            }
-        }
-        if (best_splits < 0 || splits < best_splits) { best_splits = splits; best_r = r; }
+    int p0 = (tokens[0] + ATTN_PAGE - 1) / ATTN_PAGE;
+    bool equal = true;
+    for (int i = 0; i < n; ++i) {
+        const int pages = (tokens[i] + ATTN_PAGE - 1) / ATTN_PAGE;
+        equal = equal && pages == p0;
+        cum_out[i + 1] = cum_out[i] + n_kv_heads * pages;
     }
-    cum_out[n + 1] = best_r;
+    const long long U = cum_out[n];
+    const int workers = grid * ATTN_WARPS;
+    const int even = (int)((U + workers - 1) / workers);
+    if (equal) {
+        const int r = (even + p0 - 1) / p0 * p0;            // whole items per range
+        if (r <= even + (even + 3) / 4) { cum_out[n + 1] = r; return; }
+    }
+    const int rc = std::max(ATTN_CTA_MIN, (int)((U + grid - 1) / grid));
+    cum_out[n + 1] = -rc;
 }
 
 #ifdef ATT_PROBE        // timing-probe builds only: eight timestamps per warp of the last attention launch (entry, schedule in
@@ -127,29 +131,33 @@ __device__ __forceinline__ void split2(float v, uint32_t& hi, uint32_t& lo) {
     }
 }
 
-// The work of one warp: work range w of the step's (game, KV head, page) units.  `bars` are this
-// warp's ATTN_STAGES "stage full" mbarriers, `ring` its stages in shared memory, `ring_it0` the
-// number of stages the warp has consumed through these barriers before (0 right after their
-// initialisation); returns the new count.  cum_sm / len_sm / game_sm: the step's schedule, tokens
-// attended and game per slot, in shared memory.
+// What a CTA's warps leave for each other in the block form.
+struct AttnShared {
+    int item[ATTN_WARPS][2];                // shared items of each warp: [0] began before its range, [1] begins in it; or -1
+    float m[ATTN_WARPS][2][8], l[ATTN_WARPS][2][8];
+    int open_item[2];                       // items this CTA shares with earlier / later CTAs, or -1
+    int last[2];                            // this CTA is the one that adds the item's partials up
+};
+
+// The work of one warp: units [u0, u1) of the step's (game, KV head, page) list.  `bars` are this warp's ATTN_STAGES
+// "stage full" mbarriers, `ring` its stages in shared memory, `part0` / `part1` its partial outputs in shared memory
+// (block form; part1 may overlap the ring: it is written once every load has been consumed).  cum_sm / len_sm / game_sm:
+// the step's schedule, tokens attended and game per slot, in shared memory.
 // `dependency_wait` is called once by every thread, at the point from which data written by the kernels ahead (block
 // table entries of new pages, queries, appended keys/values) is read; what comes before it uses the schedule only.
 template <int HD, bool F16, class WaitFn>
-__device__ __forceinline__ uint32_t attn_warp_work(const CUtensorMap* tmKV, const AttnParams& p, const int* cum_sm,
-                                                   const int* len_sm, const int* game_sm, uint64_t* bars, uint32_t ring,
-                                                   uint32_t ring_it0, volatile int* abort_flag, int w, WaitFn dependency_wait) {
+__device__ __forceinline__ void attn_warp_work(const CUtensorMap* tmKV, const AttnParams& p, const int* cum_sm,
+                                               const int* len_sm, const int* game_sm, uint64_t* bars, uint32_t ring,
+                                               float* part0, float* part1, AttnShared* shared, volatile int* abort_flag,
+                                               int u0, int u1, int warp, WaitFn dependency_wait) {
     constexpr int HALVES = HD / 64;                 // TMA boxes (64 elements wide) per stage
     constexpr int STAGE_BYTES = HALVES * 4096;      // 32 rows (16 K + 16 V) x 128 bytes per half
     constexpr int KSTEPS = HD / 16;                 // k-steps of Q.K^T
     constexpr int NT = HD / 8;                      // 8-column output tiles of P.V
     const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
     const int G = p.group, Hkv = p.n_kv_heads;
-    const int U = cum_sm[p.n];
-    const int R = cum_sm[p.n + 1];
-    const long long u0l = (long long)w * R;
-    if (u0l >= U) { dependency_wait(); return ring_it0; }
-    const int u0 = (int)u0l;
-    const int cnt = min(U, u0 + R) - u0;
+    const int cnt = u1 - u0;
+    if (cnt <= 0) { dependency_wait(); return; }
 
     // slot that holds unit u: largest s with cum[s] <= u
     auto slot_of = [&](int u) {
@@ -196,8 +204,8 @@ __device__ __forceinline__ uint32_t attn_warp_work(const CUtensorMap* tmKV, cons
     auto issue = [&](int j) {          // unit index j (relative to u0) into stage j % STAGES; all lanes call
         const int y = __shfl_sync(0xffffffffu, row_cur, j & 31);     // j lies in window `win`
         if (lane == 0) {
-            const uint32_t bar = smem_u32(&bars[(ring_it0 + (uint32_t)j) % ATTN_STAGES]);
-            const uint32_t dst = ring + (uint32_t)(((ring_it0 + (uint32_t)j) % ATTN_STAGES) * STAGE_BYTES);
+            const uint32_t bar = smem_u32(&bars[(uint32_t)j % ATTN_STAGES]);
+            const uint32_t dst = ring + (uint32_t)(((uint32_t)j % ATTN_STAGES) * STAGE_BYTES);
             mbar_expect_tx(bar, STAGE_BYTES);
             if (p.skip_first_load && j == 0) return;
 #pragma unroll
@@ -234,8 +242,8 @@ __device__ __forceinline__ uint32_t attn_warp_work(const CUtensorMap* tmKV, cons
             for (int ks = 0; ks < KSTEPS; ++ks) {
                 float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
                 if (g < G) {
-                    a = __ldcg(reinterpret_cast<const float2*>(qp + 16 * ks));      // through L2: written by other SMs,
-                    b = __ldcg(reinterpret_cast<const float2*>(qp + 16 * ks + 8));  // possibly in this same kernel
+                    a = __ldcg(reinterpret_cast<const float2*>(qp + 16 * ks));
+                    b = __ldcg(reinterpret_cast<const float2*>(qp + 16 * ks + 8));
                 }
                 uint32_t h0, l0, h1, l1, h2, l2, h3, l3;
                 split2<F16>(a.x * p.scale_log2, h0, l0);
@@ -250,9 +258,9 @@ __device__ __forceinline__ uint32_t attn_warp_work(const CUtensorMap* tmKV, cons
             for (int t = 0; t < NT; ++t) { o[t][0] = 0.f; o[t][1] = 0.f; o[t][2] = 0.f; o[t][3] = 0.f; }
             fresh = false;
         }
-        const int st = (int)((ring_it0 + (uint32_t)i) % ATTN_STAGES);
+        const int st = (int)((uint32_t)i % ATTN_STAGES);
         const uint32_t base = ring + (uint32_t)(st * STAGE_BYTES);
-        const bool landed = mbar_wait(smem_u32(&bars[st]), ((ring_it0 + (uint32_t)i) / ATTN_STAGES) & 1u, abort_flag,
+        const bool landed = mbar_wait(smem_u32(&bars[st]), ((uint32_t)i / ATTN_STAGES) & 1u, abort_flag,
                                       p.status, STATUS_TIMEOUT_TMA);
         if (!__all_sync(0xffffffffu, landed)) break;
         if (i == 0) ATT_STAMP(4);
@@ -336,11 +344,8 @@ __device__ __forceinline__ uint32_t attn_warp_work(const CUtensorMap* tmKV, cons
         if (item_end || i + 1 == cnt) {
             l += __shfl_xor_sync(0xffffffffu, l, 1);
             l += __shfl_xor_sync(0xffffffffu, l, 2);
-            // ranges that touch this item: [w0, w1]
-            const int ua = cum_sm[slot] + kvh * pages;
-            const int w0 = ua / R, w1 = (ua + pages - 1) / R;
-            const size_t item = (size_t)slot * Hkv + kvh;
-            if (w0 == w1) {
+            const int ua = cum_sm[slot] + kvh * pages;         // the item's units: ua .. ua + pages - 1
+            if (ua >= u0 && ua + pages <= u1) {
                 // the whole item was in this range: normalise and emit
                 if (g < G) {
                     const float inv = 1.f / l;
@@ -353,69 +358,15 @@ __device__ __forceinline__ uint32_t attn_warp_work(const CUtensorMap* tmKV, cons
                     }
                 }
             } else {
-                const size_t part = (size_t)w + item;
+                const int s = ua >= u0 ? 1 : 0;
+                float* op = (s ? part1 : part0) + g * HD + 2 * c;
                 if (g < G) {
-                    float* op = p.o_part + (part * G + g) * HD + 2 * c;
 #pragma unroll
                     for (int t = 0; t < NT; ++t)
                         *reinterpret_cast<float2*>(op + 8 * t) = make_float2(o[t][0] + o[t][2], o[t][1] + o[t][3]);
-                    if (c == 0) { p.m_part[part * G + g] = m; p.l_part[part * G + g] = l; }
+                    if (c == 0) { shared->m[warp][s][g] = m; shared->l[warp][s][g] = l; }
                 }
-                // publish; the range that arrives last folds the partials of the item in range order:
-                // o = sum_i 2^(m_i-M) o_i / sum_i 2^(m_i-M) l_i
-                __threadfence();
-                __syncwarp();
-                int last = 0;
-                if (lane == 0) last = atomicAdd(p.item_cnt + item, 1) == w1 - w0;
-                last = __shfl_sync(0xffffffffu, last, 0);
-                if (last) {
-                    __threadfence();
-                    // lane (partial j, head hh) fetches that partial's m and l; the weights then go
-                    // round by shuffle, so the loads of all partials are in flight together
-                    const int np = w1 - w0 + 1;
-                    for (int gg0 = 0; gg0 < G; gg0 += 4) {              // up to 8 partials x 4 heads per pass
-                        const int pj = lane >> 2, ph = gg0 + (lane & 3);
-                        float mj = -INFINITY, lj = 0.f;
-                        if (pj < np && ph < G && np <= 8) {
-                            mj = __ldcg(p.m_part + ((size_t)(w0 + pj) + item) * G + ph);
-                            lj = __ldcg(p.l_part + ((size_t)(w0 + pj) + item) * G + ph);
-                        }
-                        for (int hh = 0; hh < 4 && gg0 + hh < G; ++hh) {
-                            const int gg = gg0 + hh;
-                            float M = -INFINITY, ls = 0.f, acc[HD / 32];
-#pragma unroll
-                            for (int k = 0; k < HD / 32; ++k) acc[k] = 0.f;
-                            if (np <= 8) {
-                                for (int j = 0; j < np; ++j) M = fmaxf(M, __shfl_sync(0xffffffffu, mj, 4 * j + hh));
-                                for (int j = 0; j < np; ++j) {
-                                    const float wt = fast_exp2(__shfl_sync(0xffffffffu, mj, 4 * j + hh) - M);
-                                    ls += wt * __shfl_sync(0xffffffffu, lj, 4 * j + hh);
-                                    const float* op = p.o_part + (((size_t)(w0 + j) + item) * G + gg) * HD + lane;
-#pragma unroll
-                                    for (int k = 0; k < HD / 32; ++k) acc[k] += wt * __ldcg(op + 32 * k);
-                                }
-                            } else {
-                                for (int ww = w0; ww <= w1; ++ww) M = fmaxf(M, __ldcg(p.m_part + (ww + item) * G + gg));
-                                for (int ww = w0; ww <= w1; ++ww) {
-                                    const float wt = fast_exp2(__ldcg(p.m_part + (ww + item) * G + gg) - M);
-                                    ls += wt * __ldcg(p.l_part + (ww + item) * G + gg);
-                                    const float* op = p.o_part + ((ww + item) * G + gg) * HD + lane;
-#pragma unroll
-                                    for (int k = 0; k < HD / 32; ++k) acc[k] += wt * __ldcg(op + 32 * k);
-                                }
-                            }
-                            const float inv = 1.f / ls;
-                            const size_t ob = ((size_t)slot * p.n_q_heads + kvh * G + gg) * HD + lane;
-#pragma unroll
-                            for (int k = 0; k < HD / 32; ++k) {
-                                const float r = acc[k] * inv;
-                                if (p.out_f16) p.out_f16[ob + 32 * k] = __ushort_as_half((unsigned short)float_to_f16_bits(r));
-                                if (p.out_f32) p.out_f32[ob + 32 * k] = r;
-                            }
-                        }
-                    }
-                    if (lane == 0) p.item_cnt[item] = 0;
-                }
+                if (lane == 0) shared->item[warp][s] = slot * Hkv + kvh;
             }
             fresh = true;
         }
@@ -437,7 +388,153 @@ __device__ __forceinline__ uint32_t attn_warp_work(const CUtensorMap* tmKV, cons
                    global_ns() - t0 < g_wait_limit_ns) {}
         }
     }
-    return ring_it0 + (uint32_t)cnt;
+}
+
+// One query head of `cnt` partial results -> elements EL lane .. of the head, EL = HD / 32: o = sum_i 2^(m_i - M) o_i,
+// ls = sum_i 2^(m_i - M) l_i with M the largest m_i.  m_of / l_of / o_of: where partial i keeps its values.
+template <int HD, class MF, class LF, class OF>
+__device__ __forceinline__ void attn_fold(int cnt, MF m_of, LF l_of, OF o_of, float& M, float& ls, float (&acc)[HD / 32]) {
+    constexpr int EL = HD / 32;
+    M = -INFINITY; ls = 0.f;
+#pragma unroll
+    for (int e = 0; e < EL; ++e) acc[e] = 0.f;
+    for (int i0 = 0; i0 < cnt; i0 += 4) {               // four partials at a time: their loads are in flight together
+        float mi[4], li[4], oi[4][EL];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool in = i0 + k < cnt;
+            mi[k] = in ? m_of(i0 + k) : -INFINITY;
+            li[k] = in ? l_of(i0 + k) : 0.f;
+#pragma unroll
+            for (int e = 0; e < EL; ++e) oi[k][e] = 0.f;
+            if (in) o_of(i0 + k, oi[k]);
+        }
+        float Mn = fmaxf(fmaxf(fmaxf(mi[0], mi[1]), fmaxf(mi[2], mi[3])), M);
+        const float a = fast_exp2(M - Mn);
+        ls *= a;
+#pragma unroll
+        for (int e = 0; e < EL; ++e) acc[e] *= a;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float wt = fast_exp2(mi[k] - Mn);
+            ls += wt * li[k];
+#pragma unroll
+            for (int e = 0; e < EL; ++e) acc[e] += wt * oi[k][e];
+        }
+        M = Mn;
+    }
+}
+
+template <int HD>
+__device__ __forceinline__ void attn_emit(const AttnParams& p, int slot, int head, int lane, float ls, const float (&acc)[HD / 32]) {
+    constexpr int EL = HD / 32;
+    const float inv = 1.f / ls;
+    const size_t ob = ((size_t)slot * p.n_q_heads + head) * HD + EL * lane;
+#pragma unroll
+    for (int e = 0; e < EL; e += 2) {
+        const float r0 = acc[e] * inv, r1 = acc[e + 1] * inv;
+        if (p.out_f16) *reinterpret_cast<uint32_t*>(p.out_f16 + ob + e) = pack_f16(r0, r1);
+        if (p.out_f32) *reinterpret_cast<float2*>(p.out_f32 + ob + e) = make_float2(r0, r1);
+    }
+}
+
+// Block form, after the warps' ranges: adds up what the warps of the CTA [c0, c1) and, through global memory, the CTAs
+// left of shared items.  parts: [ATTN_WARPS][2] pointers' bases, see the kernel.  Called by every thread of the CTA.
+template <int HD, class PartFn>
+__device__ __forceinline__ void attn_join(const AttnParams& p, const int* cum_sm, const int* len_sm, AttnShared* sh, PartFn part_of,
+                                          int Rc, int c0, int c1) {
+    constexpr int EL = HD / 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int G = p.group, Hkv = p.n_kv_heads;
+    auto span = [&](int item, int& slot, int& kvh, int& ua) -> int {        // pages of the item; its first unit
+        slot = item / Hkv;
+        kvh = item - slot * Hkv;
+        const int pages = (len_sm[slot] + ATTN_PAGE - 1) / ATTN_PAGE;
+        ua = cum_sm[slot] + kvh * pages;
+        return pages;
+    };
+    __syncthreads();
+    // groups: 0 = the item that began before the CTA (warps 0, 1, ... [0]); 1 + w = the shared item that begins in warp w
+    for (int t = warp; t < (ATTN_WARPS + 1) * G; t += ATTN_WARPS) {
+        const int grp = t / G, g = t - grp * G;
+        int first = grp ? grp - 1 : 0, fs = grp ? 1 : 0;
+        if (grp == 0) while (first < ATTN_WARPS && sh->item[first][0] < 0 && sh->item[first][1] < 0) ++first;   // warps without work
+        if (first >= ATTN_WARPS) continue;
+        const int item = sh->item[first][fs];
+        if (item < 0) continue;
+        int slot, kvh, ua;
+        const int pages = span(item, slot, kvh, ua);
+        if (grp == 0 && ua >= c0) continue;                 // (cannot happen: the first warp's range starts at c0)
+        unsigned idx = (unsigned)(first * 2 + fs);          // the partials, one hex digit each, in k order
+        int cnt = 1;
+        unsigned long long list = idx;
+        for (int w = first + 1; w < ATTN_WARPS; ++w)
+            if (sh->item[w][0] == item) { list |= (unsigned long long)(unsigned)(w * 2) << (4 * cnt); ++cnt; }
+        auto at = [&](int i) { return (int)((list >> (4 * i)) & 15u); };
+        float M, ls, acc[EL];
+        attn_fold<HD>(cnt, [&](int i) { return sh->m[at(i) >> 1][at(i) & 1][g]; }, [&](int i) { return sh->l[at(i) >> 1][at(i) & 1][g]; },
+                      [&](int i, float (&o)[EL]) {
+                          const float* src = part_of(at(i) >> 1, at(i) & 1) + g * HD + EL * lane;
+#pragma unroll
+                          for (int e = 0; e < EL; e += 2) {
+                              const float2 v = *reinterpret_cast<const float2*>(src + e);
+                              o[e] = v.x; o[e + 1] = v.y;
+                          }
+                      }, M, ls, acc);
+        if (ua >= c0 && ua + pages <= c1) {
+            attn_emit<HD>(p, slot, kvh * G + g, lane, ls, acc);
+        } else {
+            const int side = ua >= c0 ? 1 : 0;
+            const size_t part = (size_t)(2 * blockIdx.x + side) * G + g;
+#pragma unroll
+            for (int e = 0; e < EL; e += 2) *reinterpret_cast<float2*>(p.o_part + part * HD + EL * lane + e) = make_float2(acc[e], acc[e + 1]);
+            if (lane == 0) {
+                p.m_part[part] = M; p.l_part[part] = ls;
+                sh->open_item[side] = item;                 // (every head of the item writes the same)
+            }
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        const int item = sh->open_item[threadIdx.x];
+        int last = 0;
+        if (item >= 0) {
+            int slot, kvh, ua;
+            const int pages = span(item, slot, kvh, ua);
+            const int n_cta = (ua + pages - 1) / Rc - ua / Rc + 1;
+            last = atomicAdd(p.item_cnt + item, 1) == n_cta - 1;
+            if (last) p.item_cnt[item] = 0;
+        }
+        sh->last[threadIdx.x] = last;
+    }
+    __syncthreads();
+    for (int t = warp; t < 2 * G; t += ATTN_WARPS) {
+        const int side = t / G, g = t - side * G;
+        if (!sh->last[side]) continue;
+        __threadfence();
+        int slot, kvh, ua;
+        const int item = sh->open_item[side];
+        const int pages = span(item, slot, kvh, ua);
+        const int ca = ua / Rc, cnt = (ua + pages - 1) / Rc - ca + 1;
+        auto at = [&](int i) { return (size_t)(2 * (ca + i) + (i ? 0 : 1)) * G + g; };      // (the first CTA keeps it as "goes on")
+        float M, ls, acc[EL];
+        attn_fold<HD>(cnt, [&](int i) { return __ldcg(p.m_part + at(i)); }, [&](int i) { return __ldcg(p.l_part + at(i)); },
+                      [&](int i, float (&o)[EL]) {
+                          const float* src = p.o_part + at(i) * HD + EL * lane;
+#pragma unroll
+                          for (int e = 0; e < EL; e += 2) {
+                              const float2 v = __ldcg(reinterpret_cast<const float2*>(src + e));
+                              o[e] = v.x; o[e + 1] = v.y;
+                          }
+                      }, M, ls, acc);
+        attn_emit<HD>(p, slot, kvh * G + g, lane, ls, acc);
+    }
+}
+
+// Shared memory: the warps' rings, then their [0] partial outputs (the [1] partials reuse the ring of their warp)
+inline size_t attn_smem_bytes(int head_dim, int group) {
+    return (size_t)ATTN_WARPS * ATTN_STAGES * (head_dim / 64) * 4096 + (size_t)ATTN_WARPS * group * head_dim * sizeof(float) + 1024;
 }
 
 template <int HD, bool F16>
@@ -451,6 +548,7 @@ __global__ void __launch_bounds__(ATTN_WARPS * 32, 1) attn_decode_kernel(const _
     __shared__ int len_sm[ATTN_MAX_SLOTS];
     __shared__ int game_sm[ATTN_MAX_SLOTS];
     __shared__ int abort_sm;
+    __shared__ AttnShared join_sm;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     TRACE_BEGIN(7);
@@ -463,6 +561,10 @@ __global__ void __launch_bounds__(ATTN_WARPS * 32, 1) attn_decode_kernel(const _
     if (threadIdx.x == 0) {
         abort_sm = 0;
         tmap_prefetch(&tmKV);
+    }
+    if (lane < 2) {
+        join_sm.item[warp][lane] = -1;
+        if (warp == 0) join_sm.open_item[lane] = -1;
     }
     // The schedule (range starts, lengths, games) is what the host uploaded before the first kernel of the step: a
     // copy, not a kernel, so it is complete before any kernel of the step starts and can be staged while the kernel
@@ -477,13 +579,33 @@ __global__ void __launch_bounds__(ATTN_WARPS * 32, 1) attn_decode_kernel(const _
 #ifdef ATT_PROBE
     if (lane == 0) { g_att_probe[(size_t)(warp * gridDim.x + blockIdx.x) * 8 + 0] = t_entry__; g_att_probe[(size_t)(warp * gridDim.x + blockIdx.x) * 8 + 1] = global_ns(); }
 #endif
-    const int w = warp * gridDim.x + blockIdx.x;       // consecutive ranges on different SMs: when fewer
-                                                       // ranges than warps have work, every SM still streams
-    const uint32_t ring = ((smem_u32(attn_smem_raw) + 1023u) & ~1023u) + (uint32_t)(warp * ATTN_STAGES * STAGE_BYTES);
-    attn_warp_work<HD, F16>(&tmKV, p, cum_sm, len_sm, game_sm, full_bar[warp], ring, 0u, &abort_sm, w, [&]() {
+    uint8_t* const smem0 = attn_smem_raw + ((1024u - (smem_u32(attn_smem_raw) & 1023u)) & 1023u);
+    uint8_t* const ring_p = smem0 + warp * ATTN_STAGES * STAGE_BYTES;
+    float* const part0 = reinterpret_cast<float*>(smem0 + ATTN_WARPS * ATTN_STAGES * STAGE_BYTES) + warp * p.group * HD;
+    const int U = cum_sm[p.n], R = cum_sm[p.n + 1];
+    const bool block = R < 0;
+    int u0, u1, c0 = 0, c1 = 0;
+    if (block) {
+        c0 = min(U, (int)blockIdx.x * -R);
+        c1 = min(U, c0 - R);
+        u0 = c0 + (c1 - c0) * warp / ATTN_WARPS;
+        u1 = c0 + (c1 - c0) * (warp + 1) / ATTN_WARPS;
+    } else {
+        // consecutive ranges on different SMs: when fewer ranges than warps have work, every SM still streams
+        const long long a = (long long)(warp * gridDim.x + blockIdx.x) * R;
+        u0 = (int)min((long long)U, a);
+        u1 = (int)min((long long)U, a + R);
+    }
+    attn_warp_work<HD, F16>(&tmKV, p, cum_sm, len_sm, game_sm, full_bar[warp], smem_u32(ring_p), part0,
+                            reinterpret_cast<float*>(ring_p), &join_sm, &abort_sm, u0, u1, warp, [&]() {
         grid_dependency_wait();
         TRACE_WAITED();
     });
+    if (block && c0 < c1)
+        attn_join<HD>(p, cum_sm, len_sm, &join_sm, [&](int w, int s) {
+            return s ? reinterpret_cast<const float*>(smem0 + w * ATTN_STAGES * STAGE_BYTES)
+                     : reinterpret_cast<const float*>(smem0 + ATTN_WARPS * ATTN_STAGES * STAGE_BYTES) + w * p.group * HD;
+        }, -R, c0, c1);
 }
 
 }  // namespace spiral

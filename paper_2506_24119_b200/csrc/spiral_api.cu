@@ -290,7 +290,7 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
         CU_TRY(cudaGetDeviceProperties(&prop, device));
         c->n_sm = prop.multiProcessorCount;
     }
-    const size_t parts = ((size_t)c->n_sm * ATTN_WARPS + MB * d->n_kv_heads) * c->group;
+    const size_t parts = (size_t)2 * c->n_sm * c->group;
     const int half = d->head_dim / 2;
     cudaError_t e = cudaSuccess;
     auto A = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
@@ -338,7 +338,7 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
         return SPIRAL_ERR_CUDA;
     }
     {
-        const int attn_smem = ATTN_WARPS * ATTN_STAGES * 2 * 4096 + 1024;
+        const int attn_smem = (int)attn_smem_bytes(128, 8);
         e = cudaFuncSetAttribute(attn_decode_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(attn_decode_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_smem);
@@ -696,13 +696,12 @@ static int launch_attention(spiral_ctx* c, spiral_kv* kv, int layer, int n, cons
     p.q = q; p.block_table = kv->table_dev; p.game = game_dev; p.ctx_len = len_dev; p.cum = meta_cum_dev(c);
     p.len_add = len_add; p.n = n; p.max_pages = kv->max_pages; p.n_pages = kv->n_pages; p.layer = layer;
     p.n_q_heads = d.n_q_heads; p.n_kv_heads = d.n_kv_heads; p.group = c->group;
-    p.n_workers = c->n_sm * ATTN_WARPS;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)d.head_dim));
     p.o_part = c->o_part; p.m_part = c->m_part; p.l_part = c->l_part; p.status = c->status;
     p.item_cnt = c->attn_item_cnt; p.out_f16 = out_f16; p.out_f32 = out_f32;
     p.skip_first_load = c->attn_skip_once ? 1 : 0;
     c->attn_skip_once = false;
-    const size_t smem = (size_t)ATTN_WARPS * ATTN_STAGES * (d.head_dim / 64) * 4096 + 1024;
+    const size_t smem = attn_smem_bytes(d.head_dim, c->group);
     int rec = prof_begin(c, SPIRAL_KC_ATTN, st);
     auto attn = d.head_dim == 128 ? (kv->kv_f16 ? attn_decode_kernel<128, true> : attn_decode_kernel<128, false>)
                                   : (kv->kv_f16 ? attn_decode_kernel<64, true> : attn_decode_kernel<64, false>);
@@ -922,7 +921,7 @@ static int decode_step_impl(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t
         kv->seq_len[g] = len + 1;
         attended[i] = len + 1;
     }
-    attn_host_plan(attended, n, ctx->d.n_kv_heads, ctx->n_sm * ATTN_WARPS, meta_cum_host(ctx, mh));
+    attn_host_plan(attended, n, ctx->d.n_kv_heads, ctx->n_sm, meta_cum_host(ctx, mh));
     sa->tokens = tok_in; sa->gumbel = gumbel; sa->tok_out = tok_out; sa->logits = logits_dbg;
     sa->temperature = temperature; sa->logprob = logprob;
     if (nucleus) { sa->logits = ctx->logits; sa->defer_sampling = 1; sa->top_p = top_p; }
@@ -1310,7 +1309,7 @@ extern "C" int spiral_prefill(spiral_ctx* ctx, spiral_kv* kv, int n, const int32
             ++nt;
             if (++gt == cnt) { gt = 0; ++gi; }
         }
-        attn_host_plan(attended, nt, d.n_kv_heads, ctx->n_sm * ATTN_WARPS, meta_cum_host(ctx, mh));
+        attn_host_plan(attended, nt, d.n_kv_heads, ctx->n_sm, meta_cum_host(ctx, mh));
         sa->tokens = tokens_dev;
         sa->logits = (last_logits && any_last) ? ctx->logits : nullptr;     // no sampling: logits only
         rc = meta_upload(ctx, slot, st);
@@ -1376,7 +1375,7 @@ extern "C" int spiral_attention(spiral_ctx* ctx, spiral_kv* kv, int layer, int n
     if (slot < 0) return slot;
     const int MB = ctx->max_batch;
     for (int i = 0; i < n; ++i) { mh[i] = ids[i]; mh[MB + i] = ctx_len[i]; mh[2 * MB + i] = -1; mh[3 * MB + i] = -1; }
-    attn_host_plan(ctx_len, n, ctx->d.n_kv_heads, ctx->n_sm * ATTN_WARPS, meta_cum_host(ctx, mh));
+    attn_host_plan(ctx_len, n, ctx->d.n_kv_heads, ctx->n_sm, meta_cum_host(ctx, mh));
     rc = meta_upload(ctx, slot, st);
     if (rc) return rc;
     return launch_attention(ctx, kv, layer, n, meta_i32(ctx), meta_i32(ctx) + MB, 0, q_dev, nullptr, out_dev, st);
@@ -1397,8 +1396,7 @@ namespace {
 constexpr int NA_MAX_SEQS = SPIRAL_STATIC_ATTN_MAX_SEQS;          // sequences per call
 constexpr int NA_MAX_ITEMS = SPIRAL_STATIC_ATTN_MAX_ITEMS;        // sequences x KV heads per call
 constexpr int NA_MAX_CTAS = 64;                                    // grid of the attention kernel here
-constexpr int NA_WORKERS = NA_MAX_CTAS * ATTN_WARPS;
-constexpr int NA_PARTS = NA_WORKERS + NA_MAX_ITEMS;                // partial slots, each <= 8 heads x 128 floats
+constexpr int NA_PARTS = 2 * NA_MAX_CTAS;                          // partial slots, each <= 8 heads x 128 floats
 struct NoAllocScratch {
     float o_part[(size_t)NA_PARTS * 8 * 128];
     float m_part[(size_t)NA_PARTS * 8];
@@ -1440,7 +1438,7 @@ int noalloc_setup(int device) {
     CU_TRY(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device));
     if (major != 10) return SPIRAL_ERR_UNSUPPORTED;
     CU_TRY(cudaDeviceGetAttribute(&nd.n_sm, cudaDevAttrMultiProcessorCount, device));
-    const int attn_smem = ATTN_WARPS * ATTN_STAGES * 2 * 4096 + 1024;
+    const int attn_smem = (int)attn_smem_bytes(128, 8);
     CU_TRY(cudaFuncSetAttribute(attn_decode_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_smem));
     CU_TRY(cudaFuncSetAttribute(attn_decode_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_smem));
     CU_TRY(cudaFuncSetAttribute(attn_decode_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_smem));
@@ -1496,7 +1494,7 @@ extern "C" int spiral_attention_static(int device, const void* pool_dev, int n_p
     const int grid = std::min(nd.n_sm, NA_MAX_CTAS);
     int32_t game_h[NA_MAX_SEQS], cum_h[NA_MAX_SEQS + 2];
     for (int i = 0; i < n; ++i) game_h[i] = i;
-    attn_host_plan(ctx_len_host, n, n_kv_heads, grid * ATTN_WARPS, cum_h);
+    attn_host_plan(ctx_len_host, n, n_kv_heads, grid, cum_h);
     CU_TRY(cudaMemcpyAsync(sc->game, game_h, (size_t)n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     CU_TRY(cudaMemcpyAsync(sc->len, ctx_len_host, (size_t)n * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     CU_TRY(cudaMemcpyAsync(sc->cum, cum_h, (size_t)(n + 2) * sizeof(int32_t), cudaMemcpyHostToDevice, st));
@@ -1508,11 +1506,10 @@ extern "C" int spiral_attention_static(int device, const void* pool_dev, int n_p
     p.q = q_dev; p.block_table = block_table_dev; p.game = sc->game; p.ctx_len = sc->len; p.cum = sc->cum;
     p.len_add = 0; p.n = n; p.max_pages = max_pages; p.n_pages = n_pages; p.layer = layer;
     p.n_q_heads = n_q_heads; p.n_kv_heads = n_kv_heads; p.group = n_q_heads / n_kv_heads;
-    p.n_workers = grid * ATTN_WARPS;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)head_dim));
     p.o_part = sc->o_part; p.m_part = sc->m_part; p.l_part = sc->l_part; p.item_cnt = sc->item_cnt;
     p.out_f16 = nullptr; p.out_f32 = out_dev; p.status = &sc->status; p.skip_first_load = 0;
-    const size_t smem = (size_t)ATTN_WARPS * ATTN_STAGES * (head_dim / 64) * 4096 + 1024;
+    const size_t smem = attn_smem_bytes(head_dim, p.group);
     const bool f16 = kv_dtype == SPIRAL_KV_F16;
     auto attn = head_dim == 128 ? (f16 ? attn_decode_kernel<128, true> : attn_decode_kernel<128, false>)
                                 : (f16 ? attn_decode_kernel<64, true> : attn_decode_kernel<64, false>);
@@ -1652,7 +1649,7 @@ extern "C" int spiral_selftest_wait_timeout(spiral_ctx* ctx, spiral_kv* kv, int 
             const int MB = ctx->max_batch;
             const int len = kv->seq_len[0];
             mh[0] = 0; mh[MB] = len; mh[2 * MB] = -1; mh[3 * MB] = -1;
-            attn_host_plan(&len, 1, d.n_kv_heads, ctx->n_sm * ATTN_WARPS, meta_cum_host(ctx, mh));
+            attn_host_plan(&len, 1, d.n_kv_heads, ctx->n_sm, meta_cum_host(ctx, mh));
             rc = meta_upload(ctx, slot, st);
         }
         if (rc == SPIRAL_OK) {
