@@ -122,7 +122,7 @@ struct spiral_ctx {
     cudaEvent_t meta_ev[META_RING];
     bool meta_ev_used[META_RING];
     int meta_next = 0;
-    cudaStream_t copy_stream = nullptr;    // *_host entry point: carries the noise while the layers run
+    cudaStream_t copy_stream = nullptr;    // *_host entry point: carries the noise while the layers run; records step graphs
     cudaEvent_t copy_ev = nullptr;
     int32_t* tok_stage = nullptr;      // device staging of the *_host entry point
     float* gumbel_stage = nullptr;
@@ -810,10 +810,12 @@ static int run_step_body(spiral_ctx* c, spiral_kv* kv, int n, int variant, cudaS
 
 // One decode step for n slots whose metadata and StepArgs are already on their way to the device.
 // The launch sequence depends on n only, so from its second use on a batch size is replayed from a
-// CUDA graph recorded on the caller's stream (not on the legacy default stream, which cannot be
-// captured; not while per-kernel timing is on; not inside a capture the caller has begun).
+// CUDA graph.  It is recorded on a stream of the context's own, so that callers on the legacy default stream, which
+// cannot be captured, have it too (launching a recorded graph there is allowed): with plain launches the host needs
+// longer than the GPU for a step of the two-layer decoder.  Not while per-kernel timing is on, not inside a capture
+// the caller has begun.
 static int run_step(spiral_ctx* c, spiral_kv* kv, int n, int variant, cudaStream_t st) {
-    bool graph_ok = c->use_graph && c->prof_mask == 0 && st != nullptr && st != cudaStreamLegacy;
+    bool graph_ok = c->use_graph && c->prof_mask == 0;
     if (graph_ok) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
@@ -831,10 +833,11 @@ static int run_step(spiral_ctx* c, spiral_kv* kv, int n, int variant, cudaStream
         if (!g.failed && ++g.uses >= 2) {
             // record: the first (eager) use has created every plan and tensor map this size needs
             const int64_t l0 = c->launches;
-            CU_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            int rc = run_step_body(c, kv, n, variant, st);
+            cudaStream_t rec = c->copy_stream;
+            CU_TRY(cudaStreamBeginCapture(rec, cudaStreamCaptureModeThreadLocal));
+            int rc = run_step_body(c, kv, n, variant, rec);
             cudaGraph_t graph = nullptr;
-            cudaError_t e = cudaStreamEndCapture(st, &graph);
+            cudaError_t e = cudaStreamEndCapture(rec, &graph);
             c->launches = l0;
             if (rc == SPIRAL_OK && e == cudaSuccess && graph) {
                 e = cudaGraphInstantiate(&g.exec, graph, 0);
