@@ -947,7 +947,7 @@ inline int tc_linear(TcState& tc, const __nv_bfloat16* W, int rows, int K, const
     TC_TRY(launch_kernel(true, tc_gemm_kernel<0>, dim3(pl->grid), dim3(tc_threads(0)), smem, st, w->map, *xm, *om, p));
     if (launches) ++*launches;
     out->base = pieces; out->stride = p.piece_stride; out->ld = rows; out->n_pieces = pl->max_pieces;
-    out->sk_KB = p.KB; out->sk_G = pl->grid;
+    out->sk_KB = p.KB; out->sk_G = pl->grid; out->sk_shift = 7; out->sk_tt = 1; out->sk_BN = N;
     return SPIRAL_OK;
 }
 

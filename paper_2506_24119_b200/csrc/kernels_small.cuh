@@ -24,29 +24,38 @@ struct Pieces {
     int ld;             // features per batch row
     int n_pieces;
     int sk_KB, sk_G;    // k blocks per tile and grid of the stream-K GEMM (sk_G == 0: not stream-K)
+    int sk_shift;       // log2 of the features per tile (7 or 8)
+    int sk_tt, sk_BN;   // tiles along the batch rows (fastest in the tile order) and batch rows per tile
 };
 
-__device__ __forceinline__ int piece_count(const Pieces& P, int r) {
+// tile that holds feature r of batch row b; pieces of a tile
+__device__ __forceinline__ int piece_tile(const Pieces& P, int b, int r) {
+    return P.sk_tt == 1 ? r >> P.sk_shift : (r >> P.sk_shift) * P.sk_tt + b / P.sk_BN;
+}
+__device__ __forceinline__ int piece_tiles(const Pieces& P) { return ((P.ld + (1 << P.sk_shift) - 1) >> P.sk_shift) * P.sk_tt; }
+__device__ __forceinline__ int piece_count_tile(const Pieces& P, int tile) {
     if (P.sk_G == 0) return P.n_pieces;
-    const long long U = (long long)((P.ld + 127) >> 7) * P.sk_KB;
-    const long long first = (long long)(r >> 7) * P.sk_KB;
+    const long long U = (long long)piece_tiles(P) * P.sk_KB;
+    const long long first = (long long)tile * P.sk_KB;
     return streamk_cta_of(first + P.sk_KB - 1, P.sk_G, U) - streamk_cta_of(first, P.sk_G, U) + 1;
 }
+__device__ __forceinline__ int piece_count(const Pieces& P, int b, int r) { return piece_count_tile(P, piece_tile(P, b, r)); }
 
-// The kernels that consume pieces look the count of each 128-feature tile up in a shared-memory
+// The kernels that consume pieces look the count of each tile up in a shared-memory
 // table filled once per CTA (the divisions above are too slow to repeat per element).
 constexpr int PIECE_TABLE = 512;        // tiles covered by the table; beyond it the count is recomputed
 struct PieceCounts {
     const unsigned char* tab;
-    __device__ __forceinline__ int of(const Pieces& P, int r) const {
-        const int t = r >> 7;
-        return t < PIECE_TABLE ? (int)tab[t] : piece_count(P, r);
+    __device__ __forceinline__ int of(const Pieces& P, int b, int r) const {
+        if (P.sk_G == 0) return P.n_pieces;
+        const int t = piece_tile(P, b, r);
+        return t < PIECE_TABLE ? (int)tab[t] : piece_count_tile(P, t);
     }
 };
 // fills `tab` (PIECE_TABLE bytes of shared memory) and synchronises the CTA
 __device__ __forceinline__ PieceCounts piece_counts_init(const Pieces& P, unsigned char* tab) {
-    const int tiles = min(PIECE_TABLE, (P.ld + 127) >> 7);
-    for (int t = threadIdx.x; t < tiles; t += blockDim.x) tab[t] = (unsigned char)piece_count(P, t << 7);
+    const int tiles = P.sk_G == 0 ? 0 : min(PIECE_TABLE, piece_tiles(P));
+    for (int t = threadIdx.x; t < tiles; t += blockDim.x) tab[t] = (unsigned char)piece_count_tile(P, t);
     __syncthreads();
     return PieceCounts{tab};
 }
@@ -165,7 +174,7 @@ __global__ void __launch_bounds__(RMS_THREADS) rmsnorm_kernel(float* __restrict_
         if (c < nc) {
             v[k] = reinterpret_cast<float4*>(xr)[c];
             if (has_pieces) {
-                float4 p = piece_sum4(pieces, pcnt.of(pieces, 4 * c), b, 4 * c);
+                float4 p = piece_sum4(pieces, pcnt.of(pieces, b, 4 * c), b, 4 * c);
                 v[k].x += p.x; v[k].y += p.y; v[k].z += p.z; v[k].w += p.w;
                 reinterpret_cast<float4*>(xr)[c] = v[k];
             }
@@ -266,7 +275,7 @@ __device__ __forceinline__ void qkv_post_task(const Pieces& pieces, const PieceC
                                               int n_kv_heads, float* q_out, uint16_t* pool, int kv_f16, int* status) {
     constexpr int HD = 32 * EPL, HALF = HD / 2;
     const int pos = meta.pos[slot];
-    const int cnt = pcnt.of(pieces, head * HD);            // head_dim <= 128: a head lies in one 128-row tile
+    const int cnt = pcnt.of(pieces, slot, head * HD);            // head_dim <= 128: a head lies in one 128-row tile
     const int i0 = EPL * l16;                              // this lane's elements i0 .. i0 + EPL - 1 and + HALF
     const bool is_q = head < n_q_heads;
     const bool is_k = !is_q && head < n_q_heads + n_kv_heads;
@@ -387,7 +396,7 @@ __global__ void __launch_bounds__(SILU_THREADS) silu_mul_kernel(Pieces pieces, i
         const int idx = base0 + u * stride;
         row[u] = idx / per_row;
         col[u] = idx - row[u] * per_row;
-        cnt[u] = idx < total ? pcnt.of(pieces, 4 * col[u]) : 0;
+        cnt[u] = idx < total ? pcnt.of(pieces, row[u], 4 * col[u]) : 0;
     }
     grid_dependency_wait();
     TRACE_WAITED();
@@ -399,13 +408,28 @@ __global__ void __launch_bounds__(SILU_THREADS) silu_mul_kernel(Pieces pieces, i
                 const int idx = base + u * stride;
                 row[u] = idx / per_row;
                 col[u] = idx - row[u] * per_row;
-                cnt[u] = idx < total ? pcnt.of(pieces, 4 * col[u]) : 0;
+                cnt[u] = idx < total ? pcnt.of(pieces, row[u], 4 * col[u]) : 0;
             }
         }
+        // piece by piece over all tasks: a task's sum is not waited for before the next task's loads are out
+        int most = 0;
 #pragma unroll
         for (int u = 0; u < T; ++u) {
             v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (base + u * stride < total) v[u] = piece_sum4<2>(pieces, cnt[u], row[u], 4 * col[u]);
+            if (base + u * stride < total) {
+                v[u] = __ldcg(reinterpret_cast<const float4*>(pieces.base + (size_t)row[u] * pieces.ld + 4 * col[u]));
+                most = max(most, cnt[u]);
+            }
+        }
+        for (int i = 1; i < most; ++i) {
+            float4 w[T];
+#pragma unroll
+            for (int u = 0; u < T; ++u)
+                w[u] = (base + u * stride < total && i < cnt[u])
+                           ? __ldcg(reinterpret_cast<const float4*>(pieces.base + (size_t)i * pieces.stride + (size_t)row[u] * pieces.ld + 4 * col[u]))
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int u = 0; u < T; ++u) { v[u].x += w[u].x; v[u].y += w[u].y; v[u].z += w[u].z; v[u].w += w[u].w; }
         }
 #pragma unroll
         for (int u = 0; u < T; ++u) {

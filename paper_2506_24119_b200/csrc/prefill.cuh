@@ -4,11 +4,8 @@
 // weight-streaming like the decode step -- and attention reads each cached key once per block of
 // queries instead of once per query.  Kernels:
 //
-//   pf_gemm_kernel<EPI>   Y[t][r] = sum_k X[t][k] W[r][k] over output tiles of 128 weight rows x 256
-//                         token rows, tcgen05.mma (M = 128, N = 256, K = 16) with two 256-column
-//                         accumulators in tensor memory, a four-stage TMA ring (16 KB of W + 32 KB of
-//                         X per stage) and an epilogue that runs under the next tile's mainloop:
-//                         plain fp32 store, residual accumulation in place, or SwiGLU gating to fp16.
+//   pg_gemm_kernel<EPI>   (gemm_pair.cuh) the linear layers on pairs of SMs, with the residual addition or the SwiGLU
+//                         gating in the epilogue; partial sums where few token rows make stream-K the better split.
 //   attn_append_tc_kernel causal grouped-query attention of a block of new positions of one game against
 //                         everything cached for it (earlier turns and the new tokens up to each query's own
 //                         position) on tcgen05: scores and the output accumulator in tensor memory, one
@@ -20,383 +17,190 @@
 // Every wait is bounded as in the decode kernels.
 #pragma once
 #include "attn_decode.cuh"
+#include "gemm_pair.cuh"
 #include "gemm_tc.cuh"
 
 namespace spiral {
-
-// ------------------------------------------------------------------------------------------------
-// dense GEMM
-// ------------------------------------------------------------------------------------------------
-constexpr int PF_BN = 256;                                   // token rows per tile = MMA N
-constexpr int PF_STAGES = 4;
-constexpr int PF_X_BYTES = PF_BN * TC_BK * 2;                // 32 KB
-constexpr int PF_STAGE_BYTES = TC_W_BYTES + PF_X_BYTES;      // 48 KB
-constexpr int PF_THREADS = 192;                              // TMA warp, MMA warp, four epilogue warps
-constexpr size_t PF_SMEM = (size_t)PF_STAGES * PF_STAGE_BYTES + 1024;
-enum { PF_EPI_STORE = 0, PF_EPI_ADD = 1, PF_EPI_SILU = 2 };
-
-struct PfGemmParams {
-    int row_tiles, tok_tiles, KB;   // 128-row tiles of W, 256-row tiles of X, 64-wide k blocks
-    int rows, T;                    // weight rows (output features) and token rows
-    int row_fastest;                // order in which consecutive CTAs take tiles (see pf_tile_of)
-    float* out;                     // STORE: y [T][rows] written; ADD: x [T][rows] += result
-    __half* act;                    // SILU: [T][rows / 2] = SiLU(y[2i]) * y[2i+1] (gate / up rows interleaved)
-    int* status;
-};
-
-// Tiles are dealt round-robin.  Token tile fastest: the CTAs running at one time cover a few weight row
-// tiles times all token tiles, so every weight tile is fetched from HBM once and shared through L2 while
-// the activations are re-read once per wave.  Row tile fastest: the other way round.  The host picks the
-// order that re-reads the smaller operand (the activations of the down projection exceed L2).
-__device__ __forceinline__ void pf_tile_of(const int L, const int row_tiles, const int tok_tiles, const int row_fastest,
-                                           int& rt, int& tt) {
-    if (row_fastest) { tt = L / row_tiles; rt = L - tt * row_tiles; }
-    else { rt = L / tok_tiles; tt = L - rt * tok_tiles; }
-}
-template <int EPI>
-__global__ void __launch_bounds__(PF_THREADS, 1) pf_gemm_kernel(const __grid_constant__ CUtensorMap tmW,
-                                                                const __grid_constant__ CUtensorMap tmX,
-                                                                PfGemmParams p) {
-    extern __shared__ uint8_t pf_smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[PF_STAGES], empty_bar[PF_STAGES], acc_full[2], acc_empty[2];
-    __shared__ uint32_t tmem_base_sm;
-    __shared__ int abort_sm;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    grid_launch_dependents();
-    const uint32_t tiles_base = (smem_u32(pf_smem_raw) + 1023u) & ~1023u;
-    constexpr uint32_t TMEM_COLS = 2 * PF_BN;
-    const int n_tiles = p.row_tiles * p.tok_tiles;
-    const int G = (int)gridDim.x;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < PF_STAGES; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(smem_u32(&acc_full[a]), 1); mbar_init(smem_u32(&acc_empty[a]), 4); }
-        abort_sm = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        tmap_prefetch(&tmW);
-        tmap_prefetch(&tmX);
-    }
-    if (warp == 1) tmem_alloc(smem_u32(&tmem_base_sm), TMEM_COLS);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = tmem_base_sm;
-    volatile int* abort_flag = &abort_sm;
-
-    if (warp == 0) {
-        // ---------------- TMA producer ----------------
-        if (lane == 0) {
-            const uint64_t pol_w = l2_policy_evict_last(), pol_x = l2_policy_evict_last();
-            // weights are written by nobody: the first ring-full of W tiles goes out before the dependency wait
-            int pre = 0;
-            for (int L = blockIdx.x, kb = 0; pre < PF_STAGES && L < n_tiles; ++pre) {
-                const uint32_t fb = smem_u32(&full_bar[pre]);
-                mbar_expect_tx(fb, PF_STAGE_BYTES);
-                int rt, tt;
-                pf_tile_of(L, p.row_tiles, p.tok_tiles, p.row_fastest, rt, tt);
-                tma_load_2d(tiles_base + (uint32_t)pre * PF_STAGE_BYTES, &tmW, 0, (rt * p.KB + kb) * TC_BM, fb, pol_w);
-                if (++kb == p.KB) { kb = 0; L += G; }
-            }
-            grid_dependency_wait();          // X is written by the preceding kernel
-            int it = 0;
-            bool ok = true;
-            for (int L = blockIdx.x; ok && L < n_tiles; L += G) {
-                int rt, tt;
-                pf_tile_of(L, p.row_tiles, p.tok_tiles, p.row_fastest, rt, tt);
-                for (int kb = 0; kb < p.KB; ++kb, ++it) {
-                    const int s = it % PF_STAGES;
-                    const uint32_t fb = smem_u32(&full_bar[s]);
-                    const uint32_t dst = tiles_base + (uint32_t)s * PF_STAGE_BYTES;
-                    if (it >= pre) {
-                        const uint32_t ph = (uint32_t)(it / PF_STAGES) & 1u;
-                        if (!mbar_wait(smem_u32(&empty_bar[s]), ph ^ 1u, abort_flag, p.status, STATUS_TIMEOUT_MMA)) {
-                            ok = false;
-                            break;
-                        }
-                        mbar_expect_tx(fb, PF_STAGE_BYTES);
-                        tma_load_2d(dst, &tmW, 0, (rt * p.KB + kb) * TC_BM, fb, pol_w);
-                    }
-                    tma_load_2d(dst + TC_W_BYTES, &tmX, kb * TC_BK, tt * PF_BN, fb, pol_x);
-                }
-            }
-            if (!ok) {
-                // copies already issued still land in this CTA's shared memory: bounded wait for them
-                for (int back = 1; back <= PF_STAGES && back <= it; ++back) {
-                    const int j = it - back, s = j % PF_STAGES;
-                    const uint32_t ph = (uint32_t)(j / PF_STAGES) & 1u;
-                    unsigned long long t0 = global_ns();
-                    while (!mbar_try(smem_u32(&full_bar[s]), ph) && global_ns() - t0 < TMA_WAIT_NS) {}
-                }
-            }
-        }
-    } else if (warp == 1) {
-        // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            const uint32_t idesc = tc_idesc_f16(PF_BN);
-            int it = 0, acc_it = 0;
-            bool ok = true;
-            for (int L = blockIdx.x; ok && L < n_tiles; L += G, ++acc_it) {
-                const int a = acc_it & 1;
-                const uint32_t aph = (uint32_t)(acc_it >> 1) & 1u;
-                if (!mbar_wait(smem_u32(&acc_empty[a]), aph ^ 1u, abort_flag, p.status, STATUS_TIMEOUT_EPI)) break;
-                tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(a * PF_BN);
-                for (int kb = 0; kb < p.KB; ++kb, ++it) {
-                    const int s = it % PF_STAGES;
-                    const uint32_t ph = (uint32_t)(it / PF_STAGES) & 1u;
-                    if (!mbar_wait(smem_u32(&full_bar[s]), ph, abort_flag, p.status, STATUS_TIMEOUT_TMA)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t w_addr = tiles_base + (uint32_t)s * PF_STAGE_BYTES;
-                    const uint64_t da = smem_desc_sw128(w_addr), db = smem_desc_sw128(w_addr + TC_W_BYTES);
-#pragma unroll
-                    for (int k = 0; k < TC_BK / 16; ++k)
-                        tc_mma_f16(d_tmem, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc, (kb > 0 || k > 0) ? 1u : 0u);
-                    tc_commit(smem_u32(&empty_bar[s]));
-                }
-                if (ok) tc_commit(smem_u32(&acc_full[a]));
-            }
-        }
-    } else {
-        // ---------------- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 ----------------
-        const int q = warp & 3;
-        grid_dependency_wait();              // the output may still be read (or, ADD, written) by earlier kernels
-        int acc_it = 0;
-        for (int L = blockIdx.x; L < n_tiles; L += G, ++acc_it) {
-            int rt, tt;
-            pf_tile_of(L, p.row_tiles, p.tok_tiles, p.row_fastest, rt, tt);
-            const int a = acc_it & 1;
-            const uint32_t aph = (uint32_t)(acc_it >> 1) & 1u;
-            if (!mbar_wait(smem_u32(&acc_full[a]), aph, abort_flag, p.status, STATUS_TIMEOUT_MMA)) break;
-            tc_fence_after();
-            const int row = rt * TC_BM + q * 32 + lane;
-            const bool row_ok = row < p.rows;
-            const int col0 = tt * PF_BN;
-            const int n_cols = min(PF_BN, p.T - col0);                  // token rows of this tile that exist
-            const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * PF_BN);
-            if (EPI == PF_EPI_SILU) {
-                const int half_rows = p.rows >> 1;
-                const bool odd = lane & 1;
-                __half* arow = p.act + (size_t)col0 * half_rows + (row >> 1);
-#pragma unroll 1
-                for (int c0 = 0; c0 < n_cols; c0 += 32) {
-                    uint32_t v[2][16];
-                    tmem_ld16_async(t_addr + (uint32_t)c0, v[0]);
-                    tmem_ld16_async(t_addr + (uint32_t)(c0 + 16), v[1]);
-                    tmem_ld_wait();
-                    // even lanes hold gate features, odd lanes the matching up features: per pair of token
-                    // columns the even lane finishes the first and the odd lane the second
-#pragma unroll
-                    for (int h = 0; h < 2; ++h)
-#pragma unroll
-                        for (int j = 0; j < 16; j += 2) {
-                            const float m0 = __uint_as_float(v[h][j]), m1 = __uint_as_float(v[h][j + 1]);
-                            const float got = __shfl_xor_sync(0xffffffffu, odd ? m0 : m1, 1);
-                            const float gate = odd ? got : m0, up = odd ? m1 : got;
-                            const int col = c0 + 16 * h + j + (odd ? 1 : 0);
-                            if (row_ok && col < n_cols)
-                                arow[(size_t)col * half_rows] = __ushort_as_half(
-                                    (unsigned short)float_to_f16_bits(__fdividef(gate, 1.f + __expf(-gate)) * up));
-                        }
-                }
-            } else {
-                float* dst = p.out + (size_t)col0 * p.rows + row;
-#pragma unroll 1
-                for (int c0 = 0; c0 < n_cols; c0 += 16) {
-                    uint32_t v[16];
-                    float old[16];
-                    tmem_ld16_async(t_addr + (uint32_t)c0, v);
-                    float* d0 = dst + (size_t)c0 * p.rows;
-                    if (EPI == PF_EPI_ADD) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            old[j] = (row_ok && c0 + j < n_cols) ? d0[(size_t)j * p.rows] : 0.f;
-                    }
-                    tmem_ld_wait();
-                    if (row_ok) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (c0 + j < n_cols)
-                                d0[(size_t)j * p.rows] = EPI == PF_EPI_ADD ? old[j] + __uint_as_float(v[j]) : __uint_as_float(v[j]);
-                    }
-                }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&acc_empty[a]));
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
-}
-
-// y (+)= X W^T for T token rows.  W: the caller's bf16 matrix, registered (its fp16 tile-major copy is read).
-template <int EPI>
-inline int pf_gemm(TcState& tc, const __nv_bfloat16* W, int rows, int K, const __half* X, int T, float* out, __half* act,
-                   int* status, cudaStream_t st, int64_t* launches) {
-    auto it = tc.weights.find(W);
-    if (it == tc.weights.end() || !it->second.resident || it->second.rows != rows || it->second.K != K)
-        return SPIRAL_ERR_UNSUPPORTED;
-    const CUtensorMap* xm = nullptr;
-    int rc = tc_get_xmap(tc, X, K, T, PF_BN, &xm);
-    if (rc) return rc;
-    PfGemmParams p{};
-    p.row_tiles = (rows + TC_BM - 1) / TC_BM;
-    p.tok_tiles = (T + PF_BN - 1) / PF_BN;
-    p.KB = (K + TC_BK - 1) / TC_BK;
-    p.rows = rows; p.T = T; p.out = out; p.act = act; p.status = status;
-    // re-read the smaller operand: weights rows x K, activations T x K
-    p.row_fastest = (T > rows && p.row_tiles <= tc.n_sm) ? 1 : 0;
-    const int grid = std::min(tc.n_sm, p.row_tiles * p.tok_tiles);
-    TC_TRY(launch_kernel(true, pf_gemm_kernel<EPI>, dim3(grid), dim3(PF_THREADS), PF_SMEM, st, it->second.map, *xm, p));
-    if (launches) ++*launches;
-    return SPIRAL_OK;
-}
-
-inline int pf_gemm_setup() {
-    TC_TRY(cudaFuncSetAttribute(pf_gemm_kernel<PF_EPI_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PF_SMEM));
-    TC_TRY(cudaFuncSetAttribute(pf_gemm_kernel<PF_EPI_ADD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PF_SMEM));
-    TC_TRY(cudaFuncSetAttribute(pf_gemm_kernel<PF_EPI_SILU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PF_SMEM));
-    return SPIRAL_OK;
-}
 
 // ------------------------------------------------------------------------------------------------
 // element-wise kernels over thousands of token rows (the decode step's versions are built for a
 // few hundred rows at most: one CTA per row, half a warp per head)
 // ------------------------------------------------------------------------------------------------
 
-// h[t][:] = x[t][:] * rsqrt(mean(x[t]^2) + eps) * gain as fp16, one warp per token row: the row
-// stays in registers between the reduction and the scaling, no block barrier.
-constexpr int PF_RMS_MAX_V4 = 32;       // float4 per lane: d_model <= 4096
-constexpr int PF_RMS_THREADS = 256;
-template <int NV4>                      // float4 per lane the row needs, rounded up to a multiple of 4
+// h[t][:] = x[t][:] * rsqrt(mean(x[t]^2) + eps) * gain as fp16, one CTA of four warps per token row: the row stays in
+// registers between the reduction and the scaling, and a row's loads are spread thin enough (NV4 float4 per thread)
+// for ten CTAs per SM.  Bound by memory: 6 bytes read and written per element.  (With a warp per row, 20 float4 per
+// lane at d_model 2560 left room for 16 warps per SM, which went through their rows in lockstep: 54 us for 9984 rows.)
+constexpr int PF_RMS_THREADS = 128;
+template <int NV4>                      // float4 per thread
 __global__ void __launch_bounds__(PF_RMS_THREADS) pf_rmsnorm_kernel(const float* __restrict__ x,
                                                                     const __nv_bfloat16* __restrict__ gain, float eps,
-                                                                    int d_model, int T, __half* __restrict__ h) {
-    grid_dependency_sync();
-    const int lane = threadIdx.x & 31;
-    const int warps = (gridDim.x * blockDim.x) >> 5;
+                                                                    int d_model, __half* __restrict__ h) {
+    grid_launch_dependents();
+    __shared__ float red[PF_RMS_THREADS / 32];
     const int nc = d_model >> 2;
-    for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < T; t += warps) {
-        const float4* xr = reinterpret_cast<const float4*>(x + (size_t)t * d_model);
-        float4 v[NV4];
-        float ss = 0.f;
+    uint2 g[NV4];                       // (weights: nobody writes them)
 #pragma unroll
-        for (int k = 0; k < NV4; ++k) {
-            const int c = lane + 32 * k;
-            v[k] = c < nc ? __ldcs(xr + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+    for (int k = 0; k < NV4; ++k) {
+        const int c = threadIdx.x + PF_RMS_THREADS * k;
+        g[k] = c < nc ? __ldg(reinterpret_cast<const uint2*>(gain) + c) : make_uint2(0u, 0u);
+    }
+    grid_dependency_wait();
+    const size_t t = blockIdx.x;
+    const float4* xr = reinterpret_cast<const float4*>(x + t * d_model);
+    float4 v[NV4];
 #pragma unroll
-        for (int k = 0; k < NV4; ++k) ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
-        ss = warp_sum(ss);
-        const float inv = rsqrtf(ss / (float)d_model + eps);
-        __half* hr = h + (size_t)t * d_model;
+    for (int k = 0; k < NV4; ++k) {
+        const int c = threadIdx.x + PF_RMS_THREADS * k;
+        v[k] = c < nc ? __ldcs(xr + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float ss = 0.f;
 #pragma unroll
-        for (int k = 0; k < NV4; ++k) {
-            const int c = lane + 32 * k;
-            if (c < nc) {
-                const uint2 g = __ldg(reinterpret_cast<const uint2*>(gain + 4 * c));
-                uint2 o;
-                o.x = pack_f16(v[k].x * inv * bf16_lo(g.x), v[k].y * inv * bf16_hi(g.x));
-                o.y = pack_f16(v[k].z * inv * bf16_lo(g.y), v[k].w * inv * bf16_hi(g.y));
-                *reinterpret_cast<uint2*>(hr + 4 * c) = o;
-            }
+    for (int k = 0; k < NV4; ++k) ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
+    ss = warp_sum(ss);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    const float inv = rsqrtf((red[0] + red[1] + red[2] + red[3]) / (float)d_model + eps);
+    uint2* hr = reinterpret_cast<uint2*>(h + t * d_model);
+#pragma unroll
+    for (int k = 0; k < NV4; ++k) {
+        const int c = threadIdx.x + PF_RMS_THREADS * k;
+        if (c < nc) {
+            uint2 o;
+            o.x = pack_f16(v[k].x * inv * bf16_lo(g[k].x), v[k].y * inv * bf16_hi(g[k].x));
+            o.y = pack_f16(v[k].z * inv * bf16_lo(g[k].y), v[k].w * inv * bf16_hi(g[k].y));
+            hr[c] = o;
         }
     }
 }
 
-// One warp per (token row, head) of the QKV projection y [T][(Hq + 2 Hkv) * HD] (fp32): bias, per-head
-// RMSNorm of q and k, rotate-half RoPE at the token's position; then q -> fp16 [T][Hq][HD] already
-// multiplied by log2(e) / sqrt(HD) (the attention kernel works in the exp2 domain), k and v -> the
-// token's slot in its page, rounded once to fp16.  Lane l holds elements {E l .. E l + E - 1} and
-// their rotation partners HD/2 further on (E = HD / 64).
+// The QKV projection [T][(Hq + 2 Hkv) * HD] (pieces, summed here): bias, per-head RMSNorm of q and k, rotate-half RoPE at
+// the token's position; then q -> fp16 [T][Hq][HD] already multiplied by log2(e) / sqrt(HD) (the attention kernel works in
+// the exp2 domain), k and v -> the token's slot in its page, rounded once to fp16.  One warp per token row and PF_QKV_HEADS
+// heads of one kind (q, k or v): the loads of all its heads, the rotation and the page look-up are in flight together.
+// Lane l holds elements {E l .. E l + E - 1} and their rotation partners HD/2 further on (E = HD / 64).  Bound by memory
+// (4 bytes read, 2 written per element); with a warp per single head the chain position -> page -> store of every head
+// was what took the time (208 us for 9984 rows of 48 heads).
 constexpr int PF_QKV_THREADS = 256;
+constexpr int PF_QKV_HEADS = 4;
+inline int pf_qkv_groups(int n_q_heads, int n_kv_heads) {        // tasks per token row
+    return (n_q_heads + PF_QKV_HEADS - 1) / PF_QKV_HEADS + 2 * ((n_kv_heads + PF_QKV_HEADS - 1) / PF_QKV_HEADS);
+}
 template <int HD>
 __global__ void __launch_bounds__(PF_QKV_THREADS) pf_qkv_post_kernel(
-    const float* __restrict__ y, const __nv_bfloat16* __restrict__ bias, const __nv_bfloat16* __restrict__ q_gain,
+    Pieces pieces, const __nv_bfloat16* __restrict__ bias, const __nv_bfloat16* __restrict__ q_gain,
     const __nv_bfloat16* __restrict__ k_gain, float eps, const float* __restrict__ cos_tab,
     const float* __restrict__ sin_tab, const int32_t* __restrict__ game, const int32_t* __restrict__ pos_of,
     const int32_t* __restrict__ block_table, int max_pages, int n_pages, int layer, int T, int n_q_heads,
     int n_kv_heads, float q_scale, __half* __restrict__ q_out, uint16_t* __restrict__ pool, int* status) {
-    constexpr int E = HD / 64, HALF = HD / 2;
-    grid_dependency_sync();
+    constexpr int E = HD / 64, HALF = HD / 2, NH = PF_QKV_HEADS;
+    grid_launch_dependents();
+    __shared__ unsigned char cnt_tab[PIECE_TABLE];
+    const PieceCounts pcnt = piece_counts_init(pieces, cnt_tab);       // (parameters only: before the wait)
+    grid_dependency_wait();
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
-    const int n_heads = n_q_heads + 2 * n_kv_heads;
-    const int ld = n_heads * HD;
-    const long long total = (long long)T * n_heads;
-    for (long long task = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; task < total; task += warps) {
-        const int t = (int)(task / n_heads), head = (int)(task - (long long)t * n_heads);
-        const float* yr = y + (size_t)t * ld + head * HD + E * lane;
-        float lo[E], hi[E];
-        if (E == 2) {
-            const float2 a = __ldcs(reinterpret_cast<const float2*>(yr));
-            const float2 b = __ldcs(reinterpret_cast<const float2*>(yr + HALF));
-            lo[0] = a.x; lo[E - 1] = a.y; hi[0] = b.x; hi[E - 1] = b.y;
-        } else {
-            lo[0] = __ldcs(yr); hi[0] = __ldcs(yr + HALF);
+    const int gq = (n_q_heads + NH - 1) / NH, gk = (n_kv_heads + NH - 1) / NH, groups = gq + 2 * gk;
+    const int total = T * groups;
+    for (int task = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; task < total; task += warps) {
+        const int t = task / groups, grp = task - t * groups;
+        const bool is_q = grp < gq, is_k = !is_q && grp < gq + gk;
+        const int first = is_q ? grp * NH : (is_k ? grp - gq : grp - gq - gk) * NH;             // head within its kind
+        const int nh = min(NH, (is_q ? n_q_heads : n_kv_heads) - first);
+        const int head0 = first + (is_q ? 0 : is_k ? n_q_heads : n_q_heads + n_kv_heads);       // row of the projection
+        const float* yr = pieces.base + (size_t)t * pieces.ld + head0 * HD + E * lane;
+        float lo[NH][E], hi[NH][E];
+        auto fetch = [&](const float* yh, float (&l)[E], float (&h)[E]) {
+            if (E == 2) {
+                const float2 a = __ldcs(reinterpret_cast<const float2*>(yh)), b = __ldcs(reinterpret_cast<const float2*>(yh + HALF));
+                l[0] = a.x; l[E - 1] = a.y; h[0] = b.x; h[E - 1] = b.y;
+            } else {
+                l[0] = __ldcs(yh); h[0] = __ldcs(yh + HALF);
+            }
+        };
+        // the first piece of every head, then (stream-K) the second of every head, ...: no head's sum is waited for before
+        // the next head's loads are out
+        int most = 0;
+#pragma unroll
+        for (int u = 0; u < NH; ++u)
+            if (u < nh) {
+                fetch(yr + u * HD, lo[u], hi[u]);
+                most = max(most, pcnt.of(pieces, t, (head0 + u) * HD));
+            }
+        const int pos = __ldg(pos_of + t);
+        int page = 0;
+        if (!is_q) page = __ldg(block_table + (size_t)__ldg(game + t) * max_pages + pos / ATTN_PAGE);
+        for (int i = 1; i < most; ++i) {
+            float l2[NH][E], h2[NH][E];
+#pragma unroll
+            for (int u = 0; u < NH; ++u) {
+                const bool in = u < nh && i < pcnt.of(pieces, t, (head0 + u) * HD);
+#pragma unroll
+                for (int e = 0; e < E; ++e) { l2[u][e] = 0.f; h2[u][e] = 0.f; }
+                if (in) fetch(yr + u * HD + (size_t)i * pieces.stride, l2[u], h2[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < NH; ++u)
+#pragma unroll
+                for (int e = 0; e < E; ++e) { lo[u][e] += l2[u][e]; hi[u][e] += h2[u][e]; }
         }
-        const bool is_q = head < n_q_heads, is_k = !is_q && head < n_q_heads + n_kv_heads;
-        const int pos = pos_of[t];
-        if (bias) {
+        float cs[E], sn[E], gl[E], gh[E];
+        const __nv_bfloat16* gain = is_q ? q_gain : is_k ? k_gain : nullptr;
+        if (is_q || is_k) {
 #pragma unroll
             for (int e = 0; e < E; ++e) {
-                lo[e] += __bfloat162float(bias[head * HD + E * lane + e]);
-                hi[e] += __bfloat162float(bias[head * HD + E * lane + e + HALF]);
+                cs[e] = __ldg(cos_tab + (size_t)pos * HALF + E * lane + e);
+                sn[e] = __ldg(sin_tab + (size_t)pos * HALF + E * lane + e);
+                gl[e] = gain ? __bfloat162float(gain[E * lane + e]) : 1.f;
+                gh[e] = gain ? __bfloat162float(gain[E * lane + e + HALF]) : 1.f;
             }
         }
-        if (is_q || is_k) {
-            const __nv_bfloat16* gain = is_q ? q_gain : k_gain;
-            if (gain) {
-                float ss = 0.f;
 #pragma unroll
-                for (int e = 0; e < E; ++e) ss += lo[e] * lo[e] + hi[e] * hi[e];
-                ss = warp_sum(ss);
-                const float inv = rsqrtf(ss / (float)HD + eps);
+        for (int u = 0; u < NH; ++u) {
+            if (u >= nh) break;
+            if (bias) {
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
-                    lo[e] = lo[e] * inv * __bfloat162float(gain[E * lane + e]);
-                    hi[e] = hi[e] * inv * __bfloat162float(gain[E * lane + e + HALF]);
+                    lo[u][e] += __bfloat162float(bias[(head0 + u) * HD + E * lane + e]);
+                    hi[u][e] += __bfloat162float(bias[(head0 + u) * HD + E * lane + e + HALF]);
                 }
             }
+            if (is_q || is_k) {
+                if (gain) {
+                    float ss = 0.f;
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const float cs = __ldg(cos_tab + (size_t)pos * HALF + E * lane + e);
-                const float sn = __ldg(sin_tab + (size_t)pos * HALF + E * lane + e);
-                const float a = lo[e], b = hi[e];
-                lo[e] = a * cs - b * sn;
-                hi[e] = b * cs + a * sn;
+                    for (int e = 0; e < E; ++e) ss += lo[u][e] * lo[u][e] + hi[u][e] * hi[u][e];
+                    ss = warp_sum(ss);
+                    const float inv = rsqrtf(ss / (float)HD + eps);
+#pragma unroll
+                    for (int e = 0; e < E; ++e) { lo[u][e] = lo[u][e] * inv * gl[e]; hi[u][e] = hi[u][e] * inv * gh[e]; }
+                }
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const float a = lo[u][e], b = hi[u][e];
+                    lo[u][e] = a * cs[e] - b * sn[e];
+                    hi[u][e] = b * cs[e] + a * sn[e];
+                }
             }
         }
-        if (is_q) {
-            __half* q = q_out + ((size_t)t * n_q_heads + head) * HD + E * lane;
-            if (E == 2) {
-                *reinterpret_cast<uint32_t*>(q) = pack_f16(lo[0] * q_scale, lo[E - 1] * q_scale);
-                *reinterpret_cast<uint32_t*>(q + HALF) = pack_f16(hi[0] * q_scale, hi[E - 1] * q_scale);
-            } else {
-                q[0] = __ushort_as_half((unsigned short)float_to_f16_bits(lo[0] * q_scale));
-                q[HALF] = __ushort_as_half((unsigned short)float_to_f16_bits(hi[0] * q_scale));
-            }
-            continue;
-        }
-        const int kvh = is_k ? head - n_q_heads : head - n_q_heads - n_kv_heads;
-        const int page = __ldg(block_table + (size_t)game[t] * max_pages + pos / ATTN_PAGE);
-        if (page < 0 || page >= n_pages) {
+        if (!is_q && (page < 0 || page >= n_pages)) {
             if (lane == 0) record_status(status, STATUS_BAD_PAGE);
             continue;
         }
-        uint16_t* dst = pool + kv_block_offset(layer, page, kvh, n_pages, n_kv_heads, ATTN_PAGE, HD) +
-                        (is_k ? 0 : (size_t)ATTN_PAGE * HD) + (size_t)(pos % ATTN_PAGE) * HD + E * lane;
-        if (E == 2) {
-            *reinterpret_cast<uint32_t*>(dst) = pack_f16(lo[0], lo[E - 1]);
-            *reinterpret_cast<uint32_t*>(dst + HALF) = pack_f16(hi[0], hi[E - 1]);
-        } else {
-            dst[0] = (uint16_t)float_to_f16_bits(lo[0]);
-            dst[HALF] = (uint16_t)float_to_f16_bits(hi[0]);
+#pragma unroll
+        for (int u = 0; u < NH; ++u) {
+            if (u >= nh) break;
+            const float sc = is_q ? q_scale : 1.f;
+            uint16_t* dst = is_q ? reinterpret_cast<uint16_t*>(q_out) + ((size_t)t * n_q_heads + first + u) * HD + E * lane
+                                 : pool + kv_block_offset(layer, page, first + u, n_pages, n_kv_heads, ATTN_PAGE, HD) +
+                                       (is_k ? 0 : (size_t)ATTN_PAGE * HD) + (size_t)(pos % ATTN_PAGE) * HD + E * lane;
+            if (E == 2) {
+                *reinterpret_cast<uint32_t*>(dst) = pack_f16(lo[u][0] * sc, lo[u][E - 1] * sc);
+                *reinterpret_cast<uint32_t*>(dst + HALF) = pack_f16(hi[u][0] * sc, hi[u][E - 1] * sc);
+            } else {
+                dst[0] = (uint16_t)float_to_f16_bits(lo[u][0] * sc);
+                dst[HALF] = (uint16_t)float_to_f16_bits(hi[u][0] * sc);
+            }
         }
     }
 }

@@ -80,6 +80,7 @@ struct ProfRec { int cls; cudaEvent_t e0, e1; };
 // attention work list, each with a pinned host mirror.
 struct PrefillWs {
     int cap = 0;                        // token rows the buffers hold
+    size_t y_elems = 0;                 // floats of y: the QKV projection, or the pieces of whichever matrix is split
     float *x = nullptr, *y = nullptr;
     __half *q = nullptr, *h = nullptr, *attn = nullptr, *act = nullptr;
     int32_t* meta_dev = nullptr;        // [4][cap]: game, position, -1, token index; then [2][max_batch]: rows to
@@ -91,8 +92,8 @@ struct PrefillWs {
     cudaEvent_t ev = nullptr;           // the last upload from the pinned mirrors
     bool ev_used = false;
 };
-constexpr int PREFILL_CHUNK_DEFAULT = 37 * PF_BN;   // 9472 rows: 37 token tiles x (20 | 48 | 152 row tiles) fill
-                                                    // 148 SMs in whole waves for the Qwen3-4B matrices
+constexpr int PREFILL_CHUNK_DEFAULT = 12288;   // token rows of the largest dense pass (workspace: about 90 KB per row at
+                                               // the Qwen3-4B shape); prefill_dense cuts a call into equal passes below it
 }  // namespace
 
 struct spiral_ctx {
@@ -246,7 +247,7 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
         const char* off = std::getenv("SPIRAL_NO_GRAPH");
         c->use_graph = !(off && off[0] == '1');
         off = std::getenv("SPIRAL_PREFILL_CHUNK");
-        if (off) c->prefill_chunk = std::max(PF_BN, std::min(1 << 16, (atoi(off) + PF_BN - 1) / PF_BN * PF_BN));
+        if (off) c->prefill_chunk = std::max(PG_MAX_N, std::min(1 << 16, (atoi(off) + PG_MAX_N - 1) / PG_MAX_N * PG_MAX_N));
         off = std::getenv("SPIRAL_PREFILL_DENSE");
         c->prefill_dense = !(off && off[0] == '0');
         off = std::getenv("SPIRAL_APPEND_ATTN");
@@ -392,7 +393,7 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
         for (const M& m : mats)
             if (m.w != c->lm_head && !tc_usable(c->tc, m.rows, m.k, max_batch)) c->pf_ready = false;
         if (c->pf_ready) {
-            rc = pf_gemm_setup();
+            rc = pg_gemm_setup();
             e = cudaSuccess;
             if (rc == SPIRAL_OK) e = cudaFuncSetAttribute(attn_append_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem_bytes(128));
             if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute(attn_append_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem_bytes(64));
@@ -685,6 +686,7 @@ static int launch_linear_impl(spiral_ctx* c, const bf16* W, int rows, int K, con
     dim3 grid((rows + 2 * GEMV_WARPS - 1) / (2 * GEMV_WARPS), (n + GEMV_BC - 1) / GEMV_BC);
     LAUNCH(c, gemv_kernel, grid, GEMV_WARPS * 32, 0, st, W, rows, K, X, n, y);
     out->base = y; out->stride = (size_t)n * rows; out->ld = rows; out->n_pieces = 1; out->sk_KB = 0; out->sk_G = 0;
+    out->sk_shift = 7; out->sk_tt = 1; out->sk_BN = n;
     return SPIRAL_OK;
 }
 
@@ -1024,38 +1026,71 @@ extern "C" int spiral_decode_step_host(spiral_ctx* ctx, spiral_kv* kv, int n, co
     return SPIRAL_OK;
 }
 
-// dst[pairs[stride + b]][:] = src[pairs[b]][:]
-__global__ void gather_rows_kernel(const float* __restrict__ src, const int32_t* __restrict__ pairs, int stride,
-                                   int d_model, float* __restrict__ dst) {
+// dst[pairs[stride + b]][:] = src[pairs[b]][:] + the pieces the last projection has left for that row (when given)
+__global__ void gather_rows_kernel(const float* __restrict__ src, Pieces pieces, int has_pieces, const int32_t* __restrict__ pairs,
+                                   int stride, int d_model, float* __restrict__ dst) {
     grid_dependency_sync();
-    const int b = blockIdx.x;
-    const float4* s = reinterpret_cast<const float4*>(src + (size_t)pairs[b] * d_model);
+    const int b = blockIdx.x, row = pairs[b];
+    const float4* s = reinterpret_cast<const float4*>(src + (size_t)row * d_model);
     float4* d = reinterpret_cast<float4*>(dst + (size_t)pairs[stride + b] * d_model);
-    for (int c = threadIdx.x; c < d_model / 4; c += blockDim.x) d[c] = s[c];
+    for (int c = threadIdx.x; c < d_model / 4; c += blockDim.x) {
+        float4 v = s[c];
+        if (has_pieces) {
+            const float4 p = piece_sum4(pieces, piece_count(pieces, row, 4 * c), row, 4 * c);
+            v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
+        }
+        d[c] = v;
+    }
 }
 
-// h = RMSNorm(x) * gain over T token rows (warp per row while the row fits a warp's registers)
+// h = RMSNorm(x) * gain over T token rows
 static int launch_rmsnorm_rows(spiral_ctx* c, const float* x, const bf16* gain, int T, __half* h, cudaStream_t st) {
     const spiral_model_desc& d = c->d;
     const float eps = (float)d.rms_eps;
-    const int need = (d.d_model / 4 + 31) / 32;
-    const int grid = std::max(1, std::min((T + PF_RMS_THREADS / 32 - 1) / (PF_RMS_THREADS / 32), 8 * c->n_sm));
+    const int need = (d.d_model / 4 + PF_RMS_THREADS - 1) / PF_RMS_THREADS;
 #define PF_RMS_CASE(NV)                                                                                               \
     if (need <= NV) {                                                                                                 \
-        LAUNCH(c, pf_rmsnorm_kernel<NV>, grid, PF_RMS_THREADS, 0, st, x, gain, eps, d.d_model, T, h);                 \
+        LAUNCH(c, pf_rmsnorm_kernel<NV>, T, PF_RMS_THREADS, 0, st, x, gain, eps, d.d_model, h);                       \
         return SPIRAL_OK;                                                                                             \
     }
-    PF_RMS_CASE(4) PF_RMS_CASE(8) PF_RMS_CASE(12) PF_RMS_CASE(16) PF_RMS_CASE(20) PF_RMS_CASE(24) PF_RMS_CASE(28)
-    PF_RMS_CASE(32)
+    PF_RMS_CASE(2) PF_RMS_CASE(4) PF_RMS_CASE(5) PF_RMS_CASE(6) PF_RMS_CASE(7) PF_RMS_CASE(8) PF_RMS_CASE(12) PF_RMS_CASE(16)
 #undef PF_RMS_CASE
-    Pieces none{};
-    LAUNCH(c, rmsnorm_kernel, T, rms_block(d.d_model), 0, st, const_cast<float*>(x), none, 0, gain, eps, d.d_model, h);
-    return SPIRAL_OK;
+    return SPIRAL_ERR_UNSUPPORTED;              // (d_model <= 8192 is checked in spiral_init)
 }
 
-static int prefill_ws_reserve(spiral_ctx* c, int rows) {
+// Token rows per dense pass of a call with `total` new tokens: as few passes as the largest pass allows, all of (nearly)
+// the same length -- a short last pass costs all weights again -- and within that the length at which the whole-tile
+// GEMMs waste the least of their last wave.
+static int prefill_pass_rows(const spiral_ctx* c, long long total) {
+    const spiral_model_desc& d = c->d;
+    const long long passes = (total + c->prefill_chunk - 1) / c->prefill_chunk;
+    const int even = (int)((total + passes - 1) / passes);
+    if (passes == 1) return even;
+    const int lo = (even + PG_MAX_N - 1) / PG_MAX_N, hi = std::max(lo, c->prefill_chunk / PG_MAX_N);
+    const int pairs = std::max(1, c->n_sm / 2);
+    const int rows[4] = {c->qkv_rows, d.d_model, 2 * d.d_ff, d.d_model};
+    const int ks[4] = {d.d_model, d.n_q_heads * d.head_dim, d.d_model, d.d_ff};
+    auto cost = [&](long long T) {               // waves x k over the four matrices
+        const long long tt = (T + PG_MAX_N - 1) / PG_MAX_N;
+        double s = 0;
+        for (int m = 0; m < 4; ++m) s += (double)(((rows[m] + PG_BM - 1) / PG_BM * tt + pairs - 1) / pairs) * ks[m];
+        return s;
+    };
+    int best = lo;
+    double best_cost = -1;
+    for (int tt = lo; tt <= hi; ++tt) {
+        const long long T = (long long)tt * PG_MAX_N, full = total / T, rest = total - full * T;
+        const double s = full * cost(T) + (rest ? cost(rest) : 0.0);
+        if (best_cost < 0 || s < best_cost) { best_cost = s; best = tt; }
+    }
+    return best * PG_MAX_N;
+}
+
+static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems) {
     PrefillWs& w = c->pf;
-    if (rows <= w.cap) return SPIRAL_OK;
+    if (rows <= w.cap && y_elems <= w.y_elems) return SPIRAL_OK;
+    rows = std::max(rows, w.cap);
+    y_elems = std::max(y_elems, w.y_elems);
     CU_TRY(cudaDeviceSynchronize());
     cudaFree(w.x); cudaFree(w.y); cudaFree(w.q); cudaFree(w.h); cudaFree(w.attn); cudaFree(w.act);
     cudaFree(w.meta_dev); cudaFree(w.items_dev);
@@ -1072,7 +1107,7 @@ static int prefill_ws_reserve(spiral_ctx* c, int rows) {
     cudaError_t e = cudaSuccess;
     auto A = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
     A((void**)&w.x, R * d.d_model * sizeof(float));
-    A((void**)&w.y, R * c->qkv_rows * sizeof(float));
+    A((void**)&w.y, y_elems * sizeof(float));
     A((void**)&w.q, R * qd * sizeof(__half));
     A((void**)&w.h, R * d.d_model * sizeof(__half));
     A((void**)&w.attn, R * qd * sizeof(__half));
@@ -1087,7 +1122,7 @@ static int prefill_ws_reserve(spiral_ctx* c, int rows) {
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? SPIRAL_ERR_OOM : SPIRAL_ERR_CUDA;    // cap stays 0: freed with the context
     }
-    w.cap = rows; w.items_cap = items_cap; w.meta_elems = meta_elems; w.ev_used = false;
+    w.cap = rows; w.y_elems = y_elems; w.items_cap = items_cap; w.meta_elems = meta_elems; w.ev_used = false;
     return SPIRAL_OK;
 }
 
@@ -1099,14 +1134,23 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
     const spiral_model_desc& d = ctx->d;
     long long total = 0;
     for (int i = 0; i < n; ++i) total += offsets[i + 1] - offsets[i];
-    const int chunk = (int)std::min<long long>(ctx->prefill_chunk, (total + PF_BN - 1) / PF_BN * PF_BN);
-    int rc = prefill_ws_reserve(ctx, chunk);
+    const int chunk = prefill_pass_rows(ctx, total);
+    const int qd = d.n_q_heads * d.head_dim;
+    // pieces are left by the last, shorter pass too: its split is another one
+    size_t y_elems = 0;
+    for (long long T : {(long long)chunk, total % chunk ? total % chunk : (long long)chunk}) {
+        const int shapes[4][2] = {{ctx->qkv_rows, d.d_model}, {d.d_model, qd}, {2 * d.d_ff, d.d_model}, {d.d_model, d.d_ff}};
+        for (int m = 0; m < 4; ++m) {
+            const PgPlan pl = pg_plan(ctx->n_sm, shapes[m][0], shapes[m][1], (int)T, true);
+            if (m == 0 || !pl.whole) y_elems = std::max<size_t>(y_elems, (size_t)pl.max_pieces * (size_t)T * shapes[m][0]);
+        }
+    }
+    int rc = prefill_ws_reserve(ctx, (chunk + PG_MAX_N - 1) / PG_MAX_N * PG_MAX_N, y_elems);
     if (rc) return rc;
     PrefillWs& w = ctx->pf;
     const int cap = w.cap, MB = ctx->max_batch;
     const int per_item = ctx->append_attn_tc ? apt_positions_per_item(ctx->group, ctx->append_tiles)
                                              : app_positions_per_item(ctx->group);
-    const int qd = d.n_q_heads * d.head_dim;
     const float eps = (float)d.rms_eps;
     int32_t* mdev = w.meta_dev;
     StepMeta meta{mdev, mdev + cap, mdev + 2 * (size_t)cap, mdev + 3 * (size_t)cap};
@@ -1161,27 +1205,45 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
 
         LAUNCH(ctx, embed_kernel, nt, 256, 0, st, ctx->embed, meta_args(ctx), meta, kv->table_dev, kv->max_pages,
                kv->page_size, d.d_model, d.vocab, w.x, ctx->status);
+        const PgPlan pl_qkv = pg_plan(ctx->n_sm, ctx->qkv_rows, d.d_model, nt, true), pl_o = pg_plan(ctx->n_sm, d.d_model, qd, nt, true);
+        const PgPlan pl_gu = pg_plan(ctx->n_sm, 2 * d.d_ff, d.d_model, nt, true), pl_dn = pg_plan(ctx->n_sm, d.d_model, d.d_ff, nt, true);
+        Pieces pend{};                 // pieces a projection has left for the next norm to add to the residual stream
+        int has = 0;
+        // h = RMSNorm(x + pending pieces)
+        auto norm = [&](const bf16* gain) -> int {
+            if (!has) return launch_rmsnorm_rows(ctx, w.x, gain, nt, w.h, st);
+            has = 0;
+            LAUNCH(ctx, rmsnorm_kernel, nt, rms_block(d.d_model), 0, st, w.x, pend, 1, gain, eps, d.d_model, w.h);
+            return SPIRAL_OK;
+        };
+        // x += X W^T: in the epilogue, or as pieces
+        auto project = [&](int cls, const PgPlan& pl, const bf16* W, int K, const __half* X) -> int {
+            const int rec_ = prof_begin(ctx, cls, st);
+            int rc_;
+            if (pl.whole) rc_ = pg_gemm<PG_ADD>(ctx->tc, pl, W, d.d_model, K, X, nt, w.x, nullptr, ctx->status, st, &ctx->launches);
+            else {
+                rc_ = pg_gemm<PG_STORE>(ctx->tc, pl, W, d.d_model, K, X, nt, w.y, &pend, ctx->status, st, &ctx->launches);
+                has = 1;
+            }
+            prof_end(ctx, rec_, st);
+            if (rc_ == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
+            return rc_;
+        };
         for (int l = 0; l < d.n_layers; ++l) {
-            rc = launch_rmsnorm_rows(ctx, w.x, ctx->ln1[l], nt, w.h, st);
+            rc = norm(ctx->ln1[l]);
             if (rc) return rc;
+            Pieces pq;
             int rec = prof_begin(ctx, SPIRAL_KC_QKV, st);
-            rc = pf_gemm<PF_EPI_STORE>(ctx->tc, ctx->wqkv[l], ctx->qkv_rows, d.d_model, w.h, nt, w.y, nullptr, ctx->status, st,
-                                       &ctx->launches);
+            rc = pg_gemm<PG_STORE>(ctx->tc, pl_qkv, ctx->wqkv[l], ctx->qkv_rows, d.d_model, w.h, nt, w.y, &pq, ctx->status, st, &ctx->launches);
             prof_end(ctx, rec, st);
             if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
             if (rc) return rc;
             {
-                const int qgrid = 8 * ctx->n_sm;
-                if (d.head_dim == 128)
-                    LAUNCH(ctx, pf_qkv_post_kernel<128>, qgrid, PF_QKV_THREADS, 0, st, (const float*)w.y, ctx->bqkv[l],
-                           ctx->q_norm[l], ctx->k_norm[l], eps, ctx->cos_tab, ctx->sin_tab, meta.game, meta.pos,
-                           kv->table_dev, kv->max_pages, kv->n_pages, l, nt, d.n_q_heads, d.n_kv_heads, q_scale, w.q, kv->pool,
-                           ctx->status);
-                else
-                    LAUNCH(ctx, pf_qkv_post_kernel<64>, qgrid, PF_QKV_THREADS, 0, st, (const float*)w.y, ctx->bqkv[l],
-                           ctx->q_norm[l], ctx->k_norm[l], eps, ctx->cos_tab, ctx->sin_tab, meta.game, meta.pos,
-                           kv->table_dev, kv->max_pages, kv->n_pages, l, nt, d.n_q_heads, d.n_kv_heads, q_scale, w.q, kv->pool,
-                           ctx->status);
+                const int qgrid = std::min(8 * ctx->n_sm, (nt * pf_qkv_groups(d.n_q_heads, d.n_kv_heads) + PF_QKV_THREADS / 32 - 1) / (PF_QKV_THREADS / 32));
+                auto post = d.head_dim == 128 ? pf_qkv_post_kernel<128> : pf_qkv_post_kernel<64>;
+                LAUNCH(ctx, post, qgrid, PF_QKV_THREADS, 0, st, pq, ctx->bqkv[l], ctx->q_norm[l], ctx->k_norm[l], eps, ctx->cos_tab,
+                       ctx->sin_tab, meta.game, meta.pos, kv->table_dev, kv->max_pages, kv->n_pages, l, nt, d.n_q_heads, d.n_kv_heads,
+                       q_scale, w.q, kv->pool, ctx->status);
             }
             {
                 AppendParams ap{};
@@ -1211,29 +1273,29 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
                            kv->pool_map, ap);
                 prof_end(ctx, rec, st);
             }
-            rec = prof_begin(ctx, SPIRAL_KC_O, st);
-            rc = pf_gemm<PF_EPI_ADD>(ctx->tc, ctx->wo[l], d.d_model, qd, w.attn, nt, w.x, nullptr, ctx->status, st,
-                                     &ctx->launches);
-            prof_end(ctx, rec, st);
-            if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
+            rc = project(SPIRAL_KC_O, pl_o, ctx->wo[l], qd, w.attn);
             if (rc) return rc;
-            rc = launch_rmsnorm_rows(ctx, w.x, ctx->ln2[l], nt, w.h, st);
+            rc = norm(ctx->ln2[l]);
             if (rc) return rc;
             rec = prof_begin(ctx, SPIRAL_KC_GATE_UP, st);
-            rc = pf_gemm<PF_EPI_SILU>(ctx->tc, ctx->w_gate_up[l], 2 * d.d_ff, d.d_model, w.h, nt, nullptr, w.act, ctx->status,
-                                      st, &ctx->launches);
-            prof_end(ctx, rec, st);
+            if (pl_gu.whole) {
+                rc = pg_gemm<PG_SILU>(ctx->tc, pl_gu, ctx->w_gate_up[l], 2 * d.d_ff, d.d_model, w.h, nt, w.act, nullptr, ctx->status, st,
+                                      &ctx->launches);
+                prof_end(ctx, rec, st);
+            } else {
+                Pieces pg;
+                rc = pg_gemm<PG_STORE>(ctx->tc, pl_gu, ctx->w_gate_up[l], 2 * d.d_ff, d.d_model, w.h, nt, w.y, &pg, ctx->status, st,
+                                       &ctx->launches);
+                prof_end(ctx, rec, st);
+                if (rc == SPIRAL_OK) LAUNCH(ctx, silu_mul_kernel, ctx->n_sm, SILU_THREADS, 0, st, pg, nt, d.d_ff, w.act);
+            }
             if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
             if (rc) return rc;
-            rec = prof_begin(ctx, SPIRAL_KC_DOWN, st);
-            rc = pf_gemm<PF_EPI_ADD>(ctx->tc, ctx->w_down[l], d.d_model, d.d_ff, w.act, nt, w.x, nullptr, ctx->status, st,
-                                     &ctx->launches);
-            prof_end(ctx, rec, st);
-            if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
+            rc = project(SPIRAL_KC_DOWN, pl_dn, ctx->w_down[l], d.d_ff, w.act);
             if (rc) return rc;
         }
         if (last_logits && n_pairs > 0)     // residual rows of the games' last new tokens, in game order
-            LAUNCH(ctx, gather_rows_kernel, n_pairs, 256, 0, st, (const float*)w.x, pairs_dev, MB, d.d_model, ctx->x);
+            LAUNCH(ctx, gather_rows_kernel, n_pairs, 256, 0, st, (const float*)w.x, pend, has, pairs_dev, MB, d.d_model, ctx->x);
     }
     if (last_logits) {
         LAUNCH(ctx, rmsnorm_kernel, n, rms_block(d.d_model), 0, st, ctx->x, none, 0, ctx->final_norm, eps, d.d_model, ctx->h);
@@ -1341,7 +1403,7 @@ __global__ void reduce_pieces_kernel(Pieces p, int rows, float* __restrict__ y) 
     grid_dependency_sync();
     int b = blockIdx.y;
     int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < rows) y[(size_t)b * rows + r] = piece_sum1(p, piece_count(p, r), b, r);
+    if (r < rows) y[(size_t)b * rows + r] = piece_sum1(p, piece_count(p, b, r), b, r);
 }
 
 extern "C" int spiral_linear(spiral_ctx* ctx, const void* w_dev, int rows, int k_dim, const void* x_dev, int n,
