@@ -28,8 +28,6 @@ constexpr int PG_BM = 2 * TC_BM;                     // weight rows per pair til
 constexpr int PG_MAX_N = 256;                        // token rows per pair tile
 constexpr int PG_THREADS = 192;
 constexpr int PG_MAX_STAGES = 8;
-constexpr int PG_OUT_ROWS = 32;                      // token rows per staging buffer
-constexpr int PG_OUT_BYTES = PG_OUT_ROWS * TC_BM * 4;
 constexpr size_t PG_SMEM_BUDGET = 227 * 1024 - 1024;           // less the static part (barriers)
 enum { PG_STORE = 0, PG_ADD = 1, PG_SILU = 2 };
 
@@ -128,7 +126,7 @@ __device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* map, uint32
                  ::"l"(map), "r"(src), "r"(x), "r"(y), "r"(z) : "memory");
 }
 
-// tmOut: STORE: [piece][T][rows] floats; ADD: [1][T][rows] floats; box 1 x 32 x 128.  SILU: [1][T][rows / 2] fp16, box 1 x 32 x 64.
+// tmOut: STORE: [piece][T][rows] floats; ADD: [1][T][rows] floats; box 1 x 32 x 32.  SILU: [1][T][rows / 2] fp16, box 1 x 32 x 16.
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
     pg_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
@@ -287,21 +285,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
             tc_fence_after();
             const int row0 = rt * PG_BM + (int)rank * TC_BM;
             const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16) + a * (uint32_t)N;
-            for (int c0 = 0; c0 < N && tt * N + c0 < p.T; c0 += PG_OUT_ROWS, ++out_it) {
+            for (int c0 = 0; c0 < N && tt * N + c0 < p.T; c0 += TC_OUT_ROWS, ++out_it) {
                 uint32_t v[2][16];
                 tmem_ld16_async(t_addr + (uint32_t)c0, v[0]);
                 tmem_ld16_async(t_addr + (uint32_t)(c0 + 16), v[1]);
-                const uint32_t buf = out_stage + (out_it & 1u) * PG_OUT_BYTES;
+                const uint32_t buf = out_stage + (uint32_t)(2 * q + (int)(out_it & 1u)) * TC_OUT_BYTES;
                 if (out_it >= 2) {
-                    if (threadIdx.x == 64) tma_store_wait_read<1>();
-                    asm volatile("bar.sync 1, 128;" ::: "memory");
+                    if (lane == 0) tma_store_wait_read<1>();
+                    __syncwarp();
                 }
                 tmem_ld_wait();
                 if (EPI == PG_SILU) {
                     // even lanes hold gate features, odd lanes the matching up features: per pair of token columns the
                     // even lane finishes the first and the odd lane the second
                     const bool odd = lane & 1;
-                    const uint32_t base = buf + (uint32_t)(q * 16 + (lane >> 1)) * 2u + (odd ? (uint32_t)TC_BM : 0u);
+                    const uint32_t base = buf + (uint32_t)(lane >> 1) * 2u + (odd ? 32u : 0u);
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -310,23 +308,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
                             const float got = __shfl_xor_sync(0xffffffffu, odd ? m0 : m1, 1);
                             const float gate = odd ? got : m0, up = odd ? m1 : got;
                             const unsigned short r = (unsigned short)float_to_f16_bits(__fdividef(gate, 1.f + __expf(-gate)) * up);
-                            asm volatile("st.shared.b16 [%0], %1;" ::"r"(base + (uint32_t)(16 * h + j) * (uint32_t)TC_BM), "h"(r) : "memory");
+                            asm volatile("st.shared.b16 [%0], %1;" ::"r"(base + (uint32_t)(16 * h + j) * 32u), "h"(r) : "memory");
                         }
                 } else {
-                    const uint32_t base = buf + (uint32_t)(q * 32 + lane) * 4u;
+                    const uint32_t base = buf + (uint32_t)lane * 4u;
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
 #pragma unroll
                         for (int j = 0; j < 16; ++j)
-                            asm volatile("st.shared.b32 [%0], %1;" ::"r"(base + (uint32_t)(16 * h + j) * (TC_BM * 4u)), "r"(v[h][j]) : "memory");
+                            asm volatile("st.shared.b32 [%0], %1;" ::"r"(base + (uint32_t)(16 * h + j) * 128u), "r"(v[h][j]) : "memory");
                 }
                 fence_proxy_async_smem();
-                asm volatile("bar.sync 1, 128;" ::: "memory");
-                if (threadIdx.x == 64) {
-                    const int y = tt * N + c0;
-                    if (EPI == PG_ADD) tma_reduce_add_3d(&tmOut, buf, row0, y, 0);
-                    else if (EPI == PG_SILU) tma_store_3d(&tmOut, buf, row0 >> 1, y, 0);
-                    else tma_store_3d(&tmOut, buf, row0, y, sg.piece);
+                __syncwarp();
+                if (lane == 0) {
+                    const int y = tt * N + c0, x = row0 + q * 32;
+                    if (EPI == PG_ADD) tma_reduce_add_3d(&tmOut, buf, x, y, 0);
+                    else if (EPI == PG_SILU) tma_store_3d(&tmOut, buf, x >> 1, y, 0);
+                    else tma_store_3d(&tmOut, buf, x, y, sg.piece);
                     tma_store_commit();
                 }
             }
@@ -335,7 +333,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
             if (lane == 0) mbar_arrive_cluster(release0 + 8u * a);
             if ((a ^= 1u) == 0u) aph ^= 1u;
         }
-        if (threadIdx.x == 64) tma_store_wait_all();
+        if (lane == 0) tma_store_wait_all();
     }
     tc_fence_before();
     __syncthreads();
@@ -374,14 +372,14 @@ inline PgPlan pg_plan(int n_sm, int rows, int K, int T, bool may_split) {
             pl.max_pieces = std::max(pl.max_pieces, streamk_cta_of(first + pl.KB - 1, pl.G, U) - streamk_cta_of(first, pl.G, U) + 1);
         }
     }
-    const size_t blk = TC_W_BYTES + (size_t)(pl.N / 2) * 128, budget = PG_SMEM_BUDGET - 1024 - 2 * PG_OUT_BYTES;
+    const size_t blk = TC_W_BYTES + (size_t)(pl.N / 2) * 128, budget = PG_SMEM_BUDGET - 1024 - TC_OUT_BUFS * TC_OUT_BYTES;
     pl.bps = 2;                                 // half as many barrier round trips per k block: 672 -> 615 us at T = 9984, 19456 x 2560
     pl.stages = (int)std::min<size_t>(PG_MAX_STAGES, budget / (pl.bps * blk));
-    pl.smem = (size_t)pl.stages * pl.bps * blk + 2 * PG_OUT_BYTES + 1024;
+    pl.smem = (size_t)pl.stages * pl.bps * blk + TC_OUT_BUFS * TC_OUT_BYTES + 1024;
     return pl;
 }
 
-// fp16 output [T][cols] with a 1 x 32 x 64 box (SILU epilogue)
+// fp16 output [T][cols] with a 1 x 32 x 16 box (SILU epilogue)
 inline int pg_get_actmap(TcState& tc, const __half* base, int cols, int T, const CUtensorMap** out) {
     auto key = std::make_tuple((const void*)base, cols, T, -1);
     auto it = tc.omaps.find(key);
@@ -390,7 +388,7 @@ inline int pg_get_actmap(TcState& tc, const __half* base, int cols, int T, const
         CUtensorMap m;
         cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)T, 1};
         cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)T * cols * 2};
-        cuuint32_t box[3] = {64, (cuuint32_t)PG_OUT_ROWS, 1};
+        cuuint32_t box[3] = {16, (cuuint32_t)TC_OUT_ROWS, 1};
         cuuint32_t estr[3] = {1, 1, 1};
         CUresult r = tc.encode(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half*>(base), dims, strides, box, estr,
                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,

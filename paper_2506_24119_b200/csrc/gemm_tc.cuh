@@ -15,8 +15,8 @@
 //               the epilogue adds the two chains.  Batches above 128 leave no room in TMEM for four
 //               accumulators and run with one issuer.
 //   warps 2..5  epilogue: tcgen05.ld of the finished accumulator, then either fp32 partial sums
-//               ("pieces") to memory -- transposed through two 16 KB shared-memory buffers and written
-//               by TMA stores, 32 batch rows x 128 features at a time -- or, for the LM head,
+//               ("pieces") to memory -- transposed through shared memory, two 4 KB buffers per warp, and written
+//               by TMA stores, 32 batch rows x 32 features at a time -- or, for the LM head,
 //               (logit / T + gumbel) and a running argmax
 // Work is the flattened (row tile, k block) space cut into equal contiguous ranges, one per CTA
 // (stream-K): a tile whose k range spans several CTAs yields several pieces, which the consumer
@@ -50,7 +50,8 @@ constexpr int TC_MAX_STAGES = 8;
 constexpr int TC_BPS = 2;             // default number of k blocks per ring stage
 constexpr int TC_W_BYTES = TC_BM * TC_BK * 2;
 constexpr int TC_OUT_ROWS = 32;                               // batch rows per TMA store of the pieces epilogue
-constexpr int TC_OUT_BYTES = TC_OUT_ROWS * TC_BM * 4;         // one staging buffer
+constexpr int TC_OUT_BYTES = TC_OUT_ROWS * 32 * 4;            // one staging buffer: 32 rows x the 32 features of a warp
+constexpr int TC_OUT_BUFS = 8;                                // two per epilogue warp
 
 struct TcSeg { int tile, kb0, kb1, piece; };
 
@@ -209,7 +210,7 @@ struct TcRun {
 // the kernel
 // ------------------------------------------------------------------------------------------------
 // tmOut (MODE 0 with p.tma_out): the pieces buffer as a tensor [piece][batch row][feature] of floats with a
-// box of 1 x 32 x 128
+// box of 1 x 32 x 32
 template <int MODE>     // 0: pieces to memory; 1: LM head with fused Gumbel-argmax
 // (register cap instead of launch bounds: at 112 registers the seven warps of a layer projection fit into an SM's
 // register file beside the CTA of the element-wise kernel before or after it, so that either can start early)
@@ -236,7 +237,7 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
     const uint32_t blk_bytes = TC_W_BYTES + (uint32_t)N * 128u;
     const uint32_t stage_bytes = (uint32_t)BPS * blk_bytes;
     const uint32_t ring = (smem_u32(tc_smem_raw) + 1023u) & ~1023u;
-    const uint32_t out_stage = ring + (uint32_t)S * stage_bytes;      // two staging buffers of the pieces epilogue
+    const uint32_t out_stage = ring + (uint32_t)S * stage_bytes;      // staging buffers of the pieces epilogue
     const int CH = p.chains;                    // accumulator (a, c): TMEM columns (a CH + c) N .. + N
     uint32_t tmem_cols = 32;
     while (tmem_cols < 2u * (uint32_t)CH * (uint32_t)N) tmem_cols <<= 1;
@@ -266,64 +267,71 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
     volatile int* abort_flag = &abort_sm;
 
     if (warp == 0) {
-        // ---------------- TMA producer ----------------
-        if (lane == 0) {
-            const uint64_t pol_w = l2_policy_evict_first(), pol_x = l2_policy_evict_last();
-            const TcRun run(p.tiles, p.KB, p.whole_tiles, blockIdx.x, gridDim.x);
-            const int n_stages = (run.count + BPS - 1) / BPS;
-            const uint32_t full0 = smem_u32(&full_bar[0]), done0 = smem_u32(&done_bar[0]);
-            // Weights are written by nobody: the W tiles of the first ring-full of stages are requested
-            // before the dependency wait, so that they stream in while the preceding kernel finishes.
-            int w_tile = run.y_tile, w_kb = run.kb0, w_in_tile = run.first_tile_blocks;     // next W block to request
-            auto next_w_row = [&]() {
-                const int y = w_tile + w_kb * TC_BM;
-                if (++w_kb == p.KB) w_kb = 0;
-                if (--w_in_tile == 0) { w_tile += p.KB * TC_BM; w_in_tile = p.KB; }
-                return y;
-            };
-            const int pre = n_stages < S ? n_stages : S;
-            for (int st = 0, left = run.count; st < pre; ++st) {
-                const int nb = left < BPS ? left : BPS;
-                const uint32_t fb = full0 + 8u * (uint32_t)st, dst = ring + (uint32_t)st * stage_bytes;
-                mbar_expect_tx(fb, (uint32_t)nb * blk_bytes);
-                for (int b = 0; b < nb; ++b) tma_load_2d(dst + (uint32_t)b * blk_bytes, &tmW, 0, next_w_row(), fb, pol_w);
-                left -= nb;
+        // ---------------- TMA producer (the whole warp walks the loop, one elected lane issues) ----------------
+        const uint64_t pol_w = l2_policy_evict_first(), pol_x = l2_policy_evict_last();
+        const TcRun run(p.tiles, p.KB, p.whole_tiles, blockIdx.x, gridDim.x);
+        const int n_stages = (run.count + BPS - 1) / BPS;
+        const uint32_t full0 = smem_u32(&full_bar[0]), done0 = smem_u32(&done_bar[0]);
+        // Weights are written by nobody: the W tiles of the first ring-full of stages are requested
+        // before the dependency wait, so that they stream in while the preceding kernel finishes.
+        int w_tile = run.y_tile, w_kb = run.kb0, w_in_tile = run.first_tile_blocks;     // next W block to request
+        auto next_w_row = [&]() {
+            const int y = w_tile + w_kb * TC_BM;
+            if (++w_kb == p.KB) w_kb = 0;
+            if (--w_in_tile == 0) { w_tile += p.KB * TC_BM; w_in_tile = p.KB; }
+            return y;
+        };
+        const int pre = n_stages < S ? n_stages : S;
+        for (int st = 0, left = run.count; st < pre; ++st) {
+            const int nb = left < BPS ? left : BPS;
+            const uint32_t fb = full0 + 8u * (uint32_t)st, dst = ring + (uint32_t)st * stage_bytes;
+            if (elect_one()) mbar_expect_tx(fb, (uint32_t)nb * blk_bytes);
+            for (int b = 0; b < nb; ++b) {
+                const int y = next_w_row();
+                if (elect_one()) tma_load_2d(dst + (uint32_t)b * blk_bytes, &tmW, 0, y, fb, pol_w);
             }
-            grid_dependency_wait();          // X is written by the preceding kernel
-            TC_STAMP(2);
-            TRACE_WAITED();
-            bool ok = true;
-            int x_col = run.kb0 * TC_BK, kb = run.kb0, left = run.count;
-            uint32_t s = 0, ph = 0;
-            int st = 0;
-            for (; st < n_stages; ++st) {
-                const int nb = left < BPS ? left : BPS;
-                const uint32_t fb = full0 + 8u * s, dst = ring + s * stage_bytes;
-                if (st >= S) {
-                    if (!mbar_wait(done0 + 8u * s, ph ^ 1u, abort_flag, p.status, STATUS_TIMEOUT_MMA)) {
-                        ok = false;
-                        break;
-                    }
-                    mbar_expect_tx(fb, (uint32_t)nb * blk_bytes);
-                    for (int b = 0; b < nb; ++b) tma_load_2d(dst + (uint32_t)b * blk_bytes, &tmW, 0, next_w_row(), fb, pol_w);
+            left -= nb;
+        }
+        grid_dependency_wait();          // X is written by the preceding kernel
+        if (threadIdx.x == 0) TC_STAMP(2);
+        TRACE_WAITED();
+        bool ok = true;
+        int x_col = run.kb0 * TC_BK, kb = run.kb0, left = run.count;
+        uint32_t s = 0, ph = 0;
+        int st = 0;
+        for (; st < n_stages; ++st) {
+            const int nb = left < BPS ? left : BPS;
+            const uint32_t fb = full0 + 8u * s, dst = ring + s * stage_bytes;
+            const bool with_w = st >= S;
+            if (with_w) {
+                if (!mbar_wait_warp(done0 + 8u * s, ph ^ 1u, abort_flag, p.status, STATUS_TIMEOUT_MMA)) {
+                    ok = false;
+                    break;
                 }
-                for (int b = 0; b < nb; ++b) {
-                    if (!p.skip_x) tma_load_2d(dst + (uint32_t)b * blk_bytes + TC_W_BYTES, &tmX, x_col, 0, fb, pol_x);
-                    x_col += TC_BK;
-                    if (++kb == p.KB) { kb = 0; x_col = 0; }
-                }
-                left -= nb;
-                if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
+                if (elect_one()) mbar_expect_tx(fb, (uint32_t)nb * blk_bytes);
             }
-            if (!ok) {
-                // copies already issued still land in this CTA's shared memory: give them a bounded
-                // time to complete before the CTA may exit
-                for (int back = 1; back <= S && back <= st; ++back) {
-                    const int j = st - back;
-                    const uint32_t sj = (uint32_t)(j % S), pj = (uint32_t)(j / S) & 1u;
-                    unsigned long long t1 = global_ns();
-                    while (!mbar_try(full0 + 8u * sj, pj) && global_ns() - t1 < g_wait_limit_ns) {}
+            for (int b = 0; b < nb; ++b) {
+                const uint32_t d = dst + (uint32_t)b * blk_bytes;
+                const int y = with_w ? next_w_row() : 0;
+                if (elect_one()) {
+                    if (with_w) tma_load_2d(d, &tmW, 0, y, fb, pol_w);
+                    if (!p.skip_x) tma_load_2d(d + TC_W_BYTES, &tmX, x_col, 0, fb, pol_x);
                 }
+                x_col += TC_BK;
+                if (++kb == p.KB) { kb = 0; x_col = 0; }
+            }
+            __syncwarp();
+            left -= nb;
+            if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
+        }
+        if (!ok && lane == 0) {
+            // copies already issued still land in this CTA's shared memory: give them a bounded
+            // time to complete before the CTA may exit
+            for (int back = 1; back <= S && back <= st; ++back) {
+                const int j = st - back;
+                const uint32_t sj = (uint32_t)(j % S), pj = (uint32_t)(j / S) & 1u;
+                unsigned long long t1 = global_ns();
+                while (!mbar_try(full0 + 8u * sj, pj) && global_ns() - t1 < g_wait_limit_ns) {}
             }
         }
     } else if (warp == 1 || warp == 2 + tc_epi_warps(MODE)) {
@@ -335,7 +343,7 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
         // completes when the MMAs of both chains have.  Waiting for the release also in segments an issuer adds
         // nothing to keeps it within one phase of the epilogue, which the parity waits rely on.
         const int id = warp == 1 ? 0 : 1;
-        if (lane == 0 && id < CH) {
+        if (id < CH) {
             const uint32_t idesc = tc_idesc_f16(N);
             const TcRun run(p.tiles, p.KB, p.whole_tiles, blockIdx.x, gridDim.x);
             const uint32_t full0 = smem_u32(&full_bar[0]), done0 = smem_u32(&done_bar[0]);
@@ -361,15 +369,15 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                 const bool mine = turn == id;
                 // (the other issuer's stages are waited for too: a parity wait is only sound for a thread that has
                 // seen every earlier phase of the barrier complete, and tiles need not land in the order requested)
-                if (!mbar_wait(full0 + 8u * s, ph, abort_flag, p.status, STATUS_TIMEOUT_TMA)) break;
+                if (!mbar_wait_warp(full0 + 8u * s, ph, abort_flag, p.status, STATUS_TIMEOUT_TMA)) break;
                 if (mine) tc_fence_after();
-                if (id == 0 && left == run.count) TC_STAMP(3);
+                if (id == 0 && lane == 0 && left == run.count) TC_STAMP(3);
                 if (seg_open && nb < in_tile && nb < left) {
                     // the whole stage lies inside the open segment and does not end it (all but one or two stages
                     // of a segment): no per-block bookkeeping
                     if (mine) {
-                        uint64_t da = d_cur;
-                        for (int b = 0; b < nb; ++b, da += d_blk) issue_block(da, (mine_open || b > 0) ? 1u : 0u);
+                        if (elect_one())
+                            for (int b = 0; b < nb; ++b) issue_block(d_cur + d_blk * (uint64_t)b, (mine_open || b > 0) ? 1u : 0u);
                         mine_open = true;
                     }
                     in_tile -= nb;
@@ -378,7 +386,7 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                     uint64_t da = d_cur;
                     for (int b = 0; b < nb; ++b, da += d_blk) {
                         if (!seg_open) {
-                            if (!mbar_wait(smem_u32(&acc_empty[a]), aph ^ 1u, abort_flag, p.status, STATUS_TIMEOUT_EPI)) {
+                            if (!mbar_wait_warp(smem_u32(&acc_empty[a]), aph ^ 1u, abort_flag, p.status, STATUS_TIMEOUT_EPI)) {
                                 ok = false;
                                 break;
                             }
@@ -386,23 +394,24 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                             seg_open = true;
                         }
                         if (mine) {
-                            issue_block(da, mine_open ? 1u : 0u);
+                            if (elect_one()) issue_block(da, mine_open ? 1u : 0u);
                             mine_open = true;
                         }
                         --left;
                         if (--in_tile == 0 || left == 0) {        // the tile (or this CTA's part of it) is complete
                             in_tile = p.KB;
-                            tc_commit(smem_u32(&acc_full[a]));
+                            if (elect_one()) tc_commit(smem_u32(&acc_full[a]));
                             seg_open = false;
                             mine_open = false;
                             if ((a ^= 1u) == 0) aph ^= 1u;
                             d_tmem = tmem_base + (a * (uint32_t)CH + (uint32_t)id) * (uint32_t)N;
-                            if (id == 0) TC_STAMP(4);
+                            if (id == 0 && lane == 0) TC_STAMP(4);
                         }
                     }
                     if (!ok) break;
                 }
-                if (mine) tc_commit(done0 + 8u * s);
+                if (mine && elect_one()) tc_commit(done0 + 8u * s);
+                __syncwarp();
                 d_cur += d_stage;
                 if (++s == (uint32_t)S) { s = 0; ph ^= 1u; d_cur = desc0; }
                 if (++turn == CH) turn = 0;
@@ -447,11 +456,11 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
             const uint32_t t_add = t_buf + (uint32_t)N;                                                 // the one added when both
             if (MODE == 0 && p.tma_out) {
                 // lane = feature, column = batch row.  32 batch rows at a time: every thread puts its feature's 32
-                // values into a [32 rows][128 features] buffer (a warp writes 128 contiguous bytes per row), one
-                // thread hands the buffer to the TMA unit, which writes whole rows of the piece and leaves out what
-                // lies beyond the last batch row or feature.  A buffer is refilled once the store that last used
-                // it has read it.
-                const uint32_t my_col = (uint32_t)(q * 32 + lane) * 4u;
+                // values into its warp's [32 rows][32 features] buffer (a warp writes 128 contiguous bytes per row),
+                // one lane hands the buffer to the TMA unit, which writes the rows of the piece and leaves out what
+                // lies beyond the last batch row or feature.  A warp has two buffers; one is refilled once the store
+                // that last used it has read it.  (Warps do not wait for each other: with one buffer of 128 features
+                // and two barriers of the four warps per 32 rows the epilogue took 1.1 us per tile.)
                 for (int c0 = 0; c0 < N && c0 < p.n; c0 += TC_OUT_ROWS, ++out_it) {
                     uint32_t v[2][16], w[2][16];
                     tmem_ld16_async(t_addr + (uint32_t)c0, v[0]);
@@ -460,10 +469,10 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                         tmem_ld16_async(t_add + (uint32_t)c0, w[0]);
                         if (c0 + 16 < N) tmem_ld16_async(t_add + (uint32_t)(c0 + 16), w[1]);
                     }
-                    const uint32_t buf = out_stage + (out_it & 1u) * TC_OUT_BYTES;
+                    const uint32_t buf = out_stage + (uint32_t)(2 * q + (int)(out_it & 1u)) * TC_OUT_BYTES;
                     if (out_it >= 2) {
-                        if (threadIdx.x == 64) tma_store_wait_read<1>();
-                        asm volatile("bar.sync 1, 128;" ::: "memory");
+                        if (lane == 0) tma_store_wait_read<1>();
+                        __syncwarp();
                     }
                     tmem_ld_wait();
 #pragma unroll
@@ -471,12 +480,12 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
                             const uint32_t val = both ? __float_as_uint(__fadd_rn(__uint_as_float(v[h][j]), __uint_as_float(w[h][j]))) : v[h][j];
-                            asm volatile("st.shared.b32 [%0], %1;" ::"r"(buf + (uint32_t)(16 * h + j) * (TC_BM * 4u) + my_col), "r"(val) : "memory");
+                            asm volatile("st.shared.b32 [%0], %1;" ::"r"(buf + (uint32_t)((16 * h + j) * 32 + lane) * 4u), "r"(val) : "memory");
                         }
                     fence_proxy_async_smem();
-                    asm volatile("bar.sync 1, 128;" ::: "memory");
-                    if (threadIdx.x == 64) {
-                        tma_store_3d(&tmOut, buf, sg.tile * TC_BM, c0, sg.piece);
+                    __syncwarp();
+                    if (lane == 0) {
+                        tma_store_3d(&tmOut, buf, sg.tile * TC_BM + q * 32, c0, sg.piece);
                         tma_store_commit();
                     }
                 }
@@ -616,7 +625,7 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
             }
         }
     }
-    if (MODE == 0 && threadIdx.x == 64) tma_store_wait_all();     // the staging buffers are read, the pieces written
+    if (MODE == 0 && warp >= 2 && warp < 6 && lane == 0) tma_store_wait_all();     // the staging buffers are read, the pieces written
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, tmem_cols);
@@ -878,7 +887,7 @@ inline int tc_get_xmap(TcState& tc, const void* X, int K, int x_rows, int N, con
 inline void tc_launch_shape(const TcState& tc, int N, TcParams* p, size_t* smem, bool lm_head = false) {
     // an SM's 227 KB less the static part (barriers; the LM head's argmax and log-sum-exp scratch), the alignment
     // slack and, for the pieces epilogue, its two staging buffers
-    const size_t tail = lm_head ? 0 : 2 * TC_OUT_BYTES;
+    const size_t tail = lm_head ? 0 : TC_OUT_BUFS * TC_OUT_BYTES;
     const size_t budget = 227 * 1024 - (lm_head ? 18 * 1024 : 1024) - 1024 - tail;
     const size_t blk_bytes = TC_W_BYTES + (size_t)N * 128;
     int bps = std::max(1, std::min(tc.bps, 4));
@@ -889,7 +898,7 @@ inline void tc_launch_shape(const TcState& tc, int N, TcParams* p, size_t* smem,
     *smem = (size_t)p->stages * bps * blk_bytes + 1024 + tail;
 }
 
-// the pieces buffer [pieces][n][rows] of floats as a 3-d tensor map with a box of 1 x 32 x 128 (rows % 4 == 0)
+// a buffer [pieces][n][rows] of floats as a 3-d tensor map with a box of 1 x 32 x 32 (rows % 4 == 0)
 inline int tc_get_omap(TcState& tc, const float* base, int rows, int n, int pieces, const CUtensorMap** out) {
     auto key = std::make_tuple((const void*)base, rows, n, pieces);
     auto it = tc.omaps.find(key);
@@ -898,7 +907,7 @@ inline int tc_get_omap(TcState& tc, const float* base, int rows, int n, int piec
         CUtensorMap m;
         cuuint64_t dims[3] = {(cuuint64_t)rows, (cuuint64_t)n, (cuuint64_t)pieces};
         cuuint64_t strides[2] = {(cuuint64_t)rows * 4, (cuuint64_t)n * rows * 4};
-        cuuint32_t box[3] = {(cuuint32_t)TC_BM, (cuuint32_t)TC_OUT_ROWS, 1};
+        cuuint32_t box[3] = {32, (cuuint32_t)TC_OUT_ROWS, 1};
         cuuint32_t estr[3] = {1, 1, 1};
         CUresult r = tc.encode(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims, strides, box, estr,
                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
