@@ -75,6 +75,21 @@ __device__ __forceinline__ float warp_max(float v) {
     return v;
 }
 
+// Thread-block clusters: rank in the cluster, barrier of all its threads, the same shared address in another CTA
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {       // the same shared address in another CTA
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+
 // Programmatic dependent launch: launch_dependents lets the next kernel of the stream start its
 // prologue (and prefetch data nobody writes, such as weights) while this one runs; wait blocks
 // until every kernel this one depends on has completed and its writes are visible.  Both are

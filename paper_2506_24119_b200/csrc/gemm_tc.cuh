@@ -506,6 +506,7 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                 }
             } else {
                 for (int c0 = cb; c0 < ce; c0 += 32) {       // two 16-column loads and 32 noise loads in flight
+                    uint32_t zm = 0u;                       // largest logit/T of column c0 + lane (ordered key; log-probabilities)
                     uint32_t km = 0u, kw = 0u;              // column c0 + lane over this warp's 32 rows: best score, rows that have it
                     uint32_t v[2][16], w[2][16];
                     float gm[2][16];
@@ -549,20 +550,39 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                             // memory is updated once per group, by all lanes together
                             if (lane == 16 * h + j) { km = m; kw = who; }
                             if (sa.logprob) {
-                                // running log-sum-exp of logit/T over the rows this warp has seen
+                                // exp(logit/T - the largest of this column's 32 rows); the columns are summed below
                                 const float zt = unit_t ? lg : __fdiv_rn(lg, sa.temperature);
                                 uint32_t uz = __float_as_uint(zt);
                                 uz = (!ok || zt != zt) ? 0u : ((uz & 0x80000000u) ? ~uz : (uz | 0x80000000u));
                                 const uint32_t mz = __reduce_max_sync(0xffffffffu, uz);
                                 const float mw = __uint_as_float((mz & 0x80000000u) ? (mz ^ 0x80000000u) : ~mz);
-                                float e = (ok && zt == zt) ? __expf(zt - mw) : 0.f;
-                                e = warp_sum(e);
-                                if (lane == (b & 31) && b < p.n && mz != 0u) {
-                                    const float m_old = lse_m[q][b], M = fmaxf(m_old, mw);
-                                    lse_s[q][b] = lse_s[q][b] * __expf(m_old - M) + e * __expf(mw - M);
-                                    lse_m[q][b] = M;
-                                }
+                                if (lane == 16 * h + j) zm = mz;
+                                v[h][j] = __float_as_uint((ok && zt == zt) ? __expf(zt - mw) : 0.f);
                             }
+                        }
+                    }
+                    if (sa.logprob) {
+                        // 32 columns x 32 rows (lanes) -> lane j holds the sum of column c0 + j: halves are exchanged so
+                        // that 31 shuffles do it (a reduction per column took five each and most of the epilogue's time:
+                        // the LM head of 213 rows 460 us with log-probabilities)
+                        float e[32];
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) e[j] = c0 + 16 * (j >> 4) < ce ? __uint_as_float(v[j >> 4][j & 15]) : 0.f;
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) {
+                            const bool up = lane & o;
+#pragma unroll
+                            for (int j = 0; j < o; ++j) {
+                                const float got = __shfl_xor_sync(0xffffffffu, up ? e[j] : e[j + o], o);
+                                e[j] = (up ? e[j + o] : e[j]) + got;
+                            }
+                        }
+                        const int b = c0 + lane;
+                        if (b < ce && b < p.n && zm != 0u) {
+                            const float mw = __uint_as_float((zm & 0x80000000u) ? (zm ^ 0x80000000u) : ~zm);
+                            const float m_old = lse_m[q][b], M = fmaxf(m_old, mw);
+                            lse_s[q][b] = lse_s[q][b] * __expf(m_old - M) + e[0] * __expf(mw - M);
+                            lse_m[q][b] = M;
                         }
                     }
                     const int bcol = c0 + lane;

@@ -523,116 +523,182 @@ __global__ void __launch_bounds__(1024) gumbel_argmax_kernel(const float* __rest
 // top_p (the smallest most-probable-first prefix reaching top_p, plus whatever ties its last
 // member; the most probable token is always kept), and the draw is argmax over the kept tokens of
 // z_v + gumbel_v, lowest index on ties -- a sample from the renormalised kept distribution.
-// The kept set is {v : key(z_v) >= K} for a threshold K on the order-preserving 32-bit keys of z,
-// found by a 16-way search: 8-9 passes over the row, each with 15 trial thresholds and a deterministic
-// block reduction of the mass above every one of them.  One CTA per batch row.
+// The kept set is {v : key(z_v) >= K} for a threshold K on the order-preserving 32-bit keys of z, found by a 16-way search:
+// each pass tries 15 thresholds inside what is left of the key range and looks only at the values in that range; the mass
+// above it is known from the pass before.  The first pass cuts at fixed distances below the maximum, which leaves a few
+// percent of the row; every thread then copies its values of the range to a short list, and the passes that follow (four
+// bits of the key each) read the lists.  A cluster of C CTAs works on one batch row, each with its slice of z in shared
+// memory; sums are exchanged through distributed shared memory and added in a fixed order, so every CTA takes the same
+// decisions and a call is reproducible.  Bound by latency (eight exchanges) and, in the first pass, by instruction issue.
+// (One CTA per row read the row from L2 eleven times and had 18 of 148 SMs at work for 18 rows: 450 us at 152 064 tokens.)
 __device__ __forceinline__ uint32_t ordered_key(float z) {          // larger float <=> larger key; NaN -> 0
     const uint32_t u = __float_as_uint(z);
     return z != z ? 0u : ((u & 0x80000000u) ? ~u : (u | 0x80000000u));
 }
-constexpr int NUCLEUS_THREADS = 1024;
+constexpr int NUCLEUS_THREADS = 512;
 constexpr int NUCLEUS_WAYS = 15;         // thresholds tried per pass of the search
-__device__ __forceinline__ float nucleus_block_sum(float v, float* red) {     // fixed order: same result every run
-    v = warp_sum(v);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    float tot = 0.f;
-#pragma unroll
-    for (int w = 0; w < NUCLEUS_THREADS / 32; ++w) tot += red[w];
-    return tot;
+constexpr int NUCLEUS_CLUSTER = 8;
+constexpr int NUCLEUS_ONE_CTA = 16384;   // rows up to this length take one CTA: the exchange would cost more than the scan
+constexpr int NUCLEUS_LIST = 8;          // values of the range a thread can list; more: the slice is scanned again
+constexpr int NUCLEUS_MAX_SLICE = 44 * 1024;      // floats of a slice kept in shared memory; longer slices are read again
+inline int nucleus_slice(int vocab, int C) { return (vocab + C - 1) / C; }
+inline size_t nucleus_smem(int vocab, int C) {
+    const int slice = nucleus_slice(vocab, C);
+    return (size_t)NUCLEUS_LIST * NUCLEUS_THREADS * sizeof(float) + (slice <= NUCLEUS_MAX_SLICE ? (size_t)slice * sizeof(float) : 0);
 }
-__global__ void __launch_bounds__(NUCLEUS_THREADS) nucleus_sample_kernel(const float* __restrict__ logits,
-                                                                         const StepArgs* __restrict__ args, int vocab) {
+
+template <int C>
+__global__ void __cluster_dims__(C, 1, 1) __launch_bounds__(NUCLEUS_THREADS, 2)
+    nucleus_sample_kernel(const float* __restrict__ logits, const StepArgs* __restrict__ args, int vocab, int cached) {
+    extern __shared__ float nucleus_sm[];
+    float* const list_sm = nucleus_sm + threadIdx.x;             // [NUCLEUS_LIST][threads]
+    float* const z_sm = nucleus_sm + NUCLEUS_LIST * NUCLEUS_THREADS;
+    constexpr int WARPS = NUCLEUS_THREADS / 32;
+    __shared__ float part_sm[WARPS][NUCLEUS_WAYS + 1];
+    __shared__ float xch_sm[2][C][NUCLEUS_WAYS + 1];             // what every CTA of the cluster contributes, two passes
+    __shared__ unsigned long long redk[WARPS], xchk_sm[C];
     grid_dependency_sync();
     const StepArgs sa = *args;
-    __shared__ float red[NUCLEUS_THREADS / 32];
-    __shared__ unsigned long long redk[NUCLEUS_THREADS / 32];
-    const int b = blockIdx.x;
-    const float* lg = logits + (size_t)b * vocab;
+    const int b = blockIdx.x / C, rank = C == 1 ? 0 : (int)cluster_rank();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int slice = (vocab + C - 1) / C, v0 = rank * slice, cnt = max(0, min(slice, vocab - v0));
+    const float* lg = logits + (size_t)b * vocab + v0;
     const float T = sa.temperature;
-    float mx = -INFINITY;
-    for (int v = threadIdx.x; v < vocab; v += NUCLEUS_THREADS) mx = fmaxf(mx, __fdiv_rn(lg[v], T));
-    mx = warp_max(mx);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    mx = red[0];
+    auto z_of = [&](int i) { return cached ? z_sm[i] : __fdiv_rn(lg[i], T); };
+    auto sync_all = [&]() {
+        if (C == 1) __syncthreads();
+        else cluster_sync();
+    };
+    int pass = 0;
+    // part_sm[warp][k], k < nk -> out(k, value of the whole row), with `add` folding two values
+    auto exchange = [&](int nk, auto add) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < nk * C; i += NUCLEUS_THREADS) {
+            const int k = i / C, to = i - k * C;
+            float t = part_sm[0][k];
+            for (int w = 1; w < WARPS; ++w) t = add(t, part_sm[w][k]);
+            if (C == 1) xch_sm[pass & 1][0][k] = t;
+            else
+                asm volatile("st.shared::cluster.f32 [%0], %1;"
+                             ::"r"(map_to_rank((uint32_t)__cvta_generic_to_shared(&xch_sm[pass & 1][rank][k]), (uint32_t)to)), "f"(t) : "memory");
+        }
+        sync_all();
+    };
+    auto total_of = [&](int k) {                     // after an exchange: every CTA adds in rank order
+        float t = xch_sm[pass & 1][0][k];
 #pragma unroll
-    for (int w = 1; w < NUCLEUS_THREADS / 32; ++w) mx = fmaxf(mx, red[w]);
-    float part = 0.f;
-    for (int v = threadIdx.x; v < vocab; v += NUCLEUS_THREADS) {
-        const float z = __fdiv_rn(lg[v], T);
-        if (z == z) part += __expf(z - mx);
+        for (int r = 1; r < C; ++r) t += xch_sm[pass & 1][r][k];
+        return t;
+    };
+    float mx = -INFINITY;
+#pragma unroll 8
+    for (int i = threadIdx.x; i < cnt; i += NUCLEUS_THREADS) {
+        const float z = __fdiv_rn(__ldcs(lg + i), T);
+        if (cached) z_sm[i] = z;
+        mx = fmaxf(mx, z);
     }
-    const float total = nucleus_block_sum(part, red);
-    const float target = sa.top_p * total;
-    const uint32_t key_max = ordered_key(mx);
-    uint32_t lo = 0u, hi = key_max;                  // the mass above key_max is zero: always below a positive target
+    mx = warp_max(mx);
+    if (lane == 0) part_sm[warp][0] = mx;
+    if (C > 1) cluster_sync();                       // every CTA has started: its shared memory may be written
+    exchange(1, [](float x, float y) { return fmaxf(x, y); });
+    mx = xch_sm[0][0][0];
+#pragma unroll
+    for (int r = 1; r < C; ++r) mx = fmaxf(mx, xch_sm[0][r][0]);
+    ++pass;
+    auto plus = [](float x, float y) { return x + y; };
+    uint32_t lo = 0u, hi = ordered_key(mx);          // the mass above the maximum is zero: always below a positive target
+    float base = 0.f, target = 0.f;                  // mass of the keys above hi; top_p of the whole mass
     if (!(sa.top_p < 1.f)) hi = 0u;                  // top_p >= 1: keep everything
-    // Each pass over the row tries 15 thresholds that cut [lo, hi] into 16 parts (four bits of the key per
-    // pass: 8-9 passes instead of 32), each threshold with its own fixed-order sum.
-    __shared__ float part_sm[NUCLEUS_THREADS / 32][NUCLEUS_WAYS];
-    __shared__ float tot_sm[NUCLEUS_WAYS];
-    while (lo < hi) {
+    int listed = -1;                                 // values on this thread's list; -1: it scans its slice
+    for (bool first_pass = true; lo < hi; first_pass = false) {
+        uint32_t cut[NUCLEUS_WAYS];                  // ascending, in [lo, hi)
+        float above[NUCLEUS_WAYS], all = 0.f;
         const uint32_t span = hi - lo;
-        uint32_t cut[NUCLEUS_WAYS];
-        float above[NUCLEUS_WAYS];
 #pragma unroll
         for (int k = 0; k < NUCLEUS_WAYS; ++k) {
-            cut[k] = lo + (uint32_t)(((unsigned long long)span * (unsigned)(k + 1)) >> 4);       // in [lo, hi)
+            constexpr float below_max[NUCLEUS_WAYS] = {20.f, 15.f, 12.f, 10.f, 9.f, 8.f, 7.f, 6.f, 5.f, 4.f, 3.f, 2.f, 1.5f, 1.f, 0.5f};
+            cut[k] = first_pass ? min(hi - 1u, ordered_key(mx - below_max[k]))
+                                : lo + (uint32_t)(((unsigned long long)span * (unsigned)(k + 1)) >> 4);
             above[k] = 0.f;
         }
-        for (int v = threadIdx.x; v < vocab; v += NUCLEUS_THREADS) {
-            const float z = __fdiv_rn(lg[v], T);
+        auto count = [&](float z) {
             const uint32_t key = ordered_key(z);
-            if (key > lo) {                         // below every threshold otherwise (and NaN: key 0)
+            if (key > lo && key <= hi) {             // below every threshold or above the range otherwise (and NaN: key 0)
                 const float e = __expf(z - mx);
+                if (first_pass) all += e;
 #pragma unroll
                 for (int k = 0; k < NUCLEUS_WAYS; ++k) above[k] += key > cut[k] ? e : 0.f;
             }
-        }
+        };
+        if (listed >= 0)
+            for (int i = 0; i < listed; ++i) count(list_sm[i * NUCLEUS_THREADS]);
+        else
+#pragma unroll 2
+            for (int i = threadIdx.x; i < cnt; i += NUCLEUS_THREADS) count(z_of(i));
 #pragma unroll
-        for (int k = 0; k < NUCLEUS_WAYS; ++k) above[k] = warp_sum(above[k]);
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-            for (int k = 0; k < NUCLEUS_WAYS; ++k) part_sm[threadIdx.x >> 5][k] = above[k];
+        for (int k = 0; k < NUCLEUS_WAYS; ++k) {
+            const float t = warp_sum(above[k]);
+            if (lane == 0) part_sm[warp][k] = t;
         }
-        __syncthreads();
-        if (threadIdx.x < NUCLEUS_WAYS) {
-            float tot = 0.f;
-            for (int w = 0; w < NUCLEUS_THREADS / 32; ++w) tot += part_sm[w][threadIdx.x];
-            tot_sm[threadIdx.x] = tot;
+        if (first_pass) {
+            all = warp_sum(all);
+            if (lane == 0) part_sm[warp][NUCLEUS_WAYS] = all;
         }
-        __syncthreads();
+        exchange(first_pass ? NUCLEUS_WAYS + 1 : NUCLEUS_WAYS, plus);
+        if (first_pass) target = sa.top_p * total_of(NUCLEUS_WAYS);
         // the smallest threshold whose mass above is below the target becomes the new upper end
-        int first = NUCLEUS_WAYS;
+        uint32_t lo_new = cut[NUCLEUS_WAYS - 1] + 1u, hi_new = hi;
+        float mass = base;
 #pragma unroll
-        for (int k = NUCLEUS_WAYS - 1; k >= 0; --k)
-            if (tot_sm[k] < target) first = k;
-        if (first < NUCLEUS_WAYS) hi = cut[first];
-        if (first > 0) lo = cut[first - 1] + 1u;
+        for (int k = NUCLEUS_WAYS - 1; k >= 0; --k) {
+            const float m = base + total_of(k);
+            if (m < target) { hi_new = cut[k]; mass = m; lo_new = k > 0 ? cut[k > 0 ? k - 1 : 0] + 1u : lo; }
+        }
+        lo = min(lo_new, hi_new); hi = hi_new; base = mass;      // (equal thresholds of the first pass)
+        ++pass;
+        if (listed < 0 && lo < hi) {
+            int c = 0;
+#pragma unroll 4
+            for (int i = threadIdx.x; i < cnt; i += NUCLEUS_THREADS) {
+                const float z = z_of(i);
+                const uint32_t key = ordered_key(z);
+                if (key > lo && key <= hi) {
+                    if (c < NUCLEUS_LIST) list_sm[c * NUCLEUS_THREADS] = z;
+                    ++c;
+                }
+            }
+            if (c <= NUCLEUS_LIST) listed = c;
+        }
     }
     const uint32_t K = lo;
-    const float* gm = sa.gumbel ? sa.gumbel + (size_t)b * vocab : nullptr;
+    const float* gm = sa.gumbel ? sa.gumbel + (size_t)b * vocab + v0 : nullptr;
     unsigned long long best = 0ull;
-    for (int v = threadIdx.x; v < vocab; v += NUCLEUS_THREADS) {
-        const float z = __fdiv_rn(lg[v], T);
-        if (ordered_key(z) >= K && z == z) {
-            const unsigned long long k = argmax_key(__fadd_rn(z, gm ? gm[v] : 0.f), v);
-            best = k > best ? k : best;
-        }
+#pragma unroll 8
+    for (int i = threadIdx.x; i < cnt; i += NUCLEUS_THREADS) {
+        const float z = z_of(i);
+        const bool kept = ordered_key(z) >= K && z == z;
+        const float g = (gm && kept) ? __ldg(gm + i) : 0.f;
+        const unsigned long long k = kept ? argmax_key(__fadd_rn(z, g), v0 + i) : 0ull;
+        best = k > best ? k : best;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
         best = other > best ? other : best;
     }
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) redk[threadIdx.x >> 5] = best;
+    if (lane == 0) redk[warp] = best;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < NUCLEUS_THREADS / 32; ++w) best = redk[w] > best ? redk[w] : best;
+        for (int w = 1; w < WARPS; ++w) best = redk[w] > best ? redk[w] : best;
+        if (C == 1) xchk_sm[0] = best;
+        else
+            asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(map_to_rank((uint32_t)__cvta_generic_to_shared(&xchk_sm[rank]), 0u)), "l"(best) : "memory");
+    }
+    sync_all();
+    if (rank == 0 && threadIdx.x == 0) {
+        best = xchk_sm[0];
+#pragma unroll
+        for (int r = 1; r < C; ++r) best = xchk_sm[r] > best ? xchk_sm[r] : best;
         if (sa.tok_out) sa.tok_out[b] = argmax_key_index(best);
     }
 }

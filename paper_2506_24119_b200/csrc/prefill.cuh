@@ -641,39 +641,42 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
             }
         }
     } else if (warp == 1 || (TILES == 2 && warp == APT_THREADS / 32 - 1)) {
-        // ---------------- MMA issuers: one thread per tile (issuing is serial work per thread) ----------------
+        // ---------------- MMA issuers: one warp per tile (the whole warp walks the loop, one elected lane issues) ----------------
         const int t = warp == 1 ? 0 : 1;
-        if (lane == 0 && t < n_tiles) {
+        if (t < n_tiles) {
             const uint32_t idesc_qk = tc_idesc_f16(APT_BN);
             const uint32_t idesc_pv = tc_idesc_f16(HD) | (1u << 16);          // B (V) is MN-major
 #ifdef APT_PROBE
-            const bool probe_on = t == 0;
+            const bool probe_on = t == 0 && lane == 0;
             long long probe_t = clock64();
 #endif
-            bool ok = mbar_wait(smem_u32(&q_ready), 0u, abort_flag, p.status, STATUS_TIMEOUT_EPI);
-            APT_STAMP(6);           // MMA thread: wait for Q
+            bool ok = mbar_wait_warp(smem_u32(&q_ready), 0u, abort_flag, p.status, STATUS_TIMEOUT_EPI);
+            APT_STAMP(6);           // MMA warp: wait for Q
+            const uint64_t da0 = smem_desc_sw128(q_base + (uint32_t)t * Q_TILE);
+            const uint64_t dp = smem_desc_sw128(p_base + (uint32_t)t * P_TILE);
             auto issue_qk = [&](int j) -> bool {
                 const int s = j % APT_STAGES, b = j & 1;
-                if (!mbar_wait(smem_u32(&kv_full[s]), (uint32_t)(j / APT_STAGES) & 1u, abort_flag, p.status, STATUS_TIMEOUT_TMA))
+                if (!mbar_wait_warp(smem_u32(&kv_full[s]), (uint32_t)(j / APT_STAGES) & 1u, abort_flag, p.status, STATUS_TIMEOUT_TMA))
                     return false;
-                APT_STAMP(7);       // MMA thread: wait for K/V
-                if (j >= 2 && !mbar_wait(smem_u32(&s_empty[t][b]), (uint32_t)((j >> 1) - 1) & 1u, abort_flag, p.status,
-                                         STATUS_TIMEOUT_EPI))
+                APT_STAMP(7);       // MMA warp: wait for K/V
+                if (j >= 2 && !mbar_wait_warp(smem_u32(&s_empty[t][b]), (uint32_t)((j >> 1) - 1) & 1u, abort_flag, p.status,
+                                              STATUS_TIMEOUT_EPI))
                     return false;
-                APT_STAMP(8);       // MMA thread: wait for the S buffer
+                APT_STAMP(8);       // MMA warp: wait for the S buffer
                 tc_fence_after();
-                const uint32_t kst = ring + (uint32_t)s * STAGE_BYTES;
+                const uint64_t db0 = smem_desc_sw128(ring + (uint32_t)s * STAGE_BYTES);
+                const uint32_t d_s = tmem_base + (uint32_t)((2 * t + b) * APT_BN);
+                if (elect_one()) {
 #pragma unroll
-                for (int h = 0; h < SLABS; ++h) {
-                    const uint64_t da = smem_desc_sw128(q_base + (uint32_t)t * Q_TILE + h * APT_QSLAB);
-                    const uint64_t db = smem_desc_sw128(kst + h * APT_KSLAB);
+                    for (int h = 0; h < SLABS; ++h)
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        tc_mma_f16(tmem_base + (uint32_t)((2 * t + b) * APT_BN), da + (uint64_t)(2 * k), db + (uint64_t)(2 * k),
-                                   idesc_qk, (h > 0 || k > 0) ? 1u : 0u);
+                        for (int k = 0; k < 4; ++k)
+                            tc_mma_f16(d_s, da0 + (uint64_t)(h * (APT_QSLAB >> 4) + 2 * k), db0 + (uint64_t)(h * (APT_KSLAB >> 4) + 2 * k),
+                                       idesc_qk, (h > 0 || k > 0) ? 1u : 0u);
+                    tc_commit(smem_u32(&s_full[t][b]));
                 }
-                tc_commit(smem_u32(&s_full[t][b]));
-                APT_STAMP(9);       // MMA thread: issue of Q.K
+                __syncwarp();
+                APT_STAMP(9);       // MMA warp: issue of Q.K
                 return true;
             };
             ok = ok && issue_qk(0);
@@ -681,21 +684,23 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                 if (j + 1 < n_blk && !issue_qk(j + 1)) break;
                 const int s = j % APT_STAGES;
                 const int npg = min(APT_PAGES, n_pg - APT_PAGES * j);
-                const uint32_t vst = ring + (uint32_t)s * STAGE_BYTES + KV_BYTES;
-                const uint64_t dv = smem_desc_sw128_mn(vst, APT_KSLAB, 1024u);
-                if (!mbar_wait(smem_u32(&p_full[t]), (uint32_t)j & 1u, abort_flag, p.status, STATUS_TIMEOUT_EPI)) break;
+                const uint64_t dv = smem_desc_sw128_mn(ring + (uint32_t)s * STAGE_BYTES + KV_BYTES, APT_KSLAB, 1024u);
+                if (!mbar_wait_warp(smem_u32(&p_full[t]), (uint32_t)j & 1u, abort_flag, p.status, STATUS_TIMEOUT_EPI)) break;
                 tc_fence_after();
-                APT_STAMP(10);      // MMA thread: wait for P
-                const uint64_t dp = smem_desc_sw128(p_base + (uint32_t)t * P_TILE);
-                for (int ks = 0; ks < npg; ++ks)             // one page = 16 keys = one k step
-                    tc_mma_f16(tmem_base + TM_O + (uint32_t)(t * HD), dp + (uint64_t)(2 * ks),
-                               dv + (uint64_t)(ks * (PAGE_ROWS_BYTES >> 4)), idesc_pv, (j > 0 || ks > 0) ? 1u : 0u);
-                tc_commit(smem_u32(&o_full[t]));
-                tc_commit(smem_u32(&p_empty[t]));
-                // the stage is free once both tiles' MMAs on it have completed (one tile: it arrives for both)
-                tc_commit(smem_u32(&kv_empty[s]));
-                if (TILES == 2 && n_tiles == 1) tc_commit(smem_u32(&kv_empty[s]));
-                APT_STAMP(11);      // MMA thread: issue of P.V
+                APT_STAMP(10);      // MMA warp: wait for P
+                if (elect_one()) {
+                    const uint32_t d_o = tmem_base + TM_O + (uint32_t)(t * HD);
+                    for (int ks = 0; ks < npg; ++ks)             // one page = 16 keys = one k step
+                        tc_mma_f16(d_o, dp + (uint64_t)(2 * ks), dv + (uint64_t)(ks * (PAGE_ROWS_BYTES >> 4)), idesc_pv,
+                                   (j > 0 || ks > 0) ? 1u : 0u);
+                    tc_commit(smem_u32(&o_full[t]));
+                    tc_commit(smem_u32(&p_empty[t]));
+                    // the stage is free once both tiles' MMAs on it have completed (one tile: it arrives for both)
+                    tc_commit(smem_u32(&kv_empty[s]));
+                    if (TILES == 2 && n_tiles == 1) tc_commit(smem_u32(&kv_empty[s]));
+                }
+                __syncwarp();
+                APT_STAMP(11);      // MMA warp: issue of P.V
             }
         }
     } else {

@@ -339,8 +339,12 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
         return SPIRAL_ERR_CUDA;
     }
     {
-        const int attn_smem = (int)attn_smem_bytes(128, 8);
-        e = cudaFuncSetAttribute(attn_decode_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_smem);
+        const int attn_smem = (int)attn_smem_bytes(128, 8), nuc_smem = (NUCLEUS_MAX_SLICE + NUCLEUS_LIST * NUCLEUS_THREADS) * (int)sizeof(float);
+        e = cudaFuncSetAttribute(nucleus_sample_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, nuc_smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(nucleus_sample_kernel<NUCLEUS_CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize, nuc_smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(attn_decode_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(attn_decode_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_smem);
         if (e == cudaSuccess)
@@ -796,6 +800,14 @@ static int run_head(spiral_ctx* c, int n, cudaStream_t st) {
     return rc;
 }
 
+static int launch_nucleus(spiral_ctx* c, int n, const float* logits, cudaStream_t st) {
+    const int V = c->d.vocab, C = V <= NUCLEUS_ONE_CTA ? 1 : NUCLEUS_CLUSTER;
+    const size_t smem = nucleus_smem(V, C);
+    auto kern = C == 1 ? nucleus_sample_kernel<1> : nucleus_sample_kernel<NUCLEUS_CLUSTER>;
+    LAUNCH(c, kern, n * C, NUCLEUS_THREADS, smem, st, logits, meta_args(c), V, nucleus_slice(V, C) <= NUCLEUS_MAX_SLICE ? 1 : 0);
+    return SPIRAL_OK;
+}
+
 // Launch sequences of a decode step (each with its own recorded graph per batch size)
 enum StepVariant { STEP_FUSED_SAMPLER = 0, STEP_NUCLEUS = 1, STEP_LAYERS_ONLY = 2 };
 
@@ -806,8 +818,7 @@ static int run_step_body(spiral_ctx* c, spiral_kv* kv, int n, int variant, cudaS
     rc2 = run_head(c, n, st);
     if (rc2 || !nucleus) return rc2;
     // the LM head left the logits in ctx->logits (StepArgs.defer_sampling): draw from the nucleus
-    LAUNCH(c, nucleus_sample_kernel, n, NUCLEUS_THREADS, 0, st, (const float*)c->logits, meta_args(c), c->d.vocab);
-    return SPIRAL_OK;
+    return launch_nucleus(c, n, c->logits, st);
 }
 
 // One decode step for n slots whose metadata and StepArgs are already on their way to the device.
@@ -979,8 +990,7 @@ extern "C" int spiral_sample_nucleus(spiral_ctx* ctx, int n, const float* logits
     sa->gumbel = gumbel_dev; sa->tok_out = tok_out_dev; sa->temperature = temperature; sa->top_p = top_p;
     int rc = meta_upload(ctx, slot, st);
     if (rc) return rc;
-    LAUNCH(ctx, nucleus_sample_kernel, n, NUCLEUS_THREADS, 0, st, logits_dev, meta_args(ctx), ctx->d.vocab);
-    return SPIRAL_OK;
+    return launch_nucleus(ctx, n, logits_dev, st);
 }
 
 // Role-conditioned advantage estimation: host arithmetic, no device work.
@@ -1156,7 +1166,6 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
     StepMeta meta{mdev, mdev + cap, mdev + 2 * (size_t)cap, mdev + 3 * (size_t)cap};
     const int32_t* pairs_dev = mdev + 4 * (size_t)cap;
     const float q_scale = (float)(1.4426950408889634 / std::sqrt((double)d.head_dim));
-    Pieces none{};
 
     int gi = 0, gt = 0;
     while (gi < n) {
@@ -1298,6 +1307,7 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
             LAUNCH(ctx, gather_rows_kernel, n_pairs, 256, 0, st, (const float*)w.x, pend, has, pairs_dev, MB, d.d_model, ctx->x);
     }
     if (last_logits) {
+        Pieces none{};
         LAUNCH(ctx, rmsnorm_kernel, n, rms_block(d.d_model), 0, st, ctx->x, none, 0, ctx->final_norm, eps, d.d_model, ctx->h);
         rc = run_head(ctx, n, st);
         if (rc) return rc;
