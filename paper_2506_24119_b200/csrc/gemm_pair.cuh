@@ -28,6 +28,7 @@ constexpr int PG_BM = 2 * TC_BM;                     // weight rows per pair til
 constexpr int PG_MAX_N = 256;                        // token rows per pair tile
 constexpr int PG_THREADS = 192;
 constexpr int PG_MAX_STAGES = 8;
+constexpr int PG_BPS = 2;                            // k blocks per stage = per TMA box
 constexpr size_t PG_SMEM_BUDGET = 227 * 1024 - 1024;           // less the static part (barriers)
 enum { PG_STORE = 0, PG_ADD = 1, PG_SILU = 2 };
 
@@ -35,7 +36,8 @@ struct PgParams {
     int row_tiles, tok_tiles, KB;   // 256-row tiles of W, N-row tiles of X, 64-wide k blocks
     int T, N;                       // token rows; token rows per tile
     int whole, row_fastest;         // whole tiles or stream-K; order of whole tiles (see pg_tile_of)
-    int stages, bps;                // ring depth, k blocks per stage
+    int stages;                     // ring depth
+    int w_once;                     // 1: weight tiles are read by few token tiles and leave L2 first
     int* status;
 };
 
@@ -107,6 +109,12 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         " [%0], [%1, {%2, %3}], [%4], %5;"
         ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(leader_bar), "l"(policy) : "memory");
 }
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t leader_bar, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+        " [%0], [%1, {%2, %3, %4}], [%5], %6;"
+        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(z), "r"(leader_bar), "l"(policy) : "memory");
+}
 // element-wise addition of a dense fp32 box in shared memory to global memory (same rules as tma_store_3d)
 __device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* map, uint32_t src, int x, int y, int z) {
     asm volatile("cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4}], [%1];"
@@ -127,9 +135,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
     const uint32_t rank = cluster_rank();
     const int pair = (int)(blockIdx.x >> 1), G = (int)(gridDim.x >> 1);
     grid_launch_dependents();
-    const int S = p.stages, BPS = p.bps, N = p.N;
-    const uint32_t x_bytes = (uint32_t)(N / 2) * 128u, blk_bytes = TC_W_BYTES + x_bytes;
-    const uint32_t stage_bytes = (uint32_t)BPS * blk_bytes;
+    constexpr int BPS = PG_BPS;
+    const int S = p.stages, N = p.N;
+    // a stage: the W halves of PG_BPS k blocks, then their X halves, each group one TMA box
+    const uint32_t x_bytes = (uint32_t)(N / 2) * 128u, stage_bytes = PG_BPS * (TC_W_BYTES + x_bytes);
     const uint32_t ring = (smem_u32(pg_smem_raw) + 1023u) & ~1023u;
     const uint32_t out_stage = ring + (uint32_t)S * stage_bytes;
     uint32_t tmem_cols = 32;
@@ -154,7 +163,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
 
     if (warp == 0) {
         // ---------------- TMA producer (the whole warp walks the loop, one elected lane issues) ----------------
-        const uint64_t pol_w = l2_policy_evict_last(), pol_x = l2_policy_evict_last();
+        const uint64_t pol_w = p.w_once ? l2_policy_evict_first() : l2_policy_evict_last(), pol_x = l2_policy_evict_last();
         const uint32_t full_leader = map_to_rank(smem_u32(&full_bar[0]), 0), full_own = smem_u32(&full_bar[0]);
         const uint32_t empty_own = smem_u32(&empty_bar[0]);
         const int n_tiles = p.row_tiles * p.tok_tiles;
@@ -168,18 +177,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
             while (more && pre < S) {
                 int rt, tt;
                 pg_tile_of(sg.tile, p, rt, tt);
-                const int nb = min(BPS, sg.kb1 - kb);            // a stage never crosses a segment
+                // (a stage never crosses a segment: where one has an odd number of blocks, its last stage fetches a block
+                // that is not used)
                 const int y_w = ((2 * rt + (int)rank) * p.KB + kb) * TC_BM;
                 const uint32_t dst = ring + (uint32_t)pre * stage_bytes;
                 if (elect_one()) {
-                    if (rank == 0) mbar_expect_tx(full_own + 8u * (uint32_t)pre, 2u * (uint32_t)nb * blk_bytes);
-                    for (int b = 0; b < nb; ++b)
-                        tma_load_2d_pair(dst + (uint32_t)b * blk_bytes, &tmW, 0, y_w + b * TC_BM, full_leader + 8u * (uint32_t)pre, pol_w);
+                    if (rank == 0) mbar_expect_tx(full_own + 8u * (uint32_t)pre, 2u * stage_bytes);
+                    tma_load_2d_pair(dst, &tmW, 0, y_w, full_leader + 8u * (uint32_t)pre, pol_w);
                 }
                 __syncwarp();
                 ++pre;
-                kb += nb;
-                if (kb == sg.kb1) { more = sched.next(sg); kb = more ? sg.kb0 : 0; }
+                kb += BPS;
+                if (kb >= sg.kb1) { more = sched.next(sg); kb = more ? sg.kb0 : 0; }
             }
         }
         grid_dependency_wait();                                  // X is written by the preceding kernel
@@ -193,17 +202,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
             pg_tile_of(sg.tile, p, rt, tt);
             const int y_x = tt * N + (int)rank * (N / 2), y_w0 = (2 * rt + (int)rank) * p.KB * TC_BM;
             for (int kb = sg.kb0; kb < sg.kb1; kb += BPS, ++st) {
-                const int nb = min(BPS, sg.kb1 - kb);
                 const uint32_t dst = ring + s * stage_bytes, fb = full_leader + 8u * s;
                 const bool with_w = st >= pre;
                 if (with_w && !mbar_wait_warp(empty_own + 8u * s, ph ^ 1u, abort_flag, p.status, STATUS_TIMEOUT_MMA)) { ok = false; break; }
                 if (elect_one()) {
-                    if (with_w && rank == 0) mbar_expect_tx(full_own + 8u * s, 2u * (uint32_t)nb * blk_bytes);
-                    for (int b = 0; b < nb; ++b) {
-                        const uint32_t d = dst + (uint32_t)b * blk_bytes;
-                        if (with_w) tma_load_2d_pair(d, &tmW, 0, y_w0 + (kb + b) * TC_BM, fb, pol_w);
-                        tma_load_2d_pair(d + TC_W_BYTES, &tmX, (kb + b) * TC_BK, y_x, fb, pol_x);
+                    if (with_w) {
+                        if (rank == 0) mbar_expect_tx(full_own + 8u * s, 2u * stage_bytes);
+                        tma_load_2d_pair(dst, &tmW, 0, y_w0 + kb * TC_BM, fb, pol_w);
                     }
+                    tma_load_3d_pair(dst + PG_BPS * TC_W_BYTES, &tmX, 0, y_x, kb, fb, pol_x);
                 }
                 __syncwarp();
                 if (++s == (uint32_t)S) { s = 0; ph ^= 1u; }
@@ -223,7 +230,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
         if (rank == 0) {
             const uint32_t idesc = (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(PG_BM >> 4) << 24);
             const uint64_t desc0 = smem_desc_sw128(ring);
-            const uint64_t d_blk = (uint64_t)(blk_bytes >> 4), d_stage = (uint64_t)(stage_bytes >> 4);
+            const uint64_t d_x0 = (uint64_t)((PG_BPS * TC_W_BYTES) >> 4), d_x = (uint64_t)(x_bytes >> 4), d_stage = (uint64_t)(stage_bytes >> 4);
             PgSchedule sched(p.row_tiles * p.tok_tiles, p.KB, p.whole, pair, G);
             PgSeg sg;
             uint32_t s = 0, ph = 0, a = 0, aph = 0;
@@ -240,7 +247,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
                     const uint64_t da = desc0 + d_stage * s;
                     if (elect_one()) {
                         for (int b = 0; b < nb; ++b) {
-                            const uint64_t dab = da + d_blk * (uint64_t)b, db = dab + (uint64_t)(TC_W_BYTES >> 4);
+                            const uint64_t dab = da + (uint64_t)(b * (TC_W_BYTES >> 4)), db = da + d_x0 + d_x * (uint64_t)b;
 #pragma unroll
                             for (int k = 0; k < TC_BK / 16; ++k)
                                 tc_mma_f16_pair(d_tmem, dab + (uint64_t)(2 * k), db + (uint64_t)(2 * k), idesc,
@@ -330,7 +337,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
 
 // ---- host side -----------------------------------------------------------------------------------
 struct PgPlan {
-    int N = 0, tok_tiles = 0, row_tiles = 0, KB = 0, G = 0, whole = 1, max_pieces = 1, stages = 0, bps = 1;
+    int N = 0, tok_tiles = 0, row_tiles = 0, KB = 0, G = 0, whole = 1, max_pieces = 1, stages = 0;
     size_t smem = 0;
 };
 
@@ -360,10 +367,52 @@ inline PgPlan pg_plan(int n_sm, int rows, int K, int T, bool may_split) {
         }
     }
     const size_t blk = TC_W_BYTES + (size_t)(pl.N / 2) * 128, budget = PG_SMEM_BUDGET - 1024 - TC_OUT_BUFS * TC_OUT_BYTES;
-    pl.bps = 2;                                 // half as many barrier round trips per k block: 672 -> 615 us at T = 9984, 19456 x 2560
-    pl.stages = (int)std::min<size_t>(PG_MAX_STAGES, budget / (pl.bps * blk));
-    pl.smem = (size_t)pl.stages * pl.bps * blk + TC_OUT_BUFS * TC_OUT_BYTES + 1024;
+    pl.stages = (int)std::min<size_t>(PG_MAX_STAGES, budget / (PG_BPS * blk));
+    pl.smem = (size_t)pl.stages * PG_BPS * blk + TC_OUT_BUFS * TC_OUT_BYTES + 1024;
     return pl;
+}
+
+// a tensor of fp16 values as [outer][mid][64] with a box of box_outer x box_mid x 64, 128-byte swizzle
+inline int pg_encode(TcState& tc, CUtensorMap* m, const void* base, uint64_t mid, uint64_t mid_bytes, uint64_t outer, uint64_t outer_bytes,
+                     uint32_t box_mid, uint32_t box_outer) {
+    cuuint64_t dims[3] = {(cuuint64_t)TC_BK, (cuuint64_t)mid, (cuuint64_t)outer};
+    cuuint64_t strides[2] = {(cuuint64_t)mid_bytes, (cuuint64_t)outer_bytes};
+    cuuint32_t box[3] = {(cuuint32_t)TC_BK, box_mid, box_outer};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = tc.encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+        g_tc_error = "cuTensorMapEncodeTiled (pair operand) failed (" + std::to_string((int)r) + ")";
+        return SPIRAL_ERR_CUDA;
+    }
+    return SPIRAL_OK;
+}
+// X [T][K] as [k block][T][64]: one box is PG_BPS k blocks of box_rows rows.  Where K is no multiple of 64 the last block of
+// a row runs into the next row (the buffer is that much longer and zeroed once): finite values that meet the zeros of the
+// weight copy.
+inline int pg_get_xmap(TcState& tc, const __half* X, int K, int T, int box_rows, const CUtensorMap** out) {
+    auto key = std::make_tuple((const void*)X, K, T, -box_rows);
+    auto it = tc.xmaps.find(key);
+    if (it == tc.xmaps.end()) {
+        if (tc.xmaps.size() > 4096) tc.xmaps.clear();
+        CUtensorMap m;
+        int rc = pg_encode(tc, &m, X, (uint64_t)T, (uint64_t)K * 2, (uint64_t)((K + TC_BK - 1) / TC_BK), 128, (uint32_t)box_rows, PG_BPS);
+        if (rc) return rc;
+        it = tc.xmaps.emplace(key, m).first;
+    }
+    *out = &it->second;
+    return SPIRAL_OK;
+}
+// the tile-major weight copy as rows of 64 elements, a box of PG_BPS tiles (beyond the last tile: zeros)
+inline int pg_get_wmap(TcState& tc, TcWeight& w, const CUtensorMap** out) {
+    if (!w.has_map2) {
+        int rc = tc_encode(tc, &w.map2, w.w16, (uint64_t)TC_BK, (uint64_t)(tc_tiled_elems(w.rows, w.K) / TC_BK), PG_BPS * TC_BM);
+        if (rc) return rc;
+        w.has_map2 = true;
+    }
+    *out = &w.map2;
+    return SPIRAL_OK;
 }
 
 // fp16 output [T][cols] with a 1 x 32 x 16 box (SILU epilogue)
@@ -398,7 +447,10 @@ inline int pg_gemm(TcState& tc, const PgPlan& pl, const __nv_bfloat16* W, int ro
     auto it = tc.weights.find(W);
     if (it == tc.weights.end() || !it->second.resident || it->second.rows != rows || it->second.K != K) return SPIRAL_ERR_UNSUPPORTED;
     const CUtensorMap *xm = nullptr, *om = nullptr;
-    int rc = tc_get_xmap(tc, X, K, T, pl.N / 2, &xm);
+    int rc = pg_get_xmap(tc, X, K, T, pl.N / 2, &xm);
+    if (rc) return rc;
+    const CUtensorMap* wm = nullptr;
+    rc = pg_get_wmap(tc, it->second, &wm);
     if (rc) return rc;
     if (EPI == PG_SILU) rc = pg_get_actmap(tc, (const __half*)out, rows / 2, T, &om);
     else rc = tc_get_omap(tc, (const float*)out, rows, T, EPI == PG_STORE ? pl.max_pieces : 1, &om);
@@ -406,8 +458,8 @@ inline int pg_gemm(TcState& tc, const PgPlan& pl, const __nv_bfloat16* W, int ro
     PgParams p{};
     p.row_tiles = pl.row_tiles; p.tok_tiles = pl.tok_tiles; p.KB = pl.KB; p.T = T; p.N = pl.N; p.whole = pl.whole;
     p.row_fastest = (pl.whole && T > rows) ? 1 : 0;              // re-read the smaller operand: weights rows x K, activations T x K
-    p.stages = pl.stages; p.bps = pl.bps; p.status = status;
-    TC_TRY(launch_kernel(true, pg_gemm_kernel<EPI>, dim3(2 * pl.G), dim3(PG_THREADS), pl.smem, st, it->second.map, *xm, *om, p));
+    p.stages = pl.stages; p.w_once = pl.tok_tiles <= 2; p.status = status;
+    TC_TRY(launch_kernel(true, pg_gemm_kernel<EPI>, dim3(2 * pl.G), dim3(PG_THREADS), pl.smem, st, *wm, *xm, *om, p));
     if (launches) ++*launches;
     if (pieces) {
         pieces->base = (const float*)out; pieces->stride = (size_t)T * rows; pieces->ld = rows; pieces->n_pieces = pl.max_pieces;

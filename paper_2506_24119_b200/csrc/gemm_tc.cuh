@@ -683,7 +683,8 @@ __global__ void bf16_to_f16_tiled_kernel(const __nv_bfloat16* __restrict__ src, 
 // ------------------------------------------------------------------------------------------------
 struct TcWeight {
     __half* w16 = nullptr;
-    CUtensorMap map;
+    CUtensorMap map, map2;      // boxes of one 128 x 64 tile / of two (append path, made at its first use)
+    bool has_map2 = false;
     int rows = 0, K = 0;
     bool resident = false;      // registered at init: the fp16 copy is converted once
 };

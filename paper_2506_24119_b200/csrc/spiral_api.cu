@@ -1121,7 +1121,8 @@ static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems) {
     A((void**)&w.q, R * qd * sizeof(__half));
     A((void**)&w.h, R * d.d_model * sizeof(__half));
     A((void**)&w.attn, R * qd * sizeof(__half));
-    A((void**)&w.act, R * d.d_ff * sizeof(__half));
+    A((void**)&w.act, R * d.d_ff * sizeof(__half) + 128);      // (see pg_get_xmap)
+    if (e == cudaSuccess && d.d_ff % TC_BK != 0) e = cudaMemset(w.act, 0, R * d.d_ff * sizeof(__half) + 128);
     A((void**)&w.meta_dev, meta_elems * sizeof(int32_t));
     A((void**)&w.items_dev, (size_t)items_cap * sizeof(AppendItem));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&w.meta_host, meta_elems * sizeof(int32_t));
