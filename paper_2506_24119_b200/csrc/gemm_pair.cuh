@@ -341,25 +341,49 @@ struct PgPlan {
     size_t smem = 0;
 };
 
-// How a [rows][K] matrix meets T token rows.  Stream-K is taken when whole tiles would leave more than a quarter of the
-// pair-time idle (last wave nearly empty, or fewer tiles than pairs) and the epilogue may leave pieces; the pieces of
-// more than PG_SPLIT_MAX_T token rows cost more traffic than the idle pairs.
-constexpr int PG_SPLIT_MAX_T = 1024;
-inline PgPlan pg_plan(int n_sm, int rows, int K, int T, bool may_split) {
+// Time of one 64-wide k block of a pair tile of N token rows, us: measured on a pair working alone (the 9728-wide down
+// projection, T = N).  Up to N = 128 the weight half of the tile sets it (an SM takes at most 67 bytes per clock from L2).
+inline double pg_block_us(int N) {
+    static const double at[][2] = {{32, 0.195}, {64, 0.20}, {128, 0.208}, {160, 0.27}, {192, 0.295}, {224, 0.31}, {256, 0.325}};
+    for (int i = 1; i < 7; ++i)
+        if (N <= at[i][0]) return at[i - 1][1] + (at[i][1] - at[i - 1][1]) * (N - at[i - 1][0]) / (at[i][0] - at[i - 1][0]);
+    return at[6][1];
+}
+
+// How a [rows][K] matrix meets T token rows: the token tile N and whole tiles or stream-K, whichever the estimate below
+// makes shorter.  Whole tiles cost their waves over the pairs; stream-K fills every pair but writes each piece and has it
+// read again (both at about 3 TB/s, from L2), and where the epilogue would have gated (`gated`) the gating becomes a
+// kernel of its own.  E.g. 331 rows: gate/up whole with N = 112 (4 waves of 76 x 3 tiles; 47 us against 47 + 18 for
+// stream-K and its gating kernel), QKV whole with N = 112 (72 tiles, 21 against 25 us), output and down projection
+// stream-K (21 and 29 against 25 and 41 us).
+constexpr int PG_SPLIT_MAX_T = 1024;                 // bounds the pieces buffer
+constexpr int PG_SEARCH_MAX_T = 2048;                // beyond: many waves, and the widest tile moves the fewest bytes per flop
+enum { PG_OUT_PIECES = 0, PG_OUT_ADD = 1, PG_OUT_GATED = 2 };      // what a whole tile's epilogue writes
+inline PgPlan pg_plan(int n_sm, int rows, int K, int T, int out) {
     PgPlan pl;
-    pl.tok_tiles = (T + PG_MAX_N - 1) / PG_MAX_N;
-    pl.N = ((T + pl.tok_tiles - 1) / pl.tok_tiles + 31) & ~31;
-    pl.tok_tiles = (T + pl.N - 1) / pl.N;
     pl.row_tiles = (rows + PG_BM - 1) / PG_BM;
     pl.KB = (K + TC_BK - 1) / TC_BK;
-    const int pairs = std::max(1, n_sm / 2), tiles = pl.row_tiles * pl.tok_tiles;
-    const int waves = (tiles + pairs - 1) / pairs;
-    pl.whole = !(may_split && T <= PG_SPLIT_MAX_T && tiles * 4 < waves * pairs * 3);
+    const int pairs = std::max(1, n_sm / 2), fewest = (T + PG_MAX_N - 1) / PG_MAX_N;
+    double best = -1;
+    const int most = T <= PG_SEARCH_MAX_T ? fewest + 3 : fewest;
+    for (int tt = fewest; tt <= most; ++tt) {
+        const int N = ((T + tt - 1) / tt + 31) & ~31, tok_tiles = (T + N - 1) / N;
+        if (tok_tiles != tt) continue;
+        const double t = pg_block_us(N);
+        const int tiles = pl.row_tiles * tok_tiles, waves = (tiles + pairs - 1) / pairs;
+        const double whole = (double)waves * pl.KB * t;
+        if (best < 0 || whole < best) { best = whole; pl.N = N; pl.tok_tiles = tok_tiles; pl.whole = 1; }
+        const long long U = (long long)tiles * pl.KB;
+        const int G = (int)std::min<long long>(pairs, std::max<long long>(1, U / 4));   // no ranges under four k blocks
+        const double pieces = 1.0 + (double)G / tiles, one = (double)T * rows * 4 / 3e6;
+        const double split = (double)U / G * t + one * (out == PG_OUT_PIECES ? pieces - 1.0 : pieces) + (out == PG_OUT_GATED ? 5.0 + one : 1.0);
+        if (T <= PG_SPLIT_MAX_T && split < best) { best = split; pl.N = N; pl.tok_tiles = tok_tiles; pl.whole = 0; pl.G = G; }
+    }
+    const int tiles = pl.row_tiles * pl.tok_tiles;
     if (pl.whole) {
         pl.G = std::min(pairs, tiles);
     } else {
         const long long U = (long long)tiles * pl.KB;
-        pl.G = (int)std::min<long long>(pairs, std::max<long long>(1, U / 4));          // no ranges under four k blocks
         pl.max_pieces = 0;
         for (int t = 0; t < tiles; ++t) {
             const long long first = (long long)t * pl.KB;

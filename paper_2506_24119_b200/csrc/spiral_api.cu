@@ -1152,7 +1152,7 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
     for (long long T : {(long long)chunk, total % chunk ? total % chunk : (long long)chunk}) {
         const int shapes[4][2] = {{ctx->qkv_rows, d.d_model}, {d.d_model, qd}, {2 * d.d_ff, d.d_model}, {d.d_model, d.d_ff}};
         for (int m = 0; m < 4; ++m) {
-            const PgPlan pl = pg_plan(ctx->n_sm, shapes[m][0], shapes[m][1], (int)T, true);
+            const PgPlan pl = pg_plan(ctx->n_sm, shapes[m][0], shapes[m][1], (int)T, m == 0 ? PG_OUT_PIECES : m == 2 ? PG_OUT_GATED : PG_OUT_ADD);
             if (m == 0 || !pl.whole) y_elems = std::max<size_t>(y_elems, (size_t)pl.max_pieces * (size_t)T * shapes[m][0]);
         }
     }
@@ -1215,8 +1215,8 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
 
         LAUNCH(ctx, embed_kernel, nt, 256, 0, st, ctx->embed, meta_args(ctx), meta, kv->table_dev, kv->max_pages,
                kv->page_size, d.d_model, d.vocab, w.x, ctx->status);
-        const PgPlan pl_qkv = pg_plan(ctx->n_sm, ctx->qkv_rows, d.d_model, nt, true), pl_o = pg_plan(ctx->n_sm, d.d_model, qd, nt, true);
-        const PgPlan pl_gu = pg_plan(ctx->n_sm, 2 * d.d_ff, d.d_model, nt, true), pl_dn = pg_plan(ctx->n_sm, d.d_model, d.d_ff, nt, true);
+        const PgPlan pl_qkv = pg_plan(ctx->n_sm, ctx->qkv_rows, d.d_model, nt, PG_OUT_PIECES), pl_o = pg_plan(ctx->n_sm, d.d_model, qd, nt, PG_OUT_ADD);
+        const PgPlan pl_gu = pg_plan(ctx->n_sm, 2 * d.d_ff, d.d_model, nt, PG_OUT_GATED), pl_dn = pg_plan(ctx->n_sm, d.d_model, d.d_ff, nt, PG_OUT_ADD);
         Pieces pend{};                 // pieces a projection has left for the next norm to add to the residual stream
         int has = 0;
         // h = RMSNorm(x + pending pieces)
