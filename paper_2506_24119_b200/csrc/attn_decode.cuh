@@ -61,6 +61,8 @@ struct AttnParams {
     __half* out_f16;                // [n][n_q_heads * head_dim] (input of the output projection) and / or
     float* out_f32;                 // the same in fp32; either may be null
     int* status;
+    int early;                      // 1: decode step: the block table and all pages but the last of each game (the one the
+                                    // step appends to) were complete before the kernels ahead started, see rmsnorm_kernel
     int skip_first_load;            // wait-timeout self-test only: every range leaves its first page load out, so its
                                     // first wait has to run out and the warp has to unwind
 };
@@ -168,13 +170,13 @@ __device__ __forceinline__ void attn_warp_work(const CUtensorMap* tmKV, const At
         }
         return lo;
     };
-    // where unit u's page id sits in the block table, and its KV head (schedule only)
+    // where unit u's page id sits in the block table, and its KV head (schedule only); -1 - head for a game's last page
     auto locate = [&](int u, int& kvh_out) -> size_t {
         int s = slot_of(u);
         int pages = (len_sm[s] + ATTN_PAGE - 1) / ATTN_PAGE;
         int off = u - cum_sm[s];
         int kvh = off / pages, pg = off - kvh * pages;
-        kvh_out = kvh;
+        kvh_out = pg + 1 < pages ? kvh : -1 - kvh;
         return (size_t)game_sm[s] * p.max_pages + pg;
     };
     // first pool row (TMA y coordinate) of the (page, head) block whose page id is table entry `at`
@@ -184,7 +186,7 @@ __device__ __forceinline__ void attn_warp_work(const CUtensorMap* tmKV, const At
             record_status(p.status, STATUS_BAD_PAGE);
             page = 0;
         }
-        return (((p.layer * p.n_pages + page) * Hkv) + kvh) * 32;
+        return (((p.layer * p.n_pages + page) * Hkv) + (kvh < 0 ? -1 - kvh : kvh)) * 32;
     };
     auto fetch_row = [&](int u) -> int {
         int kvh;
@@ -192,14 +194,17 @@ __device__ __forceinline__ void attn_warp_work(const CUtensorMap* tmKV, const At
         return row_of(at, kvh);
     };
     // rows of the current and of the next window of 32 units, one unit per lane: located while the kernel ahead may
-    // still run, read from the block table once it has finished
+    // still run, and in a decode step looked up then, too
     int kvh_c = 0, kvh_n = 0;
     const size_t at_c = lane < cnt ? locate(u0 + lane, kvh_c) : 0;
     const size_t at_n = 32 + lane < cnt ? locate(u0 + 32 + lane, kvh_n) : 0;
-    dependency_wait();
-    int row_cur = lane < cnt ? row_of(at_c, kvh_c) : 0;
-    int row_nxt = 32 + lane < cnt ? row_of(at_n, kvh_n) : 0;
-    int win = 0;
+    int row_cur = 0, row_nxt = 0, win = 0;
+    auto look_up = [&]() {
+        row_cur = lane < cnt ? row_of(at_c, kvh_c) : 0;
+        row_nxt = 32 + lane < cnt ? row_of(at_n, kvh_n) : 0;
+    };
+    if (p.early) look_up();
+    else { dependency_wait(); look_up(); }
 
     auto issue = [&](int j) {          // unit index j (relative to u0) into stage j % STAGES; all lanes call
         const int y = __shfl_sync(0xffffffffu, row_cur, j & 31);     // j lies in window `win`
@@ -213,7 +218,17 @@ __device__ __forceinline__ void attn_warp_work(const CUtensorMap* tmKV, const At
         }
     };
     ATT_STAMP(2);
-    for (int j = 0; j < ATTN_STAGES && j < cnt; ++j) issue(j);
+    // In a decode step the first pages are requested ahead of the dependency wait, where they are not a game's last:
+    // with few games the CTA is resident early and the trip from DRAM is hidden (one game at 900 tokens: 13 us per
+    // layer before, most of it a chain of such trips).
+    unsigned asked = 0;
+    if (p.early) {
+        for (int j = 0; j < ATTN_STAGES && j < cnt; ++j)
+            if (__shfl_sync(0xffffffffu, kvh_c, j) >= 0) { issue(j); asked |= 1u << j; }
+        dependency_wait();
+    }
+    for (int j = 0; j < ATTN_STAGES && j < cnt; ++j)
+        if (!(asked >> j & 1u)) issue(j);
     ATT_STAMP(3);
 
     // consumer cursor

@@ -147,34 +147,50 @@ __global__ void embed_kernel(const __nv_bfloat16* __restrict__ embed, const Step
 }
 
 // x <- x + sum(pieces) (when pieces are given), then h = x * rsqrt(mean(x^2) + eps) * gain as fp16.
-// One CTA per batch row, one pass: every thread keeps its (up to RMS_PER_THREAD) float4 columns of
-// the row in registers between the reduction and the scaling.
+// One CTA per batch row, one pass: every thread keeps its PT float4 columns of the row in registers between the
+// reduction and the scaling.  Bound by a chain of load latencies (10 KB of x, up to nine pieces of it in L2): DEPTH
+// pieces are in flight together, and with EARLY the gains, weights that nobody writes, come from DRAM ahead of the
+// dependency wait.  <1, 10, true>, which needs d_model <= 4096, against <2, 8, false>, us per step of the Qwen3-4B shape:
+// 1 game 2408 -> 2385, 11 games 2893 -> 2854, 128 games 4462 -> 4422; wider rows leave no registers for it.
 constexpr int RMS_THREADS = 1024;       // upper bound; launched with d_model / 4 threads rounded up to a warp
-constexpr int RMS_PER_THREAD = 2;       // d_model <= 2 * 4 * 1024 = 8192
+constexpr int RMS_MAX_PER_THREAD = 2;   // d_model <= 2 * 4 * 1024 = 8192
 inline int rms_block(int d_model) { return std::min(RMS_THREADS, ((d_model / 4 + 31) / 32) * 32); }
+template <int PT, int DEPTH, bool EARLY>
 __global__ void __launch_bounds__(RMS_THREADS) rmsnorm_kernel(float* __restrict__ x, Pieces pieces, int has_pieces,
                                                               const __nv_bfloat16* __restrict__ gain, float eps,
                                                               int d_model, __half* __restrict__ h) {
     TRACE_BEGIN(2);
     // the table of piece counts depends on the launch's parameters only: it is built while the kernel ahead runs
-    grid_launch_dependents();
+    if (has_pieces) grid_launch_dependents();
     __shared__ unsigned char cnt_tab[PIECE_TABLE];
     PieceCounts pcnt{cnt_tab};
+    const int b = blockIdx.x, nc = d_model >> 2;
+    uint2 g[PT];
+    auto fetch_gains = [&]() {
+#pragma unroll
+        for (int k = 0; k < PT; ++k) {
+            const int c = threadIdx.x + k * blockDim.x;
+            g[k] = c < nc ? *reinterpret_cast<const uint2*>(gain + 4 * c) : make_uint2(0u, 0u);
+        }
+    };
+    if (EARLY) fetch_gains();
     if (has_pieces) pcnt = piece_counts_init(pieces, cnt_tab);
     grid_dependency_wait();
     TRACE_WAITED();
-    const int b = blockIdx.x, nc = d_model >> 2;
+    // The step's first norm (no pieces yet) lets the next kernel start only now: every later kernel of the step then
+    // starts after the embedding kernel has published the block table, and may read it ahead of its own wait.
+    if (!has_pieces) grid_launch_dependents();
     float* xr = x + (size_t)b * d_model;
-    float4 v[RMS_PER_THREAD];
+    float4 v[PT];
     float ss = 0.f;
 #pragma unroll
-    for (int k = 0; k < RMS_PER_THREAD; ++k) {
+    for (int k = 0; k < PT; ++k) {
         const int c = threadIdx.x + k * blockDim.x;
         v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (c < nc) {
             v[k] = reinterpret_cast<float4*>(xr)[c];
             if (has_pieces) {
-                float4 p = piece_sum4(pieces, pcnt.of(pieces, b, 4 * c), b, 4 * c);
+                float4 p = piece_sum4<DEPTH>(pieces, pcnt.of(pieces, b, 4 * c), b, 4 * c);
                 v[k].x += p.x; v[k].y += p.y; v[k].z += p.z; v[k].w += p.w;
                 reinterpret_cast<float4*>(xr)[c] = v[k];
             }
@@ -182,12 +198,7 @@ __global__ void __launch_bounds__(RMS_THREADS) rmsnorm_kernel(float* __restrict_
         }
     }
     // the gains are fetched before the reduction's barrier, not after it: one round of latency less
-    uint2 g[RMS_PER_THREAD];
-#pragma unroll
-    for (int k = 0; k < RMS_PER_THREAD; ++k) {
-        const int c = threadIdx.x + k * blockDim.x;
-        g[k] = c < nc ? *reinterpret_cast<const uint2*>(gain + 4 * c) : make_uint2(0u, 0u);
-    }
+    if (!EARLY) fetch_gains();
     __shared__ float red[RMS_THREADS / 32];
     ss = warp_sum(ss);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
@@ -198,7 +209,7 @@ __global__ void __launch_bounds__(RMS_THREADS) rmsnorm_kernel(float* __restrict_
     const float inv = rsqrtf(tot / (float)d_model + eps);
     __half* hr = h + (size_t)b * d_model;
 #pragma unroll
-    for (int k = 0; k < RMS_PER_THREAD; ++k) {
+    for (int k = 0; k < PT; ++k) {
         const int c = threadIdx.x + k * blockDim.x;
         if (c < nc) {
             uint2 o;
@@ -373,6 +384,133 @@ __global__ void __maxnreg__(56) qkv_post_kernel(      // 56 registers: see QKV_P
     }
 }
 
+// The same for few rows (at most one task per half-warp of half the grid's warps): what a task needs besides the pieces
+// is fetched ahead of the dependency wait, which takes four round trips out of the chain (Qwen3-4B shape, 1 game 2478 ->
+// 2401 us per step; with two tasks per half-warp the registers it holds cost more: 213 games 5426 -> 5535).
+// What a task needs besides the projection's pieces: position, page, rotation (and, only brought near, the norm gains).
+// None of it comes from the kernel ahead: positions from the host, pages from the step's first kernel (see
+// rmsnorm_kernel), the rest is never written.
+template <int EPL>
+struct QkvAhead {
+    int pos, page;
+    QkvVec<EPL> cs, sn;
+    __device__ __forceinline__ void fetch(int slot, int head, int l16, const __nv_bfloat16* q_gain, const __nv_bfloat16* k_gain,
+                                          const float* cos_tab, const float* sin_tab, const StepMeta& meta,
+                                          const int32_t* block_table, int max_pages, int page_size, int n_q_heads, int n_kv_heads) {
+        constexpr int HALF = 16 * EPL;
+        pos = meta.pos[slot];
+        page = 0;
+        if (head >= n_q_heads) page = __ldcg(block_table + (size_t)meta.game[slot] * max_pages + pos / page_size);
+        if (head < n_q_heads + n_kv_heads) {
+            cs.load(cos_tab + (size_t)pos * HALF + EPL * l16);
+            sn.load(sin_tab + (size_t)pos * HALF + EPL * l16);
+            const __nv_bfloat16* gain = head < n_q_heads ? q_gain : k_gain;
+            if (gain) asm volatile("prefetch.global.L1 [%0];" ::"l"(gain + 2 * EPL * l16));
+        }
+    }
+};
+
+template <int EPL>
+__device__ __forceinline__ void qkv_post_few_task(const QkvAhead<EPL>& pre, const Pieces& pieces, const PieceCounts& pcnt, int slot, int head,
+                                              int l16, const __nv_bfloat16* bias, const __nv_bfloat16* q_gain,
+                                              const __nv_bfloat16* k_gain, float eps, int page_size, int n_pages, int layer,
+                                              int n_q_heads, int n_kv_heads, float* q_out, uint16_t* pool, int kv_f16, int* status) {
+    constexpr int HD = 32 * EPL, HALF = HD / 2;
+    const int pos = pre.pos;
+    const int cnt = pcnt.of(pieces, slot, head * HD);            // head_dim <= 128: a head lies in one 128-row tile
+    const int i0 = EPL * l16;                              // this lane's elements i0 .. i0 + EPL - 1 and + HALF
+    const bool is_q = head < n_q_heads;
+    const bool is_k = !is_q && head < n_q_heads + n_kv_heads;
+    const QkvVec<EPL>&cs = pre.cs, &sn = pre.sn;           // rotation of this lane's pairs
+    float lo[EPL], hi[EPL];
+    qkv_piece_sum<EPL>(pieces, cnt, slot, head * HD + i0, lo);
+    qkv_piece_sum<EPL>(pieces, cnt, slot, head * HD + i0 + HALF, hi);
+    if (bias) {
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) {
+            lo[e] += __bfloat162float(bias[head * HD + i0 + e]);
+            hi[e] += __bfloat162float(bias[head * HD + i0 + e + HALF]);
+        }
+    }
+    if (is_q || is_k) {
+        const __nv_bfloat16* gain = is_q ? q_gain : k_gain;
+        if (gain) {
+            float ss = 0.f;
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) ss += lo[e] * lo[e] + hi[e] * hi[e];
+            // sum over the 16 lanes of this head (the other half-warp may be on another branch)
+            const unsigned hm = 0xffffu << (threadIdx.x & 16);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(hm, ss, o);
+            const float inv = rsqrtf(ss / (float)HD + eps);
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) {
+                lo[e] = lo[e] * inv * __bfloat162float(gain[i0 + e]);
+                hi[e] = hi[e] * inv * __bfloat162float(gain[i0 + e + HALF]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) {
+            const float a = lo[e], b = hi[e];
+            lo[e] = a * cs.v[e] - b * sn.v[e];
+            hi[e] = b * cs.v[e] + a * sn.v[e];
+        }
+    }
+    if (is_q) {
+        float* q = q_out + ((size_t)slot * n_q_heads + head) * HD + i0;
+        QkvVec<EPL> o;
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) o.v[e] = lo[e];
+        o.store(q);
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) o.v[e] = hi[e];
+        o.store(q + HALF);
+        return;
+    }
+    const int kvh = is_k ? head - n_q_heads : head - n_q_heads - n_kv_heads;
+    const int page = pre.page;
+    if (page < 0 || page >= n_pages) {
+        if (l16 == 0) record_status(status, STATUS_BAD_PAGE);
+        return;
+    }
+    const size_t off = kv_block_offset(layer, page, kvh, n_pages, n_kv_heads, page_size, HD) +
+                       (is_k ? 0 : (size_t)page_size * HD) + (size_t)(pos % page_size) * HD + i0;
+#pragma unroll
+    for (int e = 0; e < EPL; e += 2) {
+        const uint32_t wl = kv_f16 ? pack_f16(lo[e], lo[e + 1]) : pack_bf16(lo[e], lo[e + 1]);
+        const uint32_t wh = kv_f16 ? pack_f16(hi[e], hi[e + 1]) : pack_bf16(hi[e], hi[e + 1]);
+        *reinterpret_cast<uint32_t*>(pool + off + e) = wl;
+        *reinterpret_cast<uint32_t*>(pool + off + e + HALF) = wh;
+    }
+}
+
+template <int HD>
+__global__ void __maxnreg__(56) qkv_post_few_kernel(      // 56 registers: see QKV_POST_THREADS
+    Pieces pieces, const __nv_bfloat16* __restrict__ bias, const __nv_bfloat16* __restrict__ q_gain,
+    const __nv_bfloat16* __restrict__ k_gain, float eps, const float* __restrict__ cos_tab,
+    const float* __restrict__ sin_tab, StepMeta meta, const int32_t* __restrict__ block_table, int max_pages,
+    int page_size, int n_pages, int layer, int n, int n_q_heads, int n_kv_heads, float* __restrict__ q_out,
+    uint16_t* __restrict__ pool, int kv_f16, int* status) {
+    constexpr int EPL = HD / 32;
+    TRACE_BEGIN(3);
+    grid_launch_dependents();
+    __shared__ unsigned char cnt_tab[PIECE_TABLE];
+    const int l16 = threadIdx.x & 15;
+    const int n_heads = n_q_heads + 2 * n_kv_heads;
+    const int total = n * n_heads;
+    const int task = (blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+    QkvAhead<EPL> pre;
+    const int slot = task / n_heads, head = task - slot * n_heads;
+    if (task < total)
+        pre.fetch(slot, head, l16, q_gain, k_gain, cos_tab, sin_tab, meta, block_table, max_pages, page_size, n_q_heads, n_kv_heads);
+    const PieceCounts pcnt = piece_counts_init(pieces, cnt_tab);       // (parameters only: before the wait)
+    grid_dependency_wait();
+    TRACE_WAITED();
+    if (task < total)
+        qkv_post_few_task<EPL>(pre, pieces, pcnt, slot, head, l16, bias, q_gain, k_gain, eps, page_size, n_pages, layer, n_q_heads,
+                               n_kv_heads, q_out, pool, kv_f16, status);
+}
+
 // act[b][i] = SiLU(gate_i) * up_i with gate_i / up_i the reduced features 2i / 2i+1 of the
 // gate-up GEMM (rows interleaved), written as fp16.
 // Persistent grid (one CTA per SM): a small grid is resident at once, so the kernel after this one
@@ -440,6 +578,27 @@ __global__ void __launch_bounds__(SILU_THREADS) silu_mul_kernel(Pieces pieces, i
             }
         }
     }
+}
+
+// The same for few rows (at most two CTAs per SM): a task per thread, the first pieces of a task in flight together, CTAs of 256 threads over all
+// SMs, beside which the projection behind fits (Qwen3-4B shape, 1 game 2576 -> 2492 us per step, 11 games 3019 -> 2908).
+constexpr int SILU_FEW_THREADS = 256;
+__global__ void __launch_bounds__(SILU_FEW_THREADS) silu_mul_few_kernel(Pieces pieces, int n, int d_ff, __half* __restrict__ act) {
+    TRACE_BEGIN(4);
+    grid_launch_dependents();
+    __shared__ unsigned char cnt_tab[PIECE_TABLE];
+    const PieceCounts pcnt = piece_counts_init(pieces, cnt_tab);       // (parameters only: before the wait)
+    const int per_row = d_ff >> 1, idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int row = idx / per_row, col = idx - row * per_row;
+    const bool in = idx < n * per_row;
+    const int cnt = in ? pcnt.of(pieces, row, 4 * col) : 0;
+    grid_dependency_wait();
+    TRACE_WAITED();
+    if (!in) return;
+    const float4 v = piece_sum4<4>(pieces, cnt, row, 4 * col);
+    const float a0 = v.x / (1.f + expf(-v.x)) * v.y;
+    const float a1 = v.z / (1.f + expf(-v.z)) * v.w;
+    *reinterpret_cast<uint32_t*>(act + (size_t)row * d_ff + 2 * col) = pack_f16(a0, a1);
 }
 
 // 64-bit key whose unsigned order is (score ascending, index descending): max key = best score,

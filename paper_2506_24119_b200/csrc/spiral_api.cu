@@ -234,7 +234,7 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
     if (d->qk_norm && (!w->q_norm || !w->k_norm)) return SPIRAL_ERR_INVALID;
     if (d->head_dim != 64 && d->head_dim != 128) return SPIRAL_ERR_UNSUPPORTED;
     if (d->n_q_heads % d->n_kv_heads != 0 || d->n_q_heads / d->n_kv_heads > 8) return SPIRAL_ERR_UNSUPPORTED;
-    if (d->d_model > 4 * RMS_PER_THREAD * RMS_THREADS || d->head_dim > 128) return SPIRAL_ERR_UNSUPPORTED;
+    if (d->d_model > 4 * RMS_MAX_PER_THREAD * RMS_THREADS || d->head_dim > 128) return SPIRAL_ERR_UNSUPPORTED;
     if (d->d_model % 64 != 0 || d->d_ff % 8 != 0 || (d->n_q_heads * d->head_dim) % 64 != 0)
         return SPIRAL_ERR_UNSUPPORTED;
     if (!(d->rope_theta > 0) || !(d->rms_eps >= 0)) return SPIRAL_ERR_INVALID;
@@ -696,7 +696,7 @@ static int launch_linear_impl(spiral_ctx* c, const bf16* W, int rows, int K, con
 
 static int launch_attention(spiral_ctx* c, spiral_kv* kv, int layer, int n, const int32_t* game_dev,
                             const int32_t* len_dev, int len_add, const float* q, __half* out_f16,
-                            float* out_f32, cudaStream_t st) {
+                            float* out_f32, bool early, cudaStream_t st) {
     const spiral_model_desc& d = c->d;
     AttnParams p;
     p.q = q; p.block_table = kv->table_dev; p.game = game_dev; p.ctx_len = len_dev; p.cum = meta_cum_dev(c);
@@ -707,6 +707,7 @@ static int launch_attention(spiral_ctx* c, spiral_kv* kv, int layer, int n, cons
     p.item_cnt = c->attn_item_cnt; p.out_f16 = out_f16; p.out_f32 = out_f32;
     p.skip_first_load = c->attn_skip_once ? 1 : 0;
     c->attn_skip_once = false;
+    p.early = early ? 1 : 0;
     const size_t smem = attn_smem_bytes(d.head_dim, c->group);
     int rec = prof_begin(c, SPIRAL_KC_ATTN, st);
     auto attn = d.head_dim == 128 ? (kv->kv_f16 ? attn_decode_kernel<128, true> : attn_decode_kernel<128, false>)
@@ -718,6 +719,19 @@ static int launch_attention(spiral_ctx* c, spiral_kv* kv, int layer, int n, cons
 
 // Reserve a slot of the pinned metadata ring (waits for the copy that last used it).
 static int meta_acquire(spiral_ctx* c, int32_t** host, StepArgs** args) {
+static decltype(&rmsnorm_kernel<2, 8, false>) rms_kernel(int d_model) {
+    return d_model <= 4 * RMS_THREADS ? rmsnorm_kernel<1, 10, true> : rmsnorm_kernel<2, 8, false>;
+}
+
+static int launch_silu(spiral_ctx* c, const Pieces& pg, int n, __half* act, cudaStream_t st) {
+    const long long tasks = (long long)n * (c->d.d_ff / 2);
+    if (tasks <= (long long)2 * c->n_sm * SILU_FEW_THREADS)
+        LAUNCH(c, silu_mul_few_kernel, (unsigned)((tasks + SILU_FEW_THREADS - 1) / SILU_FEW_THREADS), SILU_FEW_THREADS, 0, st, pg, n, c->d.d_ff, act);
+    else
+        LAUNCH(c, silu_mul_kernel, (unsigned)std::min<long long>(c->n_sm, (tasks + SILU_THREADS - 1) / SILU_THREADS), SILU_THREADS, 0, st, pg, n, c->d.d_ff, act);
+    return SPIRAL_OK;
+}
+
     int s = c->meta_next;
     c->meta_next = (s + 1) % META_RING;
     if (c->meta_ev_used[s]) CU_TRY(cudaEventSynchronize(c->meta_ev[s]));
@@ -738,7 +752,8 @@ static int meta_upload(spiral_ctx* c, int slot, cudaStream_t st) {
 }
 
 // All layers for n batch slots whose metadata is already in ctx->meta_dev.
-static int run_layers(spiral_ctx* c, spiral_kv* kv, int n, cudaStream_t st) {
+// `one_per_game`: no game has two of the slots, so only its last page changes during the step.
+static int run_layers(spiral_ctx* c, spiral_kv* kv, int n, bool one_per_game, cudaStream_t st) {
     const spiral_model_desc& d = c->d;
     const int MB = c->max_batch;
     int32_t* mi = meta_i32(c);
@@ -751,31 +766,40 @@ static int run_layers(spiral_ctx* c, spiral_kv* kv, int n, cudaStream_t st) {
     const int small_grid = std::max(1, std::min(c->n_sm, (n * (d.n_q_heads + 2 * d.n_kv_heads) + 43) / 44));
     Pieces pc{};          // pieces of the previous layer's down projection, folded into the next norm
     int has = 0;
+    const bool few = (long long)n * (d.n_q_heads + 2 * d.n_kv_heads) <= c->n_sm * (QKV_POST_THREADS / 32);
     int rc;
     for (int l = 0; l < d.n_layers; ++l) {
-        LAUNCH(c, rmsnorm_kernel, n, rms_block(d.d_model), 0, st, c->x, pc, has, c->ln1[l], eps, d.d_model, c->h);
+        LAUNCH(c, rms_kernel(d.d_model), n, rms_block(d.d_model), 0, st, c->x, pc, has, c->ln1[l], eps, d.d_model, c->h);
         Pieces pq;
         rc = launch_linear(c, SPIRAL_KC_QKV, c->wqkv[l], c->qkv_rows, d.d_model, c->h, n, nullptr, 0, &pq, st);
         if (rc) return rc;
-        LAUNCH(c, qkv_post_kernel, small_grid, QKV_POST_THREADS, 0, st, pq, c->bqkv[l], c->q_norm[l], c->k_norm[l], eps,
-               c->cos_tab, c->sin_tab, meta, kv->table_dev, kv->max_pages, kv->page_size, kv->n_pages, l, n,
-               d.n_q_heads, d.n_kv_heads, d.head_dim, c->q, kv->pool, kv->kv_f16, c->status);
-        rc = launch_attention(c, kv, l, n, meta.game, meta.pos, 1, c->q, c->attn_out, nullptr, st);
+        if (few) {
+            auto post = d.head_dim == 128 ? qkv_post_few_kernel<128> : qkv_post_few_kernel<64>;
+            LAUNCH(c, post, small_grid, QKV_POST_THREADS, 0, st, pq, c->bqkv[l], c->q_norm[l], c->k_norm[l], eps,
+                   c->cos_tab, c->sin_tab, meta, kv->table_dev, kv->max_pages, kv->page_size, kv->n_pages, l, n,
+                   d.n_q_heads, d.n_kv_heads, c->q, kv->pool, kv->kv_f16, c->status);
+        } else {
+            LAUNCH(c, qkv_post_kernel, small_grid, QKV_POST_THREADS, 0, st, pq, c->bqkv[l], c->q_norm[l], c->k_norm[l], eps,
+                   c->cos_tab, c->sin_tab, meta, kv->table_dev, kv->max_pages, kv->page_size, kv->n_pages, l, n,
+                   d.n_q_heads, d.n_kv_heads, d.head_dim, c->q, kv->pool, kv->kv_f16, c->status);
+        }
+        rc = launch_attention(c, kv, l, n, meta.game, meta.pos, 1, c->q, c->attn_out, nullptr, one_per_game, st);
         if (rc) return rc;
         Pieces po;
         rc = launch_linear(c, SPIRAL_KC_O, c->wo[l], d.d_model, qd, c->attn_out, n, nullptr, 0, &po, st);
         if (rc) return rc;
-        LAUNCH(c, rmsnorm_kernel, n, rms_block(d.d_model), 0, st, c->x, po, 1, c->ln2[l], eps, d.d_model, c->h);
+        LAUNCH(c, rms_kernel(d.d_model), n, rms_block(d.d_model), 0, st, c->x, po, 1, c->ln2[l], eps, d.d_model, c->h);
         Pieces pg;
         rc = launch_linear(c, SPIRAL_KC_GATE_UP, c->w_gate_up[l], 2 * d.d_ff, d.d_model, c->h, n, nullptr, 0, &pg, st);
         if (rc) return rc;
-        LAUNCH(c, silu_mul_kernel, small_grid, SILU_THREADS, 0, st, pg, n, d.d_ff, c->act);
+        rc = launch_silu(c, pg, n, c->act, st);
+        if (rc) return rc;
         rc = launch_linear(c, SPIRAL_KC_DOWN, c->w_down[l], d.d_model, d.d_ff, c->act, n, nullptr, 0, &pc, st);
         if (rc) return rc;
         has = 1;
     }
     // final norm (folds in the last down projection)
-    LAUNCH(c, rmsnorm_kernel, n, rms_block(d.d_model), 0, st, c->x, pc, has, c->final_norm, eps, d.d_model, c->h);
+    LAUNCH(c, rms_kernel(d.d_model), n, rms_block(d.d_model), 0, st, c->x, pc, has, c->final_norm, eps, d.d_model, c->h);
     return SPIRAL_OK;
 }
 
@@ -813,7 +837,7 @@ enum StepVariant { STEP_FUSED_SAMPLER = 0, STEP_NUCLEUS = 1, STEP_LAYERS_ONLY = 
 
 static int run_step_body(spiral_ctx* c, spiral_kv* kv, int n, int variant, cudaStream_t st) {
     const bool nucleus = variant == STEP_NUCLEUS;
-    int rc2 = run_layers(c, kv, n, st);
+    int rc2 = run_layers(c, kv, n, true, st);
     if (rc2 || variant == STEP_LAYERS_ONLY) return rc2;      // the caller launches the head itself
     rc2 = run_head(c, n, st);
     if (rc2 || !nucleus) return rc2;
@@ -1297,7 +1321,10 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
                 rc = pg_gemm<PG_STORE>(ctx->tc, pl_gu, ctx->w_gate_up[l], 2 * d.d_ff, d.d_model, w.h, nt, w.y, &pg, ctx->status, st,
                                        &ctx->launches);
                 prof_end(ctx, rec, st);
-                if (rc == SPIRAL_OK) LAUNCH(ctx, silu_mul_kernel, ctx->n_sm, SILU_THREADS, 0, st, pg, nt, d.d_ff, w.act);
+                if (rc == SPIRAL_OK) {
+                    rc = launch_silu(ctx, pg, nt, w.act, st);
+                    if (rc) return rc;
+                }
             }
             if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
             if (rc) return rc;
@@ -1309,7 +1336,7 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
     }
     if (last_logits) {
         Pieces none{};
-        LAUNCH(ctx, rmsnorm_kernel, n, rms_block(d.d_model), 0, st, ctx->x, none, 0, ctx->final_norm, eps, d.d_model, ctx->h);
+        LAUNCH(ctx, rms_kernel(d.d_model), n, rms_block(d.d_model), 0, st, ctx->x, none, 0, ctx->final_norm, eps, d.d_model, ctx->h);
         rc = run_head(ctx, n, st);
         if (rc) return rc;
     }
@@ -1390,7 +1417,7 @@ extern "C" int spiral_prefill(spiral_ctx* ctx, spiral_kv* kv, int n, const int32
         sa->logits = (last_logits && any_last) ? ctx->logits : nullptr;     // no sampling: logits only
         rc = meta_upload(ctx, slot, st);
         if (rc) return roll_back(rc);
-        rc = run_layers(ctx, kv, nt, st);
+        rc = run_layers(ctx, kv, nt, false, st);
         if (rc) return roll_back(rc);
         if (last_logits && any_last) {
             rc = run_head(ctx, nt, st);
@@ -1454,7 +1481,7 @@ extern "C" int spiral_attention(spiral_ctx* ctx, spiral_kv* kv, int layer, int n
     attn_host_plan(ctx_len, n, ctx->d.n_kv_heads, ctx->n_sm, meta_cum_host(ctx, mh));
     rc = meta_upload(ctx, slot, st);
     if (rc) return rc;
-    return launch_attention(ctx, kv, layer, n, meta_i32(ctx), meta_i32(ctx) + MB, 0, q_dev, nullptr, out_dev, st);
+    return launch_attention(ctx, kv, layer, n, meta_i32(ctx), meta_i32(ctx) + MB, 0, q_dev, nullptr, out_dev, false, st);
 }
 
 extern "C" int spiral_kv_block_table(const spiral_kv* kv, int game_id, int32_t* out, int max_entries) {
@@ -1730,7 +1757,7 @@ extern "C" int spiral_selftest_wait_timeout(spiral_ctx* ctx, spiral_kv* kv, int 
         }
         if (rc == SPIRAL_OK) {
             ctx->attn_skip_once = true;
-            rc = launch_attention(ctx, kv, 0, 1, meta_i32(ctx), meta_i32(ctx) + ctx->max_batch, 0, ctx->q, ctx->attn_out, nullptr, st);
+            rc = launch_attention(ctx, kv, 0, 1, meta_i32(ctx), meta_i32(ctx) + ctx->max_batch, 0, ctx->q, ctx->attn_out, nullptr, false, st);
             ctx->attn_skip_once = false;
         }
     }

@@ -600,3 +600,25 @@ def test_attention_component_at_the_longest_configured_context():
         assert rc == 0, detail
     finally:
         pair.close()
+
+
+@pytest.mark.parametrize("n,overrides", [
+    # 36 heads and d_ff 2048: with 148 SMs 74 | 75 rows and 90 | 91 rows lie on either side of the few-row gating and
+    # q/k-norm kernels' limits
+    (74, dict(n_q_heads=28, n_kv_heads=4, d_model=448, d_ff=2048)), (75, dict(n_q_heads=28, n_kv_heads=4, d_model=448, d_ff=2048)),
+    (90, dict(n_q_heads=28, n_kv_heads=4, d_model=448, d_ff=2048)), (91, dict(n_q_heads=28, n_kv_heads=4, d_model=448, d_ff=2048)),
+    (3, dict(d_model=4160, n_layers=1)),                # a row wider than one float4 per thread of its norm
+    (1, dict(n_q_heads=8, n_kv_heads=1, head_dim=128)),
+])
+def test_decode_step_at_the_edges_of_its_kernels(n, overrides):
+    """Contexts around page boundaries, so that steps append to a full page's last slot and to a fresh page's first one."""
+    desc = synth.shape("tiny", **overrides)
+    pair = Pair(desc, max_batch=n, max_ctx=64, n_games=n)
+    try:
+        games = [(7 * i + 3) % n for i in range(n)] if n % 7 else list(range(n))[::-1]
+        prompts = [synth.token_ids(synth.MASTER_SEED, 1200 + i, 14 + i % 20, desc["vocab"]).tolist() for i in range(n)]
+        res = _run_teacher_forced(pair, games, prompts, 3, synth.MASTER_SEED + 27)
+        print(n, overrides, "max|d| %.2e rel-rms %.2e agree %.4f" % res[:3], res[3])
+        _check(*res)
+    finally:
+        pair.close()
