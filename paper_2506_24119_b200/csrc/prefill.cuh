@@ -10,8 +10,8 @@
 //                         everything cached for it (earlier turns and the new tokens up to each query's own
 //                         position) on tcgen05: scores and the output accumulator in tensor memory, one
 //                         softmax thread per query row, keys/values streamed page by page by TMA.
-//   attn_append_kernel    the same attention on mma.sync.m16n8k16 (kept as an option), flash-style with the
-//                         fp32 online softmax in registers.
+//   attn_append_kernel    the same attention on mma.sync.m16n8k16, flash-style with the fp32 online softmax in
+//                         registers: bf16 pages (whose precision needs queries and weights in two parts), and an option.
 //   pf_rmsnorm_kernel, pf_qkv_post_kernel   the element-wise steps for thousands of token rows.
 //
 // Every wait is bounded as in the decode kernels.
@@ -31,13 +31,15 @@ namespace spiral {
 // registers between the reduction and the scaling, and a row's loads are spread thin enough (NV4 float4 per thread)
 // for ten CTAs per SM.  Bound by memory: 6 bytes read and written per element.  (With a warp per row, 20 float4 per
 // lane at d_model 2560 left room for 16 warps per SM, which went through their rows in lockstep: 54 us for 9984 rows.)
+// PIECES: the row is x + the pieces a projection has left (written back to x), added piece by piece over the whole row.
 constexpr int PF_RMS_THREADS = 128;
-template <int NV4>                      // float4 per thread
-__global__ void __launch_bounds__(PF_RMS_THREADS) pf_rmsnorm_kernel(const float* __restrict__ x,
+template <int NV4, bool PIECES>         // float4 per thread
+__global__ void __launch_bounds__(PF_RMS_THREADS) pf_rmsnorm_kernel(float* __restrict__ x, Pieces pieces,
                                                                     const __nv_bfloat16* __restrict__ gain, float eps,
                                                                     int d_model, __half* __restrict__ h) {
     grid_launch_dependents();
     __shared__ float red[PF_RMS_THREADS / 32];
+    __shared__ unsigned char cnt_tab[PIECES ? PIECE_TABLE : 1];
     const int nc = d_model >> 2;
     uint2 g[NV4];                       // (weights: nobody writes them)
 #pragma unroll
@@ -45,14 +47,39 @@ __global__ void __launch_bounds__(PF_RMS_THREADS) pf_rmsnorm_kernel(const float*
         const int c = threadIdx.x + PF_RMS_THREADS * k;
         g[k] = c < nc ? __ldg(reinterpret_cast<const uint2*>(gain) + c) : make_uint2(0u, 0u);
     }
+    PieceCounts pcnt{cnt_tab};
+    if (PIECES) pcnt = piece_counts_init(pieces, cnt_tab);             // (parameters only: before the wait)
     grid_dependency_wait();
     const size_t t = blockIdx.x;
-    const float4* xr = reinterpret_cast<const float4*>(x + t * d_model);
+    float4* xr = reinterpret_cast<float4*>(x + t * d_model);
     float4 v[NV4];
 #pragma unroll
     for (int k = 0; k < NV4; ++k) {
         const int c = threadIdx.x + PF_RMS_THREADS * k;
         v[k] = c < nc ? __ldcs(xr + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (PIECES) {
+        int most = 0, cnt[NV4];
+#pragma unroll
+        for (int k = 0; k < NV4; ++k) {
+            const int c = threadIdx.x + PF_RMS_THREADS * k;
+            cnt[k] = c < nc ? pcnt.of(pieces, (int)t, 4 * c) : 0;
+            most = max(most, cnt[k]);
+        }
+        for (int i = 0; i < most; ++i) {
+            const float* pr = pieces.base + (size_t)i * pieces.stride + t * pieces.ld;
+            float4 w[NV4];
+#pragma unroll
+            for (int k = 0; k < NV4; ++k)
+                w[k] = i < cnt[k] ? __ldcg(reinterpret_cast<const float4*>(pr) + threadIdx.x + PF_RMS_THREADS * k) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < NV4; ++k) { v[k].x += w[k].x; v[k].y += w[k].y; v[k].z += w[k].z; v[k].w += w[k].w; }
+        }
+#pragma unroll
+        for (int k = 0; k < NV4; ++k) {
+            const int c = threadIdx.x + PF_RMS_THREADS * k;
+            if (c < nc) xr[c] = v[k];
+        }
     }
     float ss = 0.f;
 #pragma unroll
@@ -81,18 +108,20 @@ __global__ void __launch_bounds__(PF_RMS_THREADS) pf_rmsnorm_kernel(const float*
 // Lane l holds elements {E l .. E l + E - 1} and their rotation partners HD/2 further on (E = HD / 64).  Bound by memory
 // (4 bytes read, 2 written per element); with a warp per single head the chain position -> page -> store of every head
 // was what took the time (208 us for 9984 rows of 48 heads).
+// bf16 pages (F16 = false): q leaves as a high and a low bf16 part (q_out, q_lo), k and v are rounded once to bf16.
 constexpr int PF_QKV_THREADS = 256;
 constexpr int PF_QKV_HEADS = 4;
 inline int pf_qkv_groups(int n_q_heads, int n_kv_heads) {        // tasks per token row
     return (n_q_heads + PF_QKV_HEADS - 1) / PF_QKV_HEADS + 2 * ((n_kv_heads + PF_QKV_HEADS - 1) / PF_QKV_HEADS);
 }
-template <int HD>
+template <int HD, bool F16>
 __global__ void __launch_bounds__(PF_QKV_THREADS) pf_qkv_post_kernel(
     Pieces pieces, const __nv_bfloat16* __restrict__ bias, const __nv_bfloat16* __restrict__ q_gain,
     const __nv_bfloat16* __restrict__ k_gain, float eps, const float* __restrict__ cos_tab,
     const float* __restrict__ sin_tab, const int32_t* __restrict__ game, const int32_t* __restrict__ pos_of,
     const int32_t* __restrict__ block_table, int max_pages, int n_pages, int layer, int T, int n_q_heads,
-    int n_kv_heads, float q_scale, __half* __restrict__ q_out, uint16_t* __restrict__ pool, int* status) {
+    int n_kv_heads, float q_scale, __half* __restrict__ q_out, __half* __restrict__ q_lo, uint16_t* __restrict__ pool,
+    int* status) {
     constexpr int E = HD / 64, HALF = HD / 2, NH = PF_QKV_HEADS;
     grid_launch_dependents();
     __shared__ unsigned char cnt_tab[PIECE_TABLE];
@@ -194,7 +223,21 @@ __global__ void __launch_bounds__(PF_QKV_THREADS) pf_qkv_post_kernel(
             uint16_t* dst = is_q ? reinterpret_cast<uint16_t*>(q_out) + ((size_t)t * n_q_heads + first + u) * HD + E * lane
                                  : pool + kv_block_offset(layer, page, first + u, n_pages, n_kv_heads, ATTN_PAGE, HD) +
                                        (is_k ? 0 : (size_t)ATTN_PAGE * HD) + (size_t)(pos % ATTN_PAGE) * HD + E * lane;
-            if (E == 2) {
+            if (!F16) {
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    uint32_t h0, l0, h1, l1;
+                    split2<false>(lo[u][e] * sc, h0, l0);
+                    split2<false>(hi[u][e] * sc, h1, l1);
+                    dst[e] = (uint16_t)h0;
+                    dst[e + HALF] = (uint16_t)h1;
+                    if (is_q) {
+                        uint16_t* dl = reinterpret_cast<uint16_t*>(q_lo) + ((size_t)t * n_q_heads + first + u) * HD + E * lane;
+                        dl[e] = (uint16_t)l0;
+                        dl[e + HALF] = (uint16_t)l1;
+                    }
+                }
+            } else if (E == 2) {
                 *reinterpret_cast<uint32_t*>(dst) = pack_f16(lo[u][0] * sc, lo[u][E - 1] * sc);
                 *reinterpret_cast<uint32_t*>(dst + HALF) = pack_f16(hi[u][0] * sc, hi[u][E - 1] * sc);
             } else {
@@ -212,6 +255,9 @@ constexpr int APP_ROWS = 176;              // query rows (position x head of the
                                            // the producer warp = three warps per scheduler, the register file's limit at
                                            // the ~168 registers the consumers need
 constexpr int APP_CWARPS = APP_ROWS / 16;  // consumer warps; one more warp issues the TMA loads
+// bf16 pages: a warp's 16 MMA rows are eight query rows, high parts in rows 0..7 and low parts in rows 8..15 (products
+// with a query and a softmax weight of twice bf16's mantissa, as in the decode kernel)
+constexpr int app_rows(bool f16) { return f16 ? APP_ROWS : APP_ROWS / 2; }
 constexpr int APP_THREADS = (APP_CWARPS + 1) * 32;
 constexpr int APP_BLK_PAGES = 4;           // pages (16 keys each) per ring stage
 constexpr int APP_STAGES = 4;
@@ -223,6 +269,7 @@ struct AppendItem { int game, pos0, n_pos, row0, kv_len, pad0, pad1, pad2; };
 
 struct AppendParams {
     const __half* q;                // [T][n_q_heads][head_dim] fp16: normalised, rotated, times log2(e)/sqrt(head_dim)
+    const __half* q_lo;             // bf16 pages: q and q_lo are the high and low bf16 parts of the same
     const AppendItem* items;
     const int32_t* block_table;     // [max_games][max_pages]
     int max_pages, n_pages, layer, n_q_heads, n_kv_heads, group;
@@ -230,7 +277,7 @@ struct AppendParams {
     int* status;
 };
 
-inline int app_positions_per_item(int group) { return APP_ROWS / group; }
+inline int app_positions_per_item(int group, bool f16) { return app_rows(f16) / group; }
 __device__ __forceinline__ uint32_t pack_unit_f16(float lo, float hi) {
     const __half2 h = __floats2half2_rn(lo, hi);
     return *reinterpret_cast<const uint32_t*>(&h);
@@ -239,7 +286,7 @@ inline size_t app_smem_bytes(int head_dim) {
     return (size_t)APP_STAGES * APP_BLK_PAGES * (head_dim / 64) * 4096 + 1024;
 }
 
-template <int HD>
+template <int HD, bool F16>
 __global__ void __launch_bounds__(APP_THREADS, 1) attn_append_kernel(const __grid_constant__ CUtensorMap tmKV,
                                                                      AppendParams p) {
     constexpr int HALVES = HD / 64;
@@ -317,9 +364,9 @@ __global__ void __launch_bounds__(APP_THREADS, 1) attn_append_kernel(const __gri
         return;
     }
 
-    // ---------------- consumers: warp w owns query rows 16 w .. 16 w + 15 ----------------
+    // ---------------- consumers: warp w owns query rows 16 w .. 16 w + 15 (bf16 pages: 8 w .. 8 w + 7) ----------------
     const int g = lane >> 2, c = lane & 3;
-    const int r0 = 16 * warp + g, r1 = r0 + 8;                   // this thread's two rows
+    const int r0 = (F16 ? 16 : 8) * warp + g, r1 = F16 ? r0 + 8 : r0;   // this thread's two rows (bf16: one, in two parts)
     const int po0 = r0 / G, hh0 = r0 - po0 * G;                  // position offset and head within the group
     const int po1 = r1 / G, hh1 = r1 - po1 * G;
     const bool ok0 = po0 < item.n_pos, ok1 = po1 < item.n_pos;
@@ -328,7 +375,7 @@ __global__ void __launch_bounds__(APP_THREADS, 1) attn_append_kernel(const __gri
     uint32_t qa[KSTEPS][4];
     {
         const __half* q0 = p.q + ((size_t)(item.row0 + (ok0 ? po0 : 0)) * p.n_q_heads + kvh * G + hh0) * HD + 2 * c;
-        const __half* q1 = p.q + ((size_t)(item.row0 + (ok1 ? po1 : 0)) * p.n_q_heads + kvh * G + hh1) * HD + 2 * c;
+        const __half* q1 = (F16 ? p.q : p.q_lo) + ((size_t)(item.row0 + (ok1 ? po1 : 0)) * p.n_q_heads + kvh * G + hh1) * HD + 2 * c;
 #pragma unroll
         for (int ks = 0; ks < KSTEPS; ++ks) {
             qa[ks][0] = __ldcg(reinterpret_cast<const uint32_t*>(q0 + 16 * ks));
@@ -382,10 +429,16 @@ __global__ void __launch_bounds__(APP_THREADS, 1) attn_append_kernel(const __gri
                     const int h = ks >> 2, ch = 2 * (ks & 3) + k_chk;
                     uint32_t b0, b1, b2, b3;
                     ldmatrix_x4(pb + h * 4096 + k_row_off + (uint32_t)(((ch ^ (k_tok & 7)) << 4)), b0, b1, b2, b3);
-                    mma_16816<true>(sc[2 * pgi], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b0, b1);
-                    mma_16816<true>(sc[2 * pgi + 1], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b2, b3);
+                    mma_16816<F16>(sc[2 * pgi], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b0, b1);
+                    mma_16816<F16>(sc[2 * pgi + 1], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b2, b3);
                 }
             }
+        }
+        if (!F16) {                     // the row's score = high-part row + low-part row; both halves carry it from here
+#pragma unroll
+            for (int t = 0; t < 2 * APP_BLK_PAGES; ++t)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) { sc[t][e] += sc[t][2 + e]; sc[t][2 + e] = sc[t][e]; }
         }
         // causal mask: the row at position P sees keys 0 .. P (also hides pages that were not loaded)
         if (key0 + APP_BLK_PAGES * ATTN_PAGE - 1 > item.pos0) {
@@ -432,16 +485,25 @@ __global__ void __launch_bounds__(APP_THREADS, 1) attn_append_kernel(const __gri
             if (pgi < npg) {
                 const uint32_t pb = base + (uint32_t)(pgi * PAGE_BYTES);
                 // weights lie in [0, 1]: plain round-to-nearest conversion, no saturation needed
-                const uint32_t a0 = pack_unit_f16(sc[2 * pgi][0], sc[2 * pgi][1]), a1 = pack_unit_f16(sc[2 * pgi][2], sc[2 * pgi][3]);
-                const uint32_t a2 = pack_unit_f16(sc[2 * pgi + 1][0], sc[2 * pgi + 1][1]);
-                const uint32_t a3 = pack_unit_f16(sc[2 * pgi + 1][2], sc[2 * pgi + 1][3]);
+                uint32_t a0, a1, a2, a3;
+                if (F16) {
+                    a0 = pack_unit_f16(sc[2 * pgi][0], sc[2 * pgi][1]); a1 = pack_unit_f16(sc[2 * pgi][2], sc[2 * pgi][3]);
+                    a2 = pack_unit_f16(sc[2 * pgi + 1][0], sc[2 * pgi + 1][1]);
+                    a3 = pack_unit_f16(sc[2 * pgi + 1][2], sc[2 * pgi + 1][3]);
+                } else {
+                    uint32_t h[4], lw[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) split2<false>(sc[2 * pgi + (k >> 1)][k & 1], h[k], lw[k]);
+                    a0 = h[0] | (h[1] << 16); a1 = lw[0] | (lw[1] << 16);
+                    a2 = h[2] | (h[3] << 16); a3 = lw[2] | (lw[3] << 16);
+                }
 #pragma unroll
                 for (int np = 0; np < NT / 2; ++np) {
                     const int h = np >> 2, ch = 2 * (np & 3) + v_chk;
                     uint32_t b0, b1, b2, b3;
                     ldmatrix_x4_trans(pb + h * 4096 + v_row_off + (uint32_t)(((ch ^ (v_tok & 7)) << 4)), b0, b1, b2, b3);
-                    mma_16816<true>(o[2 * np], a0, a1, a2, a3, b0, b1);
-                    mma_16816<true>(o[2 * np + 1], a0, a1, a2, a3, b2, b3);
+                    mma_16816<F16>(o[2 * np], a0, a1, a2, a3, b0, b1);
+                    mma_16816<F16>(o[2 * np + 1], a0, a1, a2, a3, b2, b3);
                 }
             }
         }
@@ -458,6 +520,10 @@ __global__ void __launch_bounds__(APP_THREADS, 1) attn_append_kernel(const __gri
     __half* o1 = p.out + ((size_t)(item.row0 + po1) * p.n_q_heads + kvh * G + hh1) * HD + 2 * c;
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
+        if (!F16) {
+            if (ok0) *reinterpret_cast<uint32_t*>(o0 + 8 * t) = pack_f16((o[t][0] + o[t][2]) * i0, (o[t][1] + o[t][3]) * i0);
+            continue;
+        }
         if (ok0) *reinterpret_cast<uint32_t*>(o0 + 8 * t) = pack_f16(o[t][0] * i0, o[t][1] * i0);
         if (ok1) *reinterpret_cast<uint32_t*>(o1 + 8 * t) = pack_f16(o[t][2] * i1, o[t][3] * i1);
     }

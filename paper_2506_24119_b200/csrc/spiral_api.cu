@@ -399,8 +399,10 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
         if (c->pf_ready) {
             rc = pg_gemm_setup();
             e = cudaSuccess;
-            if (rc == SPIRAL_OK) e = cudaFuncSetAttribute(attn_append_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem_bytes(128));
-            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute(attn_append_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem_bytes(64));
+            if (rc == SPIRAL_OK) e = cudaFuncSetAttribute((attn_append_kernel<128, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem_bytes(128));
+            if (rc == SPIRAL_OK) e = cudaFuncSetAttribute((attn_append_kernel<128, false>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem_bytes(128));
+            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_kernel<64, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem_bytes(64));
+            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_kernel<64, false>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem_bytes(64));
             if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<128, 1>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(128, 1));
             if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<128, 2>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(128, 2));
             if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<64, 1>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(64, 1));
@@ -705,9 +707,9 @@ static int launch_attention(spiral_ctx* c, spiral_kv* kv, int layer, int n, cons
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)d.head_dim));
     p.o_part = c->o_part; p.m_part = c->m_part; p.l_part = c->l_part; p.status = c->status;
     p.item_cnt = c->attn_item_cnt; p.out_f16 = out_f16; p.out_f32 = out_f32;
+    p.early = early ? 1 : 0;
     p.skip_first_load = c->attn_skip_once ? 1 : 0;
     c->attn_skip_once = false;
-    p.early = early ? 1 : 0;
     const size_t smem = attn_smem_bytes(d.head_dim, c->group);
     int rec = prof_begin(c, SPIRAL_KC_ATTN, st);
     auto attn = d.head_dim == 128 ? (kv->kv_f16 ? attn_decode_kernel<128, true> : attn_decode_kernel<128, false>)
@@ -717,8 +719,6 @@ static int launch_attention(spiral_ctx* c, spiral_kv* kv, int layer, int n, cons
     return SPIRAL_OK;
 }
 
-// Reserve a slot of the pinned metadata ring (waits for the copy that last used it).
-static int meta_acquire(spiral_ctx* c, int32_t** host, StepArgs** args) {
 static decltype(&rmsnorm_kernel<2, 8, false>) rms_kernel(int d_model) {
     return d_model <= 4 * RMS_THREADS ? rmsnorm_kernel<1, 10, true> : rmsnorm_kernel<2, 8, false>;
 }
@@ -732,6 +732,8 @@ static int launch_silu(spiral_ctx* c, const Pieces& pg, int n, __half* act, cuda
     return SPIRAL_OK;
 }
 
+// Reserve a slot of the pinned metadata ring (waits for the copy that last used it).
+static int meta_acquire(spiral_ctx* c, int32_t** host, StepArgs** args) {
     int s = c->meta_next;
     c->meta_next = (s + 1) % META_RING;
     if (c->meta_ev_used[s]) CU_TRY(cudaEventSynchronize(c->meta_ev[s]));
@@ -764,9 +766,9 @@ static int run_layers(spiral_ctx* c, spiral_kv* kv, int n, bool one_per_game, cu
            d.d_model, d.vocab, c->x, c->status);
     // persistent element-wise kernels: one CTA per SM, fewer when the batch is tiny
     const int small_grid = std::max(1, std::min(c->n_sm, (n * (d.n_q_heads + 2 * d.n_kv_heads) + 43) / 44));
+    const bool few = (long long)n * (d.n_q_heads + 2 * d.n_kv_heads) <= c->n_sm * (QKV_POST_THREADS / 32);
     Pieces pc{};          // pieces of the previous layer's down projection, folded into the next norm
     int has = 0;
-    const bool few = (long long)n * (d.n_q_heads + 2 * d.n_kv_heads) <= c->n_sm * (QKV_POST_THREADS / 32);
     int rc;
     for (int l = 0; l < d.n_layers; ++l) {
         LAUNCH(c, rms_kernel(d.d_model), n, rms_block(d.d_model), 0, st, c->x, pc, has, c->ln1[l], eps, d.d_model, c->h);
@@ -1077,14 +1079,22 @@ __global__ void gather_rows_kernel(const float* __restrict__ src, Pieces pieces,
     }
 }
 
-// h = RMSNorm(x) * gain over T token rows
-static int launch_rmsnorm_rows(spiral_ctx* c, const float* x, const bf16* gain, int T, __half* h, cudaStream_t st) {
+// x += pending pieces (if any), h = RMSNorm(x) * gain over T token rows
+static int launch_rmsnorm_rows(spiral_ctx* c, float* x, const Pieces* pend, const bf16* gain, int T, __half* h, cudaStream_t st) {
     const spiral_model_desc& d = c->d;
     const float eps = (float)d.rms_eps;
+    // a row per SM or less: a thread per float4 and all pieces of it in flight; more rows: narrow CTAs, ten per SM
+    // (331 rows of 2560 with three to four pieces: 8.5 us with the wide CTAs, of which an SM holds two)
+    if (pend && T <= c->n_sm) {
+        LAUNCH(c, rms_kernel(d.d_model), T, rms_block(d.d_model), 0, st, x, *pend, 1, gain, eps, d.d_model, h);
+        return SPIRAL_OK;
+    }
+    const Pieces pieces = pend ? *pend : Pieces{};
     const int need = (d.d_model / 4 + PF_RMS_THREADS - 1) / PF_RMS_THREADS;
 #define PF_RMS_CASE(NV)                                                                                               \
     if (need <= NV) {                                                                                                 \
-        LAUNCH(c, pf_rmsnorm_kernel<NV>, T, PF_RMS_THREADS, 0, st, x, gain, eps, d.d_model, h);                       \
+        auto kern = pend ? pf_rmsnorm_kernel<NV, true> : pf_rmsnorm_kernel<NV, false>;                                \
+        LAUNCH(c, kern, T, PF_RMS_THREADS, 0, st, x, pieces, gain, eps, d.d_model, h);                                \
         return SPIRAL_OK;                                                                                             \
     }
     PF_RMS_CASE(2) PF_RMS_CASE(4) PF_RMS_CASE(5) PF_RMS_CASE(6) PF_RMS_CASE(7) PF_RMS_CASE(8) PF_RMS_CASE(12) PF_RMS_CASE(16)
@@ -1135,14 +1145,14 @@ static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems) {
     w.ev = ev;
     const spiral_model_desc& d = c->d;
     const size_t R = rows, qd = (size_t)d.n_q_heads * d.head_dim;
-    const int per_item = std::min(app_positions_per_item(c->group), apt_positions_per_item(c->group, 1));
+    const int per_item = std::min(app_positions_per_item(c->group, false), apt_positions_per_item(c->group, 1));
     const int items_cap = (rows + per_item - 1) / per_item + c->max_batch + 1;
     const size_t meta_elems = 4 * R + 2 * (size_t)c->max_batch;
     cudaError_t e = cudaSuccess;
     auto A = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
     A((void**)&w.x, R * d.d_model * sizeof(float));
     A((void**)&w.y, y_elems * sizeof(float));
-    A((void**)&w.q, R * qd * sizeof(__half));
+    A((void**)&w.q, 2 * R * qd * sizeof(__half));              // (bf16 pages: high and low parts)
     A((void**)&w.h, R * d.d_model * sizeof(__half));
     A((void**)&w.attn, R * qd * sizeof(__half));
     A((void**)&w.act, R * d.d_ff * sizeof(__half) + 128);      // (see pg_get_xmap)
@@ -1184,8 +1194,9 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
     if (rc) return rc;
     PrefillWs& w = ctx->pf;
     const int cap = w.cap, MB = ctx->max_batch;
-    const int per_item = ctx->append_attn_tc ? apt_positions_per_item(ctx->group, ctx->append_tiles)
-                                             : app_positions_per_item(ctx->group);
+    const bool attn_tc = ctx->append_attn_tc && kv->kv_f16;
+    const int per_item = attn_tc ? apt_positions_per_item(ctx->group, ctx->append_tiles)
+                                 : app_positions_per_item(ctx->group, kv->kv_f16);
     const float eps = (float)d.rms_eps;
     int32_t* mdev = w.meta_dev;
     StepMeta meta{mdev, mdev + cap, mdev + 2 * (size_t)cap, mdev + 3 * (size_t)cap};
@@ -1245,10 +1256,9 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
         int has = 0;
         // h = RMSNorm(x + pending pieces)
         auto norm = [&](const bf16* gain) -> int {
-            if (!has) return launch_rmsnorm_rows(ctx, w.x, gain, nt, w.h, st);
+            const Pieces* left = has ? &pend : nullptr;
             has = 0;
-            LAUNCH(ctx, rmsnorm_kernel, nt, rms_block(d.d_model), 0, st, w.x, pend, 1, gain, eps, d.d_model, w.h);
-            return SPIRAL_OK;
+            return launch_rmsnorm_rows(ctx, w.x, left, gain, nt, w.h, st);
         };
         // x += X W^T: in the epilogue, or as pieces
         auto project = [&](int cls, const PgPlan& pl, const bf16* W, int K, const __half* X) -> int {
@@ -1274,37 +1284,37 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
             if (rc) return rc;
             {
                 const int qgrid = std::min(8 * ctx->n_sm, (nt * pf_qkv_groups(d.n_q_heads, d.n_kv_heads) + PF_QKV_THREADS / 32 - 1) / (PF_QKV_THREADS / 32));
-                auto post = d.head_dim == 128 ? pf_qkv_post_kernel<128> : pf_qkv_post_kernel<64>;
+                auto post = d.head_dim == 128 ? (kv->kv_f16 ? pf_qkv_post_kernel<128, true> : pf_qkv_post_kernel<128, false>)
+                                              : (kv->kv_f16 ? pf_qkv_post_kernel<64, true> : pf_qkv_post_kernel<64, false>);
                 LAUNCH(ctx, post, qgrid, PF_QKV_THREADS, 0, st, pq, ctx->bqkv[l], ctx->q_norm[l], ctx->k_norm[l], eps, ctx->cos_tab,
                        ctx->sin_tab, meta.game, meta.pos, kv->table_dev, kv->max_pages, kv->n_pages, l, nt, d.n_q_heads, d.n_kv_heads,
-                       q_scale, w.q, kv->pool, ctx->status);
+                       q_scale, w.q, w.q + (size_t)cap * qd, kv->pool, ctx->status);
             }
             {
                 AppendParams ap{};
-                ap.q = w.q; ap.items = w.items_dev; ap.block_table = kv->table_dev; ap.max_pages = kv->max_pages;
+                ap.q = w.q; ap.q_lo = w.q + (size_t)cap * qd; ap.items = w.items_dev; ap.block_table = kv->table_dev; ap.max_pages = kv->max_pages;
                 ap.n_pages = kv->n_pages; ap.layer = l; ap.n_q_heads = d.n_q_heads; ap.n_kv_heads = d.n_kv_heads;
                 ap.group = ctx->group;
                 ap.out = w.attn; ap.status = ctx->status;
                 rec = prof_begin(ctx, SPIRAL_KC_ATTN, st);
                 const int tl = ctx->append_tiles;
-                if (ctx->append_attn_tc && d.head_dim == 128 && tl == 2)
+                if (attn_tc && d.head_dim == 128 && tl == 2)
                     LAUNCH(ctx, (attn_append_tc_kernel<128, 2>), dim3(n_items, d.n_kv_heads), apt_threads(2), apt_smem_bytes(128, 2),
                            st, kv->pool_map16, ap);
-                else if (ctx->append_attn_tc && d.head_dim == 128)
+                else if (attn_tc && d.head_dim == 128)
                     LAUNCH(ctx, (attn_append_tc_kernel<128, 1>), dim3(n_items, d.n_kv_heads), apt_threads(1), apt_smem_bytes(128, 1),
                            st, kv->pool_map16, ap);
-                else if (ctx->append_attn_tc && tl == 2)
+                else if (attn_tc && tl == 2)
                     LAUNCH(ctx, (attn_append_tc_kernel<64, 2>), dim3(n_items, d.n_kv_heads), apt_threads(2), apt_smem_bytes(64, 2),
                            st, kv->pool_map16, ap);
-                else if (ctx->append_attn_tc)
+                else if (attn_tc)
                     LAUNCH(ctx, (attn_append_tc_kernel<64, 1>), dim3(n_items, d.n_kv_heads), apt_threads(1), apt_smem_bytes(64, 1),
                            st, kv->pool_map16, ap);
-                else if (d.head_dim == 128)
-                    LAUNCH(ctx, attn_append_kernel<128>, dim3(n_items, d.n_kv_heads), APP_THREADS, app_smem_bytes(128), st,
-                           kv->pool_map, ap);
-                else
-                    LAUNCH(ctx, attn_append_kernel<64>, dim3(n_items, d.n_kv_heads), APP_THREADS, app_smem_bytes(64), st,
-                           kv->pool_map, ap);
+                else {
+                    auto attn = d.head_dim == 128 ? (kv->kv_f16 ? attn_append_kernel<128, true> : attn_append_kernel<128, false>)
+                                                  : (kv->kv_f16 ? attn_append_kernel<64, true> : attn_append_kernel<64, false>);
+                    LAUNCH(ctx, attn, dim3(n_items, d.n_kv_heads), APP_THREADS, app_smem_bytes(d.head_dim), st, kv->pool_map, ap);
+                }
                 prof_end(ctx, rec, st);
             }
             rc = project(SPIRAL_KC_O, pl_o, ctx->wo[l], qd, w.attn);
@@ -1377,7 +1387,7 @@ extern "C" int spiral_prefill(spiral_ctx* ctx, spiral_kv* kv, int n, const int32
         // more new tokens than one decode-shaped step holds: dense passes on the tensor cores
         long long total = 0;
         for (int i = 0; i < n; ++i) total += offsets[i + 1] - offsets[i];
-        if (ctx->prefill_dense && ctx->pf_ready && kv->kv_f16 && total > ctx->max_batch) {
+        if (ctx->prefill_dense && ctx->pf_ready && total > ctx->max_batch) {
             rc = prefill_dense(ctx, kv, n, ids, tokens_dev, offsets, start, last_logits, st);
             if (rc) return roll_back(rc);
             for (int i = 0; i < n; ++i) kv->seq_len[ids[i]] = start[i] + offsets[i + 1] - offsets[i];

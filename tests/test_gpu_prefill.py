@@ -188,3 +188,25 @@ def test_dense_append_long_contexts(monkeypatch, attn):
         assert max(w[1] for w in worst) <= TOL_REL_RMS
     finally:
         pair.close()
+
+
+@pytest.mark.parametrize("overrides,lens", [
+    ({}, [44, 1, 45, 130, 89]),                                                      # 2 heads per group: 44 positions per block
+    (dict(n_q_heads=7, n_kv_heads=1, head_dim=64, d_model=448), [12, 13, 300, 25]),  # 12 per block, rows left over
+    (dict(n_q_heads=8, n_kv_heads=1, head_dim=128), [11, 12, 64, 200]),              # 11 per block
+    (dict(n_q_heads=2, n_kv_heads=2, head_dim=128), [88, 89, 176, 177]),             # 88 per block
+])
+def test_dense_append_with_bf16_pages(overrides, lens):
+    """bf16 pages take the mma.sync attention with queries and weights in two bf16 parts; lengths around its query blocks."""
+    desc = synth.shape("tiny", **overrides)
+    pair = Pair(desc, max_batch=8, max_ctx=320, n_games=8, kv_bf16=True)
+    try:
+        games = [5, 0, 3, 7, 1][:len(lens)]
+        prompts = [synth.token_ids(synth.MASTER_SEED, 970 + i, lens[i], desc["vocab"]).tolist() for i in range(len(games))]
+        launches0 = pair.sp.spiral_launch_count(pair.ctx)
+        res = _run_teacher_forced(pair, games, prompts, 3, synth.MASTER_SEED + 25)
+        assert pair.sp.spiral_launch_count(pair.ctx) - launches0 < 6 * (9 * desc["n_layers"] + 6)     # dense, not 8 tokens a step
+        print(overrides, "max|d| %.2e rel-rms %.2e agree %.4f" % res[:3], res[3])
+        _check(*res)
+    finally:
+        pair.close()
