@@ -126,12 +126,36 @@ __global__ void __launch_bounds__(PF_QKV_THREADS) pf_qkv_post_kernel(
     grid_launch_dependents();
     __shared__ unsigned char cnt_tab[PIECE_TABLE];
     const PieceCounts pcnt = piece_counts_init(pieces, cnt_tab);       // (parameters only: before the wait)
-    grid_dependency_wait();
     const int lane = threadIdx.x & 31;
     const int warps = (gridDim.x * blockDim.x) >> 5;
     const int gq = (n_q_heads + NH - 1) / NH, gk = (n_kv_heads + NH - 1) / NH, groups = gq + 2 * gk;
     const int total = T * groups;
-    for (int task = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; task < total; task += warps) {
+    const int task0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    // position, page, rotation and gains of a task: uploaded before the pass or never written, so the first task's are
+    // fetched while the projection still runs
+    int pos = 0, page = 0;
+    float cs[E], sn[E], gl[E], gh[E];
+    auto fetch_ahead = [&](int task) {
+        const int t = task / groups, grp = task - t * groups;
+        const bool is_q = grp < gq, is_k = !is_q && grp < gq + gk;
+        pos = __ldg(pos_of + t);
+        page = 0;
+        if (!is_q) page = __ldg(block_table + (size_t)__ldg(game + t) * max_pages + pos / ATTN_PAGE);
+        const __nv_bfloat16* gain = is_q ? q_gain : is_k ? k_gain : nullptr;
+        if (is_q || is_k) {
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                cs[e] = __ldg(cos_tab + (size_t)pos * HALF + E * lane + e);
+                sn[e] = __ldg(sin_tab + (size_t)pos * HALF + E * lane + e);
+                gl[e] = gain ? __bfloat162float(gain[E * lane + e]) : 1.f;
+                gh[e] = gain ? __bfloat162float(gain[E * lane + e + HALF]) : 1.f;
+            }
+        }
+    };
+    if (task0 < total) fetch_ahead(task0);
+    grid_dependency_wait();
+    for (int task = task0; task < total; task += warps) {
+        if (task != task0) fetch_ahead(task);
         const int t = task / groups, grp = task - t * groups;
         const bool is_q = grp < gq, is_k = !is_q && grp < gq + gk;
         const int first = is_q ? grp * NH : (is_k ? grp - gq : grp - gq - gk) * NH;             // head within its kind
@@ -156,9 +180,6 @@ __global__ void __launch_bounds__(PF_QKV_THREADS) pf_qkv_post_kernel(
                 fetch(yr + u * HD, lo[u], hi[u]);
                 most = max(most, pcnt.of(pieces, t, (head0 + u) * HD));
             }
-        const int pos = __ldg(pos_of + t);
-        int page = 0;
-        if (!is_q) page = __ldg(block_table + (size_t)__ldg(game + t) * max_pages + pos / ATTN_PAGE);
         for (int i = 1; i < most; ++i) {
             float l2[NH][E], h2[NH][E];
 #pragma unroll
@@ -173,17 +194,7 @@ __global__ void __launch_bounds__(PF_QKV_THREADS) pf_qkv_post_kernel(
 #pragma unroll
                 for (int e = 0; e < E; ++e) { lo[u][e] += l2[u][e]; hi[u][e] += h2[u][e]; }
         }
-        float cs[E], sn[E], gl[E], gh[E];
         const __nv_bfloat16* gain = is_q ? q_gain : is_k ? k_gain : nullptr;
-        if (is_q || is_k) {
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                cs[e] = __ldg(cos_tab + (size_t)pos * HALF + E * lane + e);
-                sn[e] = __ldg(sin_tab + (size_t)pos * HALF + E * lane + e);
-                gl[e] = gain ? __bfloat162float(gain[E * lane + e]) : 1.f;
-                gh[e] = gain ? __bfloat162float(gain[E * lane + e + HALF]) : 1.f;
-            }
-        }
 #pragma unroll
         for (int u = 0; u < NH; ++u) {
             if (u >= nh) break;
@@ -265,7 +276,11 @@ constexpr int APP_STAGES = 4;
 // One block of consecutive new positions of one game: queries at positions pos0 .. pos0 + n_pos - 1
 // (rows row0 .. of the chunk's q / output buffers); kv_len = positions of the game whose keys and
 // values have been written (everything beyond is stale pool memory).
-struct AppendItem { int game, pos0, n_pos, row0, kv_len, pad0, pad1, pad2; };
+// tcgen05 kernel: the CTA takes the key blocks blk0 .. blk1 - 1 of the item; slot >= 0: they are a part of it, whose result
+// goes to that partial slot for attn_append_merge_kernel.
+struct AppendItem { int game, pos0, n_pos, row0, kv_len, blk0, blk1, slot; };
+// a split item: its partials are slots slot .. slot + parts - 1
+struct AppendMerge { int n_pos, row0, slot, parts; };
 
 struct AppendParams {
     const __half* q;                // [T][n_q_heads][head_dim] fp16: normalised, rotated, times log2(e)/sqrt(head_dim)
@@ -274,6 +289,8 @@ struct AppendParams {
     const int32_t* block_table;     // [max_games][max_pages]
     int max_pages, n_pages, layer, n_q_heads, n_kv_heads, group;
     __half* out;                    // [T][n_q_heads * head_dim]
+    float* o_part;                  // [slot][kv head][256 rows][head_dim] partial outputs of split items, not normalised
+    float2* ml_part;                // [slot][kv head][256 rows] their (maximum, sum)
     int* status;
 };
 
@@ -310,8 +327,8 @@ __global__ void __launch_bounds__(APP_THREADS, 1) attn_append_kernel(const __gri
     volatile int* abort_flag = &abort_sm;
     grid_dependency_wait();            // items, queries and the new keys/values come from earlier kernels / copies
 
-    const AppendItem item = p.items[blockIdx.x];
-    const int kvh = blockIdx.y;
+    const AppendItem item = p.items[blockIdx.y];          // (all heads of the longest items come first)
+    const int kvh = blockIdx.x;
     const int G = p.group;
     const int last_pos = item.pos0 + item.n_pos - 1;
     const int n_pg = last_pos / ATTN_PAGE + 1;                         // pages holding keys 0 .. last_pos
@@ -640,14 +657,15 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
     volatile int* abort_flag = &abort_sm;
     grid_dependency_wait();            // items, queries and the new keys/values come from earlier kernels / copies
 
-    const AppendItem item = p.items[blockIdx.x];
-    const int kvh = blockIdx.y;
+    const AppendItem item = p.items[blockIdx.y];          // (all heads of the longest items come first)
+    const int kvh = blockIdx.x;
     const int G = p.group;
     const int PT = 128 / G;                                       // positions per tile
     const int n_tiles = (TILES == 2 && item.n_pos > PT) ? 2 : 1;  // a second tile without rows to compute stays idle
     const int last_pos = item.pos0 + item.n_pos - 1;
     const int n_pg = last_pos / ATTN_PAGE + 1;
-    const int n_blk = (n_pg + APT_PAGES - 1) / APT_PAGES;
+    const int b0 = item.blk0, n_blk = item.blk1 - b0;             // this CTA's key blocks
+    const bool has_end = item.blk1 * APT_PAGES >= n_pg;           // ... include the last one
     const uint32_t base = (smem_u32(apt_smem_raw) + 1023u) & ~1023u;
     const uint32_t q_base = base, p_base = base + TILES * Q_TILE, ring = base + TILES * Q_TILE + TILES * P_TILE;
     {
@@ -667,7 +685,7 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
         int my_page = 0;
         for (int j = 0; j < n_blk; ++j) {
             if ((j & 7) == 0) {          // page ids of the next eight blocks, one per lane
-                const int pg = APT_PAGES * j + lane;
+                const int pg = APT_PAGES * (b0 + j) + lane;
                 my_page = 0;
                 if (pg < n_pg) {
                     my_page = __ldcg(p.block_table + (size_t)item.game * p.max_pages + pg);
@@ -683,7 +701,7 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                 ok = mbar_wait(smem_u32(&kv_empty[s]), (uint32_t)((j / APT_STAGES) - 1) & 1u, abort_flag, p.status,
                                STATUS_TIMEOUT_MMA);
             if (!__shfl_sync(0xffffffffu, ok ? 1 : 0, 0)) break;
-            const int npg = min(APT_PAGES, n_pg - APT_PAGES * j);
+            const int npg = min(APT_PAGES, n_pg - APT_PAGES * (b0 + j));
             const uint32_t stage = ring + (uint32_t)s * STAGE_BYTES;
             if (lane == 0) mbar_expect_tx(smem_u32(&kv_full[s]), (uint32_t)(npg * 2 * SLABS) * PAGE_ROWS_BYTES);
             __syncwarp();
@@ -749,7 +767,7 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
             for (int j = 0; ok && j < n_blk; ++j) {
                 if (j + 1 < n_blk && !issue_qk(j + 1)) break;
                 const int s = j % APT_STAGES;
-                const int npg = min(APT_PAGES, n_pg - APT_PAGES * j);
+                const int npg = min(APT_PAGES, n_pg - APT_PAGES * (b0 + j));
                 const uint64_t dv = smem_desc_sw128_mn(ring + (uint32_t)s * STAGE_BYTES + KV_BYTES, APT_KSLAB, 1024u);
                 if (!mbar_wait_warp(smem_u32(&p_full[t]), (uint32_t)j & 1u, abort_flag, p.status, STATUS_TIMEOUT_EPI)) break;
                 tc_fence_after();
@@ -818,7 +836,7 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                 tc_fence_after();
                 APT_STAMP(0);       // wait for S
                 const uint32_t t_s = t_lane + (uint32_t)((2 * t + b) * APT_BN);
-                const int key0 = j * APT_BN;
+                const int key0 = (b0 + j) * APT_BN;
                 const int vis = key0 + APT_BN - 1 > tile_pos0 ? pos_r - key0 : APT_BN;      // columns 0 .. vis are visible
                 uint32_t v[4][16];
 #pragma unroll
@@ -845,7 +863,7 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                 }
                 const float mx = fmaxf(fmaxf(mxs[0], mxs[1]), fmaxf(mxs[2], mxs[3]));
                 if (j == 0) {
-                    m = mx;                     // key 0 is visible to every row: finite
+                    m = mx;                     // (a later part of an item may hold no key that the row sees: -inf, weights 0)
                 } else {
                     const bool raise = mx > m + APT_RESCALE_LOG2;
                     if (__any_sync(0xffffffffu, raise)) {
@@ -912,10 +930,10 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                 // value rows of positions not written yet hold stale pool bytes (possibly NaN patterns): their
                 // weights are exactly zero, but 0 * NaN is not -- zero them (they lie in the last page loaded).
                 // Both tiles do it (the same zeros) before they release their P.V.
-                if (j == n_blk - 1 && item.kv_len < n_pg * ATTN_PAGE) {
+                if (j == n_blk - 1 && has_end && item.kv_len < n_pg * ATTN_PAGE) {
                     if (!mbar_wait(smem_u32(&kv_full[s]), (uint32_t)(j / APT_STAGES) & 1u, abort_flag, p.status, STATUS_TIMEOUT_TMA))
                         break;
-                    const int npg = n_pg - APT_PAGES * j;
+                    const int npg = n_pg - APT_PAGES * (b0 + j);
                     const int valid = item.kv_len - (n_pg - 1) * ATTN_PAGE;            // rows of the last page that exist
                     const uint32_t vpage = ring + (uint32_t)s * STAGE_BYTES + KV_BYTES + (uint32_t)(npg - 1) * PAGE_ROWS_BYTES;
                     if (qd == 0 && lane < ATTN_PAGE && lane >= valid) {
@@ -938,27 +956,47 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
             if (done_blocks == n_blk && !*abort_flag &&
                 mbar_wait(smem_u32(&o_full[t]), (uint32_t)(n_blk - 1) & 1u, abort_flag, p.status, STATUS_TIMEOUT_MMA)) {
                 tc_fence_after();
-                const float inv = 1.f / l;
                 const int hh = r - po_l * G;
-                uint4* dst = reinterpret_cast<uint4*>(p.out + ((size_t)(item.row0 + po) * p.n_q_heads + kvh * G + hh) * HD);
+                if (item.slot >= 0) {
+                    const size_t prow = ((size_t)item.slot * p.n_kv_heads + kvh) * 256 + t * 128 + r;
+                    uint4* part = reinterpret_cast<uint4*>(p.o_part + prow * HD);
+                    if (row_ok) p.ml_part[prow] = make_float2(m, l);
 #pragma unroll 1
-                for (int c0 = 0; c0 < HD; c0 += 32) {
-                    uint32_t w[2][16];
-                    tmem_ld16_async(t_o + (uint32_t)c0, w[0]);
-                    tmem_ld16_async(t_o + (uint32_t)(c0 + 16), w[1]);
-                    tmem_ld_wait();
-                    if (row_ok) {
+                    for (int c0 = 0; c0 < HD; c0 += 32) {
+                        uint32_t w[2][16];
+                        tmem_ld16_async(t_o + (uint32_t)c0, w[0]);
+                        tmem_ld16_async(t_o + (uint32_t)(c0 + 16), w[1]);
+                        tmem_ld_wait();
+                        if (row_ok) {
 #pragma unroll
-                        for (int h = 0; h < 2; ++h)
+                            for (int h = 0; h < 2; ++h)
 #pragma unroll
-                            for (int q8 = 0; q8 < 2; ++q8) {
-                                uint4 o4;
-                                o4.x = pack_f16(__uint_as_float(w[h][8 * q8]) * inv, __uint_as_float(w[h][8 * q8 + 1]) * inv);
-                                o4.y = pack_f16(__uint_as_float(w[h][8 * q8 + 2]) * inv, __uint_as_float(w[h][8 * q8 + 3]) * inv);
-                                o4.z = pack_f16(__uint_as_float(w[h][8 * q8 + 4]) * inv, __uint_as_float(w[h][8 * q8 + 5]) * inv);
-                                o4.w = pack_f16(__uint_as_float(w[h][8 * q8 + 6]) * inv, __uint_as_float(w[h][8 * q8 + 7]) * inv);
-                                dst[(c0 >> 3) + 2 * h + q8] = o4;
-                            }
+                                for (int q4 = 0; q4 < 4; ++q4)
+                                    part[(c0 >> 2) + 4 * h + q4] = make_uint4(w[h][4 * q4], w[h][4 * q4 + 1], w[h][4 * q4 + 2], w[h][4 * q4 + 3]);
+                        }
+                    }
+                } else {
+                    const float inv = 1.f / l;
+                    uint4* dst = reinterpret_cast<uint4*>(p.out + ((size_t)(item.row0 + po) * p.n_q_heads + kvh * G + hh) * HD);
+#pragma unroll 1
+                    for (int c0 = 0; c0 < HD; c0 += 32) {
+                        uint32_t w[2][16];
+                        tmem_ld16_async(t_o + (uint32_t)c0, w[0]);
+                        tmem_ld16_async(t_o + (uint32_t)(c0 + 16), w[1]);
+                        tmem_ld_wait();
+                        if (row_ok) {
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                                for (int q8 = 0; q8 < 2; ++q8) {
+                                    uint4 o4;
+                                    o4.x = pack_f16(__uint_as_float(w[h][8 * q8]) * inv, __uint_as_float(w[h][8 * q8 + 1]) * inv);
+                                    o4.y = pack_f16(__uint_as_float(w[h][8 * q8 + 2]) * inv, __uint_as_float(w[h][8 * q8 + 3]) * inv);
+                                    o4.z = pack_f16(__uint_as_float(w[h][8 * q8 + 4]) * inv, __uint_as_float(w[h][8 * q8 + 5]) * inv);
+                                    o4.w = pack_f16(__uint_as_float(w[h][8 * q8 + 6]) * inv, __uint_as_float(w[h][8 * q8 + 7]) * inv);
+                                    dst[(c0 >> 3) + 2 * h + q8] = o4;
+                                }
+                        }
                     }
                 }
                 tc_fence_before();
@@ -969,6 +1007,79 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, TM_COLS);
+}
+
+// Adds up the parts of split items: one warp per query row (position x head of the group), all parts' loads in flight.
+// Bound by L2 (4 bytes per element and part read, 2 per element written).
+constexpr int APM_THREADS = 256, APM_MAX_PARTS = 8;
+template <int HD>
+__global__ void __launch_bounds__(APM_THREADS) attn_append_merge_kernel(const AppendMerge* __restrict__ merges, AppendParams p) {
+    constexpr int EL = HD / 32;
+    grid_launch_dependents();
+    const int lane = threadIdx.x & 31, r = blockIdx.x * (APM_THREADS / 32) + (threadIdx.x >> 5);       // row of the two tiles
+    const int kvh = blockIdx.y, G = p.group, PT = 128 / G;
+    const AppendMerge mg = merges[blockIdx.z];                     // (uploaded before the pass's first kernel)
+    const int po_l = (r & 127) / G, po = (r >> 7) * PT + po_l, hh = (r & 127) - po_l * G;
+    if (po_l >= PT || po >= mg.n_pos) return;
+    grid_dependency_wait();
+    const size_t row0 = ((size_t)mg.slot * p.n_kv_heads + kvh) * 256 + r, step = (size_t)p.n_kv_heads * 256;
+    float2 ml[APM_MAX_PARTS];
+    float o[APM_MAX_PARTS][EL];
+#pragma unroll
+    for (int i = 0; i < APM_MAX_PARTS; ++i) {
+        ml[i] = make_float2(-INFINITY, 0.f);
+#pragma unroll
+        for (int e = 0; e < EL; ++e) o[i][e] = 0.f;
+        if (i < mg.parts) {
+            ml[i] = __ldcg(p.ml_part + row0 + i * step);
+            const float* src = p.o_part + (row0 + i * step) * HD + EL * lane;
+#pragma unroll
+            for (int e = 0; e < EL; e += 2) {
+                const float2 v = __ldcg(reinterpret_cast<const float2*>(src + e));
+                o[i][e] = v.x; o[i][e + 1] = v.y;
+            }
+        }
+    }
+    float M = -INFINITY, l = 0.f, acc[EL];
+#pragma unroll
+    for (int i = 0; i < APM_MAX_PARTS; ++i) M = fmaxf(M, ml[i].x);    // finite: key 0 is visible to every row
+#pragma unroll
+    for (int e = 0; e < EL; ++e) acc[e] = 0.f;
+#pragma unroll
+    for (int i = 0; i < APM_MAX_PARTS; ++i) {
+        const float w = fast_exp2(ml[i].x - M);
+        l += w * ml[i].y;
+#pragma unroll
+        for (int e = 0; e < EL; ++e) acc[e] += w * o[i][e];
+    }
+    const float inv = 1.f / l;
+    __half* dst = p.out + ((size_t)(mg.row0 + po) * p.n_q_heads + kvh * G + hh) * HD + EL * lane;
+#pragma unroll
+    for (int e = 0; e < EL; e += 2) *reinterpret_cast<uint32_t*>(dst + e) = pack_f16(acc[e] * inv, acc[e + 1] * inv);
+}
+
+// How the query blocks of a pass are cut along the keys.  A CTA takes about 1.6 us per key block; a few query blocks leave
+// most SMs idle for as long as the longest takes (100 tokens behind 2400: 16 CTAs of 40 blocks; 4967 -> 3767 us per call
+// of the Qwen3-4B shape when cut).  Costs in key blocks: 3 a CTA (prologue, epilogue), 1 more for writing a partial, 5 for
+// the merge; a cut has to win 15 %, since the SMs it fills are where the output projection would request its weights
+// early (331 tokens behind 450: attention 25.8 -> 23.5 us, the call 0.7 % slower).  `blocks`: key blocks per query block;
+// returns the most key blocks of a CTA.
+inline int append_attn_cap(const std::vector<int>& blocks, int heads, int n_sm) {
+    int longest = 0;
+    for (int b : blocks) longest = std::max(longest, b);
+    int best = longest;
+    double best_cost = -1;
+    for (int parts = 1; parts <= APM_MAX_PARTS; ++parts) {
+        const int cap = (longest + parts - 1) / parts;
+        if (parts > 1 && cap < 2) break;
+        long long ctas = 0, sum = 0;
+        for (int b : blocks) { const int n = (b + cap - 1) / cap; ctas += n; sum += b + n * (n > 1 ? 4 : 3); }
+        if (parts > 1 && ctas * heads > 4 * n_sm) break;            // (bounds the partials' buffer, too)
+        const double top = cap + (parts > 1 ? 4 : 3);
+        const double cost = (ctas * heads <= n_sm ? top : (double)sum * heads / n_sm + 0.5 * top) + (parts > 1 ? 5 : 0);
+        if (best_cost < 0 || cost < 0.85 * best_cost) { best_cost = cost; best = cap; }
+    }
+    return best;
 }
 
 }  // namespace spiral

@@ -89,6 +89,10 @@ struct PrefillWs {
     AppendItem* items_dev = nullptr;
     AppendItem* items_host = nullptr;
     int items_cap = 0;
+    std::vector<AppendItem> work;       // host scratch: query blocks of a pass before they are cut
+    size_t part_slots = 0;              // partial results (of every KV head) that o_part / ml_part hold
+    float* o_part = nullptr;
+    float2* ml_part = nullptr;
     cudaEvent_t ev = nullptr;           // the last upload from the pinned mirrors
     bool ev_used = false;
 };
@@ -214,7 +218,7 @@ static void free_ctx(spiral_ctx* c) {
     for (auto& r : c->prof_recs) { cudaEventDestroy(r.e0); cudaEventDestroy(r.e1); }
     for (auto e : c->prof_pool) cudaEventDestroy(e);
     cudaFree(c->pf.x); cudaFree(c->pf.y); cudaFree(c->pf.q); cudaFree(c->pf.h); cudaFree(c->pf.attn); cudaFree(c->pf.act);
-    cudaFree(c->pf.meta_dev); cudaFree(c->pf.items_dev);
+    cudaFree(c->pf.meta_dev); cudaFree(c->pf.items_dev); cudaFree(c->pf.o_part); cudaFree(c->pf.ml_part);
     if (c->pf.meta_host) cudaFreeHost(c->pf.meta_host);
     if (c->pf.items_host) cudaFreeHost(c->pf.items_host);
     if (c->pf.ev) cudaEventDestroy(c->pf.ev);
@@ -1137,7 +1141,7 @@ static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems) {
     y_elems = std::max(y_elems, w.y_elems);
     CU_TRY(cudaDeviceSynchronize());
     cudaFree(w.x); cudaFree(w.y); cudaFree(w.q); cudaFree(w.h); cudaFree(w.attn); cudaFree(w.act);
-    cudaFree(w.meta_dev); cudaFree(w.items_dev);
+    cudaFree(w.meta_dev); cudaFree(w.items_dev); cudaFree(w.o_part); cudaFree(w.ml_part);
     if (w.meta_host) cudaFreeHost(w.meta_host);
     if (w.items_host) cudaFreeHost(w.items_host);
     cudaEvent_t ev = w.ev;
@@ -1146,7 +1150,7 @@ static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems) {
     const spiral_model_desc& d = c->d;
     const size_t R = rows, qd = (size_t)d.n_q_heads * d.head_dim;
     const int per_item = std::min(app_positions_per_item(c->group, false), apt_positions_per_item(c->group, 1));
-    const int items_cap = (rows + per_item - 1) / per_item + c->max_batch + 1;
+    const int items_cap = ((rows + per_item - 1) / per_item + c->max_batch + 1) * APM_MAX_PARTS;      // (a query block may be cut)
     const size_t meta_elems = 4 * R + 2 * (size_t)c->max_batch;
     cudaError_t e = cudaSuccess;
     auto A = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
@@ -1158,9 +1162,9 @@ static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems) {
     A((void**)&w.act, R * d.d_ff * sizeof(__half) + 128);      // (see pg_get_xmap)
     if (e == cudaSuccess && d.d_ff % TC_BK != 0) e = cudaMemset(w.act, 0, R * d.d_ff * sizeof(__half) + 128);
     A((void**)&w.meta_dev, meta_elems * sizeof(int32_t));
-    A((void**)&w.items_dev, (size_t)items_cap * sizeof(AppendItem));
+    A((void**)&w.items_dev, (size_t)items_cap * (sizeof(AppendItem) + sizeof(AppendMerge)));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&w.meta_host, meta_elems * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&w.items_host, (size_t)items_cap * sizeof(AppendItem));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&w.items_host, (size_t)items_cap * (sizeof(AppendItem) + sizeof(AppendMerge)));
     if (e == cudaSuccess && !w.ev) e = cudaEventCreateWithFlags(&w.ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         g_cuda_error = std::string("append workspace: ") + cudaGetErrorString(e);
@@ -1168,6 +1172,25 @@ static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems) {
         return e == cudaErrorMemoryAllocation ? SPIRAL_ERR_OOM : SPIRAL_ERR_CUDA;    // cap stays 0: freed with the context
     }
     w.cap = rows; w.y_elems = y_elems; w.items_cap = items_cap; w.meta_elems = meta_elems; w.ev_used = false;
+    return SPIRAL_OK;
+}
+
+// room for the partial attention results of `slots` parts
+static int prefill_part_reserve(spiral_ctx* c, size_t slots) {
+    PrefillWs& w = c->pf;
+    if (slots <= w.part_slots) return SPIRAL_OK;
+    CU_TRY(cudaDeviceSynchronize());
+    cudaFree(w.o_part); cudaFree(w.ml_part);
+    w.o_part = nullptr; w.ml_part = nullptr; w.part_slots = 0;
+    const size_t rows = slots * c->d.n_kv_heads * 256;
+    cudaError_t e = cudaMalloc((void**)&w.o_part, rows * c->d.head_dim * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&w.ml_part, rows * sizeof(float2));
+    if (e != cudaSuccess) {
+        g_cuda_error = std::string("append partials: ") + cudaGetErrorString(e);
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? SPIRAL_ERR_OOM : SPIRAL_ERR_CUDA;
+    }
+    w.part_slots = slots;
     return SPIRAL_OK;
 }
 
@@ -1208,7 +1231,8 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
         if (w.ev_used) CU_TRY(cudaEventSynchronize(w.ev));       // the pinned mirrors are free again
         int32_t* mh = w.meta_host;
         int32_t* pairs = mh + 4 * (size_t)cap;
-        int nt = 0, n_items = 0, n_pairs = 0;
+        int nt = 0, n_items = 0, n_pairs = 0, n_merges = 0, n_slots = 0;
+        w.work.clear();
         while (nt < chunk && gi < n) {
             const int cnt = offsets[gi + 1] - offsets[gi];
             const int take = std::min(cnt - gt, chunk - nt);
@@ -1224,7 +1248,9 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
                 AppendItem it{};
                 it.game = ids[gi]; it.pos0 = pos0 + b * per_item; it.n_pos = std::min(per_item, take - b * per_item);
                 it.row0 = nt + b * per_item; it.kv_len = pos0 + take;
-                w.items_host[n_items++] = it;
+                it.blk1 = ((it.pos0 + it.n_pos - 1) / ATTN_PAGE + APT_PAGES) / APT_PAGES;       // key blocks up to the last row's own
+                it.slot = -1;
+                w.work.push_back(it);
             }
             if (gt + take == cnt) {
                 pairs[n_pairs] = nt + take - 1;
@@ -1236,7 +1262,30 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
             if (gt == cnt) { gt = 0; ++gi; }
         }
         CU_TRY(cudaMemcpyAsync(w.meta_dev, mh, w.meta_elems * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+        // longest query blocks first, so that the last CTAs to start are short ones; with few of them cut along the keys
+        std::stable_sort(w.work.begin(), w.work.end(), [](const AppendItem& a, const AppendItem& b) { return a.blk1 > b.blk1; });
+        AppendMerge* merges = (AppendMerge*)(w.items_host + w.items_cap);
+        int most = w.work[0].blk1;
+        if (attn_tc && ctx->append_tiles == 2) {
+            std::vector<int> blocks;
+            for (const AppendItem& it : w.work) blocks.push_back(it.blk1);
+            most = append_attn_cap(blocks, d.n_kv_heads, ctx->n_sm);
+        }
+        for (const AppendItem& it : w.work) {
+            const int parts = (it.blk1 + most - 1) / most;
+            for (int k = 0; k < parts; ++k) {
+                AppendItem& q = w.items_host[n_items++];
+                q = it;
+                q.blk0 = it.blk1 * k / parts; q.blk1 = it.blk1 * (k + 1) / parts;
+                if (parts > 1) q.slot = n_slots + k;
+            }
+            if (parts > 1) { merges[n_merges++] = AppendMerge{it.n_pos, it.row0, n_slots, parts}; n_slots += parts; }
+        }
+        rc = prefill_part_reserve(ctx, n_slots);
+        if (rc) return rc;
+        const AppendMerge* merges_dev = (const AppendMerge*)(w.items_dev + w.items_cap);
         CU_TRY(cudaMemcpyAsync(w.items_dev, w.items_host, (size_t)n_items * sizeof(AppendItem), cudaMemcpyHostToDevice, st));
+        if (n_merges) CU_TRY(cudaMemcpyAsync(w.items_dev + w.items_cap, merges, (size_t)n_merges * sizeof(AppendMerge), cudaMemcpyHostToDevice, st));
         CU_TRY(cudaEventRecord(w.ev, st));
         w.ev_used = true;
         int32_t* unused;
@@ -1295,25 +1344,29 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
                 ap.q = w.q; ap.q_lo = w.q + (size_t)cap * qd; ap.items = w.items_dev; ap.block_table = kv->table_dev; ap.max_pages = kv->max_pages;
                 ap.n_pages = kv->n_pages; ap.layer = l; ap.n_q_heads = d.n_q_heads; ap.n_kv_heads = d.n_kv_heads;
                 ap.group = ctx->group;
-                ap.out = w.attn; ap.status = ctx->status;
+                ap.out = w.attn; ap.o_part = w.o_part; ap.ml_part = w.ml_part; ap.status = ctx->status;
                 rec = prof_begin(ctx, SPIRAL_KC_ATTN, st);
                 const int tl = ctx->append_tiles;
                 if (attn_tc && d.head_dim == 128 && tl == 2)
-                    LAUNCH(ctx, (attn_append_tc_kernel<128, 2>), dim3(n_items, d.n_kv_heads), apt_threads(2), apt_smem_bytes(128, 2),
+                    LAUNCH(ctx, (attn_append_tc_kernel<128, 2>), dim3(d.n_kv_heads, n_items), apt_threads(2), apt_smem_bytes(128, 2),
                            st, kv->pool_map16, ap);
                 else if (attn_tc && d.head_dim == 128)
-                    LAUNCH(ctx, (attn_append_tc_kernel<128, 1>), dim3(n_items, d.n_kv_heads), apt_threads(1), apt_smem_bytes(128, 1),
+                    LAUNCH(ctx, (attn_append_tc_kernel<128, 1>), dim3(d.n_kv_heads, n_items), apt_threads(1), apt_smem_bytes(128, 1),
                            st, kv->pool_map16, ap);
                 else if (attn_tc && tl == 2)
-                    LAUNCH(ctx, (attn_append_tc_kernel<64, 2>), dim3(n_items, d.n_kv_heads), apt_threads(2), apt_smem_bytes(64, 2),
+                    LAUNCH(ctx, (attn_append_tc_kernel<64, 2>), dim3(d.n_kv_heads, n_items), apt_threads(2), apt_smem_bytes(64, 2),
                            st, kv->pool_map16, ap);
                 else if (attn_tc)
-                    LAUNCH(ctx, (attn_append_tc_kernel<64, 1>), dim3(n_items, d.n_kv_heads), apt_threads(1), apt_smem_bytes(64, 1),
+                    LAUNCH(ctx, (attn_append_tc_kernel<64, 1>), dim3(d.n_kv_heads, n_items), apt_threads(1), apt_smem_bytes(64, 1),
                            st, kv->pool_map16, ap);
                 else {
                     auto attn = d.head_dim == 128 ? (kv->kv_f16 ? attn_append_kernel<128, true> : attn_append_kernel<128, false>)
                                                   : (kv->kv_f16 ? attn_append_kernel<64, true> : attn_append_kernel<64, false>);
-                    LAUNCH(ctx, attn, dim3(n_items, d.n_kv_heads), APP_THREADS, app_smem_bytes(d.head_dim), st, kv->pool_map, ap);
+                    LAUNCH(ctx, attn, dim3(d.n_kv_heads, n_items), APP_THREADS, app_smem_bytes(d.head_dim), st, kv->pool_map, ap);
+                }
+                if (n_merges) {
+                    auto merge = d.head_dim == 128 ? attn_append_merge_kernel<128> : attn_append_merge_kernel<64>;
+                    LAUNCH(ctx, merge, dim3(256 / (APM_THREADS / 32), d.n_kv_heads, n_merges), APM_THREADS, 0, st, merges_dev, ap);
                 }
                 prof_end(ctx, rec, st);
             }
@@ -1384,10 +1437,18 @@ extern "C" int spiral_prefill(spiral_ctx* ctx, spiral_kv* kv, int n, const int32
         if (rc) return roll_back(rc);
     }
     {
-        // more new tokens than one decode-shaped step holds: dense passes on the tensor cores
-        long long total = 0;
-        for (int i = 0; i < n; ++i) total += offsets[i + 1] - offsets[i];
-        if (ctx->prefill_dense && ctx->pf_ready && total > ctx->max_batch) {
+        // Dense passes on the tensor cores where one decode-shaped step does not hold the new tokens, or where its
+        // attention, which reads a game's cache once per token, would read more than 200 MB per layer: 28 us, what the
+        // dense kernels cost more at these sizes (Qwen3-4B shape, us per call, step / dense: 40 tokens behind 500, 85 MB
+        // per layer, 3011 / 3204; 100 behind 500, 225 MB, 3751 / 3700; 200 behind 2000, 1.7 GB, 9075 / 4834).
+        long long total = 0, reads = 0;
+        for (int i = 0; i < n; ++i) {
+            const long long k = offsets[i + 1] - offsets[i];
+            total += k;
+            reads += k * (start[i] + (k + 1) / 2);
+        }
+        const double step_bytes = (double)reads * 4 * ctx->d.n_kv_heads * ctx->d.head_dim;
+        if (ctx->prefill_dense && ctx->pf_ready && (total > ctx->max_batch || step_bytes > 200e6)) {
             rc = prefill_dense(ctx, kv, n, ids, tokens_dev, offsets, start, last_logits, st);
             if (rc) return roll_back(rc);
             for (int i = 0; i < n; ++i) kv->seq_len[ids[i]] = start[i] + offsets[i + 1] - offsets[i];

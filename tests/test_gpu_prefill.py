@@ -210,3 +210,27 @@ def test_dense_append_with_bf16_pages(overrides, lens):
         _check(*res)
     finally:
         pair.close()
+
+
+@pytest.mark.parametrize("overrides,new", [
+    ({}, [1, 40, 129]),                                                    # 128 positions per query block
+    (dict(n_q_heads=7, n_kv_heads=1, head_dim=64, d_model=448), [37, 3]),  # rows left over in both tiles
+    (dict(n_q_heads=8, n_kv_heads=1, head_dim=128), [33, 16, 50]),         # 32 positions per query block
+])
+def test_dense_append_cut_along_the_keys(overrides, new):
+    """Few query blocks behind long contexts: several CTAs share one, at cuts inside the context and inside the new tokens."""
+    desc = synth.shape("tiny", **overrides)
+    pair = Pair(desc, max_batch=2, max_ctx=1300, n_games=2)
+    try:
+        V = desc["vocab"]
+        worst = [_append(pair, [1], [synth.token_ids(41, 0, 700, V).tolist()])]
+        for i, k in enumerate(new):
+            worst.append(_append(pair, [1, 0], [synth.token_ids(42, i, k, V).tolist(), synth.token_ids(43, i, 190 + i, V).tolist()]))
+        worst.append(_decode(pair, [0, 1], 2, 44))
+        rc, detail = pair.sp.spiral_last_status(pair.ctx)
+        assert rc == 0, detail
+        print("cut along the keys:", overrides, worst)
+        assert max(w[0] for w in worst) <= TOL_MAX_ABS
+        assert max(w[1] for w in worst) <= TOL_REL_RMS
+    finally:
+        pair.close()
