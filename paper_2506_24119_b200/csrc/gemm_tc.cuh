@@ -687,6 +687,7 @@ struct TcWeight {
     bool has_map2 = false;
     int rows = 0, K = 0;
     bool resident = false;      // registered at init: the fp16 copy is converted once
+    bool owned = true;          // w16 is an allocation of its own (else a part of TcState::arena)
 };
 struct TcPlan {
     int grid = 0, max_pieces = 0;
@@ -698,6 +699,8 @@ struct TcState {
     bool skip_x_once = false;   // wait-timeout self-test: the next tc_linear launch leaves its activation loads out
     PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
     std::unordered_map<const void*, TcWeight> weights;
+    __half* arena = nullptr;            // the resident copies, one allocation: with one each (145 for 36 layers) the
+    size_t arena_elems = 0, arena_used = 0;     // allocations took most of spiral_init
     std::map<std::tuple<int, int, int>, TcPlan> plans;                  // (rows, K, whole-tile mode)
     std::map<std::tuple<const void*, int, int, int>, CUtensorMap> xmaps;  // (ptr, K, rows of X, N)
     std::map<std::tuple<const void*, int, int, int>, CUtensorMap> omaps;  // pieces buffer as (ptr, rows, n, pieces)
@@ -761,7 +764,10 @@ inline int tc_init(TcState& tc, int device, int max_batch) {
 }
 
 inline void tc_destroy(TcState& tc) {
-    for (auto& kv : tc.weights) cudaFree(kv.second.w16);
+    for (auto& kv : tc.weights)
+        if (kv.second.owned) cudaFree(kv.second.w16);
+    cudaFree(tc.arena);
+    tc.arena = nullptr; tc.arena_elems = tc.arena_used = 0;
     cudaFree(tc.best);
     cudaFree(tc.done);
     cudaFree(tc.lse_part);
@@ -806,20 +812,41 @@ inline int tc_convert(const __nv_bfloat16* W, __half* w16, int rows, int K, cuda
     return SPIRAL_OK;
 }
 
+// room for the resident fp16 copies of all model weights together
+inline int tc_reserve_weights(TcState& tc, size_t elems) {
+    const cudaError_t e = cudaMalloc((void**)&tc.arena, elems * sizeof(__half));
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        tc.arena = nullptr;
+        g_tc_error = "fp16 weight copies: " + std::string(cudaGetErrorString(e));
+        return e == cudaErrorMemoryAllocation ? SPIRAL_ERR_OOM : SPIRAL_ERR_CUDA;
+    }
+    tc.arena_elems = elems;
+    return SPIRAL_OK;
+}
+
 // fp16 copy + tensor map of one weight matrix.  resident = converted now, once (model weights).
 inline int tc_register_weight(TcState& tc, const __nv_bfloat16* W, int rows, int K, bool resident, cudaStream_t st,
                               int64_t* launches, TcWeight** out) {
     auto it = tc.weights.find(W);
     if (it != tc.weights.end() && (it->second.rows != rows || it->second.K != K)) {
         if (it->second.resident) { g_tc_error = "weight registered with another shape"; return SPIRAL_ERR_INVALID; }
-        cudaFree(it->second.w16);
+        if (it->second.owned) cudaFree(it->second.w16);
         tc.weights.erase(it);
         it = tc.weights.end();
     }
     if (it == tc.weights.end()) {
         TcWeight w;
         w.rows = rows; w.K = K; w.resident = resident;
-        cudaError_t e = cudaMalloc((void**)&w.w16, tc_tiled_elems(rows, K) * sizeof(__half));
+        const size_t elems = tc_tiled_elems(rows, K);           // (a multiple of 8192: 16 KB tiles)
+        cudaError_t e = cudaSuccess;
+        if (resident && tc.arena_used + elems <= tc.arena_elems) {
+            w.w16 = tc.arena + tc.arena_used;
+            tc.arena_used += elems;
+            w.owned = false;
+        } else {
+            e = cudaMalloc((void**)&w.w16, elems * sizeof(__half));
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             g_tc_error = "fp16 weight copy: " + std::string(cudaGetErrorString(e));
@@ -827,10 +854,10 @@ inline int tc_register_weight(TcState& tc, const __nv_bfloat16* W, int rows, int
         }
         // tile-major copy seen as rows of 64 elements: tile (t, kb) = rows (t * KB + kb) * 128 ...
         int rc = tc_encode(tc, &w.map, w.w16, (uint64_t)TC_BK, (uint64_t)(tc_tiled_elems(rows, K) / TC_BK), TC_BM);
-        if (rc) { cudaFree(w.w16); return rc; }
+        if (rc) { if (w.owned) cudaFree(w.w16); return rc; }
         if (resident) {
             rc = tc_convert(W, w.w16, rows, K, st, launches);
-            if (rc) { cudaFree(w.w16); return rc; }
+            if (rc) { if (w.owned) cudaFree(w.w16); return rc; }
         }
         it = tc.weights.emplace(W, w).first;
     }

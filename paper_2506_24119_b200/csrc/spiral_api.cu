@@ -376,6 +376,14 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
             mats.push_back({c->w_down[l], d->d_model, d->d_ff});
         }
         mats.push_back({c->lm_head, d->vocab, d->d_model});
+        size_t elems = 0;
+        for (const M& m : mats)
+            if (tc_usable(c->tc, m.rows, m.k, max_batch)) elems += tc_tiled_elems(m.rows, m.k);
+        if (elems > 0 && (rc = tc_reserve_weights(c->tc, elems)) != SPIRAL_OK) {
+            if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
+            free_ctx(c);
+            return rc;
+        }
         for (const M& m : mats) {
             if (!tc_usable(c->tc, m.rows, m.k, max_batch)) continue;
             rc = tc_register_weight(c->tc, m.w, m.rows, m.k, true, 0, &c->launches, nullptr);
