@@ -234,3 +234,23 @@ def test_dense_append_cut_along_the_keys(overrides, new):
         assert max(w[1] for w in worst) <= TOL_REL_RMS
     finally:
         pair.close()
+
+
+@pytest.mark.parametrize("total", [33, 256, 257, 1024, 1025, 2049])
+def test_dense_append_at_the_edges_of_its_gemms(total):
+    """Token counts around a 256-row tile, around the limits up to which partial sums and narrow tiles are considered, and
+    11 k blocks (d_ff 688) in stages of two."""
+    desc = synth.shape("tiny")
+    pair = Pair(desc, max_batch=8, max_ctx=1200, n_games=3)
+    try:
+        V, games = desc["vocab"], [2, 0, 1]
+        lens = [total // 2, total // 3, total - total // 2 - total // 3]
+        worst = [_append(pair, games, [synth.token_ids(51, i, k, V).tolist() for i, k in enumerate(lens)])]
+        worst.append(_decode(pair, games, 2, 52))
+        rc, detail = pair.sp.spiral_last_status(pair.ctx)
+        assert rc == 0, detail
+        print("append of", total, worst)
+        assert max(w[0] for w in worst) <= TOL_MAX_ABS
+        assert max(w[1] for w in worst) <= TOL_REL_RMS
+    finally:
+        pair.close()
