@@ -72,6 +72,7 @@ struct TcParams {
     unsigned long long* best;   // [256] running argmax keys, zero between launches
     unsigned int* done;         // CTAs finished, zero between launches
     float2* lse_part;           // [grid][256] per-CTA (max, sum exp) of logit/T per batch column (log-prob output)
+    float* best_zt;             // [grid][4][256] logit/T of the best score per (CTA, lane quadrant, batch column) (log-prob output)
 #ifdef TC_PROBE
     unsigned long long* probe;  // [grid][8] timestamps (timing probe builds only)
 #endif
@@ -225,6 +226,7 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
     __shared__ unsigned long long run_sm[MODE == 1 ? 4 : 1][MODE == 1 ? 256 : 1];
     __shared__ float lse_m[MODE == 1 ? 4 : 1][MODE == 1 ? 256 : 1];    // running max / sum of exp(logit/T - max) per
     __shared__ float lse_s[MODE == 1 ? 4 : 1][MODE == 1 ? 256 : 1];    // (lane quadrant, batch column): log-prob output
+    __shared__ float win_sm[MODE == 1 ? 8 : 1][32];                    // logit/T of the best score per epilogue warp and column of a group
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     TRACE_BEGIN(MODE == 1 ? 9 : 8);
@@ -434,6 +436,7 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
             if (sa.defer_sampling) { sa.gumbel = nullptr; sa.tok_out = nullptr; sa.logprob = nullptr; }
         }
         const bool unit_t = sa.temperature == 1.0f;
+        const uint32_t lanes_below = (1u << lane) - 1u;
         TcSchedule sched(p.tiles, p.KB, p.whole_tiles, blockIdx.x, gridDim.x);
         TcSeg sg;
         int blocks_before = 0;               // k blocks of this CTA's earlier segments
@@ -552,6 +555,8 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                             if (sa.logprob) {
                                 // exp(logit/T - the largest of this column's 32 rows); the columns are summed below
                                 const float zt = unit_t ? lg : __fdiv_rn(lg, sa.temperature);
+                                // the lowest row that has the best score leaves its logit/T for lane 16 h + j
+                                if (u == m && (who & lanes_below) == 0u) win_sm[ew][16 * h + j] = zt;
                                 uint32_t uz = __float_as_uint(zt);
                                 uz = (!ok || zt != zt) ? 0u : ((uz & 0x80000000u) ? ~uz : (uz | 0x80000000u));
                                 const uint32_t mz = __reduce_max_sync(0xffffffffu, uz);
@@ -561,6 +566,7 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                             }
                         }
                     }
+                    __syncwarp();
                     if (sa.logprob) {
                         // 32 columns x 32 rows (lanes) -> lane j holds the sum of column c0 + j: halves are exchanged so
                         // that 31 shuffles do it (a reduction per column took five each and most of the epilogue's time:
@@ -588,7 +594,12 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                     const int bcol = c0 + lane;
                     const int vbest = sg.tile * TC_BM + q * 32 + (__ffs(kw) - 1);       // lowest row among equals
                     const unsigned long long kcol = ((unsigned long long)km << 32) | (uint32_t)(0xffffffffu - (uint32_t)vbest);
-                    if (bcol < ce && bcol < p.n && kcol > run_sm[q][bcol]) run_sm[q][bcol] = kcol;
+                    if (bcol < ce && bcol < p.n && kcol > run_sm[q][bcol]) {
+                        run_sm[q][bcol] = kcol;
+                        // (the same lane keeps a column through all tiles: its stores are in order, the last one stays)
+                        if (sa.logprob) p.best_zt[((size_t)blockIdx.x * 4 + q) * 256 + bcol] = win_sm[ew][lane];
+                    }
+                    __syncwarp();                            // (win_sm is written again)
                 }
             }
             tc_fence_before();
@@ -627,10 +638,11 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                     const int tok = (int)(0xffffffffu - (uint32_t)(k & 0xffffffffull));
                     if (sa.tok_out) sa.tok_out[b] = tok;
                     if (sa.logprob) {
-                        // logit/T of the winner = its score minus its noise; logsumexp from the CTAs' partials
-                        const uint32_t ub = (uint32_t)(k >> 32);
-                        const float zbest = __uint_as_float((ub & 0x80000000u) ? (ub ^ 0x80000000u) : ~ub);
-                        const float zt = zbest - (sa.gumbel ? sa.gumbel[(size_t)b * p.rows + tok] : 0.f);
+                        // logit/T of the winner, as kept by the CTA and quadrant that own its row (its score minus its
+                        // noise would have lost the digits by which the noise is larger: 3e-5 with noise of a few
+                        // hundred, everything with noise that forces a token); logsumexp from the CTAs' partials
+                        const int owner = streamk_cta_of(tok / TC_BM, (int)gridDim.x, p.tiles);
+                        const float zt = __ldcg(p.best_zt + ((size_t)owner * 4 + (tok % TC_BM) / 32) * 256 + b);
                         float M = -INFINITY;
                         for (unsigned c = 0; c < gridDim.x; ++c) M = fmaxf(M, __ldcg(&p.lse_part[(size_t)c * 256 + b]).x);
                         float S = 0.f;
@@ -707,6 +719,7 @@ struct TcState {
     unsigned long long* best = nullptr;
     unsigned int* done = nullptr;
     float2* lse_part = nullptr;         // [n_sm][256]
+    float* best_zt = nullptr;           // [n_sm][4][256]
 };
 
 #ifdef TC_PROBE         // timing-probe builds only: eight timestamps per CTA for each of the last 64 launches
@@ -754,6 +767,7 @@ inline int tc_init(TcState& tc, int device, int max_batch) {
     TC_TRY(cudaMemset(tc.best, 0, 256 * sizeof(unsigned long long)));
     TC_TRY(cudaMemset(tc.done, 0, sizeof(unsigned int)));
     TC_TRY(cudaMalloc((void**)&tc.lse_part, (size_t)tc.n_sm * 256 * sizeof(float2)));
+    TC_TRY(cudaMalloc((void**)&tc.best_zt, (size_t)tc.n_sm * 4 * 256 * sizeof(float)));
     TC_TRY(cudaFuncSetAttribute(tc_gemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024));
     TC_TRY(cudaFuncSetAttribute(tc_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 18 * 1024));
 #ifdef SPIRAL_TUNE      // tuning builds only: ring shape from the environment
@@ -771,8 +785,9 @@ inline void tc_destroy(TcState& tc) {
     cudaFree(tc.best);
     cudaFree(tc.done);
     cudaFree(tc.lse_part);
+    cudaFree(tc.best_zt);
     tc.weights.clear(); tc.plans.clear(); tc.xmaps.clear(); tc.omaps.clear();
-    tc.best = nullptr; tc.done = nullptr; tc.lse_part = nullptr; tc.ready = false;
+    tc.best = nullptr; tc.done = nullptr; tc.lse_part = nullptr; tc.best_zt = nullptr; tc.ready = false;
 }
 
 inline bool tc_usable(const TcState& tc, int rows, int K, int n) {
@@ -1028,7 +1043,7 @@ inline int tc_lm_head(TcState& tc, const __nv_bfloat16* W, int vocab, int K, con
     p.rows = vocab; p.n = n; p.N = N;
     size_t smem;
     tc_launch_shape(tc, N, &p, &smem, true);
-    p.status = status; p.args = args_dev; p.best = tc.best; p.done = tc.done; p.lse_part = tc.lse_part;
+    p.status = status; p.args = args_dev; p.best = tc.best; p.done = tc.done; p.lse_part = tc.lse_part; p.best_zt = tc.best_zt;
 #ifdef TC_PROBE
     p.probe = tc_probe_slot();
 #endif

@@ -531,6 +531,34 @@ def test_log_prob_of_the_sampled_token(shape_name, n_games, temperature):
         pair.close()
 
 
+@pytest.mark.parametrize("n_games,vocab", [(1, 4096), (5, 4100), (15, 333), (16, 4096), (130, 4100)])
+def test_log_prob_does_not_lose_digits_to_the_noise(n_games, vocab):
+    """Noise far above the logits (64 x Gumbel, or 1e6 on a token that is to be forced): the log-probability depends on the
+    logits alone.  Bound: fp32 roundings of logit / T, of the maximum plus log-sum and of their difference, each at most
+    half an ulp of values below 32 (1e-6), and of the sum of exponentials (relative 1e-6): 5e-6."""
+    desc = synth.shape("tiny", vocab=vocab)
+    pair = Pair(desc, max_batch=n_games, max_ctx=64, n_games=n_games)
+    try:
+        sp, games, T = pair.sp, list(range(n_games)), 0.7
+        tok_out = torch.empty(n_games, dtype=torch.int32, device="cuda")
+        lp = torch.full((n_games,), float("nan"), dtype=torch.float32, device="cuda")
+        logits = torch.empty(n_games, vocab, dtype=torch.float32, device="cuda")
+        forced = (torch.arange(n_games) * 977 + vocab - 1) % vocab
+        for s in range(2):
+            tok_in = synth.token_ids(22, s, n_games, vocab, stream=synth.STREAM_TEACHER)
+            noise = synth.gumbel_noise(22, s, n_games, vocab) * 64.0
+            if s == 1:
+                noise[torch.arange(n_games), forced] = 1e6
+            sp.spiral_decode_step_logprob(pair.ctx, pair.kv, games, tok_in.cuda(), noise.cuda(), T, tok_out, lp, logits)
+            if s == 1:
+                assert tok_out.cpu().tolist() == forced.tolist()
+            lg, tok = logits.cpu().numpy().astype(np.float64), tok_out.cpu().numpy()
+            ref = [pair.oracle_mod.log_prob(lg[i], int(tok[i]), T) for i in range(n_games)]
+            assert np.abs(lp.cpu().numpy().astype(np.float64) - ref).max() <= 5e-6
+    finally:
+        pair.close()
+
+
 @pytest.mark.parametrize("shape_name,n_games", [("tiny_qknorm", 5), ("tiny", 24)])
 def test_host_buffer_entry_point(shape_name, n_games):
     """spiral_decode_step_host takes tokens and noise from host memory and returns host tokens (the
