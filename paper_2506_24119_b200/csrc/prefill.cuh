@@ -109,6 +109,7 @@ __global__ void __launch_bounds__(PF_RMS_THREADS) pf_rmsnorm_kernel(float* __res
 // (4 bytes read, 2 written per element); with a warp per single head the chain position -> page -> store of every head
 // was what took the time (208 us for 9984 rows of 48 heads).
 // bf16 pages (F16 = false): q leaves as a high and a low bf16 part (q_out, q_lo), k and v are rounded once to bf16.
+// fp16 pages: q leaves as a high and a low fp16 part where q_lo is given (see attn_append_tc_kernel's TWO), else as one.
 constexpr int PF_QKV_THREADS = 256;
 constexpr int PF_QKV_HEADS = 4;
 inline int pf_qkv_groups(int n_q_heads, int n_kv_heads) {        // tasks per token row
@@ -248,12 +249,28 @@ __global__ void __launch_bounds__(PF_QKV_THREADS) pf_qkv_post_kernel(
                         dl[e + HALF] = (uint16_t)l1;
                     }
                 }
-            } else if (E == 2) {
-                *reinterpret_cast<uint32_t*>(dst) = pack_f16(lo[u][0] * sc, lo[u][E - 1] * sc);
-                *reinterpret_cast<uint32_t*>(dst + HALF) = pack_f16(hi[u][0] * sc, hi[u][E - 1] * sc);
             } else {
-                dst[0] = (uint16_t)float_to_f16_bits(lo[u][0] * sc);
-                dst[HALF] = (uint16_t)float_to_f16_bits(hi[u][0] * sc);
+                auto put = [&](uint16_t* at, const float (&l)[E], const float (&h)[E]) {
+                    if (E == 2) {
+                        *reinterpret_cast<uint32_t*>(at) = pack_f16(l[0], l[E - 1]);
+                        *reinterpret_cast<uint32_t*>(at + HALF) = pack_f16(h[0], h[E - 1]);
+                    } else {
+                        at[0] = (uint16_t)float_to_f16_bits(l[0]);
+                        at[HALF] = (uint16_t)float_to_f16_bits(h[0]);
+                    }
+                };
+                float l[E], h[E];
+#pragma unroll
+                for (int e = 0; e < E; ++e) { l[e] = lo[u][e] * sc; h[e] = hi[u][e] * sc; }
+                put(dst, l, h);
+                if (is_q && q_lo) {             // what the rounding left, rounded again
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        l[e] -= unpack_f16(float_to_f16_bits(l[e])).x;
+                        h[e] -= unpack_f16(float_to_f16_bits(h[e])).x;
+                    }
+                    put(reinterpret_cast<uint16_t*>(q_lo) + (dst - reinterpret_cast<uint16_t*>(q_out)), l, h);
+                }
             }
         }
     }
@@ -284,7 +301,8 @@ struct AppendMerge { int n_pos, row0, slot, parts; };
 
 struct AppendParams {
     const __half* q;                // [T][n_q_heads][head_dim] fp16: normalised, rotated, times log2(e)/sqrt(head_dim)
-    const __half* q_lo;             // bf16 pages: q and q_lo are the high and low bf16 parts of the same
+    const __half* q_lo;             // bf16 pages: q and q_lo are the high and low bf16 parts of the same; fp16 pages in two
+                                    // parts: the high and low fp16 parts
     const AppendItem* items;
     const int32_t* block_table;     // [max_games][max_pages]
     int max_pages, n_pages, layer, n_q_heads, n_kv_heads, group;
@@ -566,7 +584,12 @@ constexpr int APT_PAGES = APT_BN / ATTN_PAGE;
 // TILES = 2: one CTA per SM holds two query tiles that share the streamed keys and values (four K/V stages).
 // TILES = 1: one query tile per CTA, two CTAs per SM (two stages each): the keys and values are fetched
 // once per tile, but one CTA's prologue and epilogue run under the other's main loop.
-__host__ __device__ constexpr int apt_stages(int tiles) { return tiles == 1 ? 2 : 4; }
+// TWO (with TILES = 1, one CTA per SM, four stages): the queries and the softmax weights are in two fp16 parts, high and
+// low, each multiplied with the same keys and values into the same accumulator: products with a query and a weight of 22
+// bits, as in the decode kernel.  It serves the appends that a decode-shaped step could hold (prefill_dense says which),
+// so that they lose nothing against it: error of the logits against 64 bits, Qwen3-4B shape, 4 x 25 tokens behind 2000:
+// step 2.98e-3, one part 3.50e-3, two parts 2.97e-3.
+__host__ __device__ constexpr int apt_stages(int tiles, bool two) { return tiles == 1 && !two ? 2 : 4; }
 __host__ __device__ constexpr int apt_threads(int tiles) { return tiles == 1 ? 192 : 352; }   // TMA warp, MMA warp (tile 0), 4 softmax warps per
                                                                           // tile, and for two tiles the MMA warp of tile 1
 constexpr uint32_t APT_QSLAB = 128 * 128;        // 128 query rows of 128 bytes: one 64-element slab of a Q tile / one P tile
@@ -576,10 +599,10 @@ constexpr float APT_RESCALE_LOG2 = 8.f;
 // head_dim 128 fill an SM to the byte (2 x (112 KB of tiles + 1 KB reserved + the barriers)): their slack is
 // what is left, 864 bytes, which suffices where the dynamic region starts 160 bytes past a 1024-byte
 // boundary, as it does behind the kernel's static shared memory; the kernel checks and refuses otherwise.
-inline size_t apt_smem_bytes(int head_dim, int tiles) {
-    const size_t slabs = head_dim / 64;
-    return tiles * slabs * APT_QSLAB + tiles * APT_QSLAB + apt_stages(tiles) * 2 * slabs * APT_KSLAB +
-           (tiles == 1 && head_dim == 128 ? 864 : 1024);
+inline size_t apt_smem_bytes(int head_dim, int tiles, bool two) {
+    const size_t slabs = head_dim / 64, parts = two ? 2 : 1;
+    return tiles * parts * (slabs + 1) * APT_QSLAB + apt_stages(tiles, two) * 2 * slabs * APT_KSLAB +
+           (tiles == 1 && !two && head_dim == 128 ? 864 : 1024);
 }
 inline int apt_positions_per_item(int group, int tiles) { return tiles * (128 / group); }
 
@@ -620,13 +643,15 @@ __device__ unsigned long long g_apt_probe[16];
 #define APT_STAMP(i) do { } while (0)
 #endif
 
-template <int HD, int TILES>
-__global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_append_tc_kernel(const __grid_constant__ CUtensorMap tmKV16,
+template <int HD, int TILES, bool TWO>
+__global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 && !TWO ? 2 : 1) attn_append_tc_kernel(const __grid_constant__ CUtensorMap tmKV16,
                                                                         AppendParams p) {
     constexpr int SLABS = HD / 64;
     constexpr uint32_t Q_TILE = SLABS * APT_QSLAB, P_TILE = APT_QSLAB, KV_BYTES = SLABS * APT_KSLAB;
     constexpr uint32_t STAGE_BYTES = 2 * KV_BYTES;
-    constexpr int APT_STAGES = apt_stages(TILES), APT_THREADS = apt_threads(TILES);
+    constexpr int PARTS = TWO ? 2 : 1;                     // tile t: its high part, then (TWO) its low part, for Q and for P
+    static_assert(!TWO || TILES == 1, "two parts: one query tile per CTA");
+    constexpr int APT_STAGES = apt_stages(TILES, TWO), APT_THREADS = apt_threads(TILES);
     constexpr uint32_t TM_O = 2 * TILES * APT_BN;          // S: (2 tile + buffer) * 64 columns; O: TM_O + tile * HD
     constexpr uint32_t TM_COLS = TILES == 1 ? 256 : 512;
     constexpr uint32_t PAGE_ROWS_BYTES = ATTN_PAGE * 128;  // 16 rows of 128 bytes
@@ -667,7 +692,7 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
     const int b0 = item.blk0, n_blk = item.blk1 - b0;             // this CTA's key blocks
     const bool has_end = item.blk1 * APT_PAGES >= n_pg;           // ... include the last one
     const uint32_t base = (smem_u32(apt_smem_raw) + 1023u) & ~1023u;
-    const uint32_t q_base = base, p_base = base + TILES * Q_TILE, ring = base + TILES * Q_TILE + TILES * P_TILE;
+    const uint32_t q_base = base, p_base = base + TILES * PARTS * Q_TILE, ring = p_base + TILES * PARTS * P_TILE;
     {
         uint32_t dyn_bytes;
         asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_bytes));
@@ -736,8 +761,8 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
 #endif
             bool ok = mbar_wait_warp(smem_u32(&q_ready), 0u, abort_flag, p.status, STATUS_TIMEOUT_EPI);
             APT_STAMP(6);           // MMA warp: wait for Q
-            const uint64_t da0 = smem_desc_sw128(q_base + (uint32_t)t * Q_TILE);
-            const uint64_t dp = smem_desc_sw128(p_base + (uint32_t)t * P_TILE);
+            const uint64_t da0 = smem_desc_sw128(q_base + (uint32_t)(t * PARTS) * Q_TILE);
+            const uint64_t dp = smem_desc_sw128(p_base + (uint32_t)(t * PARTS) * P_TILE);
             auto issue_qk = [&](int j) -> bool {
                 const int s = j % APT_STAGES, b = j & 1;
                 if (!mbar_wait_warp(smem_u32(&kv_full[s]), (uint32_t)(j / APT_STAGES) & 1u, abort_flag, p.status, STATUS_TIMEOUT_TMA))
@@ -752,11 +777,13 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                 const uint32_t d_s = tmem_base + (uint32_t)((2 * t + b) * APT_BN);
                 if (elect_one()) {
 #pragma unroll
-                    for (int h = 0; h < SLABS; ++h)
+                    for (int part = 0; part < PARTS; ++part)
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            tc_mma_f16(d_s, da0 + (uint64_t)(h * (APT_QSLAB >> 4) + 2 * k), db0 + (uint64_t)(h * (APT_KSLAB >> 4) + 2 * k),
-                                       idesc_qk, (h > 0 || k > 0) ? 1u : 0u);
+                        for (int h = 0; h < SLABS; ++h)
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                tc_mma_f16(d_s, da0 + (uint64_t)(part * (Q_TILE >> 4) + h * (APT_QSLAB >> 4) + 2 * k),
+                                           db0 + (uint64_t)(h * (APT_KSLAB >> 4) + 2 * k), idesc_qk, (part > 0 || h > 0 || k > 0) ? 1u : 0u);
                     tc_commit(smem_u32(&s_full[t][b]));
                 }
                 __syncwarp();
@@ -775,8 +802,10 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                 if (elect_one()) {
                     const uint32_t d_o = tmem_base + TM_O + (uint32_t)(t * HD);
                     for (int ks = 0; ks < npg; ++ks)             // one page = 16 keys = one k step
-                        tc_mma_f16(d_o, dp + (uint64_t)(2 * ks), dv + (uint64_t)(ks * (PAGE_ROWS_BYTES >> 4)), idesc_pv,
-                                   (j > 0 || ks > 0) ? 1u : 0u);
+#pragma unroll
+                        for (int part = 0; part < PARTS; ++part)
+                            tc_mma_f16(d_o, dp + (uint64_t)(part * (P_TILE >> 4) + 2 * ks), dv + (uint64_t)(ks * (PAGE_ROWS_BYTES >> 4)),
+                                       idesc_pv, (j > 0 || ks > 0 || part > 0) ? 1u : 0u);
                     tc_commit(smem_u32(&o_full[t]));
                     tc_commit(smem_u32(&p_empty[t]));
                     // the stage is free once both tiles' MMAs on it have completed (one tile: it arrives for both)
@@ -810,11 +839,14 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                 const int pl = rr / G, h2 = rr - pl * G;
                 const int pp = t * PT + pl;
                 const bool okr = pl < PT && pp < item.n_pos;
-                const uint4 v = __ldcg(reinterpret_cast<const uint4*>(
-                                           p.q + ((size_t)(item.row0 + (okr ? pp : 0)) * p.n_q_heads + kvh * G + h2) * HD) + c);
-                const uint32_t dst = q_base + (uint32_t)t * Q_TILE + (uint32_t)(c >> 3) * APT_QSLAB + (uint32_t)rr * 128u +
-                                     (uint32_t)(((c & 7) ^ (rr & 7)) << 4);
-                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+                const size_t row = ((size_t)(item.row0 + (okr ? pp : 0)) * p.n_q_heads + kvh * G + h2) * HD;
+#pragma unroll
+                for (int part = 0; part < PARTS; ++part) {
+                    const uint4 v = __ldcg(reinterpret_cast<const uint4*>((part ? p.q_lo : p.q) + row) + c);
+                    const uint32_t dst = q_base + (uint32_t)(t * PARTS + part) * Q_TILE + (uint32_t)(c >> 3) * APT_QSLAB + (uint32_t)rr * 128u +
+                                         (uint32_t)(((c & 7) ^ (rr & 7)) << 4);
+                    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+                }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
@@ -893,6 +925,14 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                 APT_STAMP(2);       // maximum (and rescale)
                 float sums[4];
                 uint32_t w[4][8];               // the row of P as fp16 pairs, ready before the buffer is waited for
+                uint32_t wl[TWO ? 4 : 1][8];    // what their rounding left
+                auto keep = [&](int h, int i, float e0, float e1) {
+                    w[h][i >> 1] = pack_unit_f16(e0, e1);
+                    if (TWO) {
+                        const float2 got = unpack_f16(w[h][i >> 1]);
+                        wl[TWO ? h : 0][i >> 1] = pack_unit_f16(e0 - got.x, e1 - got.y);
+                    }
+                };
 #pragma unroll
                 for (int h = 0; h < 4; ++h) {
                     sums[h] = 0.f;
@@ -902,7 +942,7 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                             const float e0 = fast_exp2(__uint_as_float(v[h][i]) - m);
                             const float e1 = fast_exp2(__uint_as_float(v[h][i + 1]) - m);
                             sums[h] += e0 + e1;
-                            w[h][i >> 1] = pack_unit_f16(e0, e1);
+                            keep(h, i, e0, e1);
                         }
                     } else {
 #pragma unroll
@@ -911,7 +951,7 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                             const float e0 = col <= vis ? fast_exp2(__uint_as_float(v[h][i]) - m) : 0.f;
                             const float e1 = col + 1 <= vis ? fast_exp2(__uint_as_float(v[h][i + 1]) - m) : 0.f;
                             sums[h] += e0 + e1;
-                            w[h][i >> 1] = pack_unit_f16(e0, e1);
+                            keep(h, i, e0, e1);
                         }
                     }
                 }
@@ -922,10 +962,15 @@ __global__ void __launch_bounds__(apt_threads(TILES), TILES == 1 ? 2 : 1) attn_a
                 APT_STAMP(4);       // wait for the P buffer
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {           // 16-byte chunk (8 keys) of the row
-                    const uint32_t dst = p_base + (uint32_t)t * P_TILE + (uint32_t)r * 128u + (uint32_t)((c ^ (r & 7)) << 4);
+                    const uint32_t dst = p_base + (uint32_t)(t * PARTS) * P_TILE + (uint32_t)r * 128u + (uint32_t)((c ^ (r & 7)) << 4);
                     asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(w[c >> 1][4 * (c & 1)]),
                                  "r"(w[c >> 1][4 * (c & 1) + 1]), "r"(w[c >> 1][4 * (c & 1) + 2]), "r"(w[c >> 1][4 * (c & 1) + 3])
                                  : "memory");
+                    if (TWO) {
+                        const uint32_t(&x)[8] = wl[TWO ? c >> 1 : 0];
+                        asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(dst + P_TILE), "r"(x[4 * (c & 1)]),
+                                     "r"(x[4 * (c & 1) + 1]), "r"(x[4 * (c & 1) + 2]), "r"(x[4 * (c & 1) + 3]) : "memory");
+                    }
                 }
                 // value rows of positions not written yet hold stale pool bytes (possibly NaN patterns): their
                 // weights are exactly zero, but 0 * NaN is not -- zero them (they lie in the last page loaded).

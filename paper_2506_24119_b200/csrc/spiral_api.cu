@@ -415,10 +415,12 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
             if (rc == SPIRAL_OK) e = cudaFuncSetAttribute((attn_append_kernel<128, false>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem_bytes(128));
             if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_kernel<64, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem_bytes(64));
             if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_kernel<64, false>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)app_smem_bytes(64));
-            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<128, 1>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(128, 1));
-            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<128, 2>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(128, 2));
-            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<64, 1>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(64, 1));
-            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<64, 2>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(64, 2));
+            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<128, 1, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(128, 1, true));
+            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<64, 1, true>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(64, 1, true));
+            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<128, 1, false>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(128, 1, false));
+            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<128, 2, false>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(128, 2, false));
+            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<64, 1, false>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(64, 1, false));
+            if (rc == SPIRAL_OK && e == cudaSuccess) e = cudaFuncSetAttribute((attn_append_tc_kernel<64, 2, false>), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apt_smem_bytes(64, 2, false));
             if (rc != SPIRAL_OK || e != cudaSuccess) {
                 g_cuda_error = rc != SPIRAL_OK ? tc_last_error() : std::string("append attention shared memory: ") + cudaGetErrorString(e);
                 free_ctx(c);
@@ -1225,8 +1227,13 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
     if (rc) return rc;
     PrefillWs& w = ctx->pf;
     const int cap = w.cap, MB = ctx->max_batch;
-    const bool attn_tc = ctx->append_attn_tc && kv->kv_f16;
-    const int per_item = attn_tc ? apt_positions_per_item(ctx->group, ctx->append_tiles)
+    // Calls that the decode-shaped step could hold, or contexts for fewer games than a dense contraction needs: these
+    // leave the decode kernel's attention, whose queries and softmax weights are in two parts, only for another with the
+    // same precision.  Longer appends have always had them in one fp16 part.
+    const bool two = kv->kv_f16 && (total <= MB || MB < TC_MIN_BATCH);
+    const bool attn_tc = kv->kv_f16 && (two || ctx->append_attn_tc);
+    const int tiles = two ? 1 : ctx->append_tiles;
+    const int per_item = attn_tc ? apt_positions_per_item(ctx->group, tiles)
                                  : app_positions_per_item(ctx->group, kv->kv_f16);
     const float eps = (float)d.rms_eps;
     int32_t* mdev = w.meta_dev;
@@ -1274,7 +1281,7 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
         std::stable_sort(w.work.begin(), w.work.end(), [](const AppendItem& a, const AppendItem& b) { return a.blk1 > b.blk1; });
         AppendMerge* merges = (AppendMerge*)(w.items_host + w.items_cap);
         int most = w.work[0].blk1;
-        if (attn_tc && ctx->append_tiles == 2) {
+        if (attn_tc && (two || tiles == 2)) {
             std::vector<int> blocks;
             for (const AppendItem& it : w.work) blocks.push_back(it.blk1);
             most = append_attn_cap(blocks, d.n_kv_heads, ctx->n_sm);
@@ -1345,7 +1352,7 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
                                               : (kv->kv_f16 ? pf_qkv_post_kernel<64, true> : pf_qkv_post_kernel<64, false>);
                 LAUNCH(ctx, post, qgrid, PF_QKV_THREADS, 0, st, pq, ctx->bqkv[l], ctx->q_norm[l], ctx->k_norm[l], eps, ctx->cos_tab,
                        ctx->sin_tab, meta.game, meta.pos, kv->table_dev, kv->max_pages, kv->n_pages, l, nt, d.n_q_heads, d.n_kv_heads,
-                       q_scale, w.q, w.q + (size_t)cap * qd, kv->pool, ctx->status);
+                       q_scale, w.q, two || !kv->kv_f16 ? w.q + (size_t)cap * qd : nullptr, kv->pool, ctx->status);
             }
             {
                 AppendParams ap{};
@@ -1354,27 +1361,18 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
                 ap.group = ctx->group;
                 ap.out = w.attn; ap.o_part = w.o_part; ap.ml_part = w.ml_part; ap.status = ctx->status;
                 rec = prof_begin(ctx, SPIRAL_KC_ATTN, st);
-                const int tl = ctx->append_tiles;
-                if (attn_tc && d.head_dim == 128 && tl == 2)
-                    LAUNCH(ctx, (attn_append_tc_kernel<128, 2>), dim3(d.n_kv_heads, n_items), apt_threads(2), apt_smem_bytes(128, 2),
-                           st, kv->pool_map16, ap);
-                else if (attn_tc && d.head_dim == 128)
-                    LAUNCH(ctx, (attn_append_tc_kernel<128, 1>), dim3(d.n_kv_heads, n_items), apt_threads(1), apt_smem_bytes(128, 1),
-                           st, kv->pool_map16, ap);
-                else if (attn_tc && tl == 2)
-                    LAUNCH(ctx, (attn_append_tc_kernel<64, 2>), dim3(d.n_kv_heads, n_items), apt_threads(2), apt_smem_bytes(64, 2),
-                           st, kv->pool_map16, ap);
-                else if (attn_tc)
-                    LAUNCH(ctx, (attn_append_tc_kernel<64, 1>), dim3(d.n_kv_heads, n_items), apt_threads(1), apt_smem_bytes(64, 1),
-                           st, kv->pool_map16, ap);
-                else {
+                if (attn_tc) {
+                    auto attn = d.head_dim == 128 ? (two ? attn_append_tc_kernel<128, 1, true> : tiles == 2 ? attn_append_tc_kernel<128, 2, false> : attn_append_tc_kernel<128, 1, false>)
+                                                  : (two ? attn_append_tc_kernel<64, 1, true> : tiles == 2 ? attn_append_tc_kernel<64, 2, false> : attn_append_tc_kernel<64, 1, false>);
+                    LAUNCH(ctx, attn, dim3(d.n_kv_heads, n_items), apt_threads(tiles), apt_smem_bytes(d.head_dim, tiles, two), st, kv->pool_map16, ap);
+                } else {
                     auto attn = d.head_dim == 128 ? (kv->kv_f16 ? attn_append_kernel<128, true> : attn_append_kernel<128, false>)
                                                   : (kv->kv_f16 ? attn_append_kernel<64, true> : attn_append_kernel<64, false>);
                     LAUNCH(ctx, attn, dim3(d.n_kv_heads, n_items), APP_THREADS, app_smem_bytes(d.head_dim), st, kv->pool_map, ap);
                 }
                 if (n_merges) {
                     auto merge = d.head_dim == 128 ? attn_append_merge_kernel<128> : attn_append_merge_kernel<64>;
-                    LAUNCH(ctx, merge, dim3(256 / (APM_THREADS / 32), d.n_kv_heads, n_merges), APM_THREADS, 0, st, merges_dev, ap);
+                    LAUNCH(ctx, merge, dim3(128 * tiles / (APM_THREADS / 32), d.n_kv_heads, n_merges), APM_THREADS, 0, st, merges_dev, ap);
                 }
                 prof_end(ctx, rec, st);
             }

@@ -254,3 +254,41 @@ def test_dense_append_at_the_edges_of_its_gemms(total):
         assert max(w[1] for w in worst) <= TOL_REL_RMS
     finally:
         pair.close()
+
+
+@pytest.mark.parametrize("overrides,lens", [
+    ({}, [64, 3, 129, 40]),                                                          # 2 heads per group, head_dim 64
+    (dict(n_q_heads=8, n_kv_heads=2, head_dim=128), [33, 50, 16, 100]),              # 32 positions per query block
+    (dict(n_q_heads=7, n_kv_heads=1, head_dim=64, d_model=448), [37, 18, 19, 70]),   # a group that does not divide 128 rows
+])
+def test_dense_append_in_place_of_steps_loses_no_precision(monkeypatch, overrides, lens):
+    """A context for few games appends in dense passes what it would otherwise append in decode-shaped steps, whose queries
+    and softmax weights are in two parts (22 bits).  One layer without an MLP, so that the attention is what differs.
+    Bound: a value that differs by d before it is rounded to fp16 (steps of u = 2^-10.5) differs by sqrt(d u) rms after it,
+    because a share d / u of the values rounds the other way.  Another order of sums, d = 2^-20, gives 2^-15.3 in the cached
+    keys and values, that 2^-12.9 in the attention's output, and that, half of the residual stream, 2^-12.2 in the LM
+    head's input; 2^-12 is allowed.  A single fp16 rounding of queries and weights gave 2^-11.5 to 2^-11.2 here."""
+    desc = synth.shape("tiny_qknorm", n_layers=1, **overrides)
+    w = synth.perturb_gains(synth.make_weights(desc))
+    w["w_down"][0].zero_()
+    V, out = desc["vocab"], {}
+    prompts = [synth.token_ids(61, i, k, V).tolist() for i, k in enumerate(lens)]
+    games = [3, 0, 2, 1]
+    for dense in ("0", "1"):
+        monkeypatch.setenv("SPIRAL_PREFILL_DENSE", dense)
+        pair = Pair(desc, max_batch=8, max_ctx=320, n_games=4, weights_cpu=w)
+        try:
+            rows = []
+            for part in range(2):               # onto nothing, then onto the cached first half
+                new = [p[:len(p) // 2] if part == 0 else p[len(p) // 2:] for p in prompts]
+                flat = torch.tensor(sum(new, []), dtype=torch.int32).cuda()
+                offs = np.concatenate([[0], np.cumsum([len(t) for t in new])]).tolist()
+                last = torch.empty(4, V, dtype=torch.float32, device="cuda")
+                pair.sp.spiral_prefill(pair.ctx, pair.kv, games, flat, offs, last)
+                rows.append(last.cpu().numpy().astype(np.float64))
+            out[dense] = np.concatenate(rows)
+        finally:
+            pair.close()
+    rel = np.sqrt(((out["0"] - out["1"]) ** 2).sum() / (out["0"] ** 2).sum())
+    print(overrides, "dense against steps: rel %.2e" % rel)
+    assert rel <= 2.0 ** -12
