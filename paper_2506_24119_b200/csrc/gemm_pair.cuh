@@ -38,6 +38,7 @@ struct PgParams {
     int whole, row_fastest;         // whole tiles or stream-K; order of whole tiles (see pg_tile_of)
     int stages;                     // ring depth
     int w_once;                     // 1: weight tiles are read by few token tiles and leave L2 first
+    float unscale;                  // what the sums are multiplied with (TcWeight::unscale)
     int* status;
 };
 
@@ -122,7 +123,7 @@ __device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* map, uint32
 }
 
 // tmOut: STORE: [piece][T][rows] floats; ADD: [1][T][rows] floats; box 1 x 32 x 32.  SILU: [1][T][rows / 2] fp16, box 1 x 32 x 16.
-template <int EPI>
+template <int EPI, bool SCALED>           // SCALED: p.unscale != 1
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
     pg_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
                    const __grid_constant__ CUtensorMap tmOut, PgParams p) {
@@ -289,6 +290,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
                     __syncwarp();
                 }
                 tmem_ld_wait();
+                if (SCALED) tc_unscale(v, p.unscale);
                 if (EPI == PG_SILU) {
                     // even lanes hold gate features, odd lanes the matching up features: per pair of token columns the
                     // even lane finishes the first and the odd lane the second
@@ -487,8 +489,8 @@ inline int pg_gemm(TcState& tc, const PgPlan& pl, const __nv_bfloat16* W, int ro
     PgParams p{};
     p.row_tiles = pl.row_tiles; p.tok_tiles = pl.tok_tiles; p.KB = pl.KB; p.T = T; p.N = pl.N; p.whole = pl.whole;
     p.row_fastest = (pl.whole && T > rows) ? 1 : 0;              // re-read the smaller operand: weights rows x K, activations T x K
-    p.stages = pl.stages; p.w_once = pl.tok_tiles <= 2; p.status = status;
-    TC_TRY(launch_kernel(true, pg_gemm_kernel<EPI>, dim3(2 * pl.G), dim3(PG_THREADS), pl.smem, st, *wm, *xm, *om, p));
+    p.stages = pl.stages; p.w_once = pl.tok_tiles <= 2; p.status = status; p.unscale = it->second.unscale;
+    TC_TRY(launch_kernel(true, it->second.unscale != 1.f ? pg_gemm_kernel<EPI, true> : pg_gemm_kernel<EPI, false>, dim3(2 * pl.G), dim3(PG_THREADS), pl.smem, st, *wm, *xm, *om, p));
     if (launches) ++*launches;
     if (pieces) {
         pieces->base = (const float*)out; pieces->stride = (size_t)T * rows; pieces->ld = rows; pieces->n_pieces = pl.max_pieces;
@@ -499,9 +501,9 @@ inline int pg_gemm(TcState& tc, const PgPlan& pl, const __nv_bfloat16* W, int ro
 }
 
 inline int pg_gemm_setup() {
-    TC_TRY(cudaFuncSetAttribute(pg_gemm_kernel<PG_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM_BUDGET));
-    TC_TRY(cudaFuncSetAttribute(pg_gemm_kernel<PG_ADD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM_BUDGET));
-    TC_TRY(cudaFuncSetAttribute(pg_gemm_kernel<PG_SILU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM_BUDGET));
+    for (auto kern : {pg_gemm_kernel<PG_STORE, false>, pg_gemm_kernel<PG_STORE, true>, pg_gemm_kernel<PG_ADD, false>,
+                      pg_gemm_kernel<PG_ADD, true>, pg_gemm_kernel<PG_SILU, false>, pg_gemm_kernel<PG_SILU, true>})
+        TC_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM_BUDGET));
     return SPIRAL_OK;
 }
 

@@ -1,6 +1,6 @@
 // Weight-streaming skinny GEMM on the 5th-generation tensor cores (tcgen05, sm_100a):
 //     Y[b][r] = sum_k W[r][k] * X[b][k]        W fp16 [rows][K] (a private fp16 re-encoding of the
-//     caller's bf16 weights), X fp16 [n][K], fp32 accumulation in tensor memory.
+//     caller's bf16 weights, times a power of two where they need one), X fp16 [n][K], fp32 accumulation in tensor memory.
 // The weight matrix is the 128-row M operand ("swap-AB"), the batch is the N operand, so one CTA
 // reads each weight byte exactly once and the whole batch shares it.  The op is HBM-bound for
 // n <= ~200: the kernel is organised around keeping TMA loads in flight, not around the MMAs.
@@ -26,7 +26,10 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
+#include <cmath>
 #include <cstdlib>
+#include <cstring>
 #include <map>
 #include <string>
 #include <tuple>
@@ -64,6 +67,7 @@ struct TcParams {
     int tma_out;                // 1: pieces leave through shared memory and TMA stores (tmOut), 0: plain stores
     int skip_x;                 // wait-timeout self-test only: the producer leaves the activation loads out, so the
                                 // "stage full" barriers never complete and every role has to give up and unwind
+    float unscale;              // what the sums are multiplied with: a power of two (see bf16_to_f16_tiled_kernel)
     float* out;                 // pieces [piece][n][rows]
     size_t piece_stride;
     int* status;
@@ -139,6 +143,14 @@ __device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t (&r)[16
         : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// sums of a matrix that was encoded times a power of two, back to their size (powers of two: exact in any order).  Rare, and
+// therefore in kernels of their own (SCALED): multiplied always, or behind a branch, it cost 0.6 % of a step of 128 games.
+__device__ __forceinline__ void tc_unscale(uint32_t (&v)[2][16], float unscale) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[h][j] = __float_as_uint(__uint_as_float(v[h][j]) * unscale);
+}
 // Shared-memory matrix descriptor of a K-major tile whose rows are 128 bytes (64 fp16) with the
 // 128-byte swizzle TMA wrote: 8-row groups are 1024 bytes apart (stride byte offset), the leading
 // byte offset is unused for this layout, descriptor version 1, layout type 2 = SWIZZLE_128B.
@@ -212,7 +224,7 @@ struct TcRun {
 // ------------------------------------------------------------------------------------------------
 // tmOut (MODE 0 with p.tma_out): the pieces buffer as a tensor [piece][batch row][feature] of floats with a
 // box of 1 x 32 x 32
-template <int MODE>     // 0: pieces to memory; 1: LM head with fused Gumbel-argmax
+template <int MODE, bool SCALED>     // MODE 0: pieces to memory; 1: LM head with fused Gumbel-argmax.  SCALED: p.unscale != 1
 // (register cap instead of launch bounds: at 112 registers the seven warps of a layer projection fit into an SM's
 // register file beside the CTA of the element-wise kernel before or after it, so that either can start early)
 __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_constant__ CUtensorMap tmW,
@@ -478,6 +490,10 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                         __syncwarp();
                     }
                     tmem_ld_wait();
+                    if (SCALED) {
+                        tc_unscale(v, p.unscale);
+                        if (both) tc_unscale(w, p.unscale);
+                    }
 #pragma unroll
                     for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -504,7 +520,7 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                         for (int j = 0; j < 16; ++j)
                             if (c0 + j < p.n)
                                 dst[(size_t)(c0 + j) * p.rows] =
-                                    both ? __fadd_rn(__uint_as_float(v[j]), __uint_as_float(w[j])) : __uint_as_float(v[j]);
+                                    (both ? __fadd_rn(__uint_as_float(v[j]), __uint_as_float(w[j])) : __uint_as_float(v[j])) * (SCALED ? p.unscale : 1.f);
                     }
                 }
             } else {
@@ -534,6 +550,7 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
                             for (int j = 0; j < 16; ++j)
                                 if (c0 + 16 * h < ce) v[h][j] = __float_as_uint(__fadd_rn(__uint_as_float(v[h][j]), __uint_as_float(w[h][j])));
                     }
+                    if (SCALED) tc_unscale(v, p.unscale);
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         if (c0 + 16 * h >= ce) break;
@@ -664,15 +681,19 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
     if (threadIdx.x == 0) TC_STAMP(7);
 }
 
-// fp16 re-encoding of bf16 weights (exact for |w| in [2^-14, 65504]; smaller magnitudes round to
-// fp16 subnormals / zero, an absolute error below 2^-25), written TILE-MAJOR: the [128 rows x 64 k]
+// fp16 re-encoding of bf16 weights times `scale`, a power of two, written TILE-MAJOR: the [128 rows x 64 k]
 // tile (row tile t, k block kb) occupies the 16 KB starting at element ((t * KB + kb) * 128) * 64,
 // rows of 128 bytes, zero-padded at the ragged edges.  One TMA box is then one contiguous 16 KB run
 // of DRAM instead of 128 separate 128-byte row segments.
+// bf16 has three bits less than fp16, so w * scale is exact for magnitudes in [2^-14, 65504]; smaller ones round to fp16
+// subnormals / zero, an absolute error below 2^-25.  `lossy` (when given) is set where that loses, anywhere, more than
+// 2^-21 of the absolute sum of 64 weights of a row -- far below what an fp32 sum of thousands of products rounds, far above
+// what normally distributed weights of the usual sizes lose (2^-28 at a deviation of 0.02).  Such a matrix is encoded again
+// with its largest magnitude moved to [2^14, 2^15): everything down to 2^-28 of that is then exact (tc_rescale).
 __global__ void bf16_to_f16_tiled_kernel(const __nv_bfloat16* __restrict__ src, __half* __restrict__ dst, int rows,
-                                         int K, int KB, size_t n_chunks) {
+                                         int K, int KB, size_t n_chunks, float scale, int* __restrict__ lossy) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;       // one 8-element (16-byte) chunk of dst
-    if (i >= n_chunks) return;
+    if (i >= n_chunks) return;                       // (n_chunks is a multiple of 1024: whole CTAs)
     const int kc = (int)(i & 7);                     // chunk within the 64-wide row
     const size_t rowi = i >> 3;                      // row of the tiled array
     const int rr = (int)(rowi & 127);
@@ -682,12 +703,49 @@ __global__ void bf16_to_f16_tiled_kernel(const __nv_bfloat16* __restrict__ src, 
     const size_t r = t * TC_BM + rr;
     const int k0 = kb * TC_BK + kc * 8;
     uint4 o = make_uint4(0u, 0u, 0u, 0u);
+    float err = 0.f, sum = 0.f;
     if (r < (size_t)rows && k0 < K) {                // K is a multiple of 8: a chunk is inside or outside
-        uint4 v = *reinterpret_cast<const uint4*>(src + r * K + k0);
-        o.x = pack_f16(bf16_lo(v.x), bf16_hi(v.x)); o.y = pack_f16(bf16_lo(v.y), bf16_hi(v.y));
-        o.z = pack_f16(bf16_lo(v.z), bf16_hi(v.z)); o.w = pack_f16(bf16_lo(v.w), bf16_hi(v.w));
+        const uint4 v = *reinterpret_cast<const uint4*>(src + r * K + k0);
+        const uint32_t in[4] = {v.x, v.y, v.z, v.w};
+        uint32_t out[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float a = bf16_lo(in[e]) * scale, b = bf16_hi(in[e]) * scale;
+            // (a scaled matrix holds nothing finite that saturates; infinities and NaN stay what they are)
+            const __half2 h2 = __floats2half2_rn(a, b);
+            out[e] = scale == 1.f ? pack_f16(a, b) : *reinterpret_cast<const uint32_t*>(&h2);
+            const float2 got = unpack_f16(out[e]);
+            err += fabsf(a - got.x) + fabsf(b - got.y);
+            sum += fabsf(a) + fabsf(b);
+        }
+        o = make_uint4(out[0], out[1], out[2], out[3]);
     }
     *reinterpret_cast<uint4*>(dst + i * 8) = o;
+    if (lossy) {
+#pragma unroll
+        for (int d = 1; d < 8; d <<= 1) {            // the eight chunks of a row's 64 weights sit in neighbouring lanes
+            err += __shfl_xor_sync(0xffffffffu, err, d);
+            sum += __shfl_xor_sync(0xffffffffu, sum, d);
+        }
+        if (kc == 0 && !(err <= sum * 4.76837158203125e-7f)) atomicOr(lossy, 1);         // (infinities and NaN, too)
+    }
+}
+
+// largest finite magnitude of n weights (n a multiple of 8), as fp32 bits
+__global__ void __launch_bounds__(256) bf16_max_kernel(const __nv_bfloat16* __restrict__ src, size_t n, unsigned int* __restrict__ out) {
+    uint32_t m = 0u;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n / 8; i += (size_t)gridDim.x * blockDim.x) {
+        const uint4 v = reinterpret_cast<const uint4*>(src)[i];
+        const uint32_t in[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t a = (in[e] << 16) & 0x7fffffffu, b = in[e] & 0x7fff0000u;
+            if (a < 0x7f800000u) m = max(m, a);
+            if (b < 0x7f800000u) m = max(m, b);
+        }
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -698,6 +756,7 @@ struct TcWeight {
     CUtensorMap map, map2;      // boxes of one 128 x 64 tile / of two (append path, made at its first use)
     bool has_map2 = false;
     int rows = 0, K = 0;
+    float unscale = 1.f;        // w16 holds the weights divided by this
     bool resident = false;      // registered at init: the fp16 copy is converted once
     bool owned = true;          // w16 is an allocation of its own (else a part of TcState::arena)
 };
@@ -768,8 +827,10 @@ inline int tc_init(TcState& tc, int device, int max_batch) {
     TC_TRY(cudaMemset(tc.done, 0, sizeof(unsigned int)));
     TC_TRY(cudaMalloc((void**)&tc.lse_part, (size_t)tc.n_sm * 256 * sizeof(float2)));
     TC_TRY(cudaMalloc((void**)&tc.best_zt, (size_t)tc.n_sm * 4 * 256 * sizeof(float)));
-    TC_TRY(cudaFuncSetAttribute(tc_gemm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024));
-    TC_TRY(cudaFuncSetAttribute(tc_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 18 * 1024));
+    for (auto kern : {tc_gemm_kernel<0, false>, tc_gemm_kernel<0, true>})
+        TC_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024));
+    for (auto kern : {tc_gemm_kernel<1, false>, tc_gemm_kernel<1, true>})
+        TC_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 18 * 1024));
 #ifdef SPIRAL_TUNE      // tuning builds only: ring shape from the environment
     if (const char* v = std::getenv("SPIRAL_TC_BPS")) tc.bps = atoi(v);
 #endif
@@ -818,13 +879,34 @@ inline int tc_encode(TcState& tc, CUtensorMap* map, const void* base, uint64_t i
 inline size_t tc_tiled_elems(int rows, int K) {
     return (size_t)((rows + TC_BM - 1) / TC_BM) * ((K + TC_BK - 1) / TC_BK) * TC_BM * TC_BK;
 }
-inline int tc_convert(const __nv_bfloat16* W, __half* w16, int rows, int K, cudaStream_t st, int64_t* launches) {
+inline int tc_convert(const __nv_bfloat16* W, __half* w16, int rows, int K, cudaStream_t st, int64_t* launches,
+                      float scale = 1.f, int* lossy = nullptr) {
     const size_t chunks = tc_tiled_elems(rows, K) / 8;
     bf16_to_f16_tiled_kernel<<<(unsigned)((chunks + 255) / 256), 256, 0, st>>>(W, w16, rows, K, (K + TC_BK - 1) / TC_BK,
-                                                                                chunks);
+                                                                                chunks, scale, lossy);
     if (launches) ++*launches;
     TC_TRY(cudaGetLastError());
     return SPIRAL_OK;
+}
+
+// A resident matrix whose fp16 copy loses too much (see bf16_to_f16_tiled_kernel) is encoded again, times a power of two.
+// Synchronous (context creation).  max_dev: scratch on the device.
+inline int tc_rescale(TcState& tc, const __nv_bfloat16* W, unsigned int* max_dev, int64_t* launches) {
+    auto it = tc.weights.find(W);
+    if (it == tc.weights.end() || !it->second.resident) return SPIRAL_OK;
+    TcWeight& w = it->second;
+    unsigned int bits = 0;
+    TC_TRY(cudaMemset(max_dev, 0, sizeof(bits)));
+    bf16_max_kernel<<<4 * tc.n_sm, 256>>>(W, (size_t)w.rows * w.K, max_dev);
+    if (launches) ++*launches;
+    TC_TRY(cudaGetLastError());
+    TC_TRY(cudaMemcpy(&bits, max_dev, sizeof(bits), cudaMemcpyDeviceToHost));
+    float largest;
+    std::memcpy(&largest, &bits, sizeof(largest));
+    if (!(largest > 0.f)) return SPIRAL_OK;
+    const int s = std::max(-126, std::min(126, 14 - std::ilogb(largest)));
+    w.unscale = std::ldexp(1.f, -s);
+    return tc_convert(W, w.w16, w.rows, w.K, 0, launches, std::ldexp(1.f, s));
 }
 
 // room for the resident fp16 copies of all model weights together
@@ -840,9 +922,10 @@ inline int tc_reserve_weights(TcState& tc, size_t elems) {
     return SPIRAL_OK;
 }
 
-// fp16 copy + tensor map of one weight matrix.  resident = converted now, once (model weights).
+// fp16 copy + tensor map of one weight matrix.  resident = converted now, once (model weights; *lossy is set where the copy
+// wants tc_rescale).
 inline int tc_register_weight(TcState& tc, const __nv_bfloat16* W, int rows, int K, bool resident, cudaStream_t st,
-                              int64_t* launches, TcWeight** out) {
+                              int64_t* launches, TcWeight** out, int* lossy = nullptr) {
     auto it = tc.weights.find(W);
     if (it != tc.weights.end() && (it->second.rows != rows || it->second.K != K)) {
         if (it->second.resident) { g_tc_error = "weight registered with another shape"; return SPIRAL_ERR_INVALID; }
@@ -871,7 +954,7 @@ inline int tc_register_weight(TcState& tc, const __nv_bfloat16* W, int rows, int
         int rc = tc_encode(tc, &w.map, w.w16, (uint64_t)TC_BK, (uint64_t)(tc_tiled_elems(rows, K) / TC_BK), TC_BM);
         if (rc) { if (w.owned) cudaFree(w.w16); return rc; }
         if (resident) {
-            rc = tc_convert(W, w.w16, rows, K, st, launches);
+            rc = tc_convert(W, w.w16, rows, K, st, launches, 1.f, lossy);
             if (rc) { if (w.owned) cudaFree(w.w16); return rc; }
         }
         it = tc.weights.emplace(W, w).first;
@@ -1005,7 +1088,7 @@ inline int tc_linear(TcState& tc, const __nv_bfloat16* W, int rows, int K, const
     p.rows = rows; p.n = n; p.N = N;
     size_t smem;
     tc_launch_shape(tc, N, &p, &smem);
-    p.out = pieces; p.piece_stride = (size_t)n * rows; p.status = status;
+    p.out = pieces; p.piece_stride = (size_t)n * rows; p.status = status; p.unscale = w->unscale;
     p.skip_x = tc.skip_x_once ? 1 : 0;
     tc.skip_x_once = false;
     const CUtensorMap* om = &w->map;        // (unused unless tma_out)
@@ -1017,7 +1100,7 @@ inline int tc_linear(TcState& tc, const __nv_bfloat16* W, int rows, int K, const
 #ifdef TC_PROBE
     p.probe = tc_probe_slot();
 #endif
-    TC_TRY(launch_kernel(true, tc_gemm_kernel<0>, dim3(pl->grid), dim3(tc_threads(0)), smem, st, w->map, *xm, *om, p));
+    TC_TRY(launch_kernel(true, w->unscale != 1.f ? tc_gemm_kernel<0, true> : tc_gemm_kernel<0, false>, dim3(pl->grid), dim3(tc_threads(0)), smem, st, w->map, *xm, *om, p));
     if (launches) ++*launches;
     out->base = pieces; out->stride = p.piece_stride; out->ld = rows; out->n_pieces = pl->max_pieces;
     out->sk_KB = p.KB; out->sk_G = pl->grid; out->sk_shift = 7; out->sk_tt = 1; out->sk_BN = N;
@@ -1043,11 +1126,12 @@ inline int tc_lm_head(TcState& tc, const __nv_bfloat16* W, int vocab, int K, con
     p.rows = vocab; p.n = n; p.N = N;
     size_t smem;
     tc_launch_shape(tc, N, &p, &smem, true);
+    p.unscale = w->unscale;
     p.status = status; p.args = args_dev; p.best = tc.best; p.done = tc.done; p.lse_part = tc.lse_part; p.best_zt = tc.best_zt;
 #ifdef TC_PROBE
     p.probe = tc_probe_slot();
 #endif
-    TC_TRY(launch_kernel(true, tc_gemm_kernel<1>, dim3(pl->grid), dim3(tc_threads(1)), smem, st, w->map, *xm, w->map, p));
+    TC_TRY(launch_kernel(true, w->unscale != 1.f ? tc_gemm_kernel<1, true> : tc_gemm_kernel<1, false>, dim3(pl->grid), dim3(tc_threads(1)), smem, st, w->map, *xm, w->map, p));
     if (launches) ++*launches;
     return SPIRAL_OK;
 }

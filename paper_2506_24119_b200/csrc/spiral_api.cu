@@ -133,6 +133,7 @@ struct spiral_ctx {
     float* gumbel_stage = nullptr;
     int32_t* tokout_stage = nullptr;
     int* status = nullptr;
+    int* lossy = nullptr;          // [4 layers + 1] matrices whose fp16 copy needs a scale, then a scratch word (spiral_init)
     int64_t launches = 0;
     std::vector<int> scratch_len;      // host scratch: tokens attended per slot
     std::vector<int> scratch_last;     // host scratch (prefill): game whose last new token a slot carries
@@ -209,7 +210,7 @@ static void free_ctx(spiral_ctx* c) {
     cudaFree(c->x); cudaFree(c->h); cudaFree(c->attn_out); cudaFree(c->act); cudaFree(c->q);
     cudaFree(c->pieces); cudaFree(c->o_part); cudaFree(c->m_part); cudaFree(c->l_part);
     cudaFree(c->attn_item_cnt); cudaFree(c->logits); cudaFree(c->cos_tab); cudaFree(c->sin_tab); cudaFree(c->meta_dev);
-    cudaFree(c->tok_stage); cudaFree(c->gumbel_stage); cudaFree(c->tokout_stage); cudaFree(c->status);
+    cudaFree(c->tok_stage); cudaFree(c->gumbel_stage); cudaFree(c->tokout_stage); cudaFree(c->status); cudaFree(c->lossy);
     if (c->meta_host) cudaFreeHost(c->meta_host);
     if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
     if (c->copy_ev) cudaEventDestroy(c->copy_ev);
@@ -317,12 +318,14 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
     A((void**)&c->tokout_stage, MB * sizeof(int32_t));
     A((void**)&c->gumbel_stage, MB * d->vocab * sizeof(float));
     A((void**)&c->status, sizeof(int));
+    A((void**)&c->lossy, ((size_t)4 * L + 2) * sizeof(int));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&c->meta_host, (size_t)META_RING * c->meta_bytes);
     for (int i = 0; i < META_RING && e == cudaSuccess; ++i)
         e = cudaEventCreateWithFlags(&c->meta_ev[i], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->copy_ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemset(c->status, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(c->lossy, 0, ((size_t)4 * L + 2) * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->attn_item_cnt, 0, MB * d->n_kv_heads * sizeof(int));
     if (e != cudaSuccess) {
         g_cuda_error = std::string("spiral_init allocation: ") + cudaGetErrorString(e);
@@ -384,25 +387,30 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
             free_ctx(c);
             return rc;
         }
-        for (const M& m : mats) {
+        int* const lossy = c->lossy;
+        std::vector<int> lossy_h(mats.size(), 0);
+        for (size_t i = 0; i < mats.size(); ++i) {
+            const M& m = mats[i];
             if (!tc_usable(c->tc, m.rows, m.k, max_batch)) continue;
-            rc = tc_register_weight(c->tc, m.w, m.rows, m.k, true, 0, &c->launches, nullptr);
+            rc = tc_register_weight(c->tc, m.w, m.rows, m.k, true, 0, &c->launches, nullptr, lossy + i);
             if (rc == SPIRAL_OK && m.w != c->lm_head) {
                 int np = tc_max_pieces(c->tc, m.rows, m.k);
                 if (np < 0) rc = SPIRAL_ERR_CUDA;
                 else c->pieces_elems = std::max(c->pieces_elems, (size_t)np * MB * m.rows);
             }
-            if (rc != SPIRAL_OK) {
-                if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
-                free_ctx(c);
-                return rc;
-            }
+            if (rc != SPIRAL_OK) break;
         }
-        e = cudaDeviceSynchronize();
-        if (e != cudaSuccess) {
-            g_cuda_error = std::string("weight re-encoding: ") + cudaGetErrorString(e);
+        if (rc == SPIRAL_OK) {
+            e = cudaMemcpy(lossy_h.data(), lossy, mats.size() * sizeof(int), cudaMemcpyDeviceToHost);
+            for (size_t i = 0; i < mats.size() && e == cudaSuccess && rc == SPIRAL_OK; ++i)
+                if (lossy_h[i]) rc = tc_rescale(c->tc, mats[i].w, (unsigned int*)(lossy + mats.size()), &c->launches);
+            if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        }
+        if (rc != SPIRAL_OK || e != cudaSuccess) {
+            if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
+            if (rc == SPIRAL_OK) g_cuda_error = std::string("weight re-encoding: ") + cudaGetErrorString(e);
             free_ctx(c);
-            return SPIRAL_ERR_CUDA;
+            return rc != SPIRAL_OK ? rc : SPIRAL_ERR_CUDA;
         }
         // dense append path: needs every layer matrix on the tensor-core path
         c->pf_ready = true;

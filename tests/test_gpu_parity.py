@@ -414,6 +414,62 @@ def test_linear_tensor_core_path_against_oracle(rows, k, n):
         pair.close()
 
 
+@pytest.mark.parametrize("n", [1, 4, 15, 16, 40])
+def test_linear_on_model_weights_outside_the_range_of_fp16(n):
+    """The tensor-core kernel reads fp16 copies of the model's matrices.  Weights below fp16's normal range, above its
+    largest value or far apart in one matrix must not lose anything to that: the bar is that of the fp32 sums."""
+    desc = synth.shape("tiny", tied_embed=0)
+    w = synth.make_weights(desc)
+    for name in ("wq", "wk", "wv"):
+        w[name][0].mul_(2.0 ** -16)                                  # about 3e-7: fp16 keeps two or three bits
+    w["wo"][0].mul_(2.0 ** 22)                                       # about 8e4: many beyond 65504
+    w["w_gate"][0][5].mul_(2.0 ** -14)                               # one small row among usual ones
+    w["w_down"][0].mul_(2.0 ** -120)                                 # the scale itself is bounded
+    w["lm_head"].mul_(2.0 ** 100)
+    pair = Pair(desc, max_batch=n, max_ctx=32, n_games=1, weights_cpu=w)
+    try:
+        for name in ("wqkv", "wo", "w_gate_up", "w_down", "lm_head"):
+            dev = pair.packed[name][0] if name != "lm_head" else pair.packed[name]
+            m = dev.cpu()
+            x = synth.normal_bf16(3, 2, n * m.shape[1], 1.0).view(n, -1).to(torch.float16)
+            y = pair.sp.spiral_linear(pair.ctx, dev, x.cuda()).cpu().numpy()
+            for b in range(n):
+                ref = pair.oracle_mod.matvec(m, x[b].double().numpy())
+                scale = np.linalg.norm(m.double().numpy(), axis=1) * np.linalg.norm(x[b].double().numpy())       # of each row
+                assert (np.abs(y[b] - ref) <= 1e-6 * scale).all(), (name, b, (np.abs(y[b] - ref) / scale).max())
+        rc, detail = pair.sp.spiral_last_status(pair.ctx)
+        assert rc == 0, detail
+    finally:
+        pair.close()
+
+
+@pytest.mark.parametrize("n_games,max_batch", [(3, 3), (20, 20), (150, 150)])
+def test_model_with_gains_moved_into_small_weights(n_games, max_batch):
+    """A norm gain of 2^12 and a projection 2^-12 as large are the same function: every kernel that reads fp16 copies of the
+    projections (decode, append, LM head) has to stay as close to the oracle as with weights of the usual size."""
+    desc = synth.shape("tiny_qknorm", tied_embed=0)
+    w = synth.perturb_gains(synth.make_weights(desc))
+    small = {k: ([t.clone() for t in v] if isinstance(v, list) and v[0] is not None else v) for k, v in w.items()}
+    for gains, mats in (("ln1", ("wq", "wk", "wv")), ("ln2", ("w_gate", "w_up"))):
+        for t in small[gains]:
+            t.mul_(2.0 ** 12)
+        for t in sum((small[k] for k in mats), []):
+            t.mul_(2.0 ** -12)
+    small["final_norm"], small["lm_head"] = w["final_norm"] * 2.0 ** 12, w["lm_head"] * 2.0 ** -12
+    worst = {}
+    for name, weights in (("usual", w), ("small", small)):
+        pair = Pair(desc, max_batch=max_batch, max_ctx=64, n_games=n_games, weights_cpu=weights)
+        try:
+            games = list(range(n_games))
+            lens = synth.lengths(synth.MASTER_SEED, 8, n_games, 2, 12)
+            prompts = [synth.token_ids(synth.MASTER_SEED, 700 + i, lens[i], desc["vocab"]).tolist() for i in range(n_games)]
+            worst[name] = _run_teacher_forced(pair, games, prompts, 2, 71)[:2]
+        finally:
+            pair.close()
+    print(n_games, worst)
+    assert worst["small"][1] <= 1.3 * worst["usual"][1]
+
+
 @pytest.mark.parametrize("shape_name,n_games", [("tiny", 20), ("tiny_qknorm", 33), ("tiny_bias", 16)])
 def test_batched_step_on_tensor_cores(shape_name, n_games):
     """Enough games for the tensor-core GEMMs and the fused LM head + Gumbel-argmax to carry the
