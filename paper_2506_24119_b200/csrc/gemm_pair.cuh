@@ -475,8 +475,8 @@ inline int pg_get_actmap(TcState& tc, const __half* base, int cols, int T, const
 template <int EPI>
 inline int pg_gemm(TcState& tc, const PgPlan& pl, const __nv_bfloat16* W, int rows, int K, const __half* X, int T, void* out,
                    Pieces* pieces, int* status, cudaStream_t st, int64_t* launches) {
+    if (!tc_resident(tc, W, rows, K)) return SPIRAL_ERR_UNSUPPORTED;
     auto it = tc.weights.find(W);
-    if (it == tc.weights.end() || !it->second.resident || it->second.rows != rows || it->second.K != K) return SPIRAL_ERR_UNSUPPORTED;
     const CUtensorMap *xm = nullptr, *om = nullptr;
     int rc = pg_get_xmap(tc, X, K, T, pl.N / 2, &xm);
     if (rc) return rc;

@@ -854,9 +854,10 @@ inline void tc_destroy(TcState& tc) {
 inline bool tc_usable(const TcState& tc, int rows, int K, int n) {
     return tc.ready && rows >= TC_BM && K >= TC_BK && K % 8 == 0 && n >= 1 && n <= 256;
 }
-inline bool tc_resident(const TcState& tc, const __nv_bfloat16* W) {        // a model weight, converted at init
+// a model weight, converted at init (the whole matrix: its first rows have the same address)
+inline bool tc_resident(const TcState& tc, const __nv_bfloat16* W, int rows, int K) {
     auto it = tc.weights.find(W);
-    return it != tc.weights.end() && it->second.resident;
+    return it != tc.weights.end() && it->second.resident && it->second.rows == rows && it->second.K == K;
 }
 
 // 2-d tensor map [outer][inner] of 2-byte floats with a [box_outer][64] box and 128-byte swizzle

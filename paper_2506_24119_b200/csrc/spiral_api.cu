@@ -704,7 +704,7 @@ static int launch_linear_impl(spiral_ctx* c, const bf16* W, int rows, int K, con
                               int path, Pieces* out, cudaStream_t st) {
     float* y = y_direct ? y_direct : c->pieces;
     if (path != 1 && !y_direct && tc_usable(c->tc, rows, K, n) &&
-        (path == 2 || n >= TC_MIN_BATCH || tc_resident(c->tc, W))) {
+        (path == 2 || n >= TC_MIN_BATCH || tc_resident(c->tc, W, rows, K))) {
         int rc = tc_linear(c->tc, W, rows, K, X, n, c->pieces, c->pieces_elems, out, c->status, st, &c->launches);
         if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
         if (rc != SPIRAL_ERR_UNSUPPORTED || path == 2) return rc;

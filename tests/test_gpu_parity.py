@@ -443,6 +443,24 @@ def test_linear_on_model_weights_outside_the_range_of_fp16(n):
         pair.close()
 
 
+@pytest.mark.parametrize("n", [1, 15])
+def test_linear_on_the_first_rows_of_a_model_matrix(n):
+    """A few rows of input on the leading rows of a matrix the context knows (the queries' part of the QKV projection): the
+    address is that of the whole matrix, the shape is not."""
+    desc = synth.shape("tiny")
+    pair = Pair(desc, max_batch=16, max_ctx=32, n_games=1)
+    try:
+        m = pair.packed["wqkv"][0]
+        for rows in (m.shape[0], desc["n_q_heads"] * desc["head_dim"], 130, 5):
+            x = synth.normal_bf16(3, 2, n * m.shape[1], 1.0).view(n, -1).to(torch.float16)
+            y = pair.sp.spiral_linear(pair.ctx, m[:rows], x.cuda()).cpu().numpy()
+            for b in range(n):
+                ref = pair.oracle_mod.matvec(m[:rows].cpu(), x[b].double().numpy())
+                np.testing.assert_allclose(y[b], ref, rtol=0, atol=2e-5 * np.abs(ref).max() + 1e-6)
+    finally:
+        pair.close()
+
+
 @pytest.mark.parametrize("n_games,max_batch", [(3, 3), (20, 20), (150, 150)])
 def test_model_with_gains_moved_into_small_weights(n_games, max_batch):
     """A norm gain of 2^12 and a projection 2^-12 as large are the same function: every kernel that reads fp16 copies of the
