@@ -382,14 +382,20 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
         size_t elems = 0;
         for (const M& m : mats)
             if (tc_usable(c->tc, m.rows, m.k, max_batch)) elems += tc_tiled_elems(m.rows, m.k);
+        bool copies = true;
         if (elems > 0 && (rc = tc_reserve_weights(c->tc, elems)) != SPIRAL_OK) {
-            if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
-            free_ctx(c);
-            return rc;
+            // no room for a second copy of the weights: contexts for few games read the caller's bf16 matrices instead
+            if (rc != SPIRAL_ERR_OOM || max_batch >= TC_MIN_BATCH) {
+                if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
+                free_ctx(c);
+                return rc;
+            }
+            rc = SPIRAL_OK;
+            copies = false;
         }
         int* const lossy = c->lossy;
         std::vector<int> lossy_h(mats.size(), 0);
-        for (size_t i = 0; i < mats.size(); ++i) {
+        for (size_t i = 0; i < mats.size() && copies; ++i) {
             const M& m = mats[i];
             if (!tc_usable(c->tc, m.rows, m.k, max_batch)) continue;
             rc = tc_register_weight(c->tc, m.w, m.rows, m.k, true, 0, &c->launches, nullptr, lossy + i);
@@ -413,7 +419,7 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
             return rc != SPIRAL_OK ? rc : SPIRAL_ERR_CUDA;
         }
         // dense append path: needs every layer matrix on the tensor-core path
-        c->pf_ready = true;
+        c->pf_ready = copies;
         for (const M& m : mats)
             if (m.w != c->lm_head && !tc_usable(c->tc, m.rows, m.k, max_batch)) c->pf_ready = false;
         if (c->pf_ready) {
@@ -830,7 +836,7 @@ static int run_layers(spiral_ctx* c, spiral_kv* kv, int n, bool one_per_game, cu
 // LM head (+ sampling, + logits for the caller) for the n rows of ctx->h, as the step's StepArgs say.
 static int run_head_impl(spiral_ctx* c, int n, cudaStream_t st) {
     const spiral_model_desc& d = c->d;
-    if (tc_usable(c->tc, d.vocab, d.d_model, n)) {
+    if (tc_usable(c->tc, d.vocab, d.d_model, n) && tc_resident(c->tc, c->lm_head, d.vocab, d.d_model)) {
         int rc = tc_lm_head(c->tc, c->lm_head, d.vocab, d.d_model, c->h, n, meta_args(c), c->status, st, &c->launches);
         if (rc == SPIRAL_ERR_CUDA) g_cuda_error = tc_last_error();
         if (rc != SPIRAL_ERR_UNSUPPORTED) return rc;

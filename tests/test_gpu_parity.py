@@ -461,6 +461,59 @@ def test_linear_on_the_first_rows_of_a_model_matrix(n):
         pair.close()
 
 
+def test_context_for_few_games_without_room_for_weight_copies():
+    """A context for fewer than 16 games starts on a GPU that cannot hold a second copy of the weights and reads the caller's
+    matrices: prompt, steps, log-probabilities and nucleus draws as with the copies.  One for 16 games is refused."""
+    desc = synth.shape("tiny_qknorm", vocab=400000, n_layers=1)              # 205 MB of embedding, 5 MB of everything else
+    pair = Pair(desc, max_batch=3, max_ctx=64, n_games=3)
+    sp, V, ctx, kv, hog = pair.sp, desc["vocab"], None, None, None
+    try:
+        games, prompts = [2, 0, 1], [synth.token_ids(81, i, 5 + i, V).tolist() for i in range(3)]
+        flat = torch.tensor(sum(prompts, []), dtype=torch.int32).cuda()
+        offs = [0, 5, 11, 18]
+        tok_in = synth.token_ids(82, 0, 3, V, stream=synth.STREAM_TEACHER).cuda()
+        noise = synth.gumbel_noise(82, 0, 3, V).cuda()
+        tok, lp = torch.empty(3, dtype=torch.int32, device="cuda"), torch.empty(3, device="cuda")
+        last, logits = torch.empty(3, V, device="cuda"), torch.empty(3, V, device="cuda")
+        pool = torch.empty_like(pair.pool)
+        pool.copy_(pair.pool)
+        pair.close()
+        pair.ctx = pair.kv = None
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        hog = torch.empty(torch.cuda.mem_get_info()[0] - (150 << 20), dtype=torch.uint8, device="cuda")
+        before = torch.cuda.mem_get_info()[0]
+        with pytest.raises(RuntimeError):
+            sp.spiral_init(desc, pair.packed, 0, 16, 64)
+        ctx = sp.spiral_init(desc, pair.packed, 0, 3, 64)
+        assert before - torch.cuda.mem_get_info()[0] < 100 << 20
+        kv = sp.spiral_kv_alloc(ctx, pool, 16, 3, 64)
+        sp.spiral_prefill(ctx, kv, games, flat, offs, last)
+        ref = [pair.oracle.prefill(pair.oracle_cache(g), p) for g, p in zip(games, prompts)]
+        for step in range(3):                                                # (the third replays a recorded graph)
+            got = (last if step == 0 else logits).cpu().numpy()
+            for i in range(3):
+                a, r = compare_logits(got[i], ref[i])
+                assert a <= TOL_MAX_ABS and r <= TOL_REL_RMS
+            sp.spiral_decode_step_logprob(ctx, kv, games, tok_in, noise, 0.8, tok, lp, logits)
+            ref = [pair.oracle.decode_step(pair.oracle_cache(g), int(tok_in[i])) for i, g in enumerate(games)]
+            lg = logits.cpu().numpy().astype(np.float64)
+            for i in range(3):
+                assert int(tok[i]) == pair.oracle_mod.sample(lg[i], noise[i].cpu().numpy(), 0.8)[0]
+                assert abs(float(lp[i]) - pair.oracle_mod.log_prob(lg[i], int(tok[i]), 0.8)) <= 5e-6
+        x = synth.normal_bf16(3, 2, 3 * desc["d_model"], 1.0).view(3, -1).to(torch.float16)
+        y = sp.spiral_linear(ctx, pair.packed["wo"][0], x[:, :pair.packed["wo"][0].shape[1]].contiguous().cuda()).cpu().numpy()
+        want = pair.oracle_mod.matvec(pair.packed["wo"][0].cpu(), x[0].double().numpy())
+        np.testing.assert_allclose(y[0], want, rtol=0, atol=2e-5 * np.abs(want).max() + 1e-6)
+        assert sp.spiral_last_status(ctx)[0] == 0
+    finally:
+        del hog
+        sp.spiral_free(ctx, kv)
+        if pair.ctx is not None:
+            pair.close()
+        torch.cuda.empty_cache()
+
+
 @pytest.mark.parametrize("n_games,max_batch", [(3, 3), (20, 20), (150, 150)])
 def test_model_with_gains_moved_into_small_weights(n_games, max_batch):
     """A norm gain of 2^12 and a projection 2^-12 as large are the same function: every kernel that reads fp16 copies of the
