@@ -1158,7 +1158,7 @@ static int prefill_pass_rows(const spiral_ctx* c, long long total) {
     return best * PG_MAX_N;
 }
 
-static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems) {
+static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems, cudaStream_t st) {
     PrefillWs& w = c->pf;
     if (rows <= w.cap && y_elems <= w.y_elems) return SPIRAL_OK;
     rows = std::max(rows, w.cap);
@@ -1184,7 +1184,8 @@ static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems) {
     A((void**)&w.h, R * d.d_model * sizeof(__half));
     A((void**)&w.attn, R * qd * sizeof(__half));
     A((void**)&w.act, R * d.d_ff * sizeof(__half) + 128);      // (see pg_get_xmap)
-    if (e == cudaSuccess && d.d_ff % TC_BK != 0) e = cudaMemset(w.act, 0, R * d.d_ff * sizeof(__half) + 128);
+    // (on the caller's stream: the legacy default stream is not ordered with it)
+    if (e == cudaSuccess && d.d_ff % TC_BK != 0) e = cudaMemsetAsync(w.act, 0, R * d.d_ff * sizeof(__half) + 128, st);
     A((void**)&w.meta_dev, meta_elems * sizeof(int32_t));
     A((void**)&w.items_dev, (size_t)items_cap * (sizeof(AppendItem) + sizeof(AppendMerge)));
     if (e == cudaSuccess) e = cudaMallocHost((void**)&w.meta_host, meta_elems * sizeof(int32_t));
@@ -1237,7 +1238,7 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
             if (m == 0 || !pl.whole) y_elems = std::max<size_t>(y_elems, (size_t)pl.max_pieces * (size_t)T * shapes[m][0]);
         }
     }
-    int rc = prefill_ws_reserve(ctx, (chunk + PG_MAX_N - 1) / PG_MAX_N * PG_MAX_N, y_elems);
+    int rc = prefill_ws_reserve(ctx, (chunk + PG_MAX_N - 1) / PG_MAX_N * PG_MAX_N, y_elems, st);
     if (rc) return rc;
     PrefillWs& w = ctx->pf;
     const int cap = w.cap, MB = ctx->max_batch;

@@ -292,3 +292,25 @@ def test_dense_append_in_place_of_steps_loses_no_precision(monkeypatch, override
     rel = np.sqrt(((out["0"] - out["1"]) ** 2).sum() / (out["0"] ** 2).sum())
     print(overrides, "dense against steps: rel %.2e" % rel)
     assert rel <= 2.0 ** -12
+
+
+@pytest.mark.parametrize("d_ff", [688, 200, 704])
+def test_first_appends_on_a_side_stream(d_ff):
+    """Calls that make or enlarge the append workspace, on a stream that the legacy default stream does not wait for: with a
+    d_ff that is no multiple of 64 the activations are cleared before they are written."""
+    desc = synth.shape("tiny", d_ff=d_ff)
+    pair = Pair(desc, max_batch=8, max_ctx=1500, n_games=2)
+    try:
+        V, stream = desc["vocab"], torch.cuda.Stream()
+        for i, k in enumerate((33, 300, 900)):
+            new = [synth.token_ids(91 + i, g, k // 2 + g, V).tolist() for g in range(2)]
+            flat = torch.tensor(sum(new, []), dtype=torch.int32).cuda()
+            last = torch.empty(2, V, dtype=torch.float32, device="cuda")
+            torch.cuda.synchronize()
+            pair.sp.spiral_prefill(pair.ctx, pair.kv, [1, 0], flat, [0, len(new[0]), len(new[0]) + len(new[1])], last, stream)
+            stream.synchronize()
+            for j, g in enumerate((1, 0)):
+                a, r = compare_logits(last[j].cpu().numpy(), pair.oracle.prefill(pair.oracle_cache(g), new[j]))
+                assert a <= TOL_MAX_ABS and r <= TOL_REL_RMS
+    finally:
+        pair.close()
