@@ -361,6 +361,29 @@ inline double pg_block_us(int N) {
 constexpr int PG_SPLIT_MAX_T = 1024;                 // bounds the pieces buffer
 constexpr int PG_SEARCH_MAX_T = 2048;                // beyond: many waves, and the widest tile moves the fewest bytes per flop
 enum { PG_OUT_PIECES = 0, PG_OUT_ADD = 1, PG_OUT_GATED = 2 };      // what a whole tile's epilogue writes
+// Stream-K over `tiles` tiles: pairs that take part, and its estimated time (fixed + per_row x token rows, us)
+struct PgSplit { int G; double fixed, per_row; };
+inline PgSplit pg_split(int pairs, int tiles, int KB, int N, int rows, int out) {
+    const long long U = (long long)tiles * KB;
+    int G = (int)std::min<long long>(pairs, std::max<long long>(1, U / 4));       // no ranges under four k blocks
+    // Whole numbers of equal k ranges per tile where they use nearly all pairs (10 tiles x 7, 24 x 3 of 74): one segment
+    // and one epilogue per pair, as in tc_get_plan.  Qwen3-4B shape, us per call: 100 tokens 3519 -> 3347, 2 x 25
+    // 3348 -> 3239; Llama-3.1-8B shape 2 x 60 4272 -> 4183, Qwen2.5-7B shape 3871 -> 3730.
+    const int aligned = tiles <= G ? tiles * (G / tiles) : 0;
+    if (aligned * 100 >= G * 94) G = aligned;
+    const double pieces = 1.0 + (double)G / tiles, one = (double)rows * 4 / 3e6;
+    return PgSplit{G, (double)U / G * pg_block_us(N) + (out == PG_OUT_GATED ? 5.0 : 1.0),
+                   one * (out == PG_OUT_PIECES ? pieces - 1.0 : out == PG_OUT_GATED ? pieces + 1.0 : pieces)};
+}
+inline int pg_max_pieces(int tiles, int KB, int G) {
+    const long long U = (long long)tiles * KB;
+    int most = 0;
+    for (int t = 0; t < tiles; ++t) {
+        const long long first = (long long)t * KB;
+        most = std::max(most, streamk_cta_of(first + KB - 1, G, U) - streamk_cta_of(first, G, U) + 1);
+    }
+    return most;
+}
 inline PgPlan pg_plan(int n_sm, int rows, int K, int T, int out) {
     PgPlan pl;
     pl.row_tiles = (rows + PG_BM - 1) / PG_BM;
@@ -371,36 +394,43 @@ inline PgPlan pg_plan(int n_sm, int rows, int K, int T, int out) {
     for (int tt = fewest; tt <= most; ++tt) {
         const int N = ((T + tt - 1) / tt + 31) & ~31, tok_tiles = (T + N - 1) / N;
         if (tok_tiles != tt) continue;
-        const double t = pg_block_us(N);
         const int tiles = pl.row_tiles * tok_tiles, waves = (tiles + pairs - 1) / pairs;
-        const double whole = (double)waves * pl.KB * t;
+        const double whole = (double)waves * pl.KB * pg_block_us(N);
         if (best < 0 || whole < best) { best = whole; pl.N = N; pl.tok_tiles = tok_tiles; pl.whole = 1; }
-        const long long U = (long long)tiles * pl.KB;
-        int G = (int)std::min<long long>(pairs, std::max<long long>(1, U / 4));   // no ranges under four k blocks
-        // Whole numbers of equal k ranges per tile where they use nearly all pairs (10 tiles x 7, 24 x 3 of 74): one segment
-        // and one epilogue per pair, as in tc_get_plan.  Qwen3-4B shape, us per call: 100 tokens 3519 -> 3347, 2 x 25
-        // 3348 -> 3239; Llama-3.1-8B shape 2 x 60 4272 -> 4183, Qwen2.5-7B shape 3871 -> 3730.
-        const int aligned = tiles <= G ? tiles * (G / tiles) : 0;
-        if (aligned * 100 >= G * 94) G = aligned;
-        const double pieces = 1.0 + (double)G / tiles, one = (double)T * rows * 4 / 3e6;
-        const double split = (double)U / G * t + one * (out == PG_OUT_PIECES ? pieces - 1.0 : pieces) + (out == PG_OUT_GATED ? 5.0 + one : 1.0);
-        if (T <= PG_SPLIT_MAX_T && split < best) { best = split; pl.N = N; pl.tok_tiles = tok_tiles; pl.whole = 0; pl.G = G; }
+        const PgSplit sp = pg_split(pairs, tiles, pl.KB, N, rows, out);
+        const double split = sp.fixed + sp.per_row * T;
+        if (T <= PG_SPLIT_MAX_T && split < best) { best = split; pl.N = N; pl.tok_tiles = tok_tiles; pl.whole = 0; pl.G = sp.G; }
     }
     const int tiles = pl.row_tiles * pl.tok_tiles;
     if (pl.whole) {
         pl.G = std::min(pairs, tiles);
     } else {
-        const long long U = (long long)tiles * pl.KB;
-        pl.max_pieces = 0;
-        for (int t = 0; t < tiles; ++t) {
-            const long long first = (long long)t * pl.KB;
-            pl.max_pieces = std::max(pl.max_pieces, streamk_cta_of(first + pl.KB - 1, pl.G, U) - streamk_cta_of(first, pl.G, U) + 1);
-        }
+        pl.max_pieces = pg_max_pieces(tiles, pl.KB, pl.G);
     }
     const size_t blk = TC_W_BYTES + (size_t)(pl.N / 2) * 128, budget = PG_SMEM_BUDGET - 1024 - TC_OUT_BUFS * TC_OUT_BYTES;
     pl.stages = (int)std::min<size_t>(PG_MAX_STAGES, budget / (PG_BPS * blk));
     pl.smem = (size_t)pl.stages * PG_BPS * blk + TC_OUT_BUFS * TC_OUT_BYTES + 1024;
     return pl;
+}
+
+// The most floats a plan for up to `cap` token rows leaves in pieces: what the buffer has to hold for every call that the
+// rest of a workspace of `cap` rows holds.  For each token tile: the largest T at which stream-K is still estimated shorter
+// than whole tiles (pg_plan takes it for no other), times its pieces.
+inline size_t pg_piece_elems(int n_sm, int rows, int K, int cap, int out) {
+    const int row_tiles = (rows + PG_BM - 1) / PG_BM, KB = (K + TC_BK - 1) / TC_BK, pairs = std::max(1, n_sm / 2);
+    size_t most = out == PG_OUT_PIECES ? (size_t)cap * rows : 0;
+    for (int tt = 1; tt <= PG_SPLIT_MAX_T / PG_MAX_N + 3; ++tt)
+        for (int N = 32; N <= PG_MAX_N; N += 32) {
+            const int tiles = row_tiles * tt, waves = (tiles + pairs - 1) / pairs;
+            const PgSplit sp = pg_split(pairs, tiles, KB, N, rows, out);
+            const double slack = (double)waves * KB * pg_block_us(N) - sp.fixed;
+            int T = std::min(std::min(N * tt, cap), PG_SPLIT_MAX_T);
+            if (slack <= 0) continue;
+            if (sp.per_row * T > slack) T = (int)(slack / sp.per_row) + 1;
+            if (T > (N - 32) * tt && tt <= (T + PG_MAX_N - 1) / PG_MAX_N + 3)
+                most = std::max(most, (size_t)pg_max_pieces(tiles, KB, sp.G) * T * rows);
+        }
+    return most;
 }
 
 // a tensor of fp16 values as [outer][mid][64] with a box of box_outer x box_mid x 64, 128-byte swizzle

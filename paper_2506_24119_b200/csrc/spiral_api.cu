@@ -80,9 +80,9 @@ struct ProfRec { int cls; cudaEvent_t e0, e1; };
 // attention work list, each with a pinned host mirror.
 struct PrefillWs {
     int cap = 0;                        // token rows the buffers hold
-    size_t y_elems = 0;                 // floats of y: the QKV projection, or the pieces of whichever matrix is split
-    float *x = nullptr, *y = nullptr;
-    __half *q = nullptr, *h = nullptr, *attn = nullptr, *act = nullptr;
+    int lo_cap = 0;                     // token rows that q_lo holds
+    float *x = nullptr, *y = nullptr;   // y: the QKV projection, or the pieces of whichever matrix is split
+    __half *q = nullptr, *q_lo = nullptr, *h = nullptr, *attn = nullptr, *act = nullptr;
     int32_t* meta_dev = nullptr;        // [4][cap]: game, position, -1, token index; then [2][max_batch]: rows to
     int32_t* meta_host = nullptr;       // hand to the LM head (source row, destination row)
     size_t meta_elems = 0;
@@ -90,7 +90,6 @@ struct PrefillWs {
     AppendItem* items_host = nullptr;
     int items_cap = 0;
     std::vector<AppendItem> work;       // host scratch: query blocks of a pass before they are cut
-    size_t part_slots = 0;              // partial results (of every KV head) that o_part / ml_part hold
     float* o_part = nullptr;
     float2* ml_part = nullptr;
     cudaEvent_t ev = nullptr;           // the last upload from the pinned mirrors
@@ -218,7 +217,7 @@ static void free_ctx(spiral_ctx* c) {
         if (c->meta_ev[i]) cudaEventDestroy(c->meta_ev[i]);
     for (auto& r : c->prof_recs) { cudaEventDestroy(r.e0); cudaEventDestroy(r.e1); }
     for (auto e : c->prof_pool) cudaEventDestroy(e);
-    cudaFree(c->pf.x); cudaFree(c->pf.y); cudaFree(c->pf.q); cudaFree(c->pf.h); cudaFree(c->pf.attn); cudaFree(c->pf.act);
+    cudaFree(c->pf.x); cudaFree(c->pf.y); cudaFree(c->pf.q); cudaFree(c->pf.q_lo); cudaFree(c->pf.h); cudaFree(c->pf.attn); cudaFree(c->pf.act);
     cudaFree(c->pf.meta_dev); cudaFree(c->pf.items_dev); cudaFree(c->pf.o_part); cudaFree(c->pf.ml_part);
     if (c->pf.meta_host) cudaFreeHost(c->pf.meta_host);
     if (c->pf.items_host) cudaFreeHost(c->pf.items_host);
@@ -1133,12 +1132,12 @@ static int launch_rmsnorm_rows(spiral_ctx* c, float* x, const Pieces* pend, cons
 // Token rows per dense pass of a call with `total` new tokens: as few passes as the largest pass allows, all of (nearly)
 // the same length -- a short last pass costs all weights again -- and within that the length at which the whole-tile
 // GEMMs waste the least of their last wave.
-static int prefill_pass_rows(const spiral_ctx* c, long long total) {
+static int prefill_pass_rows(const spiral_ctx* c, long long total, int chunk_max) {
     const spiral_model_desc& d = c->d;
-    const long long passes = (total + c->prefill_chunk - 1) / c->prefill_chunk;
+    const long long passes = (total + chunk_max - 1) / chunk_max;
     const int even = (int)((total + passes - 1) / passes);
     if (passes == 1) return even;
-    const int lo = (even + PG_MAX_N - 1) / PG_MAX_N, hi = std::max(lo, c->prefill_chunk / PG_MAX_N);
+    const int lo = (even + PG_MAX_N - 1) / PG_MAX_N, hi = std::max(lo, chunk_max / PG_MAX_N);
     const int pairs = std::max(1, c->n_sm / 2);
     const int rows[4] = {c->qkv_rows, d.d_model, 2 * d.d_ff, d.d_model};
     const int ks[4] = {d.d_model, d.n_q_heads * d.head_dim, d.d_model, d.d_ff};
@@ -1158,29 +1157,40 @@ static int prefill_pass_rows(const spiral_ctx* c, long long total) {
     return best * PG_MAX_N;
 }
 
-static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems, cudaStream_t st) {
+// Room for passes of `rows` token rows, `lo_rows` of them with queries in two parts.  Sized by the rows alone: a shorter
+// call whose plan leaves more pieces finds them provided for (allocating again waits for the device).  With nothing left of
+// the workspace when it does not fit.
+static int prefill_ws_reserve(spiral_ctx* c, int rows, int lo_rows, cudaStream_t st) {
     PrefillWs& w = c->pf;
-    if (rows <= w.cap && y_elems <= w.y_elems) return SPIRAL_OK;
+    if (rows <= w.cap && lo_rows <= w.lo_cap) return SPIRAL_OK;
     rows = std::max(rows, w.cap);
-    y_elems = std::max(y_elems, w.y_elems);
+    lo_rows = std::max(lo_rows, w.lo_cap);
     CU_TRY(cudaDeviceSynchronize());
-    cudaFree(w.x); cudaFree(w.y); cudaFree(w.q); cudaFree(w.h); cudaFree(w.attn); cudaFree(w.act);
-    cudaFree(w.meta_dev); cudaFree(w.items_dev); cudaFree(w.o_part); cudaFree(w.ml_part);
-    if (w.meta_host) cudaFreeHost(w.meta_host);
-    if (w.items_host) cudaFreeHost(w.items_host);
-    cudaEvent_t ev = w.ev;
-    w = PrefillWs{};
-    w.ev = ev;
+    auto release = [&]() {
+        cudaFree(w.x); cudaFree(w.y); cudaFree(w.q); cudaFree(w.q_lo); cudaFree(w.h); cudaFree(w.attn); cudaFree(w.act);
+        cudaFree(w.meta_dev); cudaFree(w.items_dev);
+        if (w.meta_host) cudaFreeHost(w.meta_host);
+        if (w.items_host) cudaFreeHost(w.items_host);
+        PrefillWs left;
+        left.o_part = w.o_part; left.ml_part = w.ml_part; left.ev = w.ev;
+        w = std::move(left);
+    };
+    release();
     const spiral_model_desc& d = c->d;
     const size_t R = rows, qd = (size_t)d.n_q_heads * d.head_dim;
     const int per_item = std::min(app_positions_per_item(c->group, false), apt_positions_per_item(c->group, 1));
     const int items_cap = ((rows + per_item - 1) / per_item + c->max_batch + 1) * APM_MAX_PARTS;      // (a query block may be cut)
     const size_t meta_elems = 4 * R + 2 * (size_t)c->max_batch;
+    const size_t y_elems = std::max(std::max(pg_piece_elems(c->n_sm, c->qkv_rows, d.d_model, rows, PG_OUT_PIECES),
+                                             pg_piece_elems(c->n_sm, d.d_model, (int)qd, rows, PG_OUT_ADD)),
+                                    std::max(pg_piece_elems(c->n_sm, 2 * d.d_ff, d.d_model, rows, PG_OUT_GATED),
+                                             pg_piece_elems(c->n_sm, d.d_model, d.d_ff, rows, PG_OUT_ADD)));
     cudaError_t e = cudaSuccess;
     auto A = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
     A((void**)&w.x, R * d.d_model * sizeof(float));
     A((void**)&w.y, y_elems * sizeof(float));
-    A((void**)&w.q, 2 * R * qd * sizeof(__half));              // (bf16 pages: high and low parts)
+    A((void**)&w.q, R * qd * sizeof(__half));
+    if (lo_rows > 0) A((void**)&w.q_lo, (size_t)lo_rows * qd * sizeof(__half));
     A((void**)&w.h, R * d.d_model * sizeof(__half));
     A((void**)&w.attn, R * qd * sizeof(__half));
     A((void**)&w.act, R * d.d_ff * sizeof(__half) + 128);      // (see pg_get_xmap)
@@ -1194,28 +1204,28 @@ static int prefill_ws_reserve(spiral_ctx* c, int rows, size_t y_elems, cudaStrea
     if (e != cudaSuccess) {
         g_cuda_error = std::string("append workspace: ") + cudaGetErrorString(e);
         cudaGetLastError();
-        return e == cudaErrorMemoryAllocation ? SPIRAL_ERR_OOM : SPIRAL_ERR_CUDA;    // cap stays 0: freed with the context
+        release();
+        return e == cudaErrorMemoryAllocation ? SPIRAL_ERR_OOM : SPIRAL_ERR_CUDA;
     }
-    w.cap = rows; w.y_elems = y_elems; w.items_cap = items_cap; w.meta_elems = meta_elems; w.ev_used = false;
+    w.cap = rows; w.lo_cap = lo_rows; w.items_cap = items_cap; w.meta_elems = meta_elems; w.ev_used = false;
     return SPIRAL_OK;
 }
 
-// room for the partial attention results of `slots` parts
-static int prefill_part_reserve(spiral_ctx* c, size_t slots) {
+// room for the partial results of the most parts that append_attn_cap cuts a pass into
+static int prefill_part_reserve(spiral_ctx* c) {
     PrefillWs& w = c->pf;
-    if (slots <= w.part_slots) return SPIRAL_OK;
-    CU_TRY(cudaDeviceSynchronize());
-    cudaFree(w.o_part); cudaFree(w.ml_part);
-    w.o_part = nullptr; w.ml_part = nullptr; w.part_slots = 0;
+    if (w.ml_part) return SPIRAL_OK;
+    const size_t slots = (size_t)4 * c->n_sm / c->d.n_kv_heads;
     const size_t rows = slots * c->d.n_kv_heads * 256;
     cudaError_t e = cudaMalloc((void**)&w.o_part, rows * c->d.head_dim * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc((void**)&w.ml_part, rows * sizeof(float2));
     if (e != cudaSuccess) {
         g_cuda_error = std::string("append partials: ") + cudaGetErrorString(e);
         cudaGetLastError();
+        cudaFree(w.o_part);
+        w.o_part = nullptr; w.ml_part = nullptr;
         return e == cudaErrorMemoryAllocation ? SPIRAL_ERR_OOM : SPIRAL_ERR_CUDA;
     }
-    w.part_slots = slots;
     return SPIRAL_OK;
 }
 
@@ -1227,25 +1237,24 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
     const spiral_model_desc& d = ctx->d;
     long long total = 0;
     for (int i = 0; i < n; ++i) total += offsets[i + 1] - offsets[i];
-    const int chunk = prefill_pass_rows(ctx, total);
-    const int qd = d.n_q_heads * d.head_dim;
-    // pieces are left by the last, shorter pass too: its split is another one
-    size_t y_elems = 0;
-    for (long long T : {(long long)chunk, total % chunk ? total % chunk : (long long)chunk}) {
-        const int shapes[4][2] = {{ctx->qkv_rows, d.d_model}, {d.d_model, qd}, {2 * d.d_ff, d.d_model}, {d.d_model, d.d_ff}};
-        for (int m = 0; m < 4; ++m) {
-            const PgPlan pl = pg_plan(ctx->n_sm, shapes[m][0], shapes[m][1], (int)T, m == 0 ? PG_OUT_PIECES : m == 2 ? PG_OUT_GATED : PG_OUT_ADD);
-            if (m == 0 || !pl.whole) y_elems = std::max<size_t>(y_elems, (size_t)pl.max_pieces * (size_t)T * shapes[m][0]);
-        }
-    }
-    int rc = prefill_ws_reserve(ctx, (chunk + PG_MAX_N - 1) / PG_MAX_N * PG_MAX_N, y_elems, st);
-    if (rc) return rc;
-    PrefillWs& w = ctx->pf;
-    const int cap = w.cap, MB = ctx->max_batch;
+    const int qd = d.n_q_heads * d.head_dim, MB = ctx->max_batch;
     // Calls that the decode-shaped step could hold, or contexts for fewer games than a dense contraction needs: these
     // leave the decode kernel's attention, whose queries and softmax weights are in two parts, only for another with the
     // same precision.  Longer appends have always had them in one fp16 part.
     const bool two = kv->kv_f16 && (total <= MB || MB < TC_MIN_BATCH);
+    // as few passes as the workspace can be had for: a GPU without room for the longest passes takes shorter ones
+    int chunk, rc;
+    for (int most = ctx->prefill_chunk;; most = most / 2 / PG_MAX_N * PG_MAX_N) {
+        chunk = prefill_pass_rows(ctx, total, most);
+        const int rows = (chunk + PG_MAX_N - 1) / PG_MAX_N * PG_MAX_N;
+        // (fp16 pages: what a later call of at most max_batch tokens needs is provided for)
+        const int lo_rows = !kv->kv_f16 || MB < TC_MIN_BATCH ? rows : std::min(rows, MB);
+        rc = prefill_ws_reserve(ctx, rows, lo_rows, st);
+        if (rc != SPIRAL_ERR_OOM || most < 2 * PG_MAX_N) break;
+    }
+    if (rc) return rc;
+    PrefillWs& w = ctx->pf;
+    const int cap = w.cap;
     const bool attn_tc = kv->kv_f16 && (two || ctx->append_attn_tc);
     const int tiles = two ? 1 : ctx->append_tiles;
     const int per_item = attn_tc ? apt_positions_per_item(ctx->group, tiles)
@@ -1299,7 +1308,9 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
         if (attn_tc && (two || tiles == 2)) {
             std::vector<int> blocks;
             for (const AppendItem& it : w.work) blocks.push_back(it.blk1);
-            most = append_attn_cap(blocks, d.n_kv_heads, ctx->n_sm);
+            const int cut = append_attn_cap(blocks, d.n_kv_heads, ctx->n_sm);
+            if (cut < most && (rc = prefill_part_reserve(ctx)) == SPIRAL_OK) most = cut;
+            if (rc != SPIRAL_OK && rc != SPIRAL_ERR_OOM) return rc;         // (no room for partials: uncut)
         }
         for (const AppendItem& it : w.work) {
             const int parts = (it.blk1 + most - 1) / most;
@@ -1311,8 +1322,6 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
             }
             if (parts > 1) { merges[n_merges++] = AppendMerge{it.n_pos, it.row0, n_slots, parts}; n_slots += parts; }
         }
-        rc = prefill_part_reserve(ctx, n_slots);
-        if (rc) return rc;
         const AppendMerge* merges_dev = (const AppendMerge*)(w.items_dev + w.items_cap);
         CU_TRY(cudaMemcpyAsync(w.items_dev, w.items_host, (size_t)n_items * sizeof(AppendItem), cudaMemcpyHostToDevice, st));
         if (n_merges) CU_TRY(cudaMemcpyAsync(w.items_dev + w.items_cap, merges, (size_t)n_merges * sizeof(AppendMerge), cudaMemcpyHostToDevice, st));
@@ -1367,11 +1376,11 @@ static int prefill_dense(spiral_ctx* ctx, spiral_kv* kv, int n, const int32_t* i
                                               : (kv->kv_f16 ? pf_qkv_post_kernel<64, true> : pf_qkv_post_kernel<64, false>);
                 LAUNCH(ctx, post, qgrid, PF_QKV_THREADS, 0, st, pq, ctx->bqkv[l], ctx->q_norm[l], ctx->k_norm[l], eps, ctx->cos_tab,
                        ctx->sin_tab, meta.game, meta.pos, kv->table_dev, kv->max_pages, kv->n_pages, l, nt, d.n_q_heads, d.n_kv_heads,
-                       q_scale, w.q, two || !kv->kv_f16 ? w.q + (size_t)cap * qd : nullptr, kv->pool, ctx->status);
+                       q_scale, w.q, two || !kv->kv_f16 ? w.q_lo : nullptr, kv->pool, ctx->status);
             }
             {
                 AppendParams ap{};
-                ap.q = w.q; ap.q_lo = w.q + (size_t)cap * qd; ap.items = w.items_dev; ap.block_table = kv->table_dev; ap.max_pages = kv->max_pages;
+                ap.q = w.q; ap.q_lo = w.q_lo; ap.items = w.items_dev; ap.block_table = kv->table_dev; ap.max_pages = kv->max_pages;
                 ap.n_pages = kv->n_pages; ap.layer = l; ap.n_q_heads = d.n_q_heads; ap.n_kv_heads = d.n_kv_heads;
                 ap.group = ctx->group;
                 ap.out = w.attn; ap.o_part = w.o_part; ap.ml_part = w.ml_part; ap.status = ctx->status;
@@ -1471,10 +1480,12 @@ extern "C" int spiral_prefill(spiral_ctx* ctx, spiral_kv* kv, int n, const int32
         const double step_bytes = (double)reads * 4 * ctx->d.n_kv_heads * ctx->d.head_dim;
         if (ctx->prefill_dense && ctx->pf_ready && (total > ctx->max_batch || step_bytes > 200e6)) {
             rc = prefill_dense(ctx, kv, n, ids, tokens_dev, offsets, start, last_logits, st);
-            if (rc) return roll_back(rc);
-            for (int i = 0; i < n; ++i) kv->seq_len[ids[i]] = start[i] + offsets[i + 1] - offsets[i];
-            return SPIRAL_OK;
-        }
+            if (rc && rc != SPIRAL_ERR_OOM) return roll_back(rc);
+            if (rc == SPIRAL_OK) {
+                for (int i = 0; i < n; ++i) kv->seq_len[ids[i]] = start[i] + offsets[i + 1] - offsets[i];
+                return SPIRAL_OK;
+            }
+        }                               // (no room for even the shortest passes' workspace: steps, which need none)
     }
     // Chunked: every step carries up to max_batch (game, position) slots, game after game and in
     // position order.  Slots of the same game may share a step: each slot's keys/values are cached

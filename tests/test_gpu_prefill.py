@@ -314,3 +314,64 @@ def test_first_appends_on_a_side_stream(d_ff):
                 assert a <= TOL_MAX_ABS and r <= TOL_REL_RMS
     finally:
         pair.close()
+
+
+def test_shorter_appends_do_not_allocate_again():
+    """What a call allocates serves every call with no more tokens, also one whose GEMM plans leave more partial sums or whose
+    attention is cut along the keys: at this shape 1024 tokens leave 6 MB more of them than 1792."""
+    desc = synth.shape("llama31_8b", n_layers=1, vocab=4096)
+    pair = Pair(desc, max_batch=16, max_ctx=2100, n_games=2, gains=False, generate_on_gpu=True)
+    try:
+        sp, V = pair.sp, desc["vocab"]
+        last = torch.empty(2, V, dtype=torch.float32, device="cuda")
+        tokens = synth.token_ids(95, 0, 2048, V).cuda()
+
+        def append(k):
+            sp.spiral_prefill(pair.ctx, pair.kv, [0, 1], tokens[:k], [0, k // 2, k], last)
+            torch.cuda.synchronize()
+
+        append(1792)                                 # the largest
+        append(40)                                   # few query blocks behind 896 tokens: cut
+        free = torch.cuda.mem_get_info()[0]
+        sp.spiral_kv_truncate(pair.kv, [0, 1], [0, 0])
+        for k in (1024, 1700, 640, 300, 172, 40, 17):
+            append(k)
+            assert torch.cuda.mem_get_info()[0] == free, k
+            sp.spiral_kv_truncate(pair.kv, [0, 1], [0, 0])
+        assert sp.spiral_last_status(pair.ctx)[0] == 0
+    finally:
+        pair.close()
+
+
+@pytest.mark.parametrize("overrides,room,games,each", [
+    ({}, 20 << 20, 8, 500),
+    (dict(d_model=1024, n_q_heads=16, d_ff=8192), 6 << 20, 2, 40),       # 256 rows of workspace: more than 10 MB
+])
+def test_append_on_a_gpu_with_little_room(overrides, room, games, each):
+    """Where the workspace of one long pass does not fit, the call takes shorter passes; where none fits, steps."""
+    desc = synth.shape("tiny", **overrides)
+    warm = Pair(desc, max_batch=24, max_ctx=600, n_games=games)          # (loads the kernels)
+    pair = Pair(desc, max_batch=24, max_ctx=600, n_games=games)
+    hog = None
+    try:
+        V = desc["vocab"]
+        _append(warm, list(range(games)), [synth.token_ids(96, g, 40, V).tolist() for g in range(games)])
+        _decode(warm, list(range(games)), 1, 98)
+        new = [synth.token_ids(97, g, each + g, V).tolist() for g in range(games)]
+        flat = torch.tensor(sum(new, []), dtype=torch.int32).cuda()
+        offs = np.concatenate([[0], np.cumsum([len(t) for t in new])]).tolist()
+        last = torch.empty(games, V, dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        hog = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+        pair.sp.spiral_prefill(pair.ctx, pair.kv, list(range(games)), flat, offs, last)
+        torch.cuda.synchronize()
+        del hog
+        for g in range(games):
+            a, r = compare_logits(last[g].cpu().numpy(), pair.oracle.prefill(pair.oracle_cache(g), new[g]))
+            assert a <= TOL_MAX_ABS and r <= TOL_REL_RMS
+        assert pair.sp.spiral_last_status(pair.ctx)[0] == 0
+    finally:
+        warm.close()
+        pair.close()
+        torch.cuda.empty_cache()
