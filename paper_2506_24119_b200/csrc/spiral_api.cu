@@ -727,7 +727,7 @@ static int launch_attention(spiral_ctx* c, spiral_kv* kv, int layer, int n, cons
                             const int32_t* len_dev, int len_add, const float* q, __half* out_f16,
                             float* out_f32, bool early, cudaStream_t st) {
     const spiral_model_desc& d = c->d;
-    AttnParams p;
+    AttnParams p{};
     p.q = q; p.block_table = kv->table_dev; p.game = game_dev; p.ctx_len = len_dev; p.cum = meta_cum_dev(c);
     p.len_add = len_add; p.n = n; p.max_pages = kv->max_pages; p.n_pages = kv->n_pages; p.layer = layer;
     p.n_q_heads = d.n_q_heads; p.n_kv_heads = d.n_kv_heads; p.group = c->group;
@@ -1708,13 +1708,13 @@ extern "C" int spiral_attention_static(int device, const void* pool_dev, int n_p
     // kept: it holds the first error since spiral_attention_static_status last read it)
     CU_TRY(cudaMemsetAsync(sc->item_cnt, 0, sizeof(sc->item_cnt), st));
 
-    AttnParams p;
+    AttnParams p{};
     p.q = q_dev; p.block_table = block_table_dev; p.game = sc->game; p.ctx_len = sc->len; p.cum = sc->cum;
     p.len_add = 0; p.n = n; p.max_pages = max_pages; p.n_pages = n_pages; p.layer = layer;
     p.n_q_heads = n_q_heads; p.n_kv_heads = n_kv_heads; p.group = n_q_heads / n_kv_heads;
     p.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)head_dim));
     p.o_part = sc->o_part; p.m_part = sc->m_part; p.l_part = sc->l_part; p.item_cnt = sc->item_cnt;
-    p.out_f16 = nullptr; p.out_f32 = out_dev; p.status = &sc->status; p.skip_first_load = 0;
+    p.out_f16 = nullptr; p.out_f32 = out_dev; p.status = &sc->status; p.early = 0; p.skip_first_load = 0;
     const size_t smem = attn_smem_bytes(head_dim, p.group);
     const bool f16 = kv_dtype == SPIRAL_KV_F16;
     auto attn = head_dim == 128 ? (f16 ? attn_decode_kernel<128, true> : attn_decode_kernel<128, false>)
@@ -1753,7 +1753,7 @@ extern "C" int spiral_read_ceiling(int device, const void* buf_dev, size_t bytes
     CU_TRY(cudaGetSymbolAddress((void**)&status_dev, g_read_ceiling_status));
     CU_TRY(cudaMemsetAsync(status_dev, 0, sizeof(int), st));
     CU_TRY(cudaFuncSetAttribute(read_ceiling_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    ReadCeilingParams p;
+    ReadCeilingParams p{};
     p.buf = (const uint8_t*)buf_dev; p.chunks = bytes / (size_t)stage_bytes; p.stage_bytes = stage_bytes;
     if (blocked < 0 || blocked > 2) return SPIRAL_ERR_INVALID;
     p.stages = stages; p.passes = passes; p.blocked = blocked; p.status = status_dev;

@@ -37,3 +37,12 @@ def test_host_only_entry_points_validate_arguments():
     assert lib.spiral_kv_release(None, 0, None) == sp.SPIRAL_ERR_INVALID
     assert lib.spiral_init(None, None, None, 0, 1, 1) == sp.SPIRAL_ERR_INVALID
     assert lib.spiral_decode_step(None, None, 1, None, None, None, ctypes.c_float(1.0), None, None, None) == sp.SPIRAL_ERR_INVALID
+
+
+def test_launch_parameters_start_out_cleared():
+    """Every block of kernel parameters is value-initialised where it is declared: a field added to it later is zero in the
+    entry points that do not set it, not whatever the stack holds."""
+    csrc = os.path.join(ROOT, "paper_2506_24119_b200", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        for line in open(os.path.join(csrc, name)):
+            assert not re.match(r"\s+(\w+Params|StepArgs)\s+\w+\s*;", line), (name, line)
