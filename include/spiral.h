@@ -23,8 +23,8 @@
  *   - Weights are bf16; the KV pool holds 2-byte floats (fp16 or bf16, chosen in spiral_kv_alloc); tokens, game ids and page ids are int32; noise, logits and
  *     the temperature are fp32.  The residual stream, norms, softmax and all accumulators are fp32.
  *     Activations entering a matrix product are rounded once to fp16 (11-bit mantissa); bf16
- *     weights are exactly representable in fp16 (the tensor-core path re-encodes them once at
- *     init into a private fp16 copy; magnitudes below 2^-24 flush), so products are exact.
+ *     weights are re-encoded once, in spiral_init, into a private fp16 copy, times a power of two
+ *     where a matrix has magnitudes that fp16 would lose, so products are exact.
  *   - Calls are asynchronous on `cuda_stream` (a cudaStream_t passed as void*, NULL = the legacy
  *     default stream) unless stated otherwise.  Calls on one ctx/kv must be issued from one host
  *     thread at a time and on one stream (or on streams the caller orders).
@@ -78,7 +78,9 @@ typedef struct {
  *   w_down    [d_model][d_ff]
  *   embed     [vocab][d_model];  lm_head [vocab][d_model] or NULL when tied_embed == 1
  *   ln1, ln2, final_norm   [d_model] RMSNorm gains
- * All matrix base addresses must be 16-byte aligned.  Weights must outlive the ctx. */
+ * All matrix base addresses must be 16-byte aligned.  Weights must outlive the ctx and must not
+ * change meanwhile: matrices are read from copies made in spiral_init, embedding rows, gains and
+ * biases from here.  New weights take a new ctx. */
 typedef struct {
     const void *embed, *lm_head, *final_norm;
     const void *const *ln1, *const *wqkv, *const *bqkv, *const *q_norm, *const *k_norm;
@@ -87,8 +89,11 @@ typedef struct {
 
 /* Creates a context on CUDA device `device` for batches of at most max_batch games per step
  * (1..256) and contexts of at most max_ctx tokens (RoPE table size).  Allocates the workspace
- * (activations, split-K pieces, attention partials; tens of MB) with cudaMalloc and builds the
- * RoPE table on the device in fp64.  The kernels are written for sm_100 (tcgen05, TMEM, TMA): on any
+ * (activations, split-K pieces, attention partials; tens of MB) with cudaMalloc, makes the fp16
+ * copies of all matrices (as many bytes again as the caller's weights, one allocation) and builds
+ * the RoPE table on the device in fp64.  Where the copies do not fit, a context with max_batch
+ * below 16 reads the caller's matrices instead, more slowly (appends in steps); with 16 games and
+ * more the call returns SPIRAL_ERR_OOM.  The kernels are written for sm_100 (tcgen05, TMEM, TMA): on any
  * other device the call returns SPIRAL_ERR_UNSUPPORTED -- there is no second code path.  Synchronous.
  * *out is written only on success. */
 int spiral_init(spiral_ctx **out, const spiral_model_desc *desc, const spiral_weights *weights,
@@ -145,10 +150,15 @@ int spiral_kv_load(spiral_ctx *ctx, spiral_kv *kv, int game_id, int layer, int n
  * [n][vocab] after each game's last appended token.  All pages needed are reserved up front:
  * SPIRAL_ERR_OOM / SPIRAL_ERR_INVALID leave every game unchanged.  This is the observation every game
  * receives between two turns of Algorithm 1 (the state carries the history).  A call with more than
- * max_batch new tokens in total, on an fp16 cache and a model whose matrices are on the tensor-core
- * path, runs as dense passes of up to 9472 token rows (256-token GEMM tiles, causal block attention);
- * the first such call allocates the passes' workspace (device synchronisation; SPIRAL_ERR_OOM if it
- * does not fit).  Otherwise the new tokens are pushed through the decode kernels in chunks of up to
+ * max_batch new tokens in total, or whose tokens would together read more than 200 MB of cached
+ * keys and values per layer, runs as dense passes of up to 12288 token rows (tensor-core GEMMs of
+ * up to 256 x 256 tiles, causal block attention), if the ctx holds copies of all layer matrices.
+ * Their workspace (about 90 KB per row at the Qwen3-4B shape) is allocated by the first such call
+ * and enlarged by calls with more tokens than any before (device synchronisation); where it does
+ * not fit, shorter passes are taken.  Queries and softmax weights enter the dense attention in one
+ * fp16 part, in two (high and low, as in the decode kernels) where the call has at most max_batch
+ * tokens or max_batch is below 16, and on bf16 pages.
+ * Otherwise the new tokens are pushed through the decode kernels in chunks of up to
  * max_batch (game, position) slots; several positions of one game may share a chunk (each attends
  * to positions up to its own only). */
 int spiral_prefill(spiral_ctx *ctx, spiral_kv *kv, int n, const int32_t *game_ids_host,

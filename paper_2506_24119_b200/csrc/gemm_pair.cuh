@@ -6,7 +6,7 @@
 // tcgen05.mma (M = 256) of the leader CTA reads both halves of both, and each CTA's tensor memory receives its 128
 // weight rows x N token columns.  What bounds a dense contraction here is shared memory: with a tile of 128 x 256 per
 // CTA every k step of 16 fills and reads 12 KB in the 128 cycles its MMA takes; with the token rows halved between the
-// CTAs of a pair 8 KB.  One CTA, seven warps:
+// CTAs of a pair 8 KB.  One CTA, six warps:
 //   warp 0      TMA producer of its CTA's half; both CTAs' copies are counted on the leader's "stage full" barriers
 //   warp 1      MMA issuer (leader CTA): four MMAs per k block; completion frees the stage in both CTAs (commit with
 //               multicast) and, at a tile's last block, releases the accumulator to both epilogues
@@ -355,9 +355,9 @@ inline double pg_block_us(int N) {
 // How a [rows][K] matrix meets T token rows: the token tile N and whole tiles or stream-K, whichever the estimate below
 // makes shorter.  Whole tiles cost their waves over the pairs; stream-K fills every pair but writes each piece and has it
 // read again (both at about 3 TB/s, from L2), and where the epilogue would have gated (`gated`) the gating becomes a
-// kernel of its own.  E.g. 331 rows: gate/up whole with N = 112 (4 waves of 76 x 3 tiles; 47 us against 47 + 18 for
-// stream-K and its gating kernel), QKV whole with N = 112 (72 tiles, 21 against 25 us), output and down projection
-// stream-K (21 and 29 against 25 and 41 us).
+// kernel of its own.  E.g. 331 rows of the Qwen3-4B matrices, all with N = 128 (estimates, us, whole against stream-K):
+// gate/up whole (4 waves of 76 x 3 tiles; 33 against 51 with the gating kernel that stream-K needs), QKV whole (72 tiles; 8
+// against 12), output and down projection stream-K (10 and 18 against 13 and 32).
 constexpr int PG_SPLIT_MAX_T = 1024;                 // bounds the pieces buffer
 constexpr int PG_SEARCH_MAX_T = 2048;                // beyond: many waves, and the widest tile moves the fewest bytes per flop
 enum { PG_OUT_PIECES = 0, PG_OUT_ADD = 1, PG_OUT_GATED = 2 };      // what a whole tile's epilogue writes

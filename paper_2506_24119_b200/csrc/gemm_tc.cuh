@@ -9,11 +9,11 @@
 //   warp 0      TMA producer: per k block a W tile [128 x 64] (one contiguous 16 KB run of the tile-major
 //               fp16 copy) and an X tile [N x 64], 128-byte swizzle; a ring stage holds `bps` k blocks
 //   warp 1 and  MMA issuers: four tcgen05.mma (K = 16) per k block, accumulators in TMEM (two buffers).
-//   the last    One thread issuing every MMA of the CTA is the bottleneck of the main loop (0.39 us per k
-//   warp        block, whatever the batch: instruction issue, not tensor-core time), so two threads in two
-//               warps take alternate ring stages, each adding into an accumulator of its own ("chain");
-//               the epilogue adds the two chains.  Batches above 128 leave no room in TMEM for four
-//               accumulators and run with one issuer.
+//   the last    Two warps take alternate ring stages, each adding into an accumulator of its own ("chain"); the
+//   warp        epilogue adds the two chains.  Batches above 128 leave no room in TMEM for four accumulators and
+//               run with one issuer.  Two because one, while its loop was a single lane's, was the bottleneck of
+//               the main loop (0.39 us per k block whatever the batch); now that whole warps walk the loops (see
+//               elect_one) that limit is mostly gone, and one issuer has not been measured again.
 //   warps 2..5  epilogue: tcgen05.ld of the finished accumulator, then either fp32 partial sums
 //               ("pieces") to memory -- transposed through shared memory, two 4 KB buffers per warp, and written
 //               by TMA stores, 32 batch rows x 32 features at a time -- or, for the LM head,

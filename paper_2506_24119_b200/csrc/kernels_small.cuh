@@ -384,9 +384,6 @@ __global__ void __maxnreg__(56) qkv_post_kernel(      // 56 registers: see QKV_P
     }
 }
 
-// The same for few rows (at most one task per half-warp of half the grid's warps): what a task needs besides the pieces
-// is fetched ahead of the dependency wait, which takes four round trips out of the chain (Qwen3-4B shape, 1 game 2478 ->
-// 2401 us per step; with two tasks per half-warp the registers it holds cost more: 213 games 5426 -> 5535).
 // What a task needs besides the projection's pieces: position, page, rotation (and, only brought near, the norm gains).
 // None of it comes from the kernel ahead: positions from the host, pages from the step's first kernel (see
 // rmsnorm_kernel), the rest is never written.
@@ -484,6 +481,9 @@ __device__ __forceinline__ void qkv_post_few_task(const QkvAhead<EPL>& pre, cons
     }
 }
 
+// The same for few rows (at most one task per half-warp of half the grid's warps): what a task needs besides the pieces
+// is fetched ahead of the dependency wait, which takes four round trips out of the chain (Qwen3-4B shape, 1 game 2478 ->
+// 2401 us per step; with two tasks per half-warp the registers it holds cost more: 213 games 5426 -> 5535).
 template <int HD>
 __global__ void __maxnreg__(56) qkv_post_few_kernel(      // 56 registers: see QKV_POST_THREADS
     Pieces pieces, const __nv_bfloat16* __restrict__ bias, const __nv_bfloat16* __restrict__ q_gain,
@@ -612,8 +612,8 @@ __device__ __forceinline__ int argmax_key_index(unsigned long long k) {
     return (int)(0xffffffffu - (uint32_t)(k & 0xffffffffull));
 }
 
-// token[b] = argmax_v( logits[b][v] / T + gumbel[b][v] ) from logits stored in memory (the path of
-// batches too small for the tensor cores); also hands the logits to the caller when asked.
+// token[b] = argmax_v( logits[b][v] / T + gumbel[b][v] ) from logits stored in memory: behind the CUDA-core LM head, which
+// contexts without fp16 copies of the weights and vocabularies below 128 take; also hands the logits to the caller.
 __global__ void __launch_bounds__(1024) gumbel_argmax_kernel(const float* __restrict__ logits,
                                                             const StepArgs* __restrict__ args, int vocab) {
     TRACE_BEGIN(5);

@@ -11,7 +11,7 @@
 //                         position) on tcgen05: scores and the output accumulator in tensor memory, one
 //                         softmax thread per query row, keys/values streamed page by page by TMA.
 //   attn_append_kernel    the same attention on mma.sync.m16n8k16, flash-style with the fp32 online softmax in
-//                         registers: bf16 pages (whose precision needs queries and weights in two parts), and an option.
+//                         registers: bf16 pages (queries and weights in two bf16 parts), and an option for fp16 pages.
 //   pf_rmsnorm_kernel, pf_qkv_post_kernel   the element-wise steps for thousands of token rows.
 //
 // Every wait is bounded as in the decode kernels.

@@ -66,10 +66,11 @@ namespace {
 inline size_t meta_args_offset(int max_batch) { return (((size_t)5 * max_batch + 2) * sizeof(int32_t) + 7) & ~(size_t)7; }
 constexpr int META_RING = 16;
 constexpr int MAX_PIECES = 4;
-// Batches below this use the CUDA-core GEMV for weights the context does not own (spiral_linear on a matrix of the
-// caller's): converting the matrix for one such call costs more than the call.  The model's own weights have their
-// fp16 copies from init and go through the tensor-core kernel at every batch size: it streams them at the memory's
-// pace whatever the batch (N is padded to 16), the GEMV at 2.7 TB/s with one row and less with more.
+// Batches below this use the CUDA-core GEMV for weights the context has no copy of (spiral_linear on a matrix of the
+// caller's: converting it for one such call costs more than the call; every matrix where the copies did not fit).  The
+// model's own weights otherwise have their fp16 copies from init and go through the tensor-core kernel at every batch size:
+// it streams them at the memory's pace whatever the batch (N is padded to 16), the GEMV at 2.7 TB/s with one row and less
+// with more.
 constexpr int TC_MIN_BATCH = 16;
 
 // per-kernel timing (spiral_profile): one record = a pair of events around one launch

@@ -126,8 +126,8 @@ def test_other_attention_kernels_of_the_append_still_available(monkeypatch, attn
 
 
 def test_step_shaped_append_still_available(monkeypatch):
-    """SPIRAL_PREFILL_DENSE=0 keeps the append on decode-shaped steps (the path of small batches
-    and bf16 caches): same result within the tolerances."""
+    """SPIRAL_PREFILL_DENSE=0 keeps the append on decode-shaped steps (the path of calls that one step holds
+    and of contexts without weight copies): same result within the tolerances."""
     monkeypatch.setenv("SPIRAL_PREFILL_DENSE", "0")
     desc = synth.shape("tiny_qknorm")
     pair = Pair(desc, max_batch=24, max_ctx=160, n_games=3)
