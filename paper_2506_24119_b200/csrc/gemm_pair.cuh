@@ -1,5 +1,5 @@
 // Dense GEMM of the context append on pairs of SMs (tcgen05 cta_group::2, sm_100a):
-//     Y[t][r] = sum_k X[t][k] * W[r][k]     X fp16 [T][K], W fp16 (the tile-major copy of gemm_tc.cuh), fp32 sums
+//     Y[t][r] = sum_k X[t][k] * W[r][k]     X fp16 [T][K], W fp16 (the k-block-major copy of gemm_tc.cuh), fp32 sums
 //
 // A cluster of two CTAs works on one output tile of 256 weight rows x N token rows (N <= 256, a multiple of 32): CTA r
 // of the pair holds weight rows 128 r .. + 127 and token rows (N / 2) r .. of the tile in its shared memory, one
@@ -104,12 +104,6 @@ __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
                  ::"r"(bar), "h"(both) : "memory");
 }
 // tiled load into this CTA's shared memory whose bytes are counted on a barrier of the leader CTA
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t leader_bar, uint64_t policy) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-        " [%0], [%1, {%2, %3}], [%4], %5;"
-        ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(leader_bar), "l"(policy) : "memory");
-}
 __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t leader_bar, uint64_t policy) {
     asm volatile(
         "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
@@ -180,11 +174,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
                 pg_tile_of(sg.tile, p, rt, tt);
                 // (a stage never crosses a segment: where one has an odd number of blocks, its last stage fetches a block
                 // that is not used)
-                const int y_w = ((2 * rt + (int)rank) * p.KB + kb) * TC_BM;
+                const int y_w = (2 * rt + (int)rank) * TC_BM;
                 const uint32_t dst = ring + (uint32_t)pre * stage_bytes;
                 if (elect_one()) {
                     if (rank == 0) mbar_expect_tx(full_own + 8u * (uint32_t)pre, 2u * stage_bytes);
-                    tma_load_2d_pair(dst, &tmW, 0, y_w, full_leader + 8u * (uint32_t)pre, pol_w);
+                    tma_load_3d_pair(dst, &tmW, 0, y_w, kb, full_leader + 8u * (uint32_t)pre, pol_w);
                 }
                 __syncwarp();
                 ++pre;
@@ -201,7 +195,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
         while (ok && sched.next(sg)) {
             int rt, tt;
             pg_tile_of(sg.tile, p, rt, tt);
-            const int y_x = tt * N + (int)rank * (N / 2), y_w0 = (2 * rt + (int)rank) * p.KB * TC_BM;
+            const int y_x = tt * N + (int)rank * (N / 2), y_w = (2 * rt + (int)rank) * TC_BM;
             for (int kb = sg.kb0; kb < sg.kb1; kb += BPS, ++st) {
                 const uint32_t dst = ring + s * stage_bytes, fb = full_leader + 8u * s;
                 const bool with_w = st >= pre;
@@ -209,7 +203,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
                 if (elect_one()) {
                     if (with_w) {
                         if (rank == 0) mbar_expect_tx(full_own + 8u * s, 2u * stage_bytes);
-                        tma_load_2d_pair(dst, &tmW, 0, y_w0 + kb * TC_BM, fb, pol_w);
+                        tma_load_3d_pair(dst, &tmW, 0, y_w, kb, fb, pol_w);
                     }
                     tma_load_3d_pair(dst + PG_BPS * TC_W_BYTES, &tmX, 0, y_x, kb, fb, pol_x);
                 }
@@ -433,15 +427,16 @@ inline size_t pg_piece_elems(int n_sm, int rows, int K, int cap, int out) {
     return most;
 }
 
-// a tensor of fp16 values as [outer][mid][64] with a box of box_outer x box_mid x 64, 128-byte swizzle
+// a tensor of fp16 values as [outer][mid][64] with a box of box_outer x box_mid x 64, 128-byte swizzle (none for the weight
+// copies, which are stored swizzled)
 inline int pg_encode(TcState& tc, CUtensorMap* m, const void* base, uint64_t mid, uint64_t mid_bytes, uint64_t outer, uint64_t outer_bytes,
-                     uint32_t box_mid, uint32_t box_outer) {
+                     uint32_t box_mid, uint32_t box_outer, bool swizzle = true) {
     cuuint64_t dims[3] = {(cuuint64_t)TC_BK, (cuuint64_t)mid, (cuuint64_t)outer};
     cuuint64_t strides[2] = {(cuuint64_t)mid_bytes, (cuuint64_t)outer_bytes};
     cuuint32_t box[3] = {(cuuint32_t)TC_BK, box_mid, box_outer};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = tc.encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         g_tc_error = "cuTensorMapEncodeTiled (pair operand) failed (" + std::to_string((int)r) + ")";
@@ -465,10 +460,14 @@ inline int pg_get_xmap(TcState& tc, const __half* X, int K, int T, int box_rows,
     *out = &it->second;
     return SPIRAL_OK;
 }
-// the tile-major weight copy as rows of 64 elements, a box of PG_BPS tiles (beyond the last tile: zeros)
+// the weight copy as [k block][row][64], a box of PG_BPS k blocks of a 128-row tile (beyond the last row or block: zeros)
+inline int tc_weight_map(TcState& tc, const TcWeight& w, CUtensorMap* map, int box_rows, int box_kb) {
+    const uint64_t slab = (uint64_t)((w.rows + TC_BM - 1) / TC_BM) * TC_BM;
+    return pg_encode(tc, map, w.w16, slab, 128, (uint64_t)((w.K + TC_BK - 1) / TC_BK), slab * 128, (uint32_t)box_rows, (uint32_t)box_kb, false);
+}
 inline int pg_get_wmap(TcState& tc, TcWeight& w, const CUtensorMap** out) {
     if (!w.has_map2) {
-        int rc = tc_encode(tc, &w.map2, w.w16, (uint64_t)TC_BK, (uint64_t)(tc_tiled_elems(w.rows, w.K) / TC_BK), PG_BPS * TC_BM);
+        int rc = tc_weight_map(tc, w, &w.map2, TC_BM, PG_BPS);
         if (rc) return rc;
         w.has_map2 = true;
     }

@@ -6,8 +6,8 @@
 // n <= ~200: the kernel is organised around keeping TMA loads in flight, not around the MMAs.
 //
 // One persistent CTA per SM, seven warps (eleven for the LM head):
-//   warp 0      TMA producer: per k block a W tile [128 x 64] (one contiguous 16 KB run of the tile-major
-//               fp16 copy) and an X tile [N x 64], 128-byte swizzle; a ring stage holds `bps` k blocks
+//   warp 0      TMA producer: per k block a W tile [128 x 64] (one contiguous 16 KB run of the
+//               k-block-major fp16 copy) and an X tile [N x 64], 128-byte swizzle; a ring stage holds `bps` k blocks
 //   warp 1 and  MMA issuers: four tcgen05.mma (K = 16) per k block, accumulators in TMEM (two buffers).
 //   the last    Two warps take alternate ring stages, each adding into an accumulator of its own ("chain"); the
 //   warp        epilogue adds the two chains.  Batches above 128 leave no room in TMEM for four accumulators and
@@ -201,18 +201,17 @@ struct TcSchedule {
     }
 };
 
-// A CTA's work as a sequence of k blocks, tile after tile.  In the tile-major weight copy block (tile, kb) sits at
-// row (tile KB + kb) 128 of the copy seen as rows of 64 elements (the TMA y coordinate).  A stream-K range starts
-// somewhere inside a tile and walks k upwards: consecutive rows of the copy.  CTAs that own whole tiles (LM head)
+// A CTA's work as a sequence of k blocks, tile after tile.  In the weight copy block (tile, kb) sits at row
+// (kb tiles + tile) 128 of the copy seen as rows of 64 elements (the TMA y coordinate).  CTAs that own whole tiles (LM head)
 // would all ask for the same activation block at the same time; each starts its tiles at a k block of its own
 // instead (kb0 = KB c / G) and wraps around: the order of a sum changes, who computes it does not.
 struct TcRun {
-    int y_tile, count, kb0;         // y of the first tile's k block 0, number of blocks, first k block
+    int y_tile, count, kb0;         // first row of the first tile, number of blocks, first k block
     int first_tile_blocks;          // blocks of the first tile in the run (KB for whole tiles)
     __device__ TcRun(int tiles, int KB, int whole, int c, int G) {
         const TcSchedule sc(tiles, KB, whole, c, G);
         const long long b0 = whole ? sc.u * KB : sc.u, b1 = whole ? sc.u1 * KB : sc.u1;
-        y_tile = (int)(b0 / KB) * KB * TC_BM;
+        y_tile = (int)(b0 / KB) * TC_BM;
         count = (int)(b1 - b0);
         kb0 = whole ? (int)((long long)KB * c / G) : (int)(b0 % KB);
         first_tile_blocks = whole ? KB : KB - kb0;
@@ -288,11 +287,12 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
         const uint32_t full0 = smem_u32(&full_bar[0]), done0 = smem_u32(&done_bar[0]);
         // Weights are written by nobody: the W tiles of the first ring-full of stages are requested
         // before the dependency wait, so that they stream in while the preceding kernel finishes.
+        const int slab = p.tiles * TC_BM;           // rows of the copy per k block
         int w_tile = run.y_tile, w_kb = run.kb0, w_in_tile = run.first_tile_blocks;     // next W block to request
         auto next_w_row = [&]() {
-            const int y = w_tile + w_kb * TC_BM;
+            const int y = w_tile + w_kb * slab;
             if (++w_kb == p.KB) w_kb = 0;
-            if (--w_in_tile == 0) { w_tile += p.KB * TC_BM; w_in_tile = p.KB; }
+            if (--w_in_tile == 0) { w_tile += TC_BM; w_in_tile = p.KB; }
             return y;
         };
         const int pre = n_stages < S ? n_stages : S;
@@ -681,10 +681,11 @@ __global__ void __maxnreg__(MODE == 1 ? 168 : 112) tc_gemm_kernel(const __grid_c
     if (threadIdx.x == 0) TC_STAMP(7);
 }
 
-// fp16 re-encoding of bf16 weights times `scale`, a power of two, written TILE-MAJOR: the [128 rows x 64 k]
-// tile (row tile t, k block kb) occupies the 16 KB starting at element ((t * KB + kb) * 128) * 64,
-// rows of 128 bytes, zero-padded at the ragged edges.  One TMA box is then one contiguous 16 KB run
-// of DRAM instead of 128 separate 128-byte row segments.
+// fp16 re-encoding of bf16 weights times `scale`, a power of two, written K-BLOCK-MAJOR: a slab of all rows (padded to a
+// multiple of 128) per 64-wide k block, rows of 128 bytes, zero-padded at the ragged edges.  Any rows of a k block, a tile of
+// 128 or the few that a CTA of step_few.cuh owns, are one contiguous run of DRAM instead of separate 128-byte segments.
+// The 16-byte chunk ch of row r sits at ch ^ (r & 7), the arrangement that the 128-byte swizzle would give it in shared
+// memory: rows arrive as the matrix instructions want them wherever a box starts.
 // bf16 has three bits less than fp16, so w * scale is exact for magnitudes in [2^-14, 65504]; smaller ones round to fp16
 // subnormals / zero, an absolute error below 2^-25.  `lossy` (when given) is set where that loses, anywhere, more than
 // 2^-21 of the absolute sum of 64 weights of a row -- far below what an fp32 sum of thousands of products rounds, far above
@@ -695,12 +696,9 @@ __global__ void bf16_to_f16_tiled_kernel(const __nv_bfloat16* __restrict__ src, 
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;       // one 8-element (16-byte) chunk of dst
     if (i >= n_chunks) return;                       // (n_chunks is a multiple of 1024: whole CTAs)
     const int kc = (int)(i & 7);                     // chunk within the 64-wide row
-    const size_t rowi = i >> 3;                      // row of the tiled array
-    const int rr = (int)(rowi & 127);
-    const size_t tk = rowi >> 7;                     // t * KB + kb
-    const int kb = (int)(tk % KB);
-    const size_t t = tk / KB;
-    const size_t r = t * TC_BM + rr;
+    const size_t rowi = i >> 3, slab = n_chunks / 8 / KB;       // row of the copy; rows per k block
+    const int kb = (int)(rowi / slab);
+    const size_t r = rowi - kb * slab;
     const int k0 = kb * TC_BK + kc * 8;
     uint4 o = make_uint4(0u, 0u, 0u, 0u);
     float err = 0.f, sum = 0.f;
@@ -720,7 +718,7 @@ __global__ void bf16_to_f16_tiled_kernel(const __nv_bfloat16* __restrict__ src, 
         }
         o = make_uint4(out[0], out[1], out[2], out[3]);
     }
-    *reinterpret_cast<uint4*>(dst + i * 8) = o;
+    *reinterpret_cast<uint4*>(dst + ((i & ~(size_t)7) | (size_t)(kc ^ (int)(r & 7))) * 8) = o;
     if (lossy) {
 #pragma unroll
         for (int d = 1; d < 8; d <<= 1) {            // the eight chunks of a row's 64 weights sit in neighbouring lanes
@@ -753,7 +751,7 @@ __global__ void __launch_bounds__(256) bf16_max_kernel(const __nv_bfloat16* __re
 // ------------------------------------------------------------------------------------------------
 struct TcWeight {
     __half* w16 = nullptr;
-    CUtensorMap map, map2;      // boxes of one 128 x 64 tile / of two (append path, made at its first use)
+    CUtensorMap map, map2;      // boxes of one 128 x 64 tile / of two k blocks of one (append path, made at its first use)
     bool has_map2 = false;
     int rows = 0, K = 0;
     float unscale = 1.f;        // w16 holds the weights divided by this
@@ -860,15 +858,16 @@ inline bool tc_resident(const TcState& tc, const __nv_bfloat16* W, int rows, int
     return it != tc.weights.end() && it->second.resident && it->second.rows == rows && it->second.K == K;
 }
 
-// 2-d tensor map [outer][inner] of 2-byte floats with a [box_outer][64] box and 128-byte swizzle
+// 2-d tensor map [outer][inner] of 2-byte floats with a [box_outer][64] box and 128-byte swizzle (none for the weight
+// copies, which are stored swizzled)
 inline int tc_encode(TcState& tc, CUtensorMap* map, const void* base, uint64_t inner, uint64_t outer, uint32_t box_outer,
-                     bool bf16 = false) {
+                     bool bf16 = false, bool swizzle = true) {
     cuuint64_t dims[2] = {inner, outer};
     cuuint64_t strides[1] = {inner * 2};
     cuuint32_t box[2] = {(cuuint32_t)TC_BK, box_outer};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = tc.encode(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         g_tc_error = "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")";
@@ -951,8 +950,8 @@ inline int tc_register_weight(TcState& tc, const __nv_bfloat16* W, int rows, int
             g_tc_error = "fp16 weight copy: " + std::string(cudaGetErrorString(e));
             return e == cudaErrorMemoryAllocation ? SPIRAL_ERR_OOM : SPIRAL_ERR_CUDA;
         }
-        // tile-major copy seen as rows of 64 elements: tile (t, kb) = rows (t * KB + kb) * 128 ...
-        int rc = tc_encode(tc, &w.map, w.w16, (uint64_t)TC_BK, (uint64_t)(tc_tiled_elems(rows, K) / TC_BK), TC_BM);
+        // the copy seen as rows of 64 elements: tile (t, kb) = rows (kb * tiles + t) * 128 ...
+        int rc = tc_encode(tc, &w.map, w.w16, (uint64_t)TC_BK, (uint64_t)(tc_tiled_elems(rows, K) / TC_BK), TC_BM, false, false);
         if (rc) { if (w.owned) cudaFree(w.w16); return rc; }
         if (resident) {
             rc = tc_convert(W, w.w16, rows, K, st, launches, 1.f, lossy);
