@@ -23,6 +23,7 @@
 #include "read_ceiling.cuh"
 #include "gemm_tc.cuh"
 #include "prefill.cuh"
+#include "step_few.cuh"
 
 using namespace spiral;
 typedef __nv_bfloat16 bf16;
@@ -144,6 +145,14 @@ struct spiral_ctx {
     std::vector<cudaEvent_t> prof_pool;   // events ready for reuse
     TcState tc;
     PrefillWs pf;
+    // one-kernel step for few games (step_few.cuh)
+    bool few_ready = false;
+    FsMat few_mat[4];
+    uint8_t* few_mem = nullptr;        // layer table, then what the pointers below point to
+    float* few_ss = nullptr;           // parts of the sums of squares
+    __half *few_xn = nullptr, *few_heads = nullptr, *few_act = nullptr;    // activations (zeros behind the last element of a row)
+    unsigned int* few_bar = nullptr;
+    int few_smem = 0, few_red = 0, few_slot = 0;       // dynamic shared memory a CTA can have, see few_setup
     int prefill_chunk = PREFILL_CHUNK_DEFAULT;    // token rows per pass of the dense append path (SPIRAL_PREFILL_CHUNK)
     bool prefill_dense = true;                    // SPIRAL_PREFILL_DENSE=0: always append through decode-shaped steps
     bool pf_ready = false;                        // every layer matrix is registered for the tensor-core path
@@ -210,7 +219,7 @@ static void free_ctx(spiral_ctx* c) {
     cudaFree(c->x); cudaFree(c->h); cudaFree(c->attn_out); cudaFree(c->act); cudaFree(c->q);
     cudaFree(c->pieces); cudaFree(c->o_part); cudaFree(c->m_part); cudaFree(c->l_part);
     cudaFree(c->attn_item_cnt); cudaFree(c->logits); cudaFree(c->cos_tab); cudaFree(c->sin_tab); cudaFree(c->meta_dev);
-    cudaFree(c->tok_stage); cudaFree(c->gumbel_stage); cudaFree(c->tokout_stage); cudaFree(c->status); cudaFree(c->lossy);
+    cudaFree(c->tok_stage); cudaFree(c->gumbel_stage); cudaFree(c->tokout_stage); cudaFree(c->status); cudaFree(c->lossy); cudaFree(c->few_mem);
     if (c->meta_host) cudaFreeHost(c->meta_host);
     if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
     if (c->copy_ev) cudaEventDestroy(c->copy_ev);
@@ -225,6 +234,78 @@ static void free_ctx(spiral_ctx* c) {
     if (c->pf.ev) cudaEventDestroy(c->pf.ev);
     tc_destroy(c->tc);
     delete c;
+}
+
+typedef void (*FewKernel)(const CUtensorMap, const FsParams);
+static FewKernel few_kernel(int head_dim, bool f16) {
+    return head_dim == 128 ? (f16 ? few_step_kernel<128, true> : few_step_kernel<128, false>)
+                           : (f16 ? few_step_kernel<64, true> : few_step_kernel<64, false>);
+}
+
+// Prepares the one-kernel step for few games where the model and the device allow it; elsewhere the step stays a kernel
+// per operation.  All layer matrices have their fp16 copies when this is called.
+static int few_setup(spiral_ctx* c) {
+    const spiral_model_desc& d = c->d;
+    const int L = d.n_layers, qd = d.n_q_heads * d.head_dim, G = c->n_sm;
+    int smem_max = 0;
+    CU_TRY(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+    c->few_smem = smem_max;
+    for (bool f16 : {true, false}) {
+        cudaFuncAttributes a;
+        FewKernel k = few_kernel(d.head_dim, f16);
+        CU_TRY(cudaFuncGetAttributes(&a, k));
+        c->few_smem = std::min(c->few_smem, smem_max - (int)a.sharedSizeBytes);
+        CU_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max - (int)a.sharedSizeBytes));
+    }
+    // shared memory: alignment, the warps' sums (or the attention's partial outputs and queries), the residual columns; the rest is the ring
+    const int cols = (d.d_model + G - 1) / G;
+    c->few_red = std::max(FS_WARPS * 8 * (16 * FS_MT + 4), 2 * FS_WARPS * c->group * d.head_dim) * (int)sizeof(float);
+    c->few_slot = (c->few_smem - 1024 - c->few_red - FS_MAX_GAMES * cols * (int)sizeof(float)) / FS_SLOTS & ~1023;
+    const bool fits = fs_plan(c->few_mat[FS_QKV], c->qkv_rows, d.d_model, 1, G, c->few_slot) && fs_plan(c->few_mat[FS_O], d.d_model, qd, 1, G, c->few_slot) &&
+                      fs_plan(c->few_mat[FS_GU], 2 * d.d_ff, d.d_model, 2, G, c->few_slot) && fs_plan(c->few_mat[FS_DOWN], d.d_model, d.d_ff, 1, G, c->few_slot) &&
+                      cols <= FS_COLS && c->few_mat[FS_O].groups == 1 && c->few_mat[FS_DOWN].groups == 1 && c->few_slot >= 64 * d.head_dim;
+    // rows of activations hold whole stages; the two matrices behind a norm read the same rows
+    for (FsMat& m : c->few_mat) m.ldx = m.stages * m.m * TC_BK;
+    c->few_mat[FS_QKV].ldx = c->few_mat[FS_GU].ldx = std::max(c->few_mat[FS_QKV].ldx, c->few_mat[FS_GU].ldx);
+    int coop = 0;
+    CU_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device));
+    if (!fits || !coop) return SPIRAL_OK;
+    std::vector<FsLayer> layers(L);
+    for (int l = 0; l < L; ++l) {
+        const bf16* w[4] = {c->wqkv[l], c->wo[l], c->w_gate_up[l], c->w_down[l]};
+        for (int k = 0; k < 4; ++k) {
+            auto it = c->tc.weights.find(w[k]);
+            if (it == c->tc.weights.end() || !it->second.resident || it->second.rows != c->few_mat[k].rows || it->second.K != c->few_mat[k].K) return SPIRAL_OK;
+            const int rc = tc_weight_map(c->tc, it->second, &layers[l].w[k], c->few_mat[k].h, c->few_mat[k].m);
+            if (rc) { g_cuda_error = tc_last_error(); return rc; }
+            layers[l].v.unscale[k] = it->second.unscale;
+        }
+        layers[l].v.vec[FS_QKV] = c->bqkv[l]; layers[l].v.vec[FS_O] = c->ln2[l]; layers[l].v.vec[FS_GU] = nullptr;
+        layers[l].v.vec[FS_DOWN] = l + 1 < L ? c->ln1[l + 1] : c->final_norm;
+        layers[l].v.w[0] = c->tc.weights.find(w[FS_QKV])->second.w16; layers[l].v.w[1] = c->tc.weights.find(w[FS_GU])->second.w16;
+        layers[l].v.qk_norm[0] = c->q_norm[l]; layers[l].v.qk_norm[1] = c->k_norm[l];
+    }
+    auto padded = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };
+    const size_t table = padded((size_t)L * sizeof(FsLayer)), ss = padded((size_t)FS_MAX_GAMES * G * sizeof(float));
+    size_t act[3];                     // activations: behind the norms, heads, gated
+    for (int k = 0; k < 3; ++k) act[k] = padded((size_t)FS_MAX_GAMES * c->few_mat[k == 0 ? FS_QKV : k == 1 ? FS_O : FS_DOWN].ldx * sizeof(__half));
+    const size_t all = table + ss + 256 + act[0] + act[1] + act[2];
+    cudaError_t e = cudaMalloc((void**)&c->few_mem, all);
+    if (e == cudaErrorMemoryAllocation) { cudaGetLastError(); c->few_mem = nullptr; return SPIRAL_OK; }
+    if (e == cudaSuccess) e = cudaMemcpy(c->few_mem, layers.data(), (size_t)L * sizeof(FsLayer), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(c->few_mem + table, 0, all - table);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) {
+        g_cuda_error = std::string("one-kernel step: ") + cudaGetErrorString(e);
+        return SPIRAL_ERR_CUDA;
+    }
+    c->few_ss = (float*)(c->few_mem + table);
+    c->few_bar = (unsigned int*)(c->few_mem + table + ss);
+    c->few_xn = (__half*)(c->few_mem + table + ss + 256);
+    c->few_heads = (__half*)((uint8_t*)c->few_xn + act[0]);
+    c->few_act = (__half*)((uint8_t*)c->few_heads + act[1]);
+    c->few_ready = true;
+    return SPIRAL_OK;
 }
 
 extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const spiral_weights* w, int device,
@@ -442,6 +523,7 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
             }
         }
     }
+    if (c->pf_ready && (rc = few_setup(c)) != SPIRAL_OK) { free_ctx(c); return rc; }
     e = cudaMalloc((void**)&c->pieces, c->pieces_elems * sizeof(float));
     if (e != cudaSuccess) {
         g_cuda_error = std::string("pieces buffer: ") + cudaGetErrorString(e);
@@ -781,6 +863,54 @@ static int meta_upload(spiral_ctx* c, int slot, cudaStream_t st) {
     return SPIRAL_OK;
 }
 
+// All layers of a decode step for few games as one kernel.  SPIRAL_ERR_UNSUPPORTED: not possible here, nothing was launched.
+static int launch_few(spiral_ctx* c, spiral_kv* kv, int n, cudaStream_t st) {
+    const spiral_model_desc& d = c->d;
+    int32_t* mi = meta_i32(c);
+    const int MB = c->max_batch, cols = (d.d_model + c->n_sm - 1) / c->n_sm;
+    FsParams p{};
+    p.layers = (const FsLayer*)c->few_mem; p.n_layers = d.n_layers; p.n = n;
+    for (int k = 0; k < 4; ++k) p.mat[k] = c->few_mat[k];
+    p.d_model = d.d_model; p.d_ff = d.d_ff; p.vocab = d.vocab; p.eps = (float)d.rms_eps; p.inv_d = 1.f / d.d_model;
+    p.embed = c->embed; p.first_norm = c->ln1[0]; p.qk_norm = d.qk_norm != 0; p.args = meta_args(c);
+    p.meta = StepMeta{mi, mi + MB, mi + 2 * MB, mi + 3 * MB};
+    p.block_table = kv->table_dev; p.cos_tab = c->cos_tab; p.sin_tab = c->sin_tab; p.pool = kv->pool;
+    AttnParams& a = p.at;
+    a.block_table = kv->table_dev; a.game = mi; a.ctx_len = mi + MB; a.cum = meta_cum_dev(c);
+    a.n = n; a.max_pages = kv->max_pages; a.n_pages = kv->n_pages;
+    a.n_q_heads = d.n_q_heads; a.n_kv_heads = d.n_kv_heads; a.group = c->group;
+    a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)d.head_dim));
+    a.o_part = c->o_part; a.m_part = c->m_part; a.l_part = c->l_part; a.item_cnt = c->attn_item_cnt;
+    a.status = c->status;
+    p.qkv = c->pieces; p.xn = c->few_xn; p.heads = c->few_heads; p.act = c->few_act; p.h = c->h;
+    p.ss_part = c->few_ss; p.bar = c->few_bar;
+    p.slot_bytes = c->few_slot; p.red_bytes = c->few_red;
+    const FewKernel kernel = few_kernel(d.head_dim, kv->kv_f16 != 0);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c->n_sm);
+    cfg.blockDim = dim3(FS_THREADS);
+    cfg.dynamicSmemBytes = (size_t)(1024 + p.red_bytes + n * cols * (int)sizeof(float) + FS_SLOTS * p.slot_bytes);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;       // its CTAs wait for one another
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, kv->pool_map, p);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {     // not all SMs are ours (a partitioned device)
+        cudaGetLastError();
+        c->few_ready = false;
+        return SPIRAL_ERR_UNSUPPORTED;
+    }
+    if (e != cudaSuccess) {
+        g_cuda_error = std::string("launch of few_step_kernel: ") + cudaGetErrorString(e);
+        cudaGetLastError();
+        return SPIRAL_ERR_CUDA;
+    }
+    c->launches++;
+    return SPIRAL_OK;
+}
+
 // All layers for n batch slots whose metadata is already in ctx->meta_dev.
 // `one_per_game`: no game has two of the slots, so only its last page changes during the step.
 static int run_layers(spiral_ctx* c, spiral_kv* kv, int n, bool one_per_game, cudaStream_t st) {
@@ -790,6 +920,10 @@ static int run_layers(spiral_ctx* c, spiral_kv* kv, int n, bool one_per_game, cu
     StepMeta meta{mi, mi + MB, mi + 2 * MB, mi + 3 * MB};
     const int qd = d.n_q_heads * d.head_dim;
     const float eps = (float)d.rms_eps;
+    if (one_per_game && c->few_ready && n <= FS_MAX_GAMES && c->prof_mask == 0) {
+        const int rc = launch_few(c, kv, n, st);
+        if (rc != SPIRAL_ERR_UNSUPPORTED) return rc;
+    }
     LAUNCH(c, embed_kernel, n, 256, 0, st, c->embed, meta_args(c), meta, kv->table_dev, kv->max_pages, kv->page_size,
            d.d_model, d.vocab, c->x, c->status);
     // persistent element-wise kernels: one CTA per SM, fewer when the batch is tiny
@@ -1936,6 +2070,7 @@ extern "C" int spiral_last_status(spiral_ctx* ctx, int32_t* detail) {
     CU_TRY(cudaMemset(ctx->attn_item_cnt, 0, (size_t)ctx->max_batch * ctx->d.n_kv_heads * sizeof(int)));
     if (ctx->tc.best) CU_TRY(cudaMemset(ctx->tc.best, 0, 256 * sizeof(unsigned long long)));
     if (ctx->tc.done) CU_TRY(cudaMemset(ctx->tc.done, 0, sizeof(unsigned int)));
+    if (ctx->few_bar) CU_TRY(cudaMemset(ctx->few_bar, 0, 2 * sizeof(unsigned int)));
     return s >= STATUS_TIMEOUT_TMA ? SPIRAL_ERR_TIMEOUT : SPIRAL_ERR_DEVICE_CHECK;
 }
 
