@@ -494,11 +494,21 @@ __device__ __forceinline__ void fs_norms(const FsParams& p, FsShared* sh) {
 #pragma unroll
     for (int e = 0; e < FS_MAX_GAMES; ++e) v[e] = 0.f;
     const float4* src = reinterpret_cast<const float4*>(p.ss_part);
-#pragma unroll 5
-    for (int i = lane; i < G; i += 32) {           // (games beyond the last: zeros)
-        const float4 a = __ldcg(src + 2 * i), b = p.n > 4 ? __ldcg(src + 2 * i + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
-        v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
-        v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int i0 = lane; i0 - lane < G; i0 += 5 * 32) {     // (five CTAs' sums per lane in flight; games beyond the last: zeros)
+        float4 a[5], b[5];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            const int i = i0 + 32 * k;
+            a[k] = i < G ? __ldcg(src + 2 * i) : none;
+            b[k] = i < G && p.n > 4 ? __ldcg(src + 2 * i + 1) : none;
+        }
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            v[0] += a[k].x; v[1] += a[k].y; v[2] += a[k].z; v[3] += a[k].w;
+            v[4] += b[k].x; v[5] += b[k].y; v[6] += b[k].z; v[7] += b[k].w;
+        }
     }
     // eight sums over 32 lanes: halves are exchanged, lane l ends up with game l & 7
 #pragma unroll
