@@ -523,7 +523,6 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
             }
         }
     }
-    if (c->pf_ready && (rc = few_setup(c)) != SPIRAL_OK) { free_ctx(c); return rc; }
     e = cudaMalloc((void**)&c->pieces, c->pieces_elems * sizeof(float));
     if (e != cudaSuccess) {
         g_cuda_error = std::string("pieces buffer: ") + cudaGetErrorString(e);
@@ -531,6 +530,7 @@ extern "C" int spiral_init(spiral_ctx** out, const spiral_model_desc* d, const s
         free_ctx(c);
         return e == cudaErrorMemoryAllocation ? SPIRAL_ERR_OOM : SPIRAL_ERR_CUDA;
     }
+    if (c->pf_ready && (rc = few_setup(c)) != SPIRAL_OK) { free_ctx(c); return rc; }
     *out = c;
     return SPIRAL_OK;
 }

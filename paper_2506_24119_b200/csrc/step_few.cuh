@@ -36,8 +36,9 @@
 //
 // The products use mma.sync.m16n8k16 (weight rows are the M side, games the N side): 18 to 132 rows per CTA do not fill a
 // tcgen05 tile, whose activations would have to pass through shared memory as well, and at eight games the legacy pipe needs a
-// fraction of the time the weights need to arrive.  Activations go from L2 straight into registers, four 64-wide k blocks
-// ahead of their use (eight: 2088 -> 2285 us, the moves cost more than the latency); they are stored in an order (fs_perm) in
+// fraction of the time the weights need to arrive.  Activations go from L2 straight into registers, three 64-wide k blocks
+// ahead of their use (us per step, Qwen3-4B shape with 1 and 4 games, Llama-3.1-8B shape with 2: two blocks 2035, 2202, 2937;
+// three 1981, 2187, 2923; four 1966, 2222, 3000; eight 8 % more than four: moves cost more than latency); they are stored in an order (fs_perm) in
 // which one 16-byte load is two B fragments.
 //
 // CTAs wait for one another, so the launch is cooperative.  Every wait is bounded: after a timeout the CTA records a status
@@ -57,10 +58,10 @@ namespace spiral {
 
 constexpr int FS_WARPS = 8;                        // consumer warps
 // A third warpgroup carries the producer and the norms: with nine warps a thread could have 168 registers (three warps on one
-// of the four schedulers), with twelve the two consumer warpgroups take over what the third does not need: 256 x 216 +
-// 128 x 72 registers are the 384 x 168 of the launch.
+// of the four schedulers), with twelve the two consumer warpgroups take over what the third does not need: 256 x 224 +
+// 128 x 56 registers are the 384 x 168 of the launch.
 constexpr int FS_THREADS = 32 * (FS_WARPS + 4);
-constexpr int FS_REG_CONSUMER = 216, FS_REG_PRODUCER = 72;
+constexpr int FS_REG_CONSUMER = 224, FS_REG_PRODUCER = 56;
 constexpr int FS_MAX_GAMES = 8;
 // Slots of the ring, two per consumer warp: stage q of the step lies in slot q % 16 and is taken by warp q % 8, always.  (A
 // warp may wait for a parity of a barrier only if it has seen every earlier phase of it complete.)
@@ -336,7 +337,7 @@ struct FsGrid {
 // The products of one matrix.  prefetch() asks for the first activations, run() multiplies.  Games beyond the last are read
 // as the last one; their sums are not used.
 struct FsGemm {
-    static constexpr int P = 4;                    // k blocks of activations in flight
+    static constexpr int P = 3;                    // k blocks of activations in flight
     const FsMat& M;
     const int2* rows;                              // [groups]
     int vw, q;                                     // this warp counted from the one with the phase's first stage; its first stage
