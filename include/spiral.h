@@ -356,7 +356,8 @@ int spiral_attention_static_status(int device, int32_t *detail_out);
 /* spiral_profile: from now on every launch of a class whose bit is set in class_mask is bracketed
  * by two CUDA events on the launch stream (0 switches timing off); earlier records are dropped.
  * Synchronises the device.  The events sit between kernels, so a timed run is slightly slower than
- * an untimed one: time whole steps with the mask at 0.
+ * an untimed one: time whole steps with the mask at 0.  (A decode step of up to eight games is one kernel for
+ * all layers while the mask is 0, and a kernel per operation otherwise.)
  * spiral_profile_read: synchronises, then returns the summed device time in milliseconds and the
  * number of launches recorded for one class since the last spiral_profile. */
 int spiral_profile(spiral_ctx *ctx, uint32_t class_mask);

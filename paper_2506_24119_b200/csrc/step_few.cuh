@@ -13,7 +13,7 @@
 //
 // us per step, kernel per operation -> this kernel (contexts of 200 to 1000 tokens): Qwen3-4B shape, 1 game 2313 -> 1951, 2
 // games 2351 -> 2082, 4 games 2394 -> 2229, 8 games 2480 -> 2415; Llama-3.1-8B shape 3198 -> 2904, 3212 -> 2988, 3267 -> 3152,
-// 3325 -> 3280; two layers of 256 columns, 4 games 75.6 -> 62.6.  Of a layer's 52 us with one game the memory is idle for
+// 3325 -> 3280; two layers of 256 columns, 4 games 73.5 -> 51.8.  Of a layer's 52 us with one game the memory is idle for
 // about 14: the attention's chain (queries from L2, first page, partial results of several CTAs) is longer than the ring.
 // Beyond eight games the attention and the activations' trips through every CTA outgrow what the boundaries cost.
 //
@@ -62,7 +62,7 @@ constexpr int FS_WARPS = 8;                        // consumer warps
 // 128 x 56 registers are the 384 x 168 of the launch.
 constexpr int FS_THREADS = 32 * (FS_WARPS + 4);
 constexpr int FS_REG_CONSUMER = 224, FS_REG_PRODUCER = 56;
-constexpr int FS_MAX_GAMES = 8;
+constexpr int FS_MAX_GAMES = 8;                    // one 8-column tile of the products; figures on both sides of this line: above
 // Slots of the ring, two per consumer warp: stage q of the step lies in slot q % 16 and is taken by warp q % 8, always.  (A
 // warp may wait for a parity of a barrier only if it has seen every earlier phase of it complete.)
 constexpr int FS_SLOTS = 2 * FS_WARPS;
