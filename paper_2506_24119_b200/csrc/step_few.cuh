@@ -11,11 +11,13 @@
 //   warp 10     norms.
 //   warps 0..7  consumers: products, attention, element-wise work.
 //
-// us per step, kernel per operation -> this kernel (contexts of 200 to 1000 tokens): Qwen3-4B shape, 1 game 2313 -> 1951, 2
-// games 2351 -> 2082, 4 games 2394 -> 2229, 8 games 2480 -> 2415; Llama-3.1-8B shape 3198 -> 2904, 3212 -> 2988, 3267 -> 3152,
-// 3325 -> 3280; two layers of 256 columns, 4 games 73.5 -> 51.8.  Of a layer's 52 us with one game the memory is idle for
-// about 14: the attention's chain (queries from L2, first page, partial results of several CTAs) is longer than the ring.
-// Beyond eight games the attention and the activations' trips through every CTA outgrow what the boundaries cost.
+// us per step, kernel per operation -> this kernel (contexts of 200 to 1000 tokens): Qwen3-4B shape, 1 game 2297 -> 1940, 2
+// games 2331 -> 2009, 4 games 2398 -> 2189, 8 games 2471 -> 2342 (contexts to 5000: 2970 -> 2851); Llama-3.1-8B shape 3177 ->
+// 2862, 3205 -> 2894, 3261 -> 3119, 3349 -> 3213 (3781 -> 3725); two layers of 256 columns, 4 games 74 -> 56.  Of a layer's 52 us
+// with one game the memory is idle for about a fifth: the attention's chain (queries from L2, first page, partial results of
+// several CTAs) is longer than what the ring holds.  Nine and more games, as two tiles of the products, were slower here than
+// as kernels (11 games 3757 against 2254): every CTA reads all activations of a phase, and a stage of the attention costs the
+// same however many there are.
 //
 // A CTA owns whole rows of every matrix (rows c R / G .. (c + 1) R / G), so no partial sum leaves it: the eight warps
 // split the k blocks (and, where a CTA has more than 80 rows, the rows), and add up in shared memory.  What a phase passes
@@ -62,7 +64,7 @@ constexpr int FS_WARPS = 8;                        // consumer warps
 // 128 x 56 registers are the 384 x 168 of the launch.
 constexpr int FS_THREADS = 32 * (FS_WARPS + 4);
 constexpr int FS_REG_CONSUMER = 224, FS_REG_PRODUCER = 56;
-constexpr int FS_MAX_GAMES = 8;                    // one 8-column tile of the products; figures on both sides of this line: above
+constexpr int FS_MAX_GAMES = 8;                    // one 8-column tile of the products (figures above)
 // Slots of the ring, two per consumer warp: stage q of the step lies in slot q % 16 and is taken by warp q % 8, always.  (A
 // warp may wait for a parity of a barrier only if it has seen every earlier phase of it complete.)
 constexpr int FS_SLOTS = 2 * FS_WARPS;
